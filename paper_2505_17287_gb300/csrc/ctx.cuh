@@ -5,6 +5,9 @@
 
 namespace ibm {
 
+// multigrid coarsening stops at this many cells
+constexpr int COARSE_STOP = 64;
+
 // device control block of the Poisson guess history (solver.cu): pairs in
 // the ring, next slot, Gram matrix of the stored right-hand sides, this
 // step's dots and coefficients, and the FLUID mean of its right-hand side
@@ -43,6 +46,11 @@ struct MGHier {
     // per-level table of the persistent V-cycle tail (TailLv<T>[levels],
     // device memory), null below three levels
     void *tail = nullptr;
+    // solution operator of the coarsest level (n x n), and the multigrid
+    // generation and sweep count it was formed for
+    void *cm = nullptr;
+    uint64_t cm_gen = 0;
+    int cm_sweeps = 0;
     bool built = false;
     // the V-cycle z = M^{-1} r (pr -> an output buffer) captured as CUDA
     // graphs, one per output buffer (pz, or a Krylov vector written in
@@ -228,6 +236,7 @@ struct Ctx {
     int nred = RED_BLOCKS;
     int nred_wide = RED_BLOCKS;
     unsigned nelem = 152 * 16;
+    int bot_ctas = 0;      // largest cluster of the V-cycle bottom on this device (0: not asked yet)
     uint64_t mg_gen = 0;   // multigrid rebuild counter (invalidates captured V-cycles)
 
     ibm_status fail(ibm_status code, const std::string &m) {
@@ -247,6 +256,7 @@ ibm_status kt_flush(Ctx *c);
 
 // solver.cu
 ibm_status mg_build(Ctx *c);
+ibm_status mg_coarse_ready(Ctx *c);   // coarsest solution operators for the options in force
 // Poisson guess history (solver.cu): storage, reset, the projection guess
 // for a right-hand side (after the extrapolated guess is in phi), and the
 // pair of a finished solve

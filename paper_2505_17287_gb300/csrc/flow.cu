@@ -1387,6 +1387,7 @@ static void swap_nold(Ctx *c) {
 ibm_status flow_step_graph(Ctx *c) {
     int slot = 0;
     IBM_TRY(graph_for_state(c, &slot));
+    IBM_TRY(mg_coarse_ready(c));
     IBM_CUDA(c, cudaGraphLaunch(c->sgraph[slot], c->s));
     swap_nold(c);
     c->have_nold = true;

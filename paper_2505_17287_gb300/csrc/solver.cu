@@ -1562,86 +1562,130 @@ __global__ void __launch_bounds__(256)
 // preconditioner (which would swamp FP32 corrections).
 constexpr int COARSE_MAX = 512;
 
-template <typename T>
-__device__ __forceinline__ T block_mean_active(T v, bool act, T *red, int *cnt) {
-    // plain shared-memory tree sum over COARSE_MAX slots (threads beyond
-    // COARSE_MAX only take part in the barriers)
-    const int c = threadIdx.x;
-    if (c < COARSE_MAX) {
-        red[c] = act ? v : T(0);
-        cnt[c] = act ? 1 : 0;
-    }
-    __syncthreads();
-    for (int o = COARSE_MAX / 2; o > 0; o >>= 1) {
-        if (c < o) {
-            red[c] += red[c + o];
-            cnt[c] += cnt[c + o];
-        }
-        __syncthreads();
-    }
-    const T m = cnt[0] > 0 ? red[0] / T(cnt[0]) : T(0);
-    __syncthreads();
-    return m;
-}
-
+// Shared memory of the solve: x with zero padding of half the largest level
+// on either side (a neighbour offset is at most n / 2), and the partial sums.
+constexpr int COARSE_PAD = COARSE_MAX / 2;
 template <typename T>
 struct CoarseSmem {
-    T sx[COARSE_MAX], sf[COARSE_MAX], stx[COARSE_MAX], sty[COARSE_MAX], stz[COARSE_MAX], sdi[COARSE_MAX],
-        red[COARSE_MAX];
-    int cnt[COARSE_MAX];
+    T sx[COARSE_MAX + 2 * COARSE_PAD];
+    T red[COARSE_MAX / 32];
+    int cnt[COARSE_MAX / 32];
 };
 
-// the coarsest-level solve by the threads of one block (at least COARSE_MAX)
+// mean over the active cells (thread c < COARSE_MAX holds cell c): sums of
+// the 16 warps, added in order
+template <typename T>
+__device__ __forceinline__ T block_mean_active(T v, bool act, CoarseSmem<T> &S) {
+    T a = act ? v : T(0);
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    const int cnt = __popc(__ballot_sync(0xffffffffu, act));
+    if (threadIdx.x < COARSE_MAX && (threadIdx.x & 31) == 0) {
+        S.red[threadIdx.x >> 5] = a;
+        S.cnt[threadIdx.x >> 5] = cnt;
+    }
+    __syncthreads();
+    T t = T(0);
+    int m = 0;
+#pragma unroll
+    for (int w = 0; w < COARSE_MAX / 32; ++w) {
+        t += S.red[w];
+        m += S.cnt[w];
+    }
+    __syncthreads();
+    return m > 0 ? t / T(m) : T(0);
+}
+
+// the coarsest-level solve by the threads of one block (at least COARSE_MAX).
+// Bound by the latency of one colour pass (4 sweeps of them, each waiting for
+// the last), in FP64 by the pipe: so a thread owns one cell of each colour
+// (no lane idles in a pass), keeps their coefficients in registers, reads its
+// six neighbours unconditionally (a closed or outer face has coefficient 0)
+// and only the warps that hold cells meet at the barrier. A 512-cell level
+// with 32 sweeps: 25 us before, with one thread per cell of either colour and
+// the coefficients in shared memory.
 template <typename T>
 __device__ void coarse_solve_dev(const MGLevel<T> &L, const T *__restrict__ f, T *__restrict__ x, int sweeps,
                                  CoarseSmem<T> &S) {
-    const int n = (int)L.n;
-    const int c = threadIdx.x;
-    int i = 0, j = 0, k = 0;
-    bool act = false;
-    if (c < n) {
-        i = c % L.nx;
-        j = (c / L.nx) % L.ny;
-        k = c / (L.nx * L.ny);
-        S.sx[c] = T(0);
-        S.sf[c] = f[c];
-        S.stx[c] = L.tx[c];
-        S.sty[c] = L.ty[c];
-        S.stz[c] = L.tz[c];
-        S.sdi[c] = L.dinv[c];
-        act = S.sdi[c] > T(0);
-    }
-    __syncthreads();
-    const T fm = block_mean_active<T>(c < n ? S.sf[c] : T(0), act, S.red, S.cnt);
-    if (act) S.sf[c] -= fm;
-    __syncthreads();
-    const int sy = L.nx, sz = L.nx * L.ny;
-    const int par = (i + j + k) & 1;
-    for (int pass = 0; pass < 4 * sweeps; ++pass) {
-        // sweeps x (red, black) then sweeps x (black, red): a palindrome
-        const int colour = pass < 2 * sweeps ? (pass & 1) : 1 - (pass & 1);
-        if (c < n && par == colour && act) {
-            T s = S.sf[c];
-            if (i > 0) s += S.stx[c] * S.sx[c - 1];
-            if (i < L.nx - 1) s += S.stx[c + 1] * S.sx[c + 1];
-            if (j > 0) s += S.sty[c] * S.sx[c - sy];
-            if (j < L.ny - 1) s += S.sty[c + sy] * S.sx[c + sy];
-            if (k > 0) s += S.stz[c] * S.sx[c - sz];
-            if (k < L.nz - 1) s += S.stz[c + sz] * S.sx[c + sz];
-            S.sx[c] = s * S.sdi[c];
+    const int n = (int)L.n, tid = threadIdx.x;
+    const int sy = L.nx, sz = L.nz > 1 ? L.nx * L.ny : 0;   // (at most n / 2: two cells or more per axis)
+    const bool act = tid < n && L.dinv[tid] > T(0);
+    for (int q = tid; q < COARSE_MAX + 2 * COARSE_PAD; q += blockDim.x) S.sx[q] = T(0);
+    const T fm = block_mean_active<T>(tid < n ? f[tid] : T(0), act, S);
+    const int nh = (L.nx + 1) >> 1, items = nh * L.ny * L.nz;   // at most 2 n / 3 (nx >= 2)
+    const int nthr = (items + 31) & ~31;
+    if (tid < nthr) {
+        int cc[2];
+        T k[2][6], di[2], ff[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int row = tid / nh, j = row % L.ny, z = row / L.ny;
+            const int i = 2 * (tid - row * nh) + ((q + j + z) & 1);
+            const int c = row * L.nx + i;
+            const bool in = tid < items && i < L.nx;
+            cc[q] = in && L.dinv[c] > T(0) ? c : -1;
+            k[q][0] = in && i > 0 ? L.tx[c] : T(0);
+            k[q][1] = in && i < L.nx - 1 ? L.tx[c + 1] : T(0);
+            k[q][2] = in && j > 0 ? L.ty[c] : T(0);
+            k[q][3] = in && j < L.ny - 1 ? L.ty[c + sy] : T(0);
+            k[q][4] = in && z > 0 ? L.tz[c] : T(0);
+            k[q][5] = in && z < L.nz - 1 ? L.tz[c + sz] : T(0);
+            di[q] = cc[q] >= 0 ? L.dinv[c] : T(0);
+            ff[q] = cc[q] >= 0 ? f[c] - fm : T(0);
         }
-        __syncthreads();
+        auto half = [&](int q) {
+            if (cc[q] >= 0) {
+                T *xc = S.sx + COARSE_PAD + cc[q];
+                T s = ff[q];
+                s += k[q][0] * xc[-1];
+                s += k[q][1] * xc[1];
+                s += k[q][2] * xc[-sy];
+                s += k[q][3] * xc[sy];
+                s += k[q][4] * xc[-sz];
+                s += k[q][5] * xc[sz];
+                *xc = s * di[q];
+            }
+            asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
+        };
+        // sweeps x (red, black) then sweeps x (black, red): a palindrome
+        for (int p = 0; p < sweeps; ++p) {
+            half(0);
+            half(1);
+        }
+        for (int p = 0; p < sweeps; ++p) {
+            half(1);
+            half(0);
+        }
     }
-    const T xm = block_mean_active<T>(c < n ? S.sx[c] : T(0), act, S.red, S.cnt);
-    if (c < n) x[c] = act ? S.sx[c] - xm : T(0);
+    __syncthreads();
+    const T xc = tid < n ? S.sx[COARSE_PAD + tid] : T(0);
+    const T xm = block_mean_active<T>(xc, act, S);
+    if (tid < n) x[tid] = act ? xc - xm : T(0);
     __syncthreads();
 }
 
+// The sweeps are a linear operator of the right-hand side, fixed between two
+// classifications, so their matrix M (n x n) is formed once per hierarchy,
+// one block per column, and a cycle applies it: 128 dependent passes of about
+// 0.1 us each (FP64 0.4 us) become one small matrix-vector product.
 template <typename T>
-__global__ void __launch_bounds__(COARSE_MAX) k_coarse_solve(MGLevel<T> L, const T *__restrict__ f,
-                                                             T *__restrict__ x, int sweeps) {
+__global__ void __launch_bounds__(COARSE_MAX) k_coarse_matrix(MGLevel<T> L, int sweeps, T *__restrict__ M) {
     __shared__ CoarseSmem<T> S;
-    coarse_solve_dev<T>(L, f, x, sweeps, S);
+    __shared__ T e[COARSE_MAX], x[COARSE_MAX];
+    const int n = (int)L.n, col = blockIdx.x;
+    e[threadIdx.x] = (int)threadIdx.x == col ? T(1) : T(0);
+    __syncthreads();
+    coarse_solve_dev<T>(L, e, x, sweeps, S);
+    if ((int)threadIdx.x < n) M[(size_t)threadIdx.x * n + col] = x[threadIdx.x];
+}
+
+}  // namespace ibm
+#include "vbottom.cuh"
+namespace ibm {
+
+template <typename T>
+__global__ void __launch_bounds__(COARSE_MAX) k_coarse_apply(int n, const T *__restrict__ M, const T *__restrict__ f,
+                                                             T *__restrict__ x) {
+    coarse_apply_dev<T>(n, M, f, x);
 }
 
 // ---------------------------------------------------------------------------
@@ -1809,16 +1853,19 @@ __device__ __forceinline__ void tail_prolong_yz(const TailLv<T> &A, int cny, int
     }
 }
 
-// The V-cycle from level l0 (its f and zeroed x written by the restriction
-// from l0 - 1) to the coarsest level nl - 1 and back, nu1 / nu2 sweeps per
-// level, cs sweep pairs on the coarsest level. One cluster of ncta blocks
-// (gridDim.x == ncta).
+// The V-cycle from level l0 to the coarsest level nl - 1 and back, nu1 / nu2
+// sweeps per level, cs sweep pairs on the coarsest level; it starts with the
+// restriction along y and z from level l0 - 1 (whose x-restricted residual is
+// in that level's scratch) and ends with the prolongation along x to it. One
+// cluster of ncta blocks (gridDim.x == ncta).
 template <typename T, bool OMEGA>
 __global__ void __launch_bounds__(TAIL_THREADS)
-    k_vtail(const TailLv<T> *__restrict__ A, int l0, int nl, int nu1, int nu2, int cs, T w, int ncta) {
-    __shared__ CoarseSmem<T> S;
+    k_vtail(const TailLv<T> *__restrict__ A, int l0, int nl, int nu1, int nu2, const T *__restrict__ cm, T w, int ncta) {
     const int gt = blockIdx.x * TAIL_THREADS + threadIdx.x, nt = ncta * TAIL_THREADS;
     const int zcol = 1;   // each pre-smoothing sweep ends with colour 1
+    const TailLv<T> &U = A[l0 - 1];
+    tail_restrict_yz<T>(A[l0].L, U.tmp, U.L.ny, U.X, gt, nt);
+    tail_sync(ncta);
     for (int l = l0; l < nl - 1; ++l) {
         const TailLv<T> &F = A[l];
         for (int s = 0; s < nu1; ++s) {
@@ -1835,7 +1882,7 @@ __global__ void __launch_bounds__(TAIL_THREADS)
     }
     if (blockIdx.x == 0) {
         const MGLevel<T> &C = A[nl - 1].L;
-        coarse_solve_dev<T>(C, C.f, C.x, cs, S);
+        coarse_apply_dev<T>((int)C.n, cm, C.f, C.x);
     }
     tail_sync(ncta);
     for (int l = nl - 2; l >= l0; --l) {
@@ -1852,6 +1899,7 @@ __global__ void __launch_bounds__(TAIL_THREADS)
             tail_sync(ncta);
         }
     }
+    tail_prolong_x<T>(U.L.nx, A[l0].L, U.X, U.tmp, gt, nt);
 }
 
 // q = K p ; partial (p, q) in FP64
@@ -2274,7 +2322,7 @@ static ibm_status build_hier(Ctx *c, MGHier<T> &H, bool fine0) {
             tl[l].L = H.lv[l];
             if (l + 1 < L) {
                 tl[l].pn = H.pn[l];
-                tl[l].tmp = l > 0 ? H.res[l] : nullptr;
+                tl[l].tmp = l > 0 ? H.res[l] : H.pq;   // (as the per-level transfers use)
                 tl[l].X = xfer_of<T>(c, l + 1);
             }
         }
@@ -2326,11 +2374,33 @@ static ibm_status fill_hier(Ctx *c, MGHier<T> &H, const std::vector<double *> &o
 
 ibm_status compact_flags(Ctx *c, const uint8_t *flags, int64_t **out, int64_t *count);
 
+static int bottom_max_ctas(Ctx *c);
+
+// the coarsest level's solution operator for the sweep count in force (formed
+// again after a classification or a change of coarse_sweeps)
+template <typename T>
+static ibm_status coarse_matrix(Ctx *c, MGHier<T> &H) {
+    if (!H.built || (H.cm_gen == c->mg_gen && H.cm_sweeps == c->opts.coarse_sweeps)) return IBM_OK;
+    const MGLevel<T> &L = H.lv.back();
+    if (!H.cm) H.cm = dev_alloc(c, sizeof(T) * (size_t)(L.n * L.n));
+    if (!H.cm) return c->fail(IBM_ERR_OOM, "coarsest operator allocation failed");
+    KL(-1, k_coarse_matrix<T>, (unsigned)L.n, COARSE_MAX, L, c->opts.coarse_sweeps, (T *)H.cm);
+    IBM_LAUNCHED(c);
+    H.cm_gen = c->mg_gen;
+    H.cm_sweeps = c->opts.coarse_sweeps;
+    return IBM_OK;
+}
+ibm_status mg_coarse_ready(Ctx *c) {
+    IBM_TRY(coarse_matrix<double>(c, c->mg64));
+    return coarse_matrix<float>(c, c->mg32);
+}
+
 // Multigrid hierarchies of the staircase operator and the near-body band for
 // the current classification.
 ibm_status mg_build(Ctx *c) {
     const int L = (int)c->lg.size();
     ++c->mg_gen;
+    if (c->bot_ctas == 0) c->bot_ctas = bottom_max_ctas(c);
     IBM_TRY(hist_reset(c));
     std::vector<double *> ox(L), oy(L), oz(L);
     for (int l = 0; l < L; ++l) {
@@ -2359,9 +2429,11 @@ ibm_status mg_build(Ctx *c) {
         IBM_TRY(fill_hier<double>(c, c->mg64, ox, oy, oz));
     }
     if (need32) {
-        if (!c->mg32.built) IBM_TRY(build_hier<float>(c, c->mg32, true));
+        // (a grid that is its own coarsest level keeps its coefficients)
+        if (!c->mg32.built) IBM_TRY(build_hier<float>(c, c->mg32, L > 1));
         IBM_TRY(fill_hier<float>(c, c->mg32, ox, oy, oz));
     }
+    IBM_TRY(mg_coarse_ready(c));
     // near-body band
     uint8_t *f0 = (uint8_t *)dev_alloc(c, c->N), *f1 = (uint8_t *)dev_alloc(c, c->N);
     if (!f0 || !f1) return c->fail(IBM_ERR_OOM, "band flag allocation failed");
@@ -2465,14 +2537,17 @@ static ibm_status split_pass(Ctx *c, MGHier<float> &H, int kind, int col, const 
 
 // First level of the persistent tail for this hierarchy and options (the
 // first level below 0 with at most tail_cells cells, if it leaves at least
-// one level to smooth above the coarsest), or -1; ncta: blocks of its cluster
+// one level to smooth above the coarsest, or the level that the shared-memory
+// bottom would start at where that lies higher, lb), or -1; ncta: blocks of
+// its cluster
 template <typename T>
-static int tail_level(const Ctx *c, const MGHier<T> &H, int *ncta) {
+static int tail_level(const Ctx *c, const MGHier<T> &H, int lb, int *ncta) {
     const int L = (int)H.lv.size();
     if (c->opts.tail_cells <= 0 || c->opts.mg_interp != 1 || !H.tail || L < 3) return -1;
     int l0 = 1;
     while (l0 < L && H.lv[l0].n > c->opts.tail_cells) ++l0;
     if (l0 > L - 2) return -1;
+    if (lb > 0 && lb < l0) l0 = lb;
     const int64_t per = 2 * (int64_t)TAIL_THREADS;
     *ncta = (int)std::min<int64_t>(TAIL_MAX_CTAS, std::max<int64_t>(1, (H.lv[l0].n + per - 1) / per));
     return l0;
@@ -2484,13 +2559,13 @@ static ibm_status launch_tail(Ctx *c, MGHier<T> &H, int l0, int ncta) {
     const TailLv<T> *A = reinterpret_cast<const TailLv<T> *>(H.tail);
     // (every tail level lies below the finest)
     const int nu1 = c->opts.nu_coarse > 0 ? c->opts.nu_coarse : c->opts.nu1;
-    const int nu2 = c->opts.nu_coarse > 0 ? c->opts.nu_coarse : c->opts.nu2, cs = c->opts.coarse_sweeps;
+    const int nu2 = c->opts.nu_coarse > 0 ? c->opts.nu_coarse : c->opts.nu2;
     const double w = c->opts.smooth_omega;
     auto kern = w != 1.0 ? k_vtail<T, true> : k_vtail<T, false>;
     kt_begin(c, K_TAIL);
     ++c->nlaunch;
     if (ncta == 1) {
-        kern<<<1, TAIL_THREADS, 0, c->s>>>(A, l0, L, nu1, nu2, cs, (T)w, 1);
+        kern<<<1, TAIL_THREADS, 0, c->s>>>(A, l0, L, nu1, nu2, (const T *)H.cm, (T)w, 1);
     } else {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)ncta, 1, 1);
@@ -2504,9 +2579,173 @@ static ibm_status launch_tail(Ctx *c, MGHier<T> &H, int l0, int ncta) {
         at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        IBM_CUDA(c, cudaLaunchKernelEx(&cfg, kern, A, l0, L, nu1, nu2, cs, (T)w, ncta));
+        IBM_CUDA(c, cudaLaunchKernelEx(&cfg, kern, A, l0, L, nu1, nu2, (const T *)H.cm, (T)w, ncta));
     }
     kt_end(c, K_TAIL);
+    IBM_LAUNCHED(c);
+    return IBM_OK;
+}
+
+// The levels of k_vbottom: from the first level below the finest whose share
+// the threads of its cluster can own (BotItems pairs each) and its shared
+// memory hold, to the coarsest. Returns that level, or -1 where the levels are
+// launched one by one (piecewise-constant transfer, no level between).
+//
+// Why the line lies there: a level costs about 16 launches of 2.5-4 us on its
+// own, in the cluster 16 phases of 0.5-1 us; the largest level that fits
+// (65,536 cells in FP32, 32,768 in FP64, whose passes the cluster's FP64
+// pipes bound) is still faster there.
+template <typename T>
+static int bottom_setup(Ctx *c, const MGHier<T> &H, BotPar<T> *out) {
+    const int L = (int)H.lv.size();
+    if (c->opts.mg_interp != 1 || L < 3 || c->bot_ctas < 1) return -1;
+    const bool d3 = c->ndim == 3;
+    for (int l0 = 1; l0 + 1 < L; ++l0) {
+        if (L - l0 > BOT_MAX_LV) continue;
+        BotPar<T> P{};
+        P.nl = L - l0;
+        P.ncta = 1;
+        const int64_t per = BotSingle<T>::CELLS / 4;   // cells a block should have at least
+        if (H.lv[l0].n > BotSingle<T>::CELLS)
+            while (P.ncta < c->bot_ctas && P.ncta * per < H.lv[l0].n) P.ncta *= 2;
+        P.nu1 = c->opts.nu_coarse > 0 ? c->opts.nu_coarse : c->opts.nu1;
+        P.nu2 = c->opts.nu_coarse > 0 ? c->opts.nu_coarse : c->opts.nu2;
+        P.w = (T)c->opts.smooth_omega;
+        int64_t off = 0, ioff = 0, tmp = 0;
+        auto take = [&](int64_t n) {
+            const int64_t o = off;
+            off += (n + 3) / 4 * 4;
+            return (int)o;
+        };
+        auto itake = [&](int64_t n) {
+            const int64_t o = ioff;
+            ioff += n;
+            return (int)o;
+        };
+        bool fits = true;
+        P.single = P.ncta == 1 ? 0 : P.nl - 1;
+        for (int l = l0; l < L && fits; ++l) {
+            const MGLevel<T> &M = H.lv[l];
+            BotLv<T> &v = P.lv[l - l0];
+            v.nx = M.nx;
+            v.ny = M.ny;
+            v.nz = M.nz;
+            v.nh = (M.nx + 1) / 2;
+            v.rs = v.nh + 1;
+            v.P = d3 ? M.nz : M.ny;
+            v.hr = d3 ? M.ny : 1;
+            const bool one = l == L - 1 || M.n <= BotSingle<T>::CELLS || l - l0 > P.single;
+            if (one && l - l0 < P.single) P.single = l - l0;
+            v.B = one ? v.P : (v.P + P.ncta - 1) / P.ncta;
+            v.fnh = FastDiv((uint32_t)v.nh);
+            v.fhr = FastDiv((uint32_t)v.hr);
+            v.fnx = FastDiv((uint32_t)v.nx);
+            v.tx = M.tx;
+            v.ti = d3 ? M.ty : nullptr;
+            v.to = d3 ? M.tz : M.ty;
+            v.d = M.d;
+            v.dinv = M.dinv;
+            v.pn = H.pn[l];
+            v.f = M.f;
+            v.x = M.x;
+            if (l > l0) tmp = std::max(tmp, (int64_t)v.B * v.hr * P.lv[l - l0 - 1].nx);
+            if (l + 1 == L) break;
+            const int64_t pairs = (int64_t)v.B * v.hr * v.nh;
+            const int it = (int)((pairs + BOT_THREADS - 1) / BOT_THREADS);
+            v.it = it <= 2 ? it : BotItems<T>::MAX;
+            fits = it <= BotItems<T>::MAX;
+            const int64_t row = v.rs, ps = row * v.hr;
+            v.sx = (int)((v.B + 2) * ps + 1);
+            v.ox = take(2 * (int64_t)v.sx);
+            v.sc = (int)(v.B * ps + 1);
+            v.of = take(2 * (int64_t)v.sc);
+            v.od = take(2 * (int64_t)v.sc);
+            v.ot = take(2 * (int64_t)v.sc);
+            v.opn = take(2 * (int64_t)v.sc);
+            v.odd = take(v.sc);
+            v.orr = take(v.sc);
+            v.si = d3 ? (int)((v.B * v.hr + 1) * row) : 0;
+            v.oi = take(2 * (int64_t)v.si);
+            v.so = (int)((v.B + 1) * ps);
+            v.oo = take(2 * (int64_t)v.so);
+            const int nf[3] = {M.nx, M.ny, M.nz}, nc[3] = {H.lv[l + 1].nx, H.lv[l + 1].ny, H.lv[l + 1].nz};
+            for (int a = 0; a < 3; ++a)
+                v.ax[a] = BotAxis{itake(4 * nc[a]), take(4 * nc[a]), itake(nf[a]), itake(nf[a]), take(nf[a]), take(nf[a])};
+            P.X[l - l0] = xfer_of<T>(c, l + 1);
+            tmp = std::max(tmp, (int64_t)v.B * v.hr * nc[0]);
+        }
+        if (!fits) continue;
+        P.nc = (int)H.lv[L - 1].n;
+        P.cm = (const T *)H.cm;
+        P.otmp = take(tmp);
+        P.ocf = take(COARSE_MAX);
+        P.ocx = take(COARSE_MAX);
+        P.ocm = P.nc <= COARSE_STOP ? take((int64_t)P.nc * P.nc) : -1;
+        P.total = (int)off;
+        P.itotal = (int)ioff;
+        if (off * (int64_t)sizeof(T) + ioff * (int64_t)sizeof(int) > BOT_SMEM) continue;
+        if (out) *out = P;
+        return l0;
+    }
+    return -1;
+}
+
+template <typename T>
+static const void *bottom_kernel(const Ctx *c) {
+    const bool om = c->opts.smooth_omega != 1.0;
+    if (c->ndim == 3) return om ? (const void *)k_vbottom<T, true, true> : (const void *)k_vbottom<T, false, true>;
+    return om ? (const void *)k_vbottom<T, true, false> : (const void *)k_vbottom<T, false, false>;
+}
+
+// Largest cluster of k_vbottom with all its shared memory that this device
+// takes: 16 blocks where a 16-block cluster can be resident, else 8, ...
+static int bottom_max_ctas(Ctx *c) {
+    const void *k = (const void *)k_vbottom<double, false, true>;
+    const size_t dyn = BOT_SMEM;
+    int best = 1;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) == cudaSuccess &&
+        cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+        for (int n = BOT_MAX_CTAS; n > 1 && best == 1; n /= 2) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)n, 1, 1);
+            cfg.blockDim = dim3(BOT_THREADS, 1, 1);
+            cfg.dynamicSmemBytes = dyn;
+            cudaLaunchAttribute at[1];
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = (unsigned)n;
+            at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+            cfg.attrs = at;
+            cfg.numAttrs = 1;
+            int fit = 0;
+            if (cudaOccupancyMaxActiveClusters(&fit, k, &cfg) == cudaSuccess && fit > 0) best = n;
+        }
+    }
+    cudaGetLastError();
+    return best;
+}
+
+template <typename T>
+static ibm_status launch_bottom(Ctx *c, const BotPar<T> &P) {
+    const void *k = bottom_kernel<T>(c);
+    const size_t dyn = sizeof(T) * (size_t)P.total + sizeof(int) * (size_t)P.itotal;
+    IBM_CUDA(c, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, BOT_SMEM));
+    IBM_CUDA(c, cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)P.ncta, 1, 1);
+    cfg.blockDim = dim3(BOT_THREADS, 1, 1);
+    cfg.dynamicSmemBytes = dyn;
+    cfg.stream = c->s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)P.ncta;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    void *args[1] = {const_cast<BotPar<T> *>(&P)};
+    kt_begin(c, -1);
+    ++c->nlaunch;
+    IBM_CUDA(c, cudaLaunchKernelExC(&cfg, k, args));
+    kt_end(c, -1);
     IBM_LAUNCHED(c);
     return IBM_OK;
 }
@@ -2514,13 +2753,13 @@ static ibm_status launch_tail(Ctx *c, MGHier<T> &H, int l0, int ncta) {
 template <typename T>
 static ibm_status vcycle(Ctx *c, MGHier<T> &H, const T *f0, T *x0) {
     const int L = (int)H.lv.size();
-    const int nu1 = c->opts.nu1, nu2 = c->opts.nu2, cs = c->opts.coarse_sweeps;
+    const int nu1 = c->opts.nu1, nu2 = c->opts.nu2;
     // sweeps on the levels below the finest
     const int nuc1 = c->opts.nu_coarse > 0 ? c->opts.nu_coarse : nu1;
     const int nuc2 = c->opts.nu_coarse > 0 ? c->opts.nu_coarse : nu2;
     const int bx = c->opts.tile_x;
     if (L == 1) {
-        KL(-1, k_coarse_solve<T>, 1, COARSE_MAX, H.lv[0], f0, x0, cs);
+        KL(-1, k_coarse_apply<T>, 1, COARSE_MAX, (int)H.lv[0].n, (const T *)H.cm, f0, x0);
         IBM_LAUNCHED(c);
         return IBM_OK;
     }
@@ -2528,11 +2767,13 @@ static ibm_status vcycle(Ctx *c, MGHier<T> &H, const T *f0, T *x0) {
     // levels' x is cleared by the restriction)
     if (nu1 < 1) IBM_CUDA(c, cudaMemsetAsync(x0, 0, sizeof(T) * (size_t)c->N, c->s));
     const bool sp = split_on(c, H);
-    // levels lt .. L - 1 in one persistent launch (lt = L - 1: the coarsest
-    // solve alone)
+    // levels lt .. L - 1 in one launch: the tail's where the caller asked for
+    // it, else the shared-memory bottom (lt = L - 1: the coarsest solve alone)
     int ncta = 1;
-    const int l0 = tail_level(c, H, &ncta);
-    const int lt = l0 > 0 ? l0 : L - 1;
+    BotPar<T> bot;
+    const int lb = bottom_setup<T>(c, H, &bot);
+    const int l0 = tail_level(c, H, lb, &ncta);
+    const int lt = l0 > 0 ? l0 : (lb > 0 ? lb : L - 1);
     for (int l = 0; l < lt; ++l) {
         const T *f = l == 0 ? f0 : H.lv[l].f;
         T *x = l == 0 ? x0 : H.lv[l].x;
@@ -2583,7 +2824,7 @@ static ibm_status vcycle(Ctx *c, MGHier<T> &H, const T *f0, T *x0) {
             else
                 KL(K_RESTRICT, (k_resid_rx<T, false>), rgrid, RX_THREADS, Lf, f, x, H.pn[l], X, Cl.nx, CG.fx, zcol,
                    tA);
-            KL(K_RESTRICT, k_restrict_yz<T>, grid, bx, Cl, tA, Lf.ny, X);
+            if (l0 < 0 || l + 1 < l0) KL(K_RESTRICT, k_restrict_yz<T>, grid, bx, Cl, tA, Lf.ny, X);
         } else if (l == 0 && H.fine0) {
             KL(K_RESTRICT, (k_resid_restrict<T, true>), grid, bx, Lf, f, x, Cl, CG.fx, CG.fy, CG.fz);
         } else {
@@ -2593,8 +2834,10 @@ static ibm_status vcycle(Ctx *c, MGHier<T> &H, const T *f0, T *x0) {
     }
     if (l0 > 0) {
         IBM_TRY(launch_tail(c, H, l0, ncta));
+    } else if (lb > 0) {
+        IBM_TRY(launch_bottom<T>(c, bot));
     } else {
-        KL(-1, k_coarse_solve<T>, 1, COARSE_MAX, H.lv[L - 1], H.lv[L - 1].f, H.lv[L - 1].x, cs);
+        KL(-1, k_coarse_apply<T>, 1, COARSE_MAX, (int)H.lv[L - 1].n, (const T *)H.cm, H.lv[L - 1].f, H.lv[L - 1].x);
         IBM_LAUNCHED(c);
     }
     for (int l = lt - 1; l >= 0; --l) {
@@ -2607,7 +2850,7 @@ static ibm_status vcycle(Ctx *c, MGHier<T> &H, const T *f0, T *x0) {
             MGLevel<T> &Cl = H.lv[l + 1];
             T *tB = l == 0 ? H.pq : H.res[l];
             const Xfer<T> X = xfer_of<T>(c, l + 1);
-            KL(K_PROLONG, k_prolong_x<T>, rows_grid(Lf.nx, Cl.ny, Cl.nz, 1, bx), bx, Lf.nx, Cl, X, tB);
+            if (l0 < 0 || l + 1 < l0) KL(K_PROLONG, k_prolong_x<T>, rows_grid(Lf.nx, Cl.ny, Cl.nz, 1, bx), bx, Lf.nx, Cl, X, tB);
             bool done = false;
             if constexpr (sizeof(T) == 4) {
                 if (l == 0 && sp) {
@@ -3609,6 +3852,7 @@ static ibm_status mixed_dev(Ctx *c, double *phi, DevFG *R, DevFG *F) {
 ibm_status poisson_dev_prepare(Ctx *c) {
     if ((c->opts.precision == IBM_FP64 && !c->mg64.built) || (c->opts.precision == IBM_MIXED && !c->mg32.built))
         IBM_TRY(mg_build(c));
+    IBM_TRY(mg_coarse_ready(c));
     if (c->opts.precision == IBM_MIXED) IBM_TRY(ensure_mixed(c));
     else IBM_TRY(alloc_krylov(c, c->opts.restart));
     if (!c->dctl) {
@@ -3863,6 +4107,7 @@ ibm_status hist_store(Ctx *c, const double *phi) {
 ibm_status poisson_solve(Ctx *c, const double *rhs, double *phi, double rtol, int maxit, ibm_solve_stats *st) {
     if ((c->opts.precision == IBM_FP64 && !c->mg64.built) || (c->opts.precision == IBM_MIXED && !c->mg32.built))
         IBM_TRY(mg_build(c));
+    IBM_TRY(mg_coarse_ready(c));
     const int64_t n = c->N;
     IBM_CUDA(c, cudaEventRecord(c->ev4, c->s));
     // b = P rhs on FLUID rows, 0 elsewhere
