@@ -49,6 +49,7 @@ struct MGHier {
     // solution operator of the coarsest level (n x n), and the multigrid
     // generation and sweep count it was formed for
     void *cm = nullptr;
+    void *bimg = nullptr;   // images of the V-cycle bottom's blocks
     uint64_t cm_gen = 0;
     int cm_sweeps = 0;
     bool built = false;

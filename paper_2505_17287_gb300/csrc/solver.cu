@@ -2376,6 +2376,9 @@ ibm_status compact_flags(Ctx *c, const uint8_t *flags, int64_t **out, int64_t *c
 
 static int bottom_max_ctas(Ctx *c);
 
+template <typename T>
+static int bottom_setup(Ctx *c, const MGHier<T> &H, BotPar<T> *out);
+
 // the coarsest level's solution operator for the sweep count in force (formed
 // again after a classification or a change of coarse_sweeps)
 template <typename T>
@@ -2386,6 +2389,17 @@ static ibm_status coarse_matrix(Ctx *c, MGHier<T> &H) {
     if (!H.cm) return c->fail(IBM_ERR_OOM, "coarsest operator allocation failed");
     KL(-1, k_coarse_matrix<T>, (unsigned)L.n, COARSE_MAX, L, c->opts.coarse_sweeps, (T *)H.cm);
     IBM_LAUNCHED(c);
+    // the images of the V-cycle bottom's blocks (their layout is fixed by the grid)
+    BotPar<T> P;
+    if (bottom_setup<T>(c, H, &P) > 0) {
+        const size_t nb = (size_t)P.ncta * (size_t)P.sbytes;
+        if (!H.bimg) H.bimg = dev_alloc(c, nb);
+        if (!H.bimg) return c->fail(IBM_ERR_OOM, "coarse-level image allocation failed");
+        IBM_CUDA(c, cudaMemsetAsync(H.bimg, 0, nb, c->s));
+        if (c->ndim == 3) KL(-1, (k_bottom_image<T, true>), P.ncta, BOT_THREADS, P, (uint4 *)H.bimg);
+        else KL(-1, (k_bottom_image<T, false>), P.ncta, BOT_THREADS, P, (uint4 *)H.bimg);
+        IBM_LAUNCHED(c);
+    }
     H.cm_gen = c->mg_gen;
     H.cm_sweeps = c->opts.coarse_sweeps;
     return IBM_OK;
@@ -2598,7 +2612,7 @@ static ibm_status launch_tail(Ctx *c, MGHier<T> &H, int l0, int ncta) {
 template <typename T>
 static int bottom_setup(Ctx *c, const MGHier<T> &H, BotPar<T> *out) {
     const int L = (int)H.lv.size();
-    if (c->opts.mg_interp != 1 || L < 3 || c->bot_ctas < 1) return -1;
+    if (L < 3 || c->bot_ctas < 1) return -1;
     const bool d3 = c->ndim == 3;
     for (int l0 = 1; l0 + 1 < L; ++l0) {
         if (L - l0 > BOT_MAX_LV) continue;
@@ -2624,6 +2638,7 @@ static int bottom_setup(Ctx *c, const MGHier<T> &H, BotPar<T> *out) {
         };
         bool fits = true;
         P.single = P.ncta == 1 ? 0 : P.nl - 1;
+        // the image's part
         for (int l = l0; l < L && fits; ++l) {
             const MGLevel<T> &M = H.lv[l];
             BotLv<T> &v = P.lv[l - l0];
@@ -2640,6 +2655,7 @@ static int bottom_setup(Ctx *c, const MGHier<T> &H, BotPar<T> *out) {
             v.fnh = FastDiv((uint32_t)v.nh);
             v.fhr = FastDiv((uint32_t)v.hr);
             v.fnx = FastDiv((uint32_t)v.nx);
+            v.fB = FastDiv((uint32_t)v.B);
             v.tx = M.tx;
             v.ti = d3 ? M.ty : nullptr;
             v.to = d3 ? M.tz : M.ty;
@@ -2651,19 +2667,16 @@ static int bottom_setup(Ctx *c, const MGHier<T> &H, BotPar<T> *out) {
             if (l > l0) tmp = std::max(tmp, (int64_t)v.B * v.hr * P.lv[l - l0 - 1].nx);
             if (l + 1 == L) break;
             const int64_t pairs = (int64_t)v.B * v.hr * v.nh;
-            const int it = (int)((pairs + BOT_THREADS - 1) / BOT_THREADS);
-            v.it = it <= 2 ? it : BotItems<T>::MAX;
+            const int64_t it = (pairs + BOT_THREADS - 1) / BOT_THREADS;
+            v.it = it <= 2 ? (int)it : BotItems<T>::MAX;
             fits = it <= BotItems<T>::MAX;
+            if (!fits) break;
             const int64_t row = v.rs, ps = row * v.hr;
-            v.sx = (int)((v.B + 2) * ps + 1);
-            v.ox = take(2 * (int64_t)v.sx);
             v.sc = (int)(v.B * ps + 1);
-            v.of = take(2 * (int64_t)v.sc);
             v.od = take(2 * (int64_t)v.sc);
             v.ot = take(2 * (int64_t)v.sc);
             v.opn = take(2 * (int64_t)v.sc);
             v.odd = take(v.sc);
-            v.orr = take(v.sc);
             v.si = d3 ? (int)((v.B * v.hr + 1) * row) : 0;
             v.oi = take(2 * (int64_t)v.si);
             v.so = (int)((v.B + 1) * ps);
@@ -2677,13 +2690,26 @@ static int bottom_setup(Ctx *c, const MGHier<T> &H, BotPar<T> *out) {
         if (!fits) continue;
         P.nc = (int)H.lv[L - 1].n;
         P.cm = (const T *)H.cm;
-        P.otmp = take(tmp);
-        P.ocf = take(COARSE_MAX);
-        P.ocx = take(COARSE_MAX);
         P.ocm = P.nc <= COARSE_STOP ? take((int64_t)P.nc * P.nc) : -1;
-        P.total = (int)off;
-        P.itotal = (int)ioff;
-        if (off * (int64_t)sizeof(T) + ioff * (int64_t)sizeof(int) > BOT_SMEM) continue;
+        P.oint = (int)off;
+        off = (off * (int64_t)sizeof(T) + ioff * (int64_t)sizeof(int) + 15) / 16 * 16;
+        if (off > BOT_SMEM) continue;
+        P.sbytes = (int)off;
+        P.image = (const uint4 *)H.bimg;
+        // what a cycle writes
+        off /= (int64_t)sizeof(T);
+        for (int l = 0; l + 1 < P.nl; ++l) {
+            BotLv<T> &v = P.lv[l];
+            v.sx = (int)((v.B + 2) * (int64_t)v.hr * v.rs + 1);
+            v.ox = take(2 * (int64_t)v.sx);
+            v.of = take(2 * (int64_t)v.sc);
+            v.orr = take(v.sc);
+        }
+        P.otmp = take(tmp);
+        P.ocf = take(P.nc);
+        P.ocx = take(P.nc);
+        if (off * (int64_t)sizeof(T) > BOT_SMEM) continue;
+        P.bytes = (int)(off * (int64_t)sizeof(T));
         if (out) *out = P;
         return l0;
     }
@@ -2727,7 +2753,7 @@ static int bottom_max_ctas(Ctx *c) {
 template <typename T>
 static ibm_status launch_bottom(Ctx *c, const BotPar<T> &P) {
     const void *k = bottom_kernel<T>(c);
-    const size_t dyn = sizeof(T) * (size_t)P.total + sizeof(int) * (size_t)P.itotal;
+    const size_t dyn = (size_t)P.bytes;
     IBM_CUDA(c, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, BOT_SMEM));
     IBM_CUDA(c, cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchConfig_t cfg = {};
@@ -2771,7 +2797,7 @@ static ibm_status vcycle(Ctx *c, MGHier<T> &H, const T *f0, T *x0) {
     // it, else the shared-memory bottom (lt = L - 1: the coarsest solve alone)
     int ncta = 1;
     BotPar<T> bot;
-    const int lb = bottom_setup<T>(c, H, &bot);
+    const int lb = c->opts.mg_interp == 1 ? bottom_setup<T>(c, H, &bot) : -1;
     const int l0 = tail_level(c, H, lb, &ncta);
     const int lt = l0 > 0 ? l0 : (lb > 0 ? lb : L - 1);
     for (int l = 0; l < lt; ++l) {

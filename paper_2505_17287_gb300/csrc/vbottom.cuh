@@ -21,6 +21,12 @@
 // (distributed shared memory), and the transfers read the neighbours' rows
 // the same way.
 //
+// What does not change between cycles (coefficients, transfer tables, the
+// coarsest solution operator) is packed once per classification into one image
+// per block (k_bottom_image), which a launch copies in with 16-byte
+// asynchronous copies: gathering it from the level arrays took 7-17 us of a
+// launch, the copy of 150 KB takes about 2.
+//
 // A cluster barrier costs about 1000 cycles and a block barrier about 40, so
 // the levels that one block can take in less than that (BotPar::single on)
 // belong to block 0 alone; the other blocks wait for the way back up.
@@ -57,7 +63,7 @@ struct BotLv {
     int nh, rs;         // cells of one colour per row, and the row stride (nh + 1)
     int P, hr, B;       // planes along the outer axis, rows per plane, planes per block
     int it;             // pairs per thread (1, 2 or 4)
-    FastDiv fnh, fhr, fnx;
+    FastDiv fnh, fhr, fnx, fB;
     // offsets (in T) of colour 0 in shared memory and the distance to colour 1:
     // x (with halo planes), f / dinv / tx / pn (rows of the block), ti (one row
     // more), to (one plane more); d and the residual r of colour 0
@@ -77,7 +83,9 @@ struct BotPar {
     int nc;                      // cells of the coarsest level
     const T *cm;                 // its solution operator, nc x nc
     int otmp, ocf, ocx, ocm;     // transfer scratch; coarsest f and x, cell-ordered; cm's copy
-    int total, itotal;           // T and int entries of dynamic shared memory
+    int oint;                    // T entry at which the integer tables start
+    int sbytes, bytes;           // shared memory: the image's part (first), all of it
+    const uint4 *image;          // ncta images of sbytes bytes
     T w;
 };
 
@@ -245,14 +253,15 @@ __device__ __forceinline__ void bot_down(const BotPar<T> &P, const BotLv<T> &v, 
         const int row = (int)fcx.div((uint32_t)t), I = t - row * cnx;
         int lp;
         const int par = bot_row<T, D3>(v, row, p0, lp);
-        T acc = T(0);
+        // (a missing entry has weight 0; its index is clamped)
+        T val[4], acc = T(0);
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
-            const int i = gi[4 * I + s];
-            if (i < 0) continue;
-            const T val = ((i + par) & 1) == 0 ? R[row * v.rs + (i >> 1)] : T(0);
-            acc += gw[4 * I + s] * val;
+            const int i = max(gi[4 * I + s], 0);
+            val[s] = ((i + par) & 1) == 0 ? R[row * v.rs + (i >> 1)] : T(0);
         }
+#pragma unroll
+        for (int s = 0; s < 4; ++s) acc += gw[4 * I + s] * val[s];
         tmp[t] = acc;
     }
 }
@@ -271,44 +280,31 @@ __device__ __forceinline__ void bot_up(const BotPar<T> &P, const BotLv<T> &v, co
     }
 }
 
-template <typename T, bool OMEGA, bool D3>
-__global__ void __launch_bounds__(BOT_THREADS, 1) k_vbottom(const __grid_constant__ BotPar<T> P) {
-    extern __shared__ double bot_smem[];
-    T *sm = reinterpret_cast<T *>(bot_smem);
-    int *si = reinterpret_cast<int *>(sm + P.total);
-    BotCtx C{cg::this_cluster(), false};
-    const int r = P.ncta > 1 ? (int)C.cl.block_rank() : 0, tid = threadIdx.x;
-    for (int q = tid; q < P.total; q += BOT_THREADS) sm[q] = T(0);
-    __syncthreads();
-    // coefficients and transfer tables of every level above the coarsest (a
-    // level of one block: in that block), and the coarsest solution operator
+// the images of k_vbottom's blocks (cleared beforehand), one block each
+template <typename T, bool D3>
+__global__ void __launch_bounds__(BOT_THREADS) k_bottom_image(const __grid_constant__ BotPar<T> P, uint4 *image) {
+    const int r = blockIdx.x, tid = threadIdx.x;
+    T *sm = reinterpret_cast<T *>(reinterpret_cast<char *>(image) + (size_t)r * P.sbytes);
+    int *si = reinterpret_cast<int *>(sm + P.oint);
     for (int l = 0; l + 1 < P.nl; ++l) {
-        const BotLv<T> &v = P.lv[l];
+        const BotLv<T> &v = P.lv[l], &c = P.lv[l + 1];
         int p0, np;
         bot_planes(v, r, p0, np);
         const int rows = np * v.hr, halo = p0 + np < v.P ? v.hr : 0;
-        const int n = (rows + halo) * v.nx;
+        const int n = np > 0 ? (rows + halo) * v.nx : 0;
         const int64_t g0 = (int64_t)p0 * v.hr * v.nx;
-        if (n > 0)
-#pragma unroll 2
-            for (int t = tid; t < n; t += BOT_THREADS) {
-                const int row = (int)v.fnx.div((uint32_t)t), i = t - row * v.nx;
-                int lp;
-                const int q = (i + bot_row<T, D3>(v, row, p0, lp)) & 1, idx = row * v.rs + (i >> 1);
-                const bool in = row < rows;
-                const T a = v.to[g0 + t];
-                const T b = in ? v.tx[g0 + t] : T(0), e = in ? v.dinv[g0 + t] : T(0), pn = in ? v.pn[g0 + t] : T(0);
-                const T ci = D3 && in ? v.ti[g0 + t] : T(0), d = in && q == 0 ? v.d[g0 + t] : T(0);
-                sm[v.oo + q * v.so + idx] = a;
-                if (!in) continue;
-                sm[v.ot + q * v.sc + idx] = b;
-                sm[v.od + q * v.sc + idx] = e;
-                sm[v.opn + q * v.sc + idx] = pn;
-                if (D3) sm[v.oi + q * v.si + idx] = ci;
-                if (q == 0) sm[v.odd + idx] = d;
-            }
-        // (a block needs the tables of the levels it has rows of, on either side)
-        const BotLv<T> &c = P.lv[l + 1];
+        for (int t = tid; t < n; t += BOT_THREADS) {
+            const int row = (int)v.fnx.div((uint32_t)t), i = t - row * v.nx;
+            int lp;
+            const int q = (i + bot_row<T, D3>(v, row, p0, lp)) & 1, idx = row * v.rs + (i >> 1);
+            sm[v.oo + q * v.so + idx] = v.to[g0 + t];
+            if (row >= rows) continue;
+            sm[v.ot + q * v.sc + idx] = v.tx[g0 + t];
+            sm[v.od + q * v.sc + idx] = v.dinv[g0 + t];
+            sm[v.opn + q * v.sc + idx] = v.pn[g0 + t];
+            if (D3) sm[v.oi + q * v.si + idx] = v.ti[g0 + t];
+            if (q == 0) sm[v.odd + idx] = v.d[g0 + t];
+        }
         const Xfer<T> &X = P.X[l];
         auto axis = [&](const BotAxis &a, int nf, int nc, const int *G, const T *gw, const int *I, const int *J,
                         const T *w, const T *vv) {
@@ -323,14 +319,33 @@ __global__ void __launch_bounds__(BOT_THREADS, 1) k_vbottom(const __grid_constan
                 sm[a.v + q] = vv[q];
             }
         };
-        if (np > 0 || r * c.B < c.P) {
-            axis(v.ax[0], v.nx, c.nx, X.Gx, X.gwx, X.Ix, X.Jx, X.wx, X.vx);
-            axis(v.ax[1], v.ny, c.ny, X.Gy, X.gwy, X.Iy, X.Jy, X.wy, X.vy);
-            axis(v.ax[2], v.nz, c.nz, X.Gz, X.gwz, X.Iz, X.Jz, X.wz, X.vz);
+        axis(v.ax[0], v.nx, c.nx, X.Gx, X.gwx, X.Ix, X.Jx, X.wx, X.vx);
+        axis(v.ax[1], v.ny, c.ny, X.Gy, X.gwy, X.Iy, X.Jy, X.wy, X.vy);
+        axis(v.ax[2], v.nz, c.nz, X.Gz, X.gwz, X.Iz, X.Jz, X.wz, X.vz);
+    }
+    if (P.ocm >= 0)
+        for (int q = tid; q < P.nc * P.nc; q += BOT_THREADS) sm[P.ocm + q] = P.cm[q];
+}
+
+template <typename T, bool OMEGA, bool D3>
+__global__ void __launch_bounds__(BOT_THREADS, 1) k_vbottom(const __grid_constant__ BotPar<T> P) {
+    extern __shared__ double bot_smem[];
+    T *sm = reinterpret_cast<T *>(bot_smem);
+    const int *si = reinterpret_cast<const int *>(sm + P.oint);
+    BotCtx C{cg::this_cluster(), false};
+    const int r = P.ncta > 1 ? (int)C.cl.block_rank() : 0, tid = threadIdx.x;
+    {
+        const char *src = reinterpret_cast<const char *>(P.image) + (size_t)r * P.sbytes;
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(sm);
+        for (int q = 16 * tid; q < P.sbytes; q += 16 * BOT_THREADS)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + q), "l"(src + q) : "memory");
+        // the corrections start at zero, their halos and pads included
+        for (int l = 0; l + 1 < P.nl; ++l) {
+            const BotLv<T> &v = P.lv[l];
+            if (r * v.B < v.P)
+                for (int q = tid; q < 2 * v.sx; q += BOT_THREADS) sm[v.ox + q] = T(0);
         }
     }
-    if (r == 0 && P.ocm >= 0)
-        for (int q = tid; q < P.nc * P.nc; q += BOT_THREADS) sm[P.ocm + q] = P.cm[q];
     {
         const BotLv<T> &v = P.lv[0];
         int p0, np;
@@ -345,13 +360,14 @@ __global__ void __launch_bounds__(BOT_THREADS, 1) k_vbottom(const __grid_constan
             sm[v.of + q * v.sc + row * v.rs + (i >> 1)] = v.f[g0 + t];
         }
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     // (every block's halos are cleared before a neighbour writes into them)
     C.wide = P.ncta > 1;
     C.sync();
     T *tmp = sm + P.otmp;
     // the transfer scratch of the block that holds plane pl of level v
     auto scratch = [&](const BotLv<T> &v, int pl, int &lrow) -> const T * {
-        const int o = pl / v.B;
+        const int o = (int)v.fB.div((uint32_t)pl);
         lrow = (pl - o * v.B) * v.hr;
         return C.wide ? C.cl.map_shared_rank(tmp, o) : tmp;
     };
@@ -379,19 +395,25 @@ __global__ void __launch_bounds__(BOT_THREADS, 1) k_vbottom(const __grid_constan
             const int idx = row * c.rs + (I >> 1);
             T acc = T(0);
             if (last || pos(sm[c.od + q * c.sc + idx])) {
+                // all reads (from up to 16 rows, some in other blocks) are
+                // issued before the sums; a missing entry has weight 0
+                T val[4][4];
 #pragma unroll
-                for (int s3 = 0; s3 < 4; ++s3) {
-                    const int k = si[v.ax[2].gi + 4 * K + s3];
-                    if (k < 0) continue;
-                    T a2 = T(0);
+                for (int s3 = 0; s3 < (D3 ? 4 : 1); ++s3) {
+                    const int k = max(si[v.ax[2].gi + 4 * K + s3], 0);
 #pragma unroll
                     for (int s2 = 0; s2 < 4; ++s2) {
-                        const int j = si[v.ax[1].gi + 4 * J + s2];
-                        if (j < 0) continue;
+                        const int j = max(si[v.ax[1].gi + 4 * J + s2], 0);
                         int lrow;
                         const T *src = scratch(v, D3 ? k : j, lrow);
-                        a2 += sm[v.ax[1].gw + 4 * J + s2] * src[(lrow + (D3 ? j : 0)) * c.nx + I];
+                        val[s3][s2] = src[(lrow + (D3 ? j : 0)) * c.nx + I];
                     }
+                }
+#pragma unroll
+                for (int s3 = 0; s3 < (D3 ? 4 : 1); ++s3) {
+                    T a2 = T(0);
+#pragma unroll
+                    for (int s2 = 0; s2 < 4; ++s2) a2 += sm[v.ax[1].gw + 4 * J + s2] * val[s3][s2];
                     acc += sm[v.ax[2].gw + 4 * K + s3] * a2;
                 }
             }
@@ -442,19 +464,26 @@ __global__ void __launch_bounds__(BOT_THREADS, 1) k_vbottom(const __grid_constan
             const T p = sm[v.opn + q * v.sc + idx];
             if (!pos(p)) continue;
             const int j = D3 ? row - lp * v.hr : p0 + row, k = D3 ? p0 + lp : 0;
-            int ib[2], ic[2];
-            T wb[2], wc[2];
-            const int nb = xfer_axis(si + v.ax[1].I, si + v.ax[1].J, sm + v.ax[1].w, sm + v.ax[1].v, j, ib, wb);
-            const int nc = xfer_axis(si + v.ax[2].I, si + v.ax[2].J, sm + v.ax[2].w, sm + v.ax[2].v, k, ic, wc);
-            T acc = T(0);
-            for (int q3 = 0; q3 < nc; ++q3) {
-                T a2 = T(0);
-                for (int q2 = 0; q2 < nb; ++q2) {
-                    int lrow;
-                    const T *src = scratch(c, D3 ? ic[q3] : ib[q2], lrow);
-                    a2 += wb[q2] * src[(lrow + (D3 ? ib[q2] : 0)) * v.nx + i];
+            // (no second coarse index: weight 0, the first one's value read again)
+            T val[2][2];
+            int lrow;
+#pragma unroll
+            for (int q3 = 0; q3 < (D3 ? 2 : 1); ++q3) {
+                const int kc = D3 && q3 && si[v.ax[2].J + k] >= 0 ? si[v.ax[2].J + k] : si[v.ax[2].I + k];
+#pragma unroll
+                for (int q2 = 0; q2 < 2; ++q2) {
+                    const int jc = q2 && si[v.ax[1].J + j] >= 0 ? si[v.ax[1].J + j] : si[v.ax[1].I + j];
+                    const T *src = scratch(c, D3 ? kc : jc, lrow);
+                    val[q3][q2] = src[(lrow + (D3 ? jc : 0)) * v.nx + i];
                 }
-                acc += wc[q3] * a2;
+            }
+            T acc = T(0);
+#pragma unroll
+            for (int q3 = 0; q3 < (D3 ? 2 : 1); ++q3) {
+                T a2 = T(0);
+                a2 += sm[v.ax[1].w + j] * val[q3][0];
+                a2 += sm[v.ax[1].v + j] * val[q3][1];
+                acc += sm[(q3 ? v.ax[2].v : v.ax[2].w) + k] * a2;
             }
             const int fl = (lp == 0 ? 2 : 0) | (lp == np - 1 ? 4 : 0);
             bot_put(v, sm, dn, up, q, idx + ps, fl, np, sm[v.ox + q * v.sx + idx + ps] + acc * p);
