@@ -20,6 +20,7 @@ static thread_local std::string g_create_error;
 namespace ibm {
 
 void *dev_alloc(Ctx *c, size_t bytes) {
+    c->chain = false;
     if (bytes == 0) bytes = 16;
     void *p = nullptr;
     if (c->desc.alloc) {
@@ -38,6 +39,7 @@ void *dev_alloc(Ctx *c, size_t bytes) {
 }
 
 void dev_free(Ctx *c, void *p) {
+    c->chain = false;   // (stream-ordered allocators put work on the stream)
     if (!p) return;
     auto it = std::find(c->allocs.begin(), c->allocs.end(), p);
     if (it == c->allocs.end()) return;

@@ -32,15 +32,23 @@ struct Err {
     std::string msg;
 };
 
-// Failure helpers used by every host function of the library.
+// Failure helpers used by every host function of the library. (Any runtime
+// call may put something other than a kernel on the stream: the next kernel
+// is then not overlapped with what precedes it, see launch().)
 #define IBM_CUDA(ctx, call)                                                          \
     do {                                                                             \
+        (ctx)->chain = false;                                                        \
         cudaError_t e_ = (call);                                                     \
         if (e_ != cudaSuccess) {                                                     \
             return (ctx)->fail(IBM_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
         }                                                                            \
     } while (0)
-#define IBM_LAUNCHED(ctx) IBM_CUDA(ctx, cudaGetLastError())
+#define IBM_LAUNCHED(ctx)                                                            \
+    do {                                                                             \
+        const bool chain_ = (ctx)->chain;                                            \
+        IBM_CUDA(ctx, cudaGetLastError());                                           \
+        (ctx)->chain = chain_;                                                       \
+    } while (0)
 #define IBM_TRY(expr)                          \
     do {                                       \
         ibm_status s_ = (expr);                \
@@ -144,6 +152,28 @@ ibm_status reduce_sum(Ctx *c, const double *partials, int nparts, double *out_de
 // device helpers
 // ---------------------------------------------------------------------------
 namespace ibm {
+
+// First statement of every kernel that launch() starts: allow the next kernel
+// of the stream to be set up now, and wait until the previous one is complete
+// and its writes are visible. (A kernel that does both before it touches
+// memory keeps the stream's order: its own completion implies the completion
+// of everything before it. Their pointer parameters are not __restrict__: the
+// compiler may move loads through const __restrict__ pointers, which it takes
+// for invariant, above the wait.)
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Grids of more than OVERLAP_BLOCKS blocks (one wave of 256-thread blocks on
+// 152 SMs) are launched plainly and skip both: the two instructions cost each
+// block a few hundred cycles, 5-10% of a many-wave streaming pass whose blocks
+// live about 2 us (k_helm_rb at 25.2M cells: 159 us without, 177 with), while
+// such a pass hardly notices the launch gap.
+constexpr unsigned OVERLAP_BLOCKS = 152 * 8;
+__device__ __forceinline__ void grid_begin() {
+    if (gridDim.x * gridDim.y <= OVERLAP_BLOCKS) {
+        grid_release();
+        grid_wait();
+    }
+}
 
 __device__ __forceinline__ double warp_sum(double v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);

@@ -227,6 +227,7 @@ struct Ctx {
     cudaGraphExec_t sgraph[NSGRAPH] = {nullptr};
     uint64_t sgraph_key[NSGRAPH] = {0};
     const double *sgraph_nold[NSGRAPH] = {nullptr};
+    bool chain = false;    // the last thing put on the stream was a kernel of launch()
     int64_t nlaunch = 0;   // kernels launched by this context so far
     // launch sizes that follow the grid: reduction kernels run nred blocks of
     // RED_THREADS (about 8 cells per thread, at most RED_BLOCKS; a function
@@ -246,6 +247,33 @@ struct Ctx {
         return code;
     }
 };
+
+// Start a kernel on the context stream. Its launch overlaps the previous
+// kernel's run (programmatic dependent launch): a small grid costs 2-4 us
+// between one kernel's end and the next one's start otherwise, more than most
+// coarse-level and Krylov kernels run. Every kernel started here begins with
+// grid_begin() (common.cuh), whose rule on the grid's size is repeated here.
+// Only a kernel that directly follows another kernel is overlapped: not one
+// after a copy, a memset, an event, a graph launch or a conditional node, whose
+// completion griddepcontrol.wait does not cover. The legacy default stream and
+// the event timer take plain launches.
+inline bool overlap_launch(const Ctx *c) {
+    return c->chain && c->s != nullptr && c->s != cudaStreamLegacy && !c->kt.on;
+}
+template <typename... P, typename... A>
+inline void launch(Ctx *c, void (*kern)(P...), dim3 grid, dim3 block, A &&...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = c->s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = overlap_launch(c) && (uint64_t)grid.x * grid.y * grid.z <= OVERLAP_BLOCKS ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);   // (the callers read cudaGetLastError)
+    c->chain = true;
+}
 
 // FP64 Krylov storage on first use (api.cu)
 ibm_status alloc_krylov(Ctx *c, int m);

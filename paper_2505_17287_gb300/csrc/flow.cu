@@ -67,9 +67,10 @@ __device__ __forceinline__ P pick3(int q, P a, P b, P c) { return q == 0 ? a : (
 // over the volume is 1/width, and the viscous face coefficients are the
 // pressure operator's per-axis coefficients; a Dirichlet wall contributes
 // 2 (value - u_c) / width^2.
-__global__ void k_conv_rhs(GridDev g, const uint8_t *__restrict__ type, const double *__restrict__ dg, CFields3 u,
-                           CFields3 F, CFields3 Nold, int first, const uint8_t *__restrict__ fresh, Fields3 Nnew,
+__global__ void k_conv_rhs(GridDev g, const uint8_t * type, const double * dg, CFields3 u,
+                           CFields3 F, CFields3 Nold, int first, const uint8_t * fresh, Fields3 Nnew,
                            Fields3 rhs, BCInfo bc, double dt, double alpha, int ncomp) {
+    grid_begin();
     const int64_t sy = g.nx, sz = (int64_t)g.nx * g.ny;
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < g.n; c += (int64_t)gridDim.x * blockDim.x) {
         if (type[c] != FLUID) {
@@ -190,8 +191,9 @@ __device__ __forceinline__ double helm_D(const GridDev &g, const BCInfo &bc, int
 }
 
 // inverse diagonal of (I - alpha L0) for component q on FLUID cells
-__global__ void k_helm_diag(GridDev g, const uint8_t *__restrict__ type, BCInfo bc, int q, double alpha,
-                            double *__restrict__ hinv) {
+__global__ void k_helm_diag(GridDev g, const uint8_t * type, BCInfo bc, int q, double alpha,
+                            double * hinv) {
+    grid_begin();
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < g.n; c += (int64_t)gridDim.x * blockDim.x) {
         if (type[c] != FLUID) { hinv[c] = 0.0; continue; }
         int i, j, k;
@@ -208,7 +210,7 @@ struct HelmCoef {
 // s0 + alpha sum_f c_f u_nb over the interior faces, accumulated onto s0
 // (one FP64 FMA per face: the scaling by alpha is folded into the stored
 // coefficients)
-__device__ __forceinline__ double visc_sum(const GridDev &g, const HelmCoef &h, const double *__restrict__ u,
+__device__ __forceinline__ double visc_sum(const GridDev &g, const HelmCoef &h, const double * u,
                                            int64_t c, int i, int j, int k, double s0) {
     const int64_t sy = g.nx, sz = (int64_t)g.nx * g.ny;
     double s = s0;
@@ -223,7 +225,8 @@ __device__ __forceinline__ double visc_sum(const GridDev &g, const HelmCoef &h, 
     return s;
 }
 
-__global__ void k_scaled_copy(int n, const double *__restrict__ src, double a, double *__restrict__ dst) {
+__global__ void k_scaled_copy(int n, const double * src, double a, double * dst) {
+    grid_begin();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t < n) dst[t] = a * src[t];
 }
@@ -233,8 +236,9 @@ __global__ void k_scaled_copy(int n, const double *__restrict__ src, double a, d
 // (phi changes smoothly between steps: on the 9.4M-cell wing the linear
 // guess saves ~10% of the iterations of phi^n, the quadratic one ~6% more);
 // the history shifts by one
-__global__ void k_phi_guess(int64_t n, double *__restrict__ p, double *__restrict__ pp, double *__restrict__ pp2,
+__global__ void k_phi_guess(int64_t n, double * p, double * pp, double * pp2,
                             int order) {
+    grid_begin();
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x) {
         const double t = p[c], t1 = pp[c];
         if (order == 1) p[c] = 2.0 * t - t1;
@@ -254,8 +258,9 @@ static int phi_order(const Ctx *c) { return c->nstep >= 4 ? 2 : (c->nstep == 3 ?
 // Helmholtz (I - alpha L0) u = rhs: one red-black colour on FLUID cells;
 // SOR: u += w (Gauss-Seidel value - u)
 template <bool SOR>
-__global__ void k_helm_rb(GridDev g, HelmCoef h, const uint8_t *__restrict__ type, const double *__restrict__ rhs,
-                          const double *__restrict__ hinv, double *__restrict__ u, int col, double w) {
+__global__ void k_helm_rb(GridDev g, HelmCoef h, const uint8_t * type, const double * rhs,
+                          const double * hinv, double * u, int col, double w) {
+    grid_begin();
     const int64_t row = blockIdx.x;
     int j, k;
     row_jk((uint32_t)blockIdx.x, g.fny, g.ny, j, k);
@@ -274,9 +279,10 @@ __global__ void k_helm_rb(GridDev g, HelmCoef h, const uint8_t *__restrict__ typ
 
 // one damped-Jacobi sweep of the Helmholtz system: out = u + w (D^{-1}(rhs +
 // alpha L_off u) - u) on FLUID cells, u elsewhere (ghost rows are refreshed after)
-__global__ void k_helm_jacobi(GridDev g, HelmCoef h, const uint8_t *__restrict__ type, const double *__restrict__ rhs,
-                              const double *__restrict__ hinv, const double *__restrict__ u, double *__restrict__ out,
+__global__ void k_helm_jacobi(GridDev g, HelmCoef h, const uint8_t * type, const double * rhs,
+                              const double * hinv, const double * u, double * out,
                               double w) {
+    grid_begin();
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < g.n; c += (int64_t)gridDim.x * blockDim.x) {
         const double uc = u[c];
         if (type[c] != FLUID) { out[c] = uc; continue; }
@@ -289,9 +295,10 @@ __global__ void k_helm_jacobi(GridDev g, HelmCoef h, const uint8_t *__restrict__
 // residual of the Helmholtz system on FLUID rows; partial columns |r|^2, |rhs|^2
 // (the diagonal is formed again rather than divided out of hinv: an FP64
 // division costs several times the few adds)
-__global__ void k_helm_resid(GridDev g, HelmCoef h, const uint8_t *__restrict__ type, const double *__restrict__ rhs,
-                             BCInfo bc, int q, const double *__restrict__ u, double alpha,
-                             double *__restrict__ part) {
+__global__ void k_helm_resid(GridDev g, HelmCoef h, const uint8_t * type, const double * rhs,
+                             BCInfo bc, int q, const double * u, double alpha,
+                             double * part) {
+    grid_begin();
     __shared__ double sh[32];
     double rr = 0.0, bb = 0.0;
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < g.n; c += (int64_t)gridDim.x * blockDim.x) {
@@ -314,8 +321,9 @@ __global__ void k_helm_resid(GridDev g, HelmCoef h, const uint8_t *__restrict__ 
 // tmp[q*ng + g] = (2 - bv) u_BI - sum_m wv_m u_m, with u_BI the body velocity
 // at the intercept (ubi, 3 per ghost; null: body at rest, u_BI = 0); the
 // fields u.p[0..ncomp) are velocity components comp0, comp0 + 1, ...
-__global__ void k_vghost_compute(GhostDev gh, Fields3 u, int ncomp, const double *__restrict__ ubi, int comp0,
-                                 double *__restrict__ tmp, double *__restrict__ res, int want_res) {
+__global__ void k_vghost_compute(GhostDev gh, Fields3 u, int ncomp, const double * ubi, int comp0,
+                                 double * tmp, double * res, int want_res) {
+    grid_begin();
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     __shared__ double sh[32];
     double r2 = 0.0;
@@ -341,12 +349,14 @@ __global__ void k_vghost_compute(GhostDev gh, Fields3 u, int ncomp, const double
         }
     }
 }
-__global__ void k_vghost_scatter(GhostDev gh, Fields3 u, int ncomp, const double *__restrict__ tmp) {
+__global__ void k_vghost_scatter(GhostDev gh, Fields3 u, int ncomp, const double * tmp) {
+    grid_begin();
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (q >= gh.ng) return;
     for (int cq = 0; cq < ncomp; ++cq) u.p[cq][gh.gidx[q]] = tmp[cq * gh.ng + q];
 }
-__global__ void k_max_final(const double *__restrict__ part, int n, double *__restrict__ out) {
+__global__ void k_max_final(const double * part, int n, double * out) {
+    grid_begin();
     double m = 0.0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) m = fmax(m, part[i]);
     m = warp_max(m);
@@ -361,8 +371,9 @@ __global__ void k_max_final(const double *__restrict__ part, int n, double *__re
 }
 
 // face velocities of axis a from cell values (interior and outer faces)
-__global__ void k_faces(GridDev g, const uint8_t *__restrict__ type, const double *__restrict__ ua, int a,
-                        BCInfo bc, double *__restrict__ Fa, FastDiv fdx, FastDiv fdy) {
+__global__ void k_faces(GridDev g, const uint8_t * type, const double * ua, int a,
+                        BCInfo bc, double * Fa, FastDiv fdx, FastDiv fdy) {
+    grid_begin();
     const int nfx = g.nx + (a == 0), nfy = g.ny + (a == 1), nfz = g.nz + (a == 2);
     const int64_t nf = (int64_t)nfx * nfy * nfz;
     const int64_t st = a == 0 ? 1 : (a == 1 ? (int64_t)g.nx : (int64_t)g.nx * g.ny);
@@ -397,7 +408,8 @@ __global__ void k_faces(GridDev g, const uint8_t *__restrict__ type, const doubl
 }
 
 // net inflow through the outer faces and the FLUID outflow area
-__global__ void k_bnd_flux(GridDev g, const uint8_t *__restrict__ type, CFields3 F, BCInfo bc, double *__restrict__ part) {
+__global__ void k_bnd_flux(GridDev g, const uint8_t * type, CFields3 F, BCInfo bc, double * part) {
+    grid_begin();
     __shared__ double sh[32];
     double net = 0.0, area = 0.0;
     const int64_t nyz = (int64_t)g.ny * g.nz, nxz = (int64_t)g.nx * g.nz, nxy = (int64_t)g.nx * g.ny;
@@ -438,8 +450,9 @@ __global__ void k_bnd_flux(GridDev g, const uint8_t *__restrict__ type, CFields3
 }
 
 // uniform correction of OUTFLOW faces over FLUID cells: corr = net / area
-__global__ void k_outflow_corr(GridDev g, const uint8_t *__restrict__ type, Fields3 F, BCInfo bc,
-                               const double *__restrict__ sums) {
+__global__ void k_outflow_corr(GridDev g, const uint8_t * type, Fields3 F, BCInfo bc,
+                               const double * sums) {
+    grid_begin();
     const double area = sums[F_AREA];
     if (!(area > 0.0)) return;
     const double corr = sums[F_NET] / area;
@@ -470,8 +483,9 @@ __global__ void k_outflow_corr(GridDev g, const uint8_t *__restrict__ type, Fiel
 }
 
 // b_raw = div(F) / dt on FLUID cells, 0 elsewhere
-__global__ void k_divergence(GridDev g, const uint8_t *__restrict__ type, CFields3 F, double inv_dt,
-                             double *__restrict__ out) {
+__global__ void k_divergence(GridDev g, const uint8_t * type, CFields3 F, double inv_dt,
+                             double * out) {
+    grid_begin();
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < g.n; c += (int64_t)gridDim.x * blockDim.x) {
         if (type[c] != FLUID) { out[c] = 0.0; continue; }
         int i, j, k;
@@ -489,8 +503,9 @@ __global__ void k_divergence(GridDev g, const uint8_t *__restrict__ type, CField
 // projection of the interior faces of axis a that have a FLUID side
 // (fdx, fdy: multiply-shift dividers by the face counts along x and y; the
 // gradient multiplies by the stored reciprocal centre spacing)
-__global__ void k_project_faces(GridDev g, const uint8_t *__restrict__ type, const double *__restrict__ phi, int a,
-                                double dt, double *__restrict__ Fa, FastDiv fdx, FastDiv fdy) {
+__global__ void k_project_faces(GridDev g, const uint8_t * type, const double * phi, int a,
+                                double dt, double * Fa, FastDiv fdx, FastDiv fdy) {
+    grid_begin();
     const int nfx = g.nx + (a == 0), nfy = g.ny + (a == 1), nfz = g.nz + (a == 2);
     const int64_t nf = (int64_t)nfx * nfy * nfz;
     const int64_t st = a == 0 ? 1 : (a == 1 ? (int64_t)g.nx : (int64_t)g.nx * g.ny);
@@ -509,8 +524,9 @@ __global__ void k_project_faces(GridDev g, const uint8_t *__restrict__ type, con
 }
 
 // cell velocities on FLUID cells: u_a -= dt * mean of the two face gradients
-__global__ void k_project_cells(GridDev g, const uint8_t *__restrict__ type, const double *__restrict__ phi,
+__global__ void k_project_cells(GridDev g, const uint8_t * type, const double * phi,
                                 CFields3 us, Fields3 u, double dt) {
+    grid_begin();
     const int64_t sy = g.nx, sz = (int64_t)g.nx * g.ny;
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < g.n; c += (int64_t)gridDim.x * blockDim.x) {
         const uint8_t t = type[c];
@@ -538,8 +554,9 @@ __global__ void k_project_cells(GridDev g, const uint8_t *__restrict__ type, con
     }
 }
 
-__global__ void k_init_cells(int64_t n, const uint8_t *__restrict__ type, Fields3 u, double u0, double u1, double u2,
-                             int ncomp, double *__restrict__ p) {
+__global__ void k_init_cells(int64_t n, const uint8_t * type, Fields3 u, double u0, double u1, double u2,
+                             int ncomp, double * p) {
+    grid_begin();
     const double v[3] = {u0, u1, u2};
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x) {
         const bool fl = type[c] == FLUID;
@@ -549,8 +566,9 @@ __global__ void k_init_cells(int64_t n, const uint8_t *__restrict__ type, Fields
 }
 
 // max |div F - mean| over FLUID cells, in two passes
-__global__ void k_div_stats(GridDev g, const uint8_t *__restrict__ type, const double *__restrict__ div,
-                            const double *__restrict__ mean, double *__restrict__ part) {
+__global__ void k_div_stats(GridDev g, const uint8_t * type, const double * div,
+                            const double * mean, double * part) {
+    grid_begin();
     const double m = mean ? *mean : 0.0;
     double mx = 0.0;
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < g.n; c += (int64_t)gridDim.x * blockDim.x)
@@ -584,16 +602,16 @@ static ibm_status faces_from(Ctx *c, double *const *ucell) {
     for (int a = 0; a < c->ndim; ++a) {
         const int64_t nf = a == 0 ? c->NFx : (a == 1 ? c->NFy : c->NFz);
         const unsigned nb = (unsigned)((nf + 255) / 256 > 152 * 32 ? 152 * 32 : (nf + 255) / 256);
-        ++c->nlaunch, k_faces<<<nb, 256, 0, c->s>>>(c->g, c->type, ucell[a], a, bc, c->F[a], FastDiv((uint32_t)(c->nx + (a == 0))),
+        ++c->nlaunch, launch(c, k_faces, nb, 256, c->g, c->type, ucell[a], a, bc, c->F[a], FastDiv((uint32_t)(c->nx + (a == 0))),
                                                   FastDiv((uint32_t)(c->ny + (a == 1))));
         IBM_LAUNCHED(c);
     }
     CFields3 F{{c->F[0], c->F[1], c->F[2]}};
-    ++c->nlaunch, k_bnd_flux<<<c->nred, RED_THREADS, 0, c->s>>>(c->g, c->type, F, bc, c->part);
+    ++c->nlaunch, launch(c, k_bnd_flux, c->nred, RED_THREADS, c->g, c->type, F, bc, c->part);
     IBM_LAUNCHED(c);
     IBM_TRY(finalize(c, c->part, c->nred, 2, 1.0, c->scal + 56));
     Fields3 Fw{{c->F[0], c->F[1], c->F[2]}};
-    ++c->nlaunch, k_outflow_corr<<<c->nred, RED_THREADS, 0, c->s>>>(c->g, c->type, Fw, bc, c->scal + 56);
+    ++c->nlaunch, launch(c, k_outflow_corr, c->nred, RED_THREADS, c->g, c->type, Fw, bc, c->scal + 56);
     IBM_LAUNCHED(c);
     return IBM_OK;
 }
@@ -612,12 +630,12 @@ static ibm_status ghost_refresh_all(Ctx *c, double *const *ucell, int *passes) {
     const int check_every = 4;
     for (int it = 0; it < c->opts.ghost_maxit; ++it) {
         const int want = ((it + 1) % check_every == 0) || it + 1 == c->opts.ghost_maxit;
-        ++c->nlaunch, k_vghost_compute<<<gb, 256, 0, c->s>>>(c->gh, U, nc, ghost_ubi(c), 0, c->gtmp, c->part, want);
-        ++c->nlaunch, k_vghost_scatter<<<gb, 256, 0, c->s>>>(c->gh, U, nc, c->gtmp);
+        ++c->nlaunch, launch(c, k_vghost_compute, gb, 256, c->gh, U, nc, ghost_ubi(c), 0, c->gtmp, c->part, want);
+        ++c->nlaunch, launch(c, k_vghost_scatter, gb, 256, c->gh, U, nc, c->gtmp);
         IBM_LAUNCHED(c);
         ++*passes;
         if (want) {
-            ++c->nlaunch, k_max_final<<<1, 256, 0, c->s>>>(c->part, (int)gb, c->scal + 40);
+            ++c->nlaunch, launch(c, k_max_final, 1, 256, c->part, (int)gb, c->scal + 40);
             IBM_LAUNCHED(c);
             IBM_TRY(sync_scalars(c, 41));
             const double d = c->hscal[40];
@@ -636,7 +654,7 @@ ibm_status ghost_refresh_velocity(Ctx *c, int comp, int *iters) {
 ibm_status flow_init(Ctx *c) {
     Fields3 U{{c->u[0], c->u[1], c->u[2]}};
     const unsigned nb = 152 * 16;
-    ++c->nlaunch, k_init_cells<<<nb, 256, 0, c->s>>>(c->N, c->type, U, c->desc.u_inf[0], c->desc.u_inf[1], c->desc.u_inf[2],
+    ++c->nlaunch, launch(c, k_init_cells, nb, 256, c->N, c->type, U, c->desc.u_inf[0], c->desc.u_inf[1], c->desc.u_inf[2],
                                       c->ndim, c->p);
     IBM_LAUNCHED(c);
     int passes = 0;
@@ -671,13 +689,13 @@ static ibm_status helm_prepare(Ctx *c) {
         const int len[6] = {nx, nx, ny, ny, nz, nz};
         size_t off = 0;
         for (int a = 0; a < 6; ++a) {
-            ++c->nlaunch, k_scaled_copy<<<(len[a] + 255) / 256, 256, 0, c->s>>>(len[a], src[a], alpha, c->hac + off);
+            ++c->nlaunch, launch(c, k_scaled_copy, (len[a] + 255) / 256, 256, len[a], src[a], alpha, c->hac + off);
             off += (size_t)len[a];
         }
         for (int cq = 0; cq < c->ndim; ++cq) {
             if (!c->hinv[cq]) c->hinv[cq] = (double *)dev_alloc(c, sizeof(double) * c->N);
             if (!c->hinv[cq]) return c->fail(IBM_ERR_OOM, "Helmholtz diagonal allocation failed");
-            ++c->nlaunch, k_helm_diag<<<c->nelem, 256, 0, c->s>>>(c->g, c->type, bc, cq, alpha, c->hinv[cq]);
+            ++c->nlaunch, launch(c, k_helm_diag, c->nelem, 256, c->g, c->type, bc, cq, alpha, c->hinv[cq]);
         }
         IBM_LAUNCHED(c);
         c->hinv_ok = true;
@@ -742,12 +760,12 @@ static ibm_status helmholtz_srj(Ctx *c, int q, int *sweeps) {
     for (int it = 0; it < c->opts.helm_maxit; it += M) {
         for (int k = 0; k < M; ++k) {
             kt_begin(c, K_HELM);
-            ++c->nlaunch, k_helm_jacobi<<<c->nelem, 256, 0, c->s>>>(c->g, helm_coef(c), c->type, rhs, hinv, u, t, w[k]);
+            ++c->nlaunch, launch(c, k_helm_jacobi, c->nelem, 256, c->g, helm_coef(c), c->type, rhs, hinv, u, t, w[k]);
             kt_end(c, K_HELM);
             if (c->ng > 0) {
                 Fields3 T3{{t, t, t}};
-                ++c->nlaunch, k_vghost_compute<<<gb, 256, 0, c->s>>>(c->gh, T3, 1, ghost_ubi(c), q, c->gtmp, c->part, 0);
-                ++c->nlaunch, k_vghost_scatter<<<gb, 256, 0, c->s>>>(c->gh, T3, 1, c->gtmp);
+                ++c->nlaunch, launch(c, k_vghost_compute, gb, 256, c->gh, T3, 1, ghost_ubi(c), q, c->gtmp, c->part, 0);
+                ++c->nlaunch, launch(c, k_vghost_scatter, gb, 256, c->gh, T3, 1, c->gtmp);
             }
             IBM_LAUNCHED(c);
             double *x = u;
@@ -757,13 +775,13 @@ static ibm_status helmholtz_srj(Ctx *c, int q, int *sweeps) {
         }
         // M is even: the iterate is back in ustar[q]
         Fields3 U{{u, u, u}};
-        ++c->nlaunch, k_helm_resid<<<c->nred, RED_THREADS, 0, c->s>>>(c->g, helm_coef(c), c->type, rhs, make_bc(c), q, u, alpha, c->part);
+        ++c->nlaunch, launch(c, k_helm_resid, c->nred, RED_THREADS, c->g, helm_coef(c), c->type, rhs, make_bc(c), q, u, alpha, c->part);
         IBM_LAUNCHED(c);
         IBM_TRY(finalize(c, c->part, c->nred, 2, 1.0, c->scal + 48));
         double gmax = 0.0;
         if (c->ng > 0) {
-            ++c->nlaunch, k_vghost_compute<<<gb, 256, 0, c->s>>>(c->gh, U, 1, ghost_ubi(c), q, c->gtmp, c->part + 2 * RED_BLOCKS_MAX, 1);
-            ++c->nlaunch, k_max_final<<<1, 256, 0, c->s>>>(c->part + 2 * RED_BLOCKS_MAX, (int)gb, c->scal + 50);
+            ++c->nlaunch, launch(c, k_vghost_compute, gb, 256, c->gh, U, 1, ghost_ubi(c), q, c->gtmp, c->part + 2 * RED_BLOCKS_MAX, 1);
+            ++c->nlaunch, launch(c, k_max_final, 1, 256, c->part + 2 * RED_BLOCKS_MAX, (int)gb, c->scal + 50);
             IBM_LAUNCHED(c);
         }
         IBM_TRY(sync_scalars(c, 51));
@@ -782,8 +800,8 @@ static ibm_status helmholtz_srj(Ctx *c, int q, int *sweeps) {
 // one red-black colour pass of the Helmholtz sweeps (kernel launch)
 static void helm_rb(Ctx *c, const double *rhs, const double *hinv, double *u, int col) {
     const double w = helm_omega(c);
-    if (w != 1.0) k_helm_rb<true><<<rb_grid(c), 128, 0, c->s>>>(c->g, helm_coef(c), c->type, rhs, hinv, u, col, w);
-    else k_helm_rb<false><<<rb_grid(c), 128, 0, c->s>>>(c->g, helm_coef(c), c->type, rhs, hinv, u, col, 1.0);
+    if (w != 1.0) launch(c, k_helm_rb<true>, rb_grid(c), 128, c->g, helm_coef(c), c->type, rhs, hinv, u, col, w);
+    else launch(c, k_helm_rb<false>, rb_grid(c), 128, c->g, helm_coef(c), c->type, rhs, hinv, u, col, 1.0);
 }
 
 // one Jacobi pass of the ghost rows of component q: u_G = (2 - bv) u_BI -
@@ -795,8 +813,8 @@ static void helm_rb(Ctx *c, const double *rhs, const double *hinv, double *u, in
 // finer cells converge more slowly, still needs 6).
 static void helm_ghost_pass(Ctx *c, int q, Fields3 U, unsigned gb) {
     if (c->ng == 0) return;
-    ++c->nlaunch, k_vghost_compute<<<gb, 256, 0, c->s>>>(c->gh, U, 1, ghost_ubi(c), q, c->gtmp, c->part, 0);
-    ++c->nlaunch, k_vghost_scatter<<<gb, 256, 0, c->s>>>(c->gh, U, 1, c->gtmp);
+    ++c->nlaunch, launch(c, k_vghost_compute, gb, 256, c->gh, U, 1, ghost_ubi(c), q, c->gtmp, c->part, 0);
+    ++c->nlaunch, launch(c, k_vghost_scatter, gb, 256, c->gh, U, 1, c->gtmp);
 }
 
 static ibm_status helmholtz(Ctx *c, int q, int *sweeps) {
@@ -823,14 +841,14 @@ static ibm_status helmholtz(Ctx *c, int q, int *sweeps) {
         ++*sweeps;
         if (*sweeps == next_check || it + 1 == c->opts.helm_maxit) {
             next_check = helm_next_check(next_check);
-            ++c->nlaunch, k_helm_resid<<<c->nred, RED_THREADS, 0, c->s>>>(c->g, helm_coef(c), c->type, rhs, make_bc(c), q, u, alpha, c->part);
+            ++c->nlaunch, launch(c, k_helm_resid, c->nred, RED_THREADS, c->g, helm_coef(c), c->type, rhs, make_bc(c), q, u, alpha, c->part);
             IBM_LAUNCHED(c);
             IBM_TRY(finalize(c, c->part, c->nred, 2, 1.0, c->scal + 48));
             double gmax = 0.0;
             if (c->ng > 0) {
                 // ghost-row residual: largest change a further Jacobi pass would make
-                ++c->nlaunch, k_vghost_compute<<<gb, 256, 0, c->s>>>(c->gh, U, 1, ghost_ubi(c), q, c->gtmp, c->part + 2 * RED_BLOCKS_MAX, 1);
-                ++c->nlaunch, k_max_final<<<1, 256, 0, c->s>>>(c->part + 2 * RED_BLOCKS_MAX, (int)gb, c->scal + 50);
+                ++c->nlaunch, launch(c, k_vghost_compute, gb, 256, c->gh, U, 1, ghost_ubi(c), q, c->gtmp, c->part + 2 * RED_BLOCKS_MAX, 1);
+                ++c->nlaunch, launch(c, k_max_final, 1, 256, c->part + 2 * RED_BLOCKS_MAX, (int)gb, c->scal + 50);
                 IBM_LAUNCHED(c);
             }
             IBM_TRY(sync_scalars(c, 51));
@@ -858,7 +876,7 @@ ibm_status flow_step(Ctx *c, ibm_step_stats *st) {
     Fields3 Nn{{c->Nnew[0], c->Nnew[1], nc == 3 ? c->Nnew[2] : c->Nnew[1]}};
     Fields3 R{{c->rhs[0], c->rhs[1], nc == 3 ? c->rhs[2] : c->rhs[1]}};
     kt_begin(c, K_CONV);
-    ++c->nlaunch, k_conv_rhs<<<c->nelem, 256, 0, c->s>>>(c->g, c->type, c->dg_c, u, F, No, c->have_nold ? 0 : 1, c->fresh_pending ? c->fresh : nullptr, Nn, R, make_bc(c), dt,
+    ++c->nlaunch, launch(c, k_conv_rhs, c->nelem, 256, c->g, c->type, c->dg_c, u, F, No, c->have_nold ? 0 : 1, c->fresh_pending ? c->fresh : nullptr, Nn, R, make_bc(c), dt,
                                            alpha, nc);
     kt_end(c, K_CONV);
     IBM_LAUNCHED(c);
@@ -875,9 +893,9 @@ ibm_status flow_step(Ctx *c, ibm_step_stats *st) {
     IBM_TRY(faces_from(c, c->ustar));
     CFields3 Fs{{c->F[0], c->F[1], nc == 3 ? c->F[2] : c->F[1]}};
     double *braw = c->rhs[0];
-    ++c->nlaunch, k_divergence<<<c->nelem, 256, 0, c->s>>>(c->g, c->type, Fs, 1.0 / dt, braw);
+    ++c->nlaunch, launch(c, k_divergence, c->nelem, 256, c->g, c->type, Fs, 1.0 / dt, braw);
     IBM_LAUNCHED(c);
-    ++c->nlaunch, k_phi_guess<<<c->nelem, 256, 0, c->s>>>(c->N, c->p, c->p_prev, c->p_prev2, phi_order(c));
+    ++c->nlaunch, launch(c, k_phi_guess, c->nelem, 256, c->N, c->p, c->p_prev, c->p_prev2, phi_order(c));
     IBM_LAUNCHED(c);
     IBM_TRY(hist_guess(c, braw, c->p));
     IBM_CUDA(c, cudaEventRecord(c->ev2, c->s));
@@ -890,14 +908,14 @@ ibm_status flow_step(Ctx *c, ibm_step_stats *st) {
     for (int a = 0; a < nc; ++a) {
         const int64_t nf = a == 0 ? c->NFx : (a == 1 ? c->NFy : c->NFz);
         const unsigned nb = (unsigned)((nf + 255) / 256 > 152 * 32 ? 152 * 32 : (nf + 255) / 256);
-        ++c->nlaunch, k_project_faces<<<nb, 256, 0, c->s>>>(c->g, c->type, c->p, a, dt, c->F[a],
+        ++c->nlaunch, launch(c, k_project_faces, nb, 256, c->g, c->type, c->p, a, dt, c->F[a],
                                                           FastDiv((uint32_t)(c->nx + (a == 0))),
                                                           FastDiv((uint32_t)(c->ny + (a == 1))));
     }
     IBM_LAUNCHED(c);
     CFields3 us{{c->ustar[0], c->ustar[1], nc == 3 ? c->ustar[2] : c->ustar[1]}};
     Fields3 un{{c->u[0], c->u[1], nc == 3 ? c->u[2] : c->u[1]}};
-    ++c->nlaunch, k_project_cells<<<c->nelem, 256, 0, c->s>>>(c->g, c->type, c->p, us, un, dt);
+    ++c->nlaunch, launch(c, k_project_cells, c->nelem, 256, c->g, c->type, c->p, us, un, dt);
     IBM_LAUNCHED(c);
     int passes = 0;
     IBM_TRY(ghost_refresh_all(c, c->u, &passes));
@@ -938,18 +956,20 @@ ibm_status flow_step(Ctx *c, ibm_step_stats *st) {
 // moving body: the fields after a move (Section 2.2)
 // ---------------------------------------------------------------------------
 
-__global__ void k_fresh_flags(int64_t n, const uint8_t *__restrict__ type, const uint8_t *__restrict__ old,
-                              uint8_t *__restrict__ fresh) {
+__global__ void k_fresh_flags(int64_t n, const uint8_t * type, const uint8_t * old,
+                              uint8_t * fresh) {
+    grid_begin();
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x)
         fresh[c] = (type[c] == FLUID && old[c] != FLUID) ? 1 : 0;
 }
 
 // fresh values, one Jacobi pass over the fresh rows (all components):
 // tmp = sum_m w_m u_m + wb u_BI; res: largest change
-__global__ void k_fresh_compute(int64_t nf, const int64_t *__restrict__ fidx, const int64_t *__restrict__ sidx,
-                                const double *__restrict__ w, const double *__restrict__ wb,
-                                const double *__restrict__ ub, Fields3 u, int ncomp, double *__restrict__ tmp,
-                                double *__restrict__ res) {
+__global__ void k_fresh_compute(int64_t nf, const int64_t * fidx, const int64_t * sidx,
+                                const double * w, const double * wb,
+                                const double * ub, Fields3 u, int ncomp, double * tmp,
+                                double * res) {
+    grid_begin();
     const int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     __shared__ double sh[32];
     double r = 0.0;
@@ -971,21 +991,24 @@ __global__ void k_fresh_compute(int64_t nf, const int64_t *__restrict__ fidx, co
         if (threadIdx.x == 0) res[blockIdx.x] = t;
     }
 }
-__global__ void k_fresh_scatter(int64_t nf, const int64_t *__restrict__ fidx, Fields3 u, int ncomp,
-                                const double *__restrict__ tmp) {
+__global__ void k_fresh_scatter(int64_t nf, const int64_t * fidx, Fields3 u, int ncomp,
+                                const double * tmp) {
+    grid_begin();
     const int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (f >= nf) return;
     for (int cq = 0; cq < ncomp; ++cq) u.p[cq][fidx[f]] = tmp[cq * nf + f];
 }
 // start value of the fresh cells: the body velocity at their intercept
-__global__ void k_fresh_start(int64_t nf, const int64_t *__restrict__ fidx, const double *__restrict__ ub, Fields3 u,
+__global__ void k_fresh_start(int64_t nf, const int64_t * fidx, const double * ub, Fields3 u,
                               int ncomp) {
+    grid_begin();
     const int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (f >= nf) return;
     for (int cq = 0; cq < ncomp; ++cq) u.p[cq][fidx[f]] = ub[3 * f + cq];
 }
 
-__global__ void k_dead_zero(int64_t n, const uint8_t *__restrict__ type, Fields3 u, int ncomp) {
+__global__ void k_dead_zero(int64_t n, const uint8_t * type, Fields3 u, int ncomp) {
+    grid_begin();
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x)
         if (type[c] == DEAD)
             for (int q = 0; q < ncomp; ++q) u.p[q][c] = 0.0;
@@ -993,8 +1016,9 @@ __global__ void k_dead_zero(int64_t n, const uint8_t *__restrict__ type, Fields3
 
 // interior faces of axis a next to a cell whose type changed: the face rule
 // (mean of the two cells on faces with a FLUID side and no DEAD side, else 0)
-__global__ void k_faces_changed(GridDev g, const uint8_t *__restrict__ type, const uint8_t *__restrict__ old,
-                                const double *__restrict__ ua, int a, double *__restrict__ Fa) {
+__global__ void k_faces_changed(GridDev g, const uint8_t * type, const uint8_t * old,
+                                const double * ua, int a, double * Fa) {
+    grid_begin();
     const int nfx = g.nx + (a == 0), nfy = g.ny + (a == 1);
     const int64_t nf = (int64_t)nfx * nfy * (g.nz + (a == 2));
     const int64_t st = a == 0 ? 1 : (a == 1 ? g.nx : (int64_t)g.nx * g.ny);
@@ -1024,7 +1048,7 @@ ibm_status flow_move(Ctx *c) {
     }
     IBM_TRY(geom_body_velocity(c, c->ng, c->bi, c->ubi));
     // fresh cells: FLUID now, not FLUID before the move
-    ++c->nlaunch, k_fresh_flags<<<c->nelem, 256, 0, c->s>>>(c->N, c->type, c->type_old, c->fresh);
+    ++c->nlaunch, launch(c, k_fresh_flags, c->nelem, 256, c->N, c->type, c->type_old, c->fresh);
     IBM_LAUNCHED(c);
     int64_t *fidx = nullptr, nf = 0;
     IBM_TRY(compact_flags(c, c->fresh, &fidx, &nf));
@@ -1041,18 +1065,18 @@ ibm_status flow_move(Ctx *c) {
         IBM_TRY(geom_fresh_tables(c, nf, fidx, fbi, fk, fs, fw, fwb));
         IBM_TRY(geom_body_velocity(c, nf, fbi, fub));
         const unsigned fb = (unsigned)((nf + 255) / 256);
-        ++c->nlaunch, k_fresh_start<<<fb, 256, 0, c->s>>>(nf, fidx, fub, U, nc);
+        ++c->nlaunch, launch(c, k_fresh_start, fb, 256, nf, fidx, fub, U, nc);
         IBM_LAUNCHED(c);
         // fresh corners are implicit unknowns: Jacobi passes to ghost_tol
         double scale = 1.0;
         for (int a = 0; a < 3; ++a) scale = fmax(scale, fmax(fabs(c->desc.u_inf[a]), fabs(c->motion[a])));
         bool done = false;
         for (int it = 0; it < 4 * c->opts.ghost_maxit && !done; ++it) {
-            ++c->nlaunch, k_fresh_compute<<<fb, 256, 0, c->s>>>(nf, fidx, fs, fw, fwb, fub, U, nc, ftmp, c->part);
-            ++c->nlaunch, k_fresh_scatter<<<fb, 256, 0, c->s>>>(nf, fidx, U, nc, ftmp);
+            ++c->nlaunch, launch(c, k_fresh_compute, fb, 256, nf, fidx, fs, fw, fwb, fub, U, nc, ftmp, c->part);
+            ++c->nlaunch, launch(c, k_fresh_scatter, fb, 256, nf, fidx, U, nc, ftmp);
             IBM_LAUNCHED(c);
             if ((it + 1) % 4 == 0) {
-                ++c->nlaunch, k_max_final<<<1, 256, 0, c->s>>>(c->part, (int)fb, c->scal + 40);
+                ++c->nlaunch, launch(c, k_max_final, 1, 256, c->part, (int)fb, c->scal + 40);
                 IBM_LAUNCHED(c);
                 IBM_TRY(sync_scalars(c, 41));
                 const double d = c->hscal[40];
@@ -1070,12 +1094,12 @@ ibm_status flow_move(Ctx *c) {
         dev_free(c, fk);
     }
     dev_free(c, fidx);
-    ++c->nlaunch, k_dead_zero<<<c->nelem, 256, 0, c->s>>>(c->N, c->type, U, nc);
+    ++c->nlaunch, launch(c, k_dead_zero, c->nelem, 256, c->N, c->type, U, nc);
     IBM_LAUNCHED(c);
     int passes = 0;
     IBM_TRY(ghost_refresh_all(c, c->u, &passes));
     for (int a = 0; a < nc; ++a)
-        ++c->nlaunch, k_faces_changed<<<c->nelem, 256, 0, c->s>>>(c->g, c->type, c->type_old, c->u[a], a, c->F[a]);
+        ++c->nlaunch, launch(c, k_faces_changed, c->nelem, 256, c->g, c->type, c->type_old, c->u[a], a, c->F[a]);
     IBM_LAUNCHED(c);
     c->fresh_pending = nf > 0;
     IBM_CUDA(c, cudaStreamSynchronize(c->s));
@@ -1086,11 +1110,11 @@ ibm_status flow_move(Ctx *c) {
 ibm_status div_stat(Ctx *c, double *out) {
     CFields3 F{{c->F[0], c->F[1], c->ndim == 3 ? c->F[2] : c->F[1]}};
     double *d = c->rhs[1];
-    ++c->nlaunch, k_divergence<<<c->nelem, 256, 0, c->s>>>(c->g, c->type, F, 1.0, d);
+    ++c->nlaunch, launch(c, k_divergence, c->nelem, 256, c->g, c->type, F, 1.0, d);
     IBM_LAUNCHED(c);
     IBM_TRY(fluid_mean(c, d, false, nullptr));
-    ++c->nlaunch, k_div_stats<<<c->nred, RED_THREADS, 0, c->s>>>(c->g, c->type, d, c->scal + 5, c->part);
-    ++c->nlaunch, k_max_final<<<1, 256, 0, c->s>>>(c->part, c->nred, c->scal + 52);
+    ++c->nlaunch, launch(c, k_div_stats, c->nred, RED_THREADS, c->g, c->type, d, c->scal + 5, c->part);
+    ++c->nlaunch, launch(c, k_max_final, 1, 256, c->part, c->nred, c->scal + 52);
     IBM_LAUNCHED(c);
     IBM_TRY(sync_scalars(c, 53));
     *out = c->hscal[52];
@@ -1117,6 +1141,7 @@ struct HelmCtl {
 };
 
 __global__ void k_hc_reset(HelmCtl *H, int q, int first_check, cudaGraphConditionalHandle h) {
+    grid_begin();
     if (q == 0) H->status = 0;
     if (q >= 0) {
         H->sweeps[q] = 0;
@@ -1130,6 +1155,7 @@ __global__ void k_hc_reset(HelmCtl *H, int q, int first_check, cudaGraphConditio
 
 // after each sweep: count it and open the residual test when it is due
 __global__ void k_helm_tick(HelmCtl *H, int q, int maxit, cudaGraphConditionalHandle hif) {
+    grid_begin();
     const int s = ++H->sweeps[q];
     const bool due = s == H->next_check || s >= maxit;
     if (due) H->next_check = helm_next_check(H->next_check);
@@ -1137,8 +1163,9 @@ __global__ void k_helm_tick(HelmCtl *H, int q, int maxit, cudaGraphConditionalHa
     cudaGraphSetConditional(hif, due ? 1u : 0u);
 }
 
-__global__ void k_helm_decide(HelmCtl *H, int q, const double *__restrict__ scal, int has_ghost, double tol,
+__global__ void k_helm_decide(HelmCtl *H, int q, const double * scal, int has_ghost, double tol,
                               double scale, int maxit, cudaGraphConditionalHandle h) {
+    grid_begin();
     if (!H->due) {
         cudaGraphSetConditional(h, 1u);
         return;
@@ -1158,8 +1185,9 @@ __global__ void k_helm_decide(HelmCtl *H, int q, const double *__restrict__ scal
     cudaGraphSetConditional(h, go ? 1u : 0u);
 }
 
-__global__ void k_ghost_decide(HelmCtl *H, const double *__restrict__ d, double tol, int maxit, int trip,
+__global__ void k_ghost_decide(HelmCtl *H, const double * d, double tol, int maxit, int trip,
                                cudaGraphConditionalHandle h) {
+    grid_begin();
     H->passes += trip;
     const double v = *d;
     if (!isfinite(v)) {
@@ -1187,7 +1215,7 @@ static ibm_status helmholtz_dev(Ctx *c, int q) {
     cudaGraphConditionalHandle h, hif;
     IBM_TRY(cond_handle(c, &h));
     IBM_TRY(cond_handle(c, &hif));
-    ++c->nlaunch, k_hc_reset<<<1, 1, 0, c->s>>>(H, q, c->opts.helm_check_first, h);
+    ++c->nlaunch, launch(c, k_hc_reset, 1, 1, H, q, c->opts.helm_check_first, h);
     CondScope sc;
     IBM_TRY(cond_open(c, cudaGraphCondTypeWhile, h, &sc));
     {
@@ -1197,21 +1225,21 @@ static ibm_status helmholtz_dev(Ctx *c, int q) {
             ++c->nlaunch, helm_rb(c, rhs, hinv, u, col);
             helm_ghost_pass(c, q, U, gb);
         }
-        ++c->nlaunch, k_helm_tick<<<1, 1, 0, c->s>>>(H, q, c->opts.helm_maxit, hif);
+        ++c->nlaunch, launch(c, k_helm_tick, 1, 1, H, q, c->opts.helm_maxit, hif);
         IBM_LAUNCHED(c);
         CondScope si;
         IBM_TRY(cond_open(c, cudaGraphCondTypeIf, hif, &si));
-        ++c->nlaunch, k_helm_resid<<<c->nred, RED_THREADS, 0, c->s>>>(c->g, helm_coef(c), c->type, rhs, make_bc(c), q, u, alpha,
+        ++c->nlaunch, launch(c, k_helm_resid, c->nred, RED_THREADS, c->g, helm_coef(c), c->type, rhs, make_bc(c), q, u, alpha,
                                                                      c->part);
         IBM_LAUNCHED(c);
         IBM_TRY(finalize(c, c->part, c->nred, 2, 1.0, c->scal + 48));
         if (c->ng > 0) {
-            ++c->nlaunch, k_vghost_compute<<<gb, 256, 0, c->s>>>(c->gh, U, 1, ghost_ubi(c), q, c->gtmp, c->part + 2 * RED_BLOCKS_MAX, 1);
-            ++c->nlaunch, k_max_final<<<1, 256, 0, c->s>>>(c->part + 2 * RED_BLOCKS_MAX, (int)gb, c->scal + 50);
+            ++c->nlaunch, launch(c, k_vghost_compute, gb, 256, c->gh, U, 1, ghost_ubi(c), q, c->gtmp, c->part + 2 * RED_BLOCKS_MAX, 1);
+            ++c->nlaunch, launch(c, k_max_final, 1, 256, c->part + 2 * RED_BLOCKS_MAX, (int)gb, c->scal + 50);
             IBM_LAUNCHED(c);
         }
         IBM_TRY(cond_close(c, &si));
-        ++c->nlaunch, k_helm_decide<<<1, 1, 0, c->s>>>(H, q, c->scal, c->ng > 0, c->opts.helm_rtol, u_scale(c),
+        ++c->nlaunch, launch(c, k_helm_decide, 1, 1, H, q, c->scal, c->ng > 0, c->opts.helm_rtol, u_scale(c),
                                                      c->opts.helm_maxit, h);
         IBM_LAUNCHED(c);
     }
@@ -1228,15 +1256,15 @@ static ibm_status ghost_refresh_dev(Ctx *c) {
     const int trip = 4;
     cudaGraphConditionalHandle h;
     IBM_TRY(cond_handle(c, &h));
-    ++c->nlaunch, k_hc_reset<<<1, 1, 0, c->s>>>(H, -1, 0, h);
+    ++c->nlaunch, launch(c, k_hc_reset, 1, 1, H, -1, 0, h);
     CondScope sc;
     IBM_TRY(cond_open(c, cudaGraphCondTypeWhile, h, &sc));
     for (int t = 0; t < trip; ++t) {
-        ++c->nlaunch, k_vghost_compute<<<gb, 256, 0, c->s>>>(c->gh, U, nc, ghost_ubi(c), 0, c->gtmp, c->part, t == trip - 1);
-        ++c->nlaunch, k_vghost_scatter<<<gb, 256, 0, c->s>>>(c->gh, U, nc, c->gtmp);
+        ++c->nlaunch, launch(c, k_vghost_compute, gb, 256, c->gh, U, nc, ghost_ubi(c), 0, c->gtmp, c->part, t == trip - 1);
+        ++c->nlaunch, launch(c, k_vghost_scatter, gb, 256, c->gh, U, nc, c->gtmp);
     }
-    ++c->nlaunch, k_max_final<<<1, 256, 0, c->s>>>(c->part, (int)gb, c->scal + 40);
-    ++c->nlaunch, k_ghost_decide<<<1, 1, 0, c->s>>>(H, c->scal + 40, c->opts.ghost_tol * u_scale(c),
+    ++c->nlaunch, launch(c, k_max_final, 1, 256, c->part, (int)gb, c->scal + 40);
+    ++c->nlaunch, launch(c, k_ghost_decide, 1, 1, H, c->scal + 40, c->opts.ghost_tol * u_scale(c),
                                                   c->opts.ghost_maxit, trip, h);
     IBM_LAUNCHED(c);
     IBM_TRY(cond_close(c, &sc));
@@ -1253,7 +1281,7 @@ static ibm_status flow_step_capture(Ctx *c) {
     CFields3 No{{c->Nold[0], c->Nold[1], nc == 3 ? c->Nold[2] : c->Nold[1]}};
     Fields3 Nn{{c->Nnew[0], c->Nnew[1], nc == 3 ? c->Nnew[2] : c->Nnew[1]}};
     Fields3 R{{c->rhs[0], c->rhs[1], nc == 3 ? c->rhs[2] : c->rhs[1]}};
-    ++c->nlaunch, k_conv_rhs<<<c->nelem, 256, 0, c->s>>>(c->g, c->type, c->dg_c, u, F, No, c->have_nold ? 0 : 1, c->fresh_pending ? c->fresh : nullptr, Nn, R,
+    ++c->nlaunch, launch(c, k_conv_rhs, c->nelem, 256, c->g, c->type, c->dg_c, u, F, No, c->have_nold ? 0 : 1, c->fresh_pending ? c->fresh : nullptr, Nn, R,
                                                        make_bc(c), dt, alpha, nc);
     IBM_LAUNCHED(c);
     for (int q = 0; q < nc; ++q) {
@@ -1263,9 +1291,9 @@ static ibm_status flow_step_capture(Ctx *c) {
     IBM_TRY(faces_from(c, c->ustar));
     CFields3 Fs{{c->F[0], c->F[1], nc == 3 ? c->F[2] : c->F[1]}};
     double *braw = c->rhs[0];
-    ++c->nlaunch, k_divergence<<<c->nelem, 256, 0, c->s>>>(c->g, c->type, Fs, 1.0 / dt, braw);
+    ++c->nlaunch, launch(c, k_divergence, c->nelem, 256, c->g, c->type, Fs, 1.0 / dt, braw);
     IBM_LAUNCHED(c);
-    ++c->nlaunch, k_phi_guess<<<c->nelem, 256, 0, c->s>>>(c->N, c->p, c->p_prev, c->p_prev2, phi_order(c));
+    ++c->nlaunch, launch(c, k_phi_guess, c->nelem, 256, c->N, c->p, c->p_prev, c->p_prev2, phi_order(c));
     IBM_LAUNCHED(c);
     IBM_TRY(hist_guess(c, braw, c->p));
     IBM_TRY(poisson_solve_dev(c, braw, c->p, c->opts.rtol, c->opts.max_outer));
@@ -1273,13 +1301,13 @@ static ibm_status flow_step_capture(Ctx *c) {
     for (int a = 0; a < nc; ++a) {
         const int64_t nf = a == 0 ? c->NFx : (a == 1 ? c->NFy : c->NFz);
         const unsigned nb = (unsigned)((nf + 255) / 256 > 152 * 32 ? 152 * 32 : (nf + 255) / 256);
-        ++c->nlaunch, k_project_faces<<<nb, 256, 0, c->s>>>(c->g, c->type, c->p, a, dt, c->F[a],
+        ++c->nlaunch, launch(c, k_project_faces, nb, 256, c->g, c->type, c->p, a, dt, c->F[a],
                                                           FastDiv((uint32_t)(c->nx + (a == 0))),
                                                           FastDiv((uint32_t)(c->ny + (a == 1))));
     }
     CFields3 us{{c->ustar[0], c->ustar[1], nc == 3 ? c->ustar[2] : c->ustar[1]}};
     Fields3 un{{c->u[0], c->u[1], nc == 3 ? c->u[2] : c->u[1]}};
-    ++c->nlaunch, k_project_cells<<<c->nelem, 256, 0, c->s>>>(c->g, c->type, c->p, us, un, dt);
+    ++c->nlaunch, launch(c, k_project_cells, c->nelem, 256, c->g, c->type, c->p, us, un, dt);
     IBM_LAUNCHED(c);
     IBM_TRY(ghost_refresh_dev(c));
     IBM_TRY(step_stats_dev(c, ((HelmCtl *)c->hctl)->sweeps));

@@ -42,7 +42,7 @@ enum {
     do {                                                     \
         kt_begin(c, kid);                                    \
         ++c->nlaunch;                                        \
-        kern<<<(grid), (block), 0, c->s>>>(__VA_ARGS__);     \
+        launch(c, kern, (grid), (block), __VA_ARGS__);       \
         kt_end(c, kid);                                      \
     } while (0)
 
@@ -63,7 +63,8 @@ static inline dim3 rows_grid(int nx, int ny, int nz, int per_thread, int bx) {
 
 // out[col] = scale * sum_i part[col*nparts + i], in a fixed order; one block
 // per column
-__global__ void k_finalize(const double *__restrict__ part, int nparts, double scale, double *__restrict__ out) {
+__global__ void k_finalize(const double * part, int nparts, double scale, double * out) {
+    grid_begin();
     __shared__ double sh[32];
     const int col = blockIdx.x;
     double v = 0.0;
@@ -93,8 +94,9 @@ ibm_status sync_scalars(Ctx *c, int n) {
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < (n); c += (int64_t)gridDim.x * blockDim.x)
 
 // sum over FLUID cells of vol * x (x null: the FLUID volume)
-__global__ void k_fluid_volsum(GridDev g, const uint8_t *__restrict__ type, const double *__restrict__ x,
-                               double *__restrict__ part) {
+__global__ void k_fluid_volsum(GridDev g, const uint8_t * type, const double * x,
+                               double * part) {
+    grid_begin();
     __shared__ double sh[32];
     double acc = 0.0;
     GRID_STRIDE(c, g.n) {
@@ -108,8 +110,9 @@ __global__ void k_fluid_volsum(GridDev g, const uint8_t *__restrict__ type, cons
 }
 
 // x -= mean on FLUID (and GHOST if ghosts) cells; DEAD cells set to 0
-__global__ void k_sub_mean(int64_t n, const uint8_t *__restrict__ type, double *__restrict__ x,
-                           const double *__restrict__ mean, int ghosts) {
+__global__ void k_sub_mean(int64_t n, const uint8_t * type, double * x,
+                           const double * mean, int ghosts) {
+    grid_begin();
     const double m = *mean;
     GRID_STRIDE(c, n) {
         const uint8_t t = type[c];
@@ -157,7 +160,7 @@ struct OpT {
 // (A x)_c of a FLUID cell with the per-axis coefficients; boundary faces
 // have coefficient 0, so a wall reads the cell itself
 template <typename T>
-__device__ __forceinline__ T A_row(const GridDev &g, const OpT<T> &o, const T *__restrict__ x, int64_t c, int i,
+__device__ __forceinline__ T A_row(const GridDev &g, const OpT<T> &o, const T * x, int64_t c, int i,
                                    int j, int k) {
     const int64_t sy = g.nx, sz = (int64_t)g.nx * g.ny;
     const T xc = x[c];
@@ -186,8 +189,9 @@ __device__ __forceinline__ T A_row(const GridDev &g, const OpT<T> &o, const T *_
 // (PLAIN: b null and sgn = 1, the product of every Krylov step; two FP64
 // operations per cell fewer)
 template <typename T, bool PLAIN = false>
-__global__ void k_apply_A(GridDev g, OpT<T> o, const uint8_t *__restrict__ type, const T *__restrict__ x,
-                          const T *__restrict__ b, T sgn, T *__restrict__ y, double *__restrict__ part) {
+__global__ void k_apply_A(GridDev g, OpT<T> o, const uint8_t * type, const T * x,
+                          const T * b, T sgn, T * y, double * part) {
+    grid_begin();
     __shared__ double sh[32];
     typename Acc<T>::type acc = 0;
     GRID_STRIDE(c, g.n) {
@@ -216,8 +220,9 @@ __device__ __forceinline__ float f4get(const float4 &v, int e) { return e == 0 ?
 __device__ __forceinline__ uint8_t u4get(const uchar4 &v, int e) { return e == 0 ? v.x : e == 1 ? v.y : e == 2 ? v.z : v.w; }
 
 __global__ void __launch_bounds__(RED_THREADS)
-    k_apply_A4(GridDev g, OpT<float> o, const uint8_t *__restrict__ type, const float *__restrict__ x,
-               const float *__restrict__ b, float sgn, float *__restrict__ y, double *__restrict__ part) {
+    k_apply_A4(GridDev g, OpT<float> o, const uint8_t * type, const float * x,
+               const float * b, float sgn, float * y, double * part) {
+    grid_begin();
     __shared__ double sh[32];
     double acc = 0.0;
     const int64_t sy = g.nx, sz = (int64_t)g.nx * g.ny;
@@ -275,8 +280,9 @@ static inline bool al16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 // GHOST rows: y_g = sgn * (x_g - sum_m wp_m x_m) + b_g (b may be null = 0;
 // the pressure equation has b_g = 0, a defect-correction right-hand side not)
 template <typename T>
-__global__ void k_ghost_rows(GhostDev gh, OpT<T> o, const T *__restrict__ x, const T *__restrict__ b, T sgn,
-                             T *__restrict__ y) {
+__global__ void k_ghost_rows(GhostDev gh, OpT<T> o, const T * x, const T * b, T sgn,
+                             T * y) {
+    grid_begin();
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (q >= gh.ng) return;
     const int64_t gi = gh.gidx[q];
@@ -285,7 +291,8 @@ __global__ void k_ghost_rows(GhostDev gh, OpT<T> o, const T *__restrict__ x, con
     y[gi] = sgn * s + (b ? b[gi] : T(0));
 }
 
-__global__ void k_zero_at(int64_t m, const int64_t *__restrict__ idx, double *__restrict__ x) {
+__global__ void k_zero_at(int64_t m, const int64_t * idx, double * x) {
+    grid_begin();
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (q < m) x[idx[q]] = 0.0;
 }
@@ -293,8 +300,9 @@ __global__ void k_zero_at(int64_t m, const int64_t *__restrict__ idx, double *__
 // x -= mean on FLUID cells (precision T); DEAD cells set to 0
 // (FP32: four cells per 16-byte access, the tail one by one)
 template <typename T>
-__global__ void k_sub_meanT(int64_t n, const uint8_t *__restrict__ type, T *__restrict__ x,
-                            const double *__restrict__ mean) {
+__global__ void k_sub_meanT(int64_t n, const uint8_t * type, T * x,
+                            const double * mean) {
+    grid_begin();
     const T m = (T)*mean;
     int64_t n0 = 0;
     if constexpr (sizeof(T) == 4) {
@@ -386,8 +394,9 @@ struct VPtrs {
 // parameter so every loop is unrolled without predicates; 16-byte loads (the
 // vectors come from cudaMalloc or PyTorch's allocator, 256-byte aligned)
 template <typename T, int NC>
-__global__ void __launch_bounds__(RED_THREADS) k_mdot(int64_t n, const T *__restrict__ w, VPtrs<T> V,
-                                                      double *__restrict__ part) {
+__global__ void __launch_bounds__(RED_THREADS) k_mdot(int64_t n, const T * w, VPtrs<T> V,
+                                                      double * part) {
+    grid_begin();
     typedef typename Acc<T>::type A;
     typedef typename Vec16<T>::type VT;
     constexpr int W = Vec16<T>::W;
@@ -427,8 +436,9 @@ __global__ void __launch_bounds__(RED_THREADS) k_mdot(int64_t n, const T *__rest
 
 // w -= sum_q h_q V_q ; partial (w, w)
 template <typename T, int NC>
-__global__ void __launch_bounds__(RED_THREADS) k_orth(int64_t n, T *__restrict__ w, VPtrs<T> V, Coef h,
-                                                      double *__restrict__ part) {
+__global__ void __launch_bounds__(RED_THREADS) k_orth(int64_t n, T * w, VPtrs<T> V, Coef h,
+                                                      double * part) {
+    grid_begin();
     typedef typename Acc<T>::type A;
     typedef typename Vec16<T>::type VT;
     constexpr int W = Vec16<T>::W;
@@ -484,7 +494,7 @@ static const OrthFn<T> *orth_table(std::integer_sequence<int, I...>) {
 
 // dst = a src. FP32 to FP32 in FP32 arithmetic, four elements per 16-byte
 // access (per-element FP64 arithmetic makes an FP32 stream FP64-bound)
-__device__ __forceinline__ void scale_f32(int64_t n, float *__restrict__ dst, const float *__restrict__ src,
+__device__ __forceinline__ void scale_f32(int64_t n, float * dst, const float * src,
                                           float a) {
     GRID_STRIDE(q, n / 4) {
         float4 v = reinterpret_cast<const float4 *>(src)[q];
@@ -507,14 +517,16 @@ template <typename T>
 static unsigned mdot_blocks(const Ctx *c) { return sizeof(T) == 8 ? (unsigned)((c->nred + 1) / 2) : (unsigned)c->nred; }
 
 template <typename T, typename S>
-__global__ void k_scale(int64_t n, T *__restrict__ dst, const S *__restrict__ src, double a) {
+__global__ void k_scale(int64_t n, T * dst, const S * src, double a) {
+    grid_begin();
     if constexpr (sizeof(T) == 4 && sizeof(S) == 4) scale_f32(n, dst, src, (float)a);
     else GRID_STRIDE(c, n) dst[c] = (T)(a * (double)src[c]);
 }
 
 // x += sum_i y_i Z_i
 template <typename T>
-__global__ void k_xupd(int64_t n, T *__restrict__ x, const T *const *__restrict__ Z, int ncols, Coef y) {
+__global__ void k_xupd(int64_t n, T * x, const T *const * Z, int ncols, Coef y) {
+    grid_begin();
     T yv[17];
 #pragma unroll
     for (int q = 0; q < 17; ++q) yv[q] = (T)y.v[q];
@@ -529,8 +541,9 @@ __global__ void k_xupd(int64_t n, T *__restrict__ x, const T *const *__restrict_
 
 // phi += a * ((double) d - mean) on FLUID and GHOST cells (FP64 update of the
 // outer iterate; the constant part of the correction is discarded)
-__global__ void k_add_scaled(int64_t n, const uint8_t *__restrict__ type, double *__restrict__ phi,
-                             const float *__restrict__ d, double a, const double *__restrict__ mean) {
+__global__ void k_add_scaled(int64_t n, const uint8_t * type, double * phi,
+                             const float * d, double a, const double * mean) {
+    grid_begin();
     const double m = *mean;
     GRID_STRIDE(c, n) if (type[c] != DEAD) phi[c] += a * ((double)d[c] - m);
 }
@@ -538,8 +551,9 @@ __global__ void k_add_scaled(int64_t n, const uint8_t *__restrict__ type, double
 // FLUID volume-weighted sum of an FP32 vector: FP32 volumes and products,
 // leaves of four consecutive cells in FP32, FP64 across leaves, warps and
 // blocks
-__global__ void k_fluid_volsum32(GridDev g, OpT<float> o, const uint8_t *__restrict__ type,
-                                 const float *__restrict__ x, double *__restrict__ part) {
+__global__ void k_fluid_volsum32(GridDev g, OpT<float> o, const uint8_t * type,
+                                 const float * x, double * part) {
+    grid_begin();
     __shared__ double sh[32];
     double acc = 0.0;
     GRID_STRIDE(q, (g.n + 3) / 4) {
@@ -559,7 +573,8 @@ __global__ void k_fluid_volsum32(GridDev g, OpT<float> o, const uint8_t *__restr
 // (FP32 vectors: leaves of four consecutive products in FP32, FP64
 // per-thread partials, FP64 across warps and blocks)
 template <typename T>
-__global__ void k_dotT(int64_t n, const T *__restrict__ a, const T *__restrict__ b, double *__restrict__ part) {
+__global__ void k_dotT(int64_t n, const T * a, const T * b, double * part) {
+    grid_begin();
     __shared__ double sh[32];
     double acc = 0.0;
     if constexpr (sizeof(T) == 4) {
@@ -579,8 +594,9 @@ __global__ void k_dotT(int64_t n, const T *__restrict__ a, const T *__restrict__
 // FP64 vector kernels: BiCGStab (scalars live on the device)
 // ---------------------------------------------------------------------------
 
-__global__ void k_dot64(int64_t n, const double *__restrict__ a, const double *__restrict__ b,
-                        double *__restrict__ part) {
+__global__ void k_dot64(int64_t n, const double * a, const double * b,
+                        double * part) {
+    grid_begin();
     __shared__ double sh[32];
     double acc = 0.0;
     GRID_STRIDE(c, n) acc += a[c] * b[c];
@@ -590,22 +606,26 @@ __global__ void k_dot64(int64_t n, const double *__restrict__ a, const double *_
 
 // beta = (rho1 / rho) (alpha / omega), rho = rho1; flag 1 on breakdown
 __global__ void k_bicg_beta(double *s) {
+    grid_begin();
     const double rho1 = s[B_RHO1], rho = s[B_RHO], om = s[B_OMEGA];
     if (!(rho != 0.0) || !(om != 0.0) || !isfinite(rho1)) { s[B_FLAG] = 1.0; s[B_BETA] = 0.0; }
     else s[B_BETA] = (rho1 / rho) * (s[B_ALPHA] / om);
     s[B_RHO] = rho1;
 }
 __global__ void k_bicg_alpha(double *s) {
+    grid_begin();
     const double den = s[B_DEN];
     if (!(den != 0.0) || !isfinite(den)) { s[B_FLAG] = 1.0; s[B_ALPHA] = 0.0; }
     else s[B_ALPHA] = s[B_RHO] / den;
 }
 __global__ void k_bicg_omega(double *s) {
+    grid_begin();
     const double tt = s[B_TT];
     s[B_OMEGA] = (tt > 0.0 && isfinite(tt)) ? s[B_TS] / tt : 0.0;
     if (!(s[B_OMEGA] != 0.0)) s[B_FLAG] = 1.0;
 }
 __global__ void k_bicg_init(double *s) {
+    grid_begin();
     s[B_RHO] = 1.0;
     s[B_ALPHA] = 1.0;
     s[B_OMEGA] = 1.0;
@@ -613,20 +633,23 @@ __global__ void k_bicg_init(double *s) {
 }
 
 // p = r + beta (p - omega v)
-__global__ void k_bicg_p(int64_t n, const double *__restrict__ r, double *__restrict__ p,
-                         const double *__restrict__ v, const double *__restrict__ s) {
+__global__ void k_bicg_p(int64_t n, const double * r, double * p,
+                         const double * v, const double * s) {
+    grid_begin();
     const double be = s[B_BETA], om = s[B_OMEGA];
     GRID_STRIDE(c, n) p[c] = r[c] + be * (p[c] - om * v[c]);
 }
 // sv = r - alpha v
-__global__ void k_bicg_s(int64_t n, const double *__restrict__ r, const double *__restrict__ v,
-                         double *__restrict__ sv, const double *__restrict__ s) {
+__global__ void k_bicg_s(int64_t n, const double * r, const double * v,
+                         double * sv, const double * s) {
+    grid_begin();
     const double al = s[B_ALPHA];
     GRID_STRIDE(c, n) sv[c] = r[c] - al * v[c];
 }
 // partial (t, s) and (t, t)
-__global__ void k_bicg_tdots(int64_t n, const double *__restrict__ t, const double *__restrict__ sv,
-                             double *__restrict__ part) {
+__global__ void k_bicg_tdots(int64_t n, const double * t, const double * sv,
+                             double * part) {
+    grid_begin();
     __shared__ double sh[32];
     double ts = 0.0, tt = 0.0;
     GRID_STRIDE(c, n) {
@@ -642,9 +665,10 @@ __global__ void k_bicg_tdots(int64_t n, const double *__restrict__ t, const doub
     }
 }
 // x += alpha ph + omega sh ; r = sv - omega t ; partial (r, r)
-__global__ void k_bicg_xr(int64_t n, double *__restrict__ x, const double *__restrict__ ph,
-                          const double *__restrict__ sh_, double *__restrict__ r, const double *__restrict__ sv,
-                          const double *__restrict__ t, const double *__restrict__ s, double *__restrict__ part) {
+__global__ void k_bicg_xr(int64_t n, double * x, const double * ph,
+                          const double * sh_, double * r, const double * sv,
+                          const double * t, const double * s, double * part) {
+    grid_begin();
     __shared__ double sh[32];
     const double al = s[B_ALPHA], om = s[B_OMEGA];
     double rr = 0.0;
@@ -684,7 +708,7 @@ __device__ __forceinline__ bool pos(float v) { return v > 0.f; }
 // sum over the open faces of T_f x_nb, and the diagonal sum T_f, at cell c
 // of a level (FINE: derived from the cell types and 1D metrics)
 template <typename T, bool FINE>
-__device__ __forceinline__ T k_offdiag(const MGLevel<T> &L, const T *__restrict__ x, int64_t c, int i, int j, int k,
+__device__ __forceinline__ T k_offdiag(const MGLevel<T> &L, const T * x, int64_t c, int i, int j, int k,
                                        T &d, T s0 = T(0)) {
     const int64_t sy = L.nx, sz = (int64_t)L.nx * L.ny;
     T s = s0;
@@ -718,7 +742,8 @@ __device__ __forceinline__ bool active(const MGLevel<T> &L, int64_t c) {
 }
 
 // open-face mask of the finest level
-__global__ void k_open_mask(GridDev g, const uint8_t *__restrict__ type, uint8_t *__restrict__ m) {
+__global__ void k_open_mask(GridDev g, const uint8_t * type, uint8_t * m) {
+    grid_begin();
     GRID_STRIDE(c, g.n) {
         int i, j, k;
         split3(g, (uint32_t)c, i, j, k);
@@ -745,7 +770,8 @@ __global__ void k_open_mask(GridDev g, const uint8_t *__restrict__ type, uint8_t
 // size tile_x allows, up to 512 threads.)
 template <typename T, bool FINE, bool OMEGA = false>
 __global__ void __launch_bounds__(512, 4)
-    k_rbgs(MGLevel<T> L, const T *__restrict__ f, T *__restrict__ x, int col, T w = T(1)) {
+    k_rbgs(MGLevel<T> L, const T * f, T * x, int col, T w = T(1)) {
+    grid_begin();
     const int64_t row = blockIdx.x;
     int j, k;
     row_jk((uint32_t)blockIdx.x, L.fny, L.ny, j, k);
@@ -791,7 +817,8 @@ __device__ __forceinline__ T fine_diag(const MGLevel<T> &L, unsigned msk, int i,
 // clearing x beforehand.
 template <typename T, bool FINE, bool OMEGA = false>
 __global__ void __launch_bounds__(512, 4)
-    k_rbgs_first(MGLevel<T> L, const T *__restrict__ f, T *__restrict__ x, int col, T w, int zero_rest) {
+    k_rbgs_first(MGLevel<T> L, const T * f, T * x, int col, T w, int zero_rest) {
+    grid_begin();
     const int64_t row = blockIdx.x;
     int j, k;
     row_jk((uint32_t)blockIdx.x, L.fny, L.ny, j, k);
@@ -890,7 +917,7 @@ struct QuadNb {
     float xe;
 };
 
-__device__ __forceinline__ QuadNb split_loads(const SplitLv<float> &L, const float *__restrict__ xo, int64_t base,
+__device__ __forceinline__ QuadNb split_loads(const SplitLv<float> &L, const float * xo, int64_t base,
                                               int h0, int j, int k, int pc) {
     const int64_t sy = L.H, sz = (int64_t)L.H * L.ny;
     QuadNb q;
@@ -941,8 +968,9 @@ __device__ __forceinline__ void split_offdiag(const SplitLv<float> &L, const Qua
 // for memory once.
 template <bool OMEGA, bool NAT>
 __global__ void __launch_bounds__(256, 5)
-    k_rbgs_split(SplitLv<float> L, const float *__restrict__ fq, const uint8_t *__restrict__ mq,
-                 const float *__restrict__ xo, float *__restrict__ xq, int col, float w, float *__restrict__ xn) {
+    k_rbgs_split(SplitLv<float> L, const float * fq, const uint8_t * mq,
+                 const float * xo, float * xq, int col, float w, float * xn) {
+    grid_begin();
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (q >= L.nq) return;
     int64_t base;
@@ -999,9 +1027,10 @@ __global__ void __launch_bounds__(256, 5)
 // elsewhere, and colour 1 as 0 (the values and zeros k_rbgs_first writes).
 template <bool OMEGA>
 __global__ void __launch_bounds__(256)
-    k_rbgs_first_split(SplitLv<float> L, const float *__restrict__ f0, const uint8_t *__restrict__ m0,
-                       float *__restrict__ fs0, float *__restrict__ fs1, float *__restrict__ xs0,
-                       float *__restrict__ xs1, float w) {
+    k_rbgs_first_split(SplitLv<float> L, const float * f0, const uint8_t * m0,
+                       float * fs0, float * fs1, float * xs0,
+                       float * xs1, float w) {
+    grid_begin();
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (q >= L.nq) return;
     int64_t base;
@@ -1048,8 +1077,9 @@ __global__ void __launch_bounds__(256)
 }
 
 // cell-ordered x from the two split colours (a V-cycle without post-smoothing)
-__global__ void k_split_merge(SplitLv<float> L, const float *__restrict__ xs0, const float *__restrict__ xs1,
-                              float *__restrict__ xn) {
+__global__ void k_split_merge(SplitLv<float> L, const float * xs0, const float * xs1,
+                              float * xn) {
+    grid_begin();
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (q >= L.nq) return;
     int64_t base;
@@ -1069,8 +1099,9 @@ __global__ void k_split_merge(SplitLv<float> L, const float *__restrict__ xs0, c
 }
 
 // per-colour copies of the level-0 open-face mask
-__global__ void k_split_mask(SplitLv<float> L, const uint8_t *__restrict__ m, uint8_t *__restrict__ m0,
-                             uint8_t *__restrict__ m1) {
+__global__ void k_split_mask(SplitLv<float> L, const uint8_t * m, uint8_t * m0,
+                             uint8_t * m1) {
+    grid_begin();
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (q >= L.nq) return;
     int64_t base;
@@ -1089,8 +1120,9 @@ __global__ void k_split_mask(SplitLv<float> L, const uint8_t *__restrict__ m, ui
 
 // coarse f_C = sum over children of (f - K x); coarse x_C = 0
 template <typename T, bool FINE>
-__global__ void k_resid_restrict(MGLevel<T> L, const T *__restrict__ f, const T *__restrict__ x, MGLevel<T> C,
+__global__ void k_resid_restrict(MGLevel<T> L, const T * f, const T * x, MGLevel<T> C,
                                  int fx, int fy, int fz) {
+    grid_begin();
     const int64_t row = blockIdx.x;
     int J, K;
     row_jk((uint32_t)blockIdx.x, C.fny, C.ny, J, K);
@@ -1121,7 +1153,8 @@ __global__ void k_resid_restrict(MGLevel<T> L, const T *__restrict__ f, const T 
 
 // x_c += x_parent(c) on active cells
 template <typename T, bool FINE>
-__global__ void k_prolong(MGLevel<T> L, T *__restrict__ x, MGLevel<T> C, int fx, int fy, int fz) {
+__global__ void k_prolong(MGLevel<T> L, T * x, MGLevel<T> C, int fx, int fy, int fz) {
+    grid_begin();
     const int64_t row = blockIdx.x;
     int j, k;
     row_jk((uint32_t)blockIdx.x, L.fny, L.ny, j, k);
@@ -1166,7 +1199,8 @@ __device__ __forceinline__ int xfer_axis(const int *I, const int *J, const T *w,
 
 // pn_c = 1 / (sum of the weights of the active coarse cells of c), 0 if c inactive
 template <typename T, bool FINE>
-__global__ void k_pnorm(MGLevel<T> L, MGLevel<T> C, Xfer<T> X, T *__restrict__ pn) {
+__global__ void k_pnorm(MGLevel<T> L, MGLevel<T> C, Xfer<T> X, T * pn) {
+    grid_begin();
     const int64_t row = blockIdx.x;
     int j, k;
     row_jk((uint32_t)blockIdx.x, L.fny, L.ny, j, k);
@@ -1200,8 +1234,9 @@ __global__ void k_pnorm(MGLevel<T> L, MGLevel<T> C, Xfer<T> X, T *__restrict__ p
 constexpr int RX_THREADS = 128;
 template <typename T, bool FINE>
 __global__ void __launch_bounds__(RX_THREADS)
-    k_resid_rx(MGLevel<T> L, const T *__restrict__ f, const T *__restrict__ x, const T *__restrict__ pn, Xfer<T> X,
-               int cnx, int fx, int zcol, T *__restrict__ tA) {
+    k_resid_rx(MGLevel<T> L, const T * f, const T * x, const T * pn, Xfer<T> X,
+               int cnx, int fx, int zcol, T * tA) {
+    grid_begin();
     __shared__ T sg[2 * RX_THREADS + 2];
     const int64_t row = blockIdx.x;
     int j, k;
@@ -1260,7 +1295,8 @@ __global__ void __launch_bounds__(RX_THREADS)
 // the coarse x extent and the fine y, z extents); x_C = 0, and f_C = 0 on
 // inactive coarse cells.
 template <typename T>
-__global__ void k_restrict_yz(MGLevel<T> C, const T *__restrict__ tA, int fny, Xfer<T> X) {
+__global__ void k_restrict_yz(MGLevel<T> C, const T * tA, int fny, Xfer<T> X) {
+    grid_begin();
     const int64_t row = blockIdx.x;
     int Jc, Kc;
     row_jk((uint32_t)blockIdx.x, C.fny, C.ny, Jc, Kc);
@@ -1290,7 +1326,8 @@ __global__ void k_restrict_yz(MGLevel<T> C, const T *__restrict__ tA, int fny, X
 // cells (restriction clears it, smoothing and the coarse solve write only
 // active cells), so no mask is needed here.
 template <typename T>
-__global__ void k_prolong_x(int fnx, MGLevel<T> C, Xfer<T> X, T *__restrict__ tB) {
+__global__ void k_prolong_x(int fnx, MGLevel<T> C, Xfer<T> X, T * tB) {
+    grid_begin();
     const int64_t row = blockIdx.x;
     const int i = blockIdx.y * blockDim.x + threadIdx.x;
     if (i >= fnx) return;
@@ -1304,8 +1341,9 @@ __global__ void k_prolong_x(int fnx, MGLevel<T> C, Xfer<T> X, T *__restrict__ tB
 // Prolongation, second and third axes, and the correction:
 // x_c += pn_c * sum_z wz sum_y wy tB on fine cells with pn_c > 0
 template <typename T>
-__global__ void k_prolong_yz(MGLevel<T> L, T *__restrict__ x, const T *__restrict__ tB, int cny, Xfer<T> X,
-                             const T *__restrict__ pn) {
+__global__ void k_prolong_yz(MGLevel<T> L, T * x, const T * tB, int cny, Xfer<T> X,
+                             const T * pn) {
+    grid_begin();
     const int64_t row = blockIdx.x;
     int j, k;
     row_jk((uint32_t)blockIdx.x, L.fny, L.ny, j, k);
@@ -1339,9 +1377,10 @@ __global__ void k_prolong_yz(MGLevel<T> L, T *__restrict__ x, const T *__restric
 // k_resid_rx on level 0 in colour-split storage (x and f split; the mask and
 // pn cell-ordered): the same cells, values and order of evaluation
 __global__ void __launch_bounds__(RX_THREADS)
-    k_resid_rx_split(MGLevel<float> L, const float *__restrict__ fs0, const float *__restrict__ fs1,
-                     const float *__restrict__ xs0, const float *__restrict__ xs1, const float *__restrict__ pn,
-                     Xfer<float> X, int cnx, int fx, int zcol, float *__restrict__ tA) {
+    k_resid_rx_split(MGLevel<float> L, const float * fs0, const float * fs1,
+                     const float * xs0, const float * xs1, const float * pn,
+                     Xfer<float> X, int cnx, int fx, int zcol, float * tA) {
+    grid_begin();
     __shared__ float sg[2 * RX_THREADS + 2];
     const int64_t row = blockIdx.x;
     int j, k;
@@ -1399,9 +1438,10 @@ __global__ void __launch_bounds__(RX_THREADS)
 // restriction then sums in the gather table's order, so the result equals
 // k_resid_rx bit for bit.
 __global__ void __launch_bounds__(256)
-    k_resid_rx_split4(MGLevel<float> L, SplitLv<float> S, const float *__restrict__ fs0, const float *__restrict__ fs1,
-                      const float *__restrict__ xs0, const float *__restrict__ xs1, const float *__restrict__ pn,
-                      Xfer<float> X, float *__restrict__ tA) {
+    k_resid_rx_split4(MGLevel<float> L, SplitLv<float> S, const float * fs0, const float * fs1,
+                      const float * xs0, const float * xs1, const float * pn,
+                      Xfer<float> X, float * tA) {
+    grid_begin();
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (q >= S.nq) return;
     const int H = S.H, nx = L.nx;
@@ -1510,8 +1550,9 @@ __global__ void __launch_bounds__(256)
 // 16-byte accesses; each cell gets the expression of k_prolong_yz (cells
 // with pn = 0 keep their value)
 __global__ void __launch_bounds__(256)
-    k_prolong_yz_split8(MGLevel<float> L, SplitLv<float> S, float *__restrict__ xs0, float *__restrict__ xs1,
-                        const float *__restrict__ tB, int cny, Xfer<float> X, const float *__restrict__ pn) {
+    k_prolong_yz_split8(MGLevel<float> L, SplitLv<float> S, float * xs0, float * xs1,
+                        const float * tB, int cny, Xfer<float> X, const float * pn) {
+    grid_begin();
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (q >= S.nq) return;
     int64_t base;
@@ -1604,7 +1645,7 @@ __device__ __forceinline__ T block_mean_active(T v, bool act, CoarseSmem<T> &S) 
 // with 32 sweeps: 25 us before, with one thread per cell of either colour and
 // the coefficients in shared memory.
 template <typename T>
-__device__ void coarse_solve_dev(const MGLevel<T> &L, const T *__restrict__ f, T *__restrict__ x, int sweeps,
+__device__ void coarse_solve_dev(const MGLevel<T> &L, const T * f, T * x, int sweeps,
                                  CoarseSmem<T> &S) {
     const int n = (int)L.n, tid = threadIdx.x;
     const int sy = L.nx, sz = L.nz > 1 ? L.nx * L.ny : 0;   // (at most n / 2: two cells or more per axis)
@@ -1668,7 +1709,8 @@ __device__ void coarse_solve_dev(const MGLevel<T> &L, const T *__restrict__ f, T
 // one block per column, and a cycle applies it: 128 dependent passes of about
 // 0.1 us each (FP64 0.4 us) become one small matrix-vector product.
 template <typename T>
-__global__ void __launch_bounds__(COARSE_MAX) k_coarse_matrix(MGLevel<T> L, int sweeps, T *__restrict__ M) {
+__global__ void __launch_bounds__(COARSE_MAX) k_coarse_matrix(MGLevel<T> L, int sweeps, T * M) {
+    grid_begin();
     __shared__ CoarseSmem<T> S;
     __shared__ T e[COARSE_MAX], x[COARSE_MAX];
     const int n = (int)L.n, col = blockIdx.x;
@@ -1683,8 +1725,9 @@ __global__ void __launch_bounds__(COARSE_MAX) k_coarse_matrix(MGLevel<T> L, int 
 namespace ibm {
 
 template <typename T>
-__global__ void __launch_bounds__(COARSE_MAX) k_coarse_apply(int n, const T *__restrict__ M, const T *__restrict__ f,
-                                                             T *__restrict__ x) {
+__global__ void __launch_bounds__(COARSE_MAX) k_coarse_apply(int n, const T * M, const T * f,
+                                                             T * x) {
+    grid_begin();
     coarse_apply_dev<T>(n, M, f, x);
 }
 
@@ -1860,7 +1903,8 @@ __device__ __forceinline__ void tail_prolong_yz(const TailLv<T> &A, int cny, int
 // cluster of ncta blocks (gridDim.x == ncta).
 template <typename T, bool OMEGA>
 __global__ void __launch_bounds__(TAIL_THREADS)
-    k_vtail(const TailLv<T> *__restrict__ A, int l0, int nl, int nu1, int nu2, const T *__restrict__ cm, T w, int ncta) {
+    k_vtail(const TailLv<T> * A, int l0, int nl, int nu1, int nu2, const T * cm, T w, int ncta) {
+    grid_begin();
     const int gt = blockIdx.x * TAIL_THREADS + threadIdx.x, nt = ncta * TAIL_THREADS;
     const int zcol = 1;   // each pre-smoothing sweep ends with colour 1
     const TailLv<T> &U = A[l0 - 1];
@@ -1904,7 +1948,8 @@ __global__ void __launch_bounds__(TAIL_THREADS)
 
 // q = K p ; partial (p, q) in FP64
 template <typename T, bool FINE>
-__global__ void k_spmv_dot(MGLevel<T> L, const T *__restrict__ p, T *__restrict__ q, double *__restrict__ part) {
+__global__ void k_spmv_dot(MGLevel<T> L, const T * p, T * q, double * part) {
+    grid_begin();
     __shared__ double sh[32];
     double acc = 0.0;
     GRID_STRIDE(c, L.n) {
@@ -1926,7 +1971,8 @@ __global__ void k_spmv_dot(MGLevel<T> L, const T *__restrict__ p, T *__restrict_
 }
 
 template <typename T>
-__global__ void k_dot(int64_t n, const T *__restrict__ a, const T *__restrict__ b, double *__restrict__ part) {
+__global__ void k_dot(int64_t n, const T * a, const T * b, double * part) {
+    grid_begin();
     __shared__ double sh[32];
     double acc = 0.0;
     GRID_STRIDE(c, n) acc += (double)a[c] * (double)b[c];
@@ -1935,8 +1981,9 @@ __global__ void k_dot(int64_t n, const T *__restrict__ a, const T *__restrict__ 
 }
 
 template <typename T>
-__global__ void k_axpy2(int64_t n, T *__restrict__ x, T *__restrict__ r, const T *__restrict__ p,
-                        const T *__restrict__ q, const double *__restrict__ scal) {
+__global__ void k_axpy2(int64_t n, T * x, T * r, const T * p,
+                        const T * q, const double * scal) {
+    grid_begin();
     const T a = (T)scal[S_AL];
     GRID_STRIDE(c, n) {
         x[c] += a * p[c];
@@ -1945,17 +1992,20 @@ __global__ void k_axpy2(int64_t n, T *__restrict__ x, T *__restrict__ r, const T
 }
 
 template <typename T>
-__global__ void k_pupd(int64_t n, T *__restrict__ p, const T *__restrict__ z, const double *__restrict__ scal) {
+__global__ void k_pupd(int64_t n, T * p, const T * z, const double * scal) {
+    grid_begin();
     const T b = (T)scal[S_BE];
     GRID_STRIDE(c, n) p[c] = z[c] + b * p[c];
 }
 
 // scalar updates (one thread)
 __global__ void k_alpha(double *scal) {
+    grid_begin();
     const double pq = scal[S_PQ];
     scal[S_AL] = (pq > 0.0 && isfinite(pq)) ? scal[S_RZ] / pq : 0.0;
 }
 __global__ void k_beta(double *scal) {
+    grid_begin();
     const double rz = scal[S_RZ];
     scal[S_BE] = (rz != 0.0 && isfinite(rz)) ? scal[S_RZN] / rz : 0.0;
     scal[S_RZ] = scal[S_RZN];
@@ -1963,8 +2013,9 @@ __global__ void k_beta(double *scal) {
 
 // preconditioner input / output conversion
 template <typename T>
-__global__ void k_pre_in(GridDev g, OpT<T> o, const uint8_t *__restrict__ type, const T *__restrict__ v,
-                         T *__restrict__ f) {
+__global__ void k_pre_in(GridDev g, OpT<T> o, const uint8_t * type, const T * v,
+                         T * f) {
+    grid_begin();
     GRID_STRIDE(c, g.n) {
         if (type[c] != FLUID) { f[c] = T(0); continue; }
         int i, j, k;
@@ -1974,8 +2025,9 @@ __global__ void k_pre_in(GridDev g, OpT<T> o, const uint8_t *__restrict__ type, 
     }
 }
 // FP32 input four cells at a time (rows of a multiple of four cells)
-__global__ void k_pre_in4(GridDev g, OpT<float> o, const uint8_t *__restrict__ type, const float *__restrict__ v,
-                          float *__restrict__ f) {
+__global__ void k_pre_in4(GridDev g, OpT<float> o, const uint8_t * type, const float * v,
+                          float * f) {
+    grid_begin();
     GRID_STRIDE(q, g.n / 4) {
         const int64_t c = 4 * q;
         const uchar4 t4 = reinterpret_cast<const uchar4 *>(type)[q];
@@ -1991,7 +2043,8 @@ __global__ void k_pre_in4(GridDev g, OpT<float> o, const uint8_t *__restrict__ t
     }
 }
 template <typename T>
-__global__ void k_pre_out(int64_t n, const uint8_t *__restrict__ type, const T *__restrict__ x, T *__restrict__ z) {
+__global__ void k_pre_out(int64_t n, const uint8_t * type, const T * x, T * z) {
+    grid_begin();
     int64_t n0 = 0;
     if constexpr (sizeof(T) == 4) {
         n0 = n / 4 * 4;
@@ -2007,8 +2060,9 @@ __global__ void k_pre_out(int64_t n, const uint8_t *__restrict__ type, const T *
 }
 // ghost rows of the preconditioner: z_g = v_g + sum over FLUID corners wp z_m
 template <typename T>
-__global__ void k_pre_ghost(GhostDev gh, const T *__restrict__ wp, const uint8_t *__restrict__ type,
-                            const T *__restrict__ v, T *__restrict__ z) {
+__global__ void k_pre_ghost(GhostDev gh, const T * wp, const uint8_t * type,
+                            const T * v, T * z) {
+    grid_begin();
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (q >= gh.ng) return;
     const int64_t gi = gh.gidx[q];
@@ -2047,9 +2101,10 @@ __device__ __forceinline__ T band_value(const GridDev &g, const GhostDev &gh, co
 // tmp = the new band values (a pass over the whole band; k_band_scatter
 // then writes them into z)
 template <typename T>
-__global__ void k_band_jacobi(GridDev g, GhostDev gh, OpT<T> o, int64_t nb, const int64_t *__restrict__ band,
-                              const int64_t *__restrict__ band_g, const T *__restrict__ v, const T *__restrict__ z,
-                              T omega, T *__restrict__ tmp) {
+__global__ void k_band_jacobi(GridDev g, GhostDev gh, OpT<T> o, int64_t nb, const int64_t * band,
+                              const int64_t * band_g, const T * v, const T * z,
+                              T omega, T * tmp) {
+    grid_begin();
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (q < nb) tmp[q] = band_value<T>(g, gh, o, band, band_g, v, z, omega, q);
 }
@@ -2060,8 +2115,9 @@ __global__ void k_band_jacobi(GridDev g, GhostDev gh, OpT<T> o, int64_t nb, cons
 constexpr int BAND_BLOCK = 1024, BAND_PER_THREAD = 8;
 template <typename T>
 __global__ void __launch_bounds__(BAND_BLOCK)
-    k_band_block(GridDev g, GhostDev gh, OpT<T> o, int64_t nb, const int64_t *__restrict__ band,
-                 const int64_t *__restrict__ band_g, const T *__restrict__ v, T *z, T omega, int sweeps) {
+    k_band_block(GridDev g, GhostDev gh, OpT<T> o, int64_t nb, const int64_t * band,
+                 const int64_t * band_g, const T * v, T *z, T omega, int sweeps) {
+    grid_begin();
     T nv[BAND_PER_THREAD];
     for (int s = 0; s < sweeps; ++s) {
 #pragma unroll
@@ -2079,8 +2135,9 @@ __global__ void __launch_bounds__(BAND_BLOCK)
     }
 }
 template <typename T>
-__global__ void k_band_scatter(int64_t nb, const int64_t *__restrict__ band, const T *__restrict__ tmp,
-                               T *__restrict__ z) {
+__global__ void k_band_scatter(int64_t nb, const int64_t * band, const T * tmp,
+                               T * z) {
+    grid_begin();
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (q < nb) z[band[q]] = tmp[q];
 }
@@ -2089,8 +2146,9 @@ __global__ void k_band_scatter(int64_t nb, const int64_t *__restrict__ band, con
 
 // level 0 open face areas: face on the low side of cell c along each axis is
 // open when c and its low neighbour are both FLUID
-__global__ void k_open_area0(GridDev g, const uint8_t *__restrict__ type, double *__restrict__ ox,
-                             double *__restrict__ oy, double *__restrict__ oz) {
+__global__ void k_open_area0(GridDev g, const uint8_t * type, double * ox,
+                             double * oy, double * oz) {
+    grid_begin();
     GRID_STRIDE(c, g.n) {
         int i, j, k;
         split3(g, (uint32_t)c, i, j, k);
@@ -2104,10 +2162,11 @@ __global__ void k_open_area0(GridDev g, const uint8_t *__restrict__ type, double
 
 // coarse open areas: the coarse low face gathers the low faces of the
 // children that touch it
-__global__ void k_open_area_coarsen(int nx, int ny, int nz, const double *__restrict__ ox,
-                                    const double *__restrict__ oy, const double *__restrict__ oz, int cnx, int cny,
-                                    int cnz, int fx, int fy, int fz, double *__restrict__ cx, double *__restrict__ cy,
-                                    double *__restrict__ cz) {
+__global__ void k_open_area_coarsen(int nx, int ny, int nz, const double * ox,
+                                    const double * oy, const double * oz, int cnx, int cny,
+                                    int cnz, int fx, int fy, int fz, double * cx, double * cy,
+                                    double * cz) {
+    grid_begin();
     const int64_t cn = (int64_t)cnx * cny * cnz;
     GRID_STRIDE(cc, cn) {
         const int64_t t = cc / cnx;
@@ -2137,10 +2196,11 @@ __global__ void k_open_area_coarsen(int nx, int ny, int nz, const double *__rest
 
 // T = open area / centre spacing
 template <typename T>
-__global__ void k_level_coef(int nx, int ny, int nz, const double *__restrict__ ox, const double *__restrict__ oy,
-                             const double *__restrict__ oz, const double *__restrict__ hx,
-                             const double *__restrict__ hy, const double *__restrict__ hz, T *__restrict__ tx,
-                             T *__restrict__ ty, T *__restrict__ tz) {
+__global__ void k_level_coef(int nx, int ny, int nz, const double * ox, const double * oy,
+                             const double * oz, const double * hx,
+                             const double * hy, const double * hz, T * tx,
+                             T * ty, T * tz) {
+    grid_begin();
     const int64_t n = (int64_t)nx * ny * nz;
     GRID_STRIDE(c, n) {
         const int64_t t = c / nx;
@@ -2153,6 +2213,7 @@ __global__ void k_level_coef(int nx, int ny, int nz, const double *__restrict__ 
 // D = sum of the six faces; dinv = 1/D (0 when D = 0)
 template <typename T>
 __global__ void k_level_diag(MGLevel<T> L) {
+    grid_begin();
     GRID_STRIDE(c, L.n) {
         const int64_t t = c / L.nx;
         const int i = (int)(c - t * L.nx), j = (int)(t % L.ny), k = (int)(t / L.ny);
@@ -2167,11 +2228,13 @@ __global__ void k_level_diag(MGLevel<T> L) {
 }
 
 // band: FLUID cells within band_width faces of a ghost cell, plus the ghosts
-__global__ void k_band_seed(int64_t n, const uint8_t *__restrict__ type, uint8_t *__restrict__ f) {
+__global__ void k_band_seed(int64_t n, const uint8_t * type, uint8_t * f) {
+    grid_begin();
     GRID_STRIDE(c, n) f[c] = type[c] == GHOST;
 }
-__global__ void k_band_dilate(GridDev g, const uint8_t *__restrict__ type, const uint8_t *__restrict__ in,
-                              uint8_t *__restrict__ out) {
+__global__ void k_band_dilate(GridDev g, const uint8_t * type, const uint8_t * in,
+                              uint8_t * out) {
+    grid_begin();
     GRID_STRIDE(c, g.n) {
         int i, j, k;
         split3(g, (uint32_t)c, i, j, k);
@@ -2185,8 +2248,9 @@ __global__ void k_band_dilate(GridDev g, const uint8_t *__restrict__ type, const
     }
 }
 // band_g[q] = position of band[q] in the ascending ghost list, or -1
-__global__ void k_band_gpos(int64_t nb, const int64_t *__restrict__ band, int64_t ng, const int64_t *__restrict__ gidx,
-                            int64_t *__restrict__ band_g) {
+__global__ void k_band_gpos(int64_t nb, const int64_t * band, int64_t ng, const int64_t * gidx,
+                            int64_t * band_g) {
+    grid_begin();
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (q >= nb) return;
     const int64_t c = band[q];
@@ -2754,6 +2818,7 @@ template <typename T>
 static ibm_status launch_bottom(Ctx *c, const BotPar<T> &P) {
     const void *k = bottom_kernel<T>(c);
     const size_t dyn = (size_t)P.bytes;
+    const bool ahead = overlap_launch(c);   // (the attribute calls put nothing on the stream)
     IBM_CUDA(c, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, BOT_SMEM));
     IBM_CUDA(c, cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchConfig_t cfg = {};
@@ -2761,18 +2826,20 @@ static ibm_status launch_bottom(Ctx *c, const BotPar<T> &P) {
     cfg.blockDim = dim3(BOT_THREADS, 1, 1);
     cfg.dynamicSmemBytes = dyn;
     cfg.stream = c->s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)P.ncta;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = ahead ? 2 : 1;
     void *args[1] = {const_cast<BotPar<T> *>(&P)};
     kt_begin(c, -1);
     ++c->nlaunch;
     IBM_CUDA(c, cudaLaunchKernelExC(&cfg, k, args));
+    c->chain = true;
     kt_end(c, -1);
-    IBM_LAUNCHED(c);
     return IBM_OK;
 }
 
@@ -2974,7 +3041,8 @@ static ibm_status vcycle_graph(Ctx *c, MGHier<T> &H, T *out) {
 // bit-reversed order so large and small factors alternate. A fixed linear
 // operator: usable as the right preconditioner of BiCGStab.
 template <typename T, bool FINE>
-__global__ void k_srj_sweep(MGLevel<T> L, const T *__restrict__ f, const T *__restrict__ x, T *__restrict__ xn, T w) {
+__global__ void k_srj_sweep(MGLevel<T> L, const T * f, const T * x, T * xn, T w) {
+    grid_begin();
     GRID_STRIDE(c, L.n) {
         T v = T(0);
         if (active<T, FINE>(L, c)) {
@@ -3254,7 +3322,8 @@ static ibm_status apply_prec(Ctx *c, const double *v, double *z);
 
 // FP32 storage of mixed mode: operator coefficients, ghost weights, Krylov
 // vectors (allocated on first use)
-__global__ void k_to_float(int64_t n, const double *__restrict__ a, float *__restrict__ b) {
+__global__ void k_to_float(int64_t n, const double * a, float * b) {
+    grid_begin();
     GRID_STRIDE(q, n) b[q] = (float)a[q];
 }
 static ibm_status ensure_mixed(Ctx *c) {
@@ -3503,16 +3572,19 @@ ibm_status cond_open(Ctx *c, cudaGraphConditionalNodeType type, cudaGraphConditi
 ibm_status cond_close(Ctx *c, CondScope *sc) {
     cudaGraph_t g = nullptr;
     const cudaError_t e = cudaStreamEndCapture(c->s, &g);
+    c->chain = false;
     c->s = sc->outer;
     --c->side_depth;
     if (e != cudaSuccess) return c->fail(IBM_ERR_CUDA, std::string("conditional body capture: ") + cudaGetErrorString(e));
     return IBM_OK;
 }
 
-__global__ void k_set_cond(cudaGraphConditionalHandle h, const int *flag) { cudaGraphSetConditional(h, *flag ? 1u : 0u); }
+__global__ void k_set_cond(cudaGraphConditionalHandle h, const int *flag) {
+    grid_begin(); cudaGraphSetConditional(h, *flag ? 1u : 0u); }
 
 template <typename T, typename S>
-__global__ void k_scale_dev(int64_t n, T *__restrict__ dst, const S *__restrict__ src, const double *__restrict__ a) {
+__global__ void k_scale_dev(int64_t n, T * dst, const S * src, const double * a) {
+    grid_begin();
     const double f = *a;
     if constexpr (sizeof(T) == 4 && sizeof(S) == 4) scale_f32(n, dst, src, (float)f);
     else GRID_STRIDE(c, n) dst[c] = (T)(f * (double)src[c]);
@@ -3520,8 +3592,9 @@ __global__ void k_scale_dev(int64_t n, T *__restrict__ dst, const S *__restrict_
 
 // w -= sum_q h_q V_q with h in device memory; partial (w, w)
 template <typename T, int NC>
-__global__ void __launch_bounds__(RED_THREADS) k_orth_dev(int64_t n, T *__restrict__ w, VPtrs<T> V,
-                                                          const double *__restrict__ h, double *__restrict__ part) {
+__global__ void __launch_bounds__(RED_THREADS) k_orth_dev(int64_t n, T * w, VPtrs<T> V,
+                                                          const double * h, double * part) {
+    grid_begin();
     typedef typename Acc<T>::type A;
     typedef typename Vec16<T>::type VT;
     constexpr int W = Vec16<T>::W;
@@ -3572,7 +3645,8 @@ static const OrthDevFn<T> *orth_dev_table(std::integer_sequence<int, I...>) {
 
 // x += sum_{q < ncols} y_q Z_q with y and ncols from the control block
 template <typename T>
-__global__ void k_xupd_dev(int64_t n, T *__restrict__ x, VPtrs<T> Z, const DevFG *__restrict__ F) {
+__global__ void k_xupd_dev(int64_t n, T * x, VPtrs<T> Z, const DevFG * F) {
+    grid_begin();
     const int nc = F->ncols;
     if (nc <= 0) return;
     T yv[16];
@@ -3587,20 +3661,23 @@ __global__ void k_xupd_dev(int64_t n, T *__restrict__ x, VPtrs<T> Z, const DevFG
     }
 }
 
-__global__ void k_zero_if(int64_t n, double *__restrict__ x, const int *__restrict__ flag) {
+__global__ void k_zero_if(int64_t n, double * x, const int * flag) {
+    grid_begin();
     if (!*flag) return;
     GRID_STRIDE(c, n) x[c] = 0.0;
 }
 
 // phi += rn * ((double) d - mean) on FLUID and GHOST cells, rn from the control block
-__global__ void k_add_scaled_dev(int64_t n, const uint8_t *__restrict__ type, double *__restrict__ phi,
-                                 const float *__restrict__ d, const DevFG *__restrict__ R,
-                                 const double *__restrict__ mean) {
+__global__ void k_add_scaled_dev(int64_t n, const uint8_t * type, double * phi,
+                                 const float * d, const DevFG * R,
+                                 const double * mean) {
+    grid_begin();
     const double a = R->rn, m = *mean;
     GRID_STRIDE(c, n) if (type[c] != DEAD) phi[c] += a * ((double)d[c] - m);
 }
 
 __global__ void k_fg_setup(DevFG *F, const double *bn2, double rtol, int maxit) {
+    grid_begin();
     const double bnorm = sqrt(*bn2);
     F->bnorm = bnorm;
     // a non-finite right-hand side is reported, not solved (phi is zeroed)
@@ -3621,10 +3698,12 @@ __global__ void k_fg_setup(DevFG *F, const double *bn2, double rtol, int maxit) 
     F->ncols = 0;
 }
 
-__global__ void k_copy_inner_rtol(DevFG *R, double v) { R->inner_rtol = v; }
+__global__ void k_copy_inner_rtol(DevFG *R, double v) {
+    grid_begin(); R->inner_rtol = v; }
 
 // restart test at the top of a cycle: beta = ||r||, rel = beta / bnorm
 __global__ void k_fg_cycle(DevFG *F, const double *rn2, cudaGraphConditionalHandle h) {
+    grid_begin();
     const double beta = sqrt(*rn2);
     F->rel = F->zero ? 0.0 : beta / F->bnorm;
     if (!isfinite(F->rel)) F->status = IBM_ERR_DIVERGED;
@@ -3650,6 +3729,7 @@ __global__ void k_fg_cycle(DevFG *F, const double *rn2, cudaGraphConditionalHand
 // in *wa2; a second pass when ||w||^2 dropped to eta2 of its value before the
 // pass (||w_after||^2 + sum h^2) or below
 __global__ void k_fg_post1(DevFG *F, const double *md, const double *wa2, int j, double eta2) {
+    grid_begin();
     double h2 = 0.0;
     for (int i = 0; i <= j; ++i) {
         F->hcol[i] = md[i];
@@ -3661,6 +3741,7 @@ __global__ void k_fg_post1(DevFG *F, const double *md, const double *wa2, int j,
 }
 
 __global__ void k_fg_post2(DevFG *F, const double *md, const double *wa2, int j) {
+    grid_begin();
     for (int i = 0; i <= j; ++i) F->hcol[i] += md[i];
     F->wa = *wa2;
 }
@@ -3668,6 +3749,7 @@ __global__ void k_fg_post2(DevFG *F, const double *md, const double *wa2, int j)
 // Hessenberg column j, Givens rotations, residual estimate and the decision
 // to take step j + 1
 __global__ void k_fg_givens(DevFG *F, int j, int m) {
+    grid_begin();
     const double hn = sqrt(F->wa);
     F->outer += 1;
     double *H = F->H;
@@ -3699,6 +3781,7 @@ __global__ void k_fg_givens(DevFG *F, int j, int m) {
 
 // back substitution H y = g over the steps taken
 __global__ void k_fg_ysolve(DevFG *F, int m) {
+    grid_begin();
     const int jl = F->jlast;
     if (F->status != 0 || jl < 0) {
         if (F->status == 0) F->status = IBM_ERR_NOT_CONVERGED;
@@ -3715,6 +3798,7 @@ __global__ void k_fg_ysolve(DevFG *F, int m) {
 
 // refinement test: rel = ||P(b - A phi)|| / ||b||; sets up the FP32 cycle
 __global__ void k_ref_start(DevFG *R, DevFG *F, const double *rn2, cudaGraphConditionalHandle h) {
+    grid_begin();
     const double rn = sqrt(*rn2);
     R->rn = rn;
     R->rel = R->zero ? 0.0 : rn / R->bnorm;
@@ -3741,6 +3825,7 @@ __global__ void k_ref_start(DevFG *R, DevFG *F, const double *rn2, cudaGraphCond
 }
 
 __global__ void k_ref_after(DevFG *R, const DevFG *F) {
+    grid_begin();
     R->steps += F->outer;
     if (F->outer == 0) {
         R->status = IBM_ERR_NOT_CONVERGED;
@@ -3920,6 +4005,7 @@ ibm_status poisson_solve_dev(Ctx *c, const double *rhs, double *phi, double rtol
 // per-step statistics of the captured step: Poisson iterations and status,
 // Helmholtz sweeps (hsw[0..2], status in hsw[3]), ghost refresh status
 __global__ void k_step_stats(DevStats *S, const DevFG *R, const int *hsw) {
+    grid_begin();
     S->steps += 1;
     S->outer += R->refinements > 0 ? R->steps : R->outer;
     S->helm_sweeps += hsw[0] + hsw[1] + hsw[2];
@@ -3977,8 +4063,9 @@ static inline const MdotFn<T> *mdot_fns() {
 }
 
 // rhs - mean on FLUID cells, 0 elsewhere (the solver's P rhs)
-__global__ void k_hist_bp(int64_t n, const uint8_t *__restrict__ type, const double *__restrict__ rhs,
-                          const HistCtl *__restrict__ H, double *__restrict__ bp) {
+__global__ void k_hist_bp(int64_t n, const uint8_t * type, const double * rhs,
+                          const HistCtl * H, double * bp) {
+    grid_begin();
     const double m = H->mean;
     GRID_STRIDE(c, n) bp[c] = type[c] == FLUID ? rhs[c] - m : 0.0;
 }
@@ -3986,6 +4073,7 @@ __global__ void k_hist_bp(int64_t n, const uint8_t *__restrict__ type, const dou
 // c over the m active slots (0 elsewhere, and everywhere if the factorisation
 // meets a non-positive pivot)
 __global__ void k_hist_solve(HistCtl *H) {
+    grid_begin();
     const int m = H->count;
     for (int i = 0; i < HIST_MAX; ++i) H->c[i] = 0.0;
     if (m == 0) return;
@@ -4023,8 +4111,9 @@ __global__ void k_hist_solve(HistCtl *H) {
 
 // phi = sum over the active slots of c_i X_i (phi untouched with no pairs);
 // slot i starts at X + i ld
-__global__ void k_hist_guess(int64_t n, int64_t ld, const HistCtl *__restrict__ H, const double *__restrict__ X,
-                             double *__restrict__ phi) {
+__global__ void k_hist_guess(int64_t n, int64_t ld, const HistCtl * H, const double * X,
+                             double * phi) {
+    grid_begin();
     const int m = H->count;
     if (m == 0) return;
     GRID_STRIDE(c, n) {
@@ -4035,8 +4124,9 @@ __global__ void k_hist_guess(int64_t n, int64_t ld, const HistCtl *__restrict__ 
 }
 
 // the pair of this step into the current slot
-__global__ void k_hist_insert(int64_t n, int64_t ld, const HistCtl *__restrict__ H, const double *__restrict__ phi,
-                              const double *__restrict__ bp, double *__restrict__ X, double *__restrict__ B) {
+__global__ void k_hist_insert(int64_t n, int64_t ld, const HistCtl * H, const double * phi,
+                              const double * bp, double * X, double * B) {
+    grid_begin();
     const int64_t off = (int64_t)H->slot * ld;
     GRID_STRIDE(c, n) {
         X[off + c] = phi[c];
@@ -4046,6 +4136,7 @@ __global__ void k_hist_insert(int64_t n, int64_t ld, const HistCtl *__restrict__
 
 // Gram row and column of the new pair; advance the ring
 __global__ void k_hist_advance(HistCtl *H, int L) {
+    grid_begin();
     const int k = H->slot;
     for (int i = 0; i < L; ++i) {
         if (i == k) continue;

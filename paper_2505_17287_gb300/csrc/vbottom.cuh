@@ -283,6 +283,7 @@ __device__ __forceinline__ void bot_up(const BotPar<T> &P, const BotLv<T> &v, co
 // the images of k_vbottom's blocks (cleared beforehand), one block each
 template <typename T, bool D3>
 __global__ void __launch_bounds__(BOT_THREADS) k_bottom_image(const __grid_constant__ BotPar<T> P, uint4 *image) {
+    grid_begin();
     const int r = blockIdx.x, tid = threadIdx.x;
     T *sm = reinterpret_cast<T *>(reinterpret_cast<char *>(image) + (size_t)r * P.sbytes);
     int *si = reinterpret_cast<int *>(sm + P.oint);
@@ -332,6 +333,7 @@ __global__ void __launch_bounds__(BOT_THREADS, 1) k_vbottom(const __grid_constan
     extern __shared__ double bot_smem[];
     T *sm = reinterpret_cast<T *>(bot_smem);
     const int *si = reinterpret_cast<const int *>(sm + P.oint);
+    grid_release();
     BotCtx C{cg::this_cluster(), false};
     const int r = P.ncta > 1 ? (int)C.cl.block_rank() : 0, tid = threadIdx.x;
     {
@@ -346,6 +348,9 @@ __global__ void __launch_bounds__(BOT_THREADS, 1) k_vbottom(const __grid_constan
                 for (int q = tid; q < 2 * v.sx; q += BOT_THREADS) sm[v.ox + q] = T(0);
         }
     }
+    // (the image is older than the previous kernel: it is written while the
+    // stream is idle or before a copy that every kernel after it waits for)
+    grid_wait();
     {
         const BotLv<T> &v = P.lv[0];
         int p0, np;
