@@ -189,7 +189,8 @@ struct Ctx {
     int64_t nband = 0;
     int64_t *band = nullptr;      // cell index
     int64_t *band_g = nullptr;    // position in gidx, -1 for FLUID cells
-    double *btmp = nullptr;
+    int *band_n = nullptr;        // band positions of each cell's neighbours (band.cuh)
+    double *btmp = nullptr;       // the sweeps' vectors
     std::vector<LevelGeom> lg;
     std::vector<double *> lhx, lhy, lhz;   // per level centre spacing (device)
     // trilinear transfer from level l-1 to level l, per axis (entry 0 unused):

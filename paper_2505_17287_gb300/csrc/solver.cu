@@ -2074,73 +2074,9 @@ __global__ void k_pre_ghost(GhostDev gh, const T * wp, const uint8_t * type,
     z[gi] = s;
 }
 
-// one damped Jacobi pass of the full operator on the band, in precision T
-// (o: the operator of op_of<T>; the FP64 A_row reads its stored diagonal dg,
-// the FP32 one the per-axis sums): the new value of band cell q. z is read
-// through a plain pointer: the single-block form below writes it in place.
-template <typename T>
-__device__ __forceinline__ T band_value(const GridDev &g, const GhostDev &gh, const OpT<T> &o, const int64_t *band,
-                                        const int64_t *band_g, const T *v, const T *z, T omega, int64_t q) {
-    const int64_t c = band[q];
-    const int64_t gq = band_g[q];
-    T res, diag;
-    if (gq >= 0) {
-        T s = z[c];
-        for (int m = 0; m < 8; ++m) s -= o.wp[8 * gq + m] * z[gh.sidx[8 * gq + m]];
-        res = v[c] - s;
-        diag = T(1);
-    } else {
-        int i, j, k;
-        split3(g, (uint32_t)c, i, j, k);
-        res = v[c] - A_row<T>(g, o, z, c, i, j, k);
-        if constexpr (sizeof(T) == 8) diag = -o.dg[c];
-        else diag = -(o.cxs[i] + o.cys[j] + (g.ndim == 3 ? o.czs[k] : T(0)));
-    }
-    return z[c] + omega * res / diag;
-}
-// tmp = the new band values (a pass over the whole band; k_band_scatter
-// then writes them into z)
-template <typename T>
-__global__ void k_band_jacobi(GridDev g, GhostDev gh, OpT<T> o, int64_t nb, const int64_t * band,
-                              const int64_t * band_g, const T * v, const T * z,
-                              T omega, T * tmp) {
-    grid_begin();
-    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q < nb) tmp[q] = band_value<T>(g, gh, o, band, band_g, v, z, omega, q);
-}
-// All sweeps in one block of BAND_BLOCK threads, for bands of at most
-// BAND_BLOCK * BAND_PER_THREAD cells: each sweep computes every new value
-// into registers, then (after a block barrier) writes them; the values
-// equal those of the two-kernel form.
-constexpr int BAND_BLOCK = 1024, BAND_PER_THREAD = 8;
-template <typename T>
-__global__ void __launch_bounds__(BAND_BLOCK)
-    k_band_block(GridDev g, GhostDev gh, OpT<T> o, int64_t nb, const int64_t * band,
-                 const int64_t * band_g, const T * v, T *z, T omega, int sweeps) {
-    grid_begin();
-    T nv[BAND_PER_THREAD];
-    for (int s = 0; s < sweeps; ++s) {
-#pragma unroll
-        for (int u = 0; u < BAND_PER_THREAD; ++u) {
-            const int64_t q = threadIdx.x + (int64_t)u * BAND_BLOCK;
-            if (q < nb) nv[u] = band_value<T>(g, gh, o, band, band_g, v, z, omega, q);
-        }
-        __syncthreads();
-#pragma unroll
-        for (int u = 0; u < BAND_PER_THREAD; ++u) {
-            const int64_t q = threadIdx.x + (int64_t)u * BAND_BLOCK;
-            if (q < nb) z[band[q]] = nv[u];
-        }
-        __syncthreads();
-    }
-}
-template <typename T>
-__global__ void k_band_scatter(int64_t nb, const int64_t * band, const T * tmp,
-                               T * z) {
-    grid_begin();
-    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q < nb) z[band[q]] = tmp[q];
-}
+}  // namespace ibm
+#include "band.cuh"
+namespace ibm {
 
 // level coefficient construction ------------------------------------------
 
@@ -2528,10 +2464,14 @@ ibm_status mg_build(Ctx *c) {
     c->btmp = nullptr;
     IBM_TRY(compact_flags(c, f0, &c->band, &c->nband));
     c->band_g = (int64_t *)dev_alloc(c, sizeof(int64_t) * (c->nband > 0 ? c->nband : 1));
-    c->btmp = (double *)dev_alloc(c, sizeof(double) * (c->nband > 0 ? c->nband : 1));
-    if (!c->band_g || !c->btmp) return c->fail(IBM_ERR_OOM, "band allocation failed");
+    dev_free(c, c->band_n);
+    c->btmp = (double *)dev_alloc(c, sizeof(double) * 10 * (c->nband > 0 ? c->nband : 1));
+    c->band_n = (int *)dev_alloc(c, sizeof(int) * 8 * (c->nband > 0 ? c->nband : 1));
+    if (!c->band_g || !c->btmp || !c->band_n) return c->fail(IBM_ERR_OOM, "band allocation failed");
     if (c->nband > 0) {
         KL(-1, k_band_gpos, (unsigned)((c->nband + 255) / 256), 256, c->nband, c->band, c->ng, c->gidx, c->band_g);
+        KL(-1, k_band_nbr, dim3((unsigned)((c->nband + 255) / 256), 8), 256, c->g, c->gh, (int)c->nband, c->band, c->band_g,
+           c->band_n);
         IBM_LAUNCHED(c);
     }
     IBM_CUDA(c, cudaStreamSynchronize(c->s));
@@ -3132,6 +3072,62 @@ static ibm_status pcg(Ctx *c, MGHier<T> &H, int iters) {
     return IBM_OK;
 }
 
+// The ghost rows of z and the band sweeps. One block while it can own the
+// band (2048 cells in FP32, 1024 in FP64), a cluster of up to 16 blocks up to
+// 16 times that, one launch per sweep above.
+template <typename T>
+static ibm_status band_sweeps(Ctx *c, const T *v, T *z) {
+    const OpT<T> o = op_of<T>(c);
+    const BandDev b{(int)c->nband, c->band, c->band_g, c->band_n};
+    const T omega = (T)c->opts.band_omega;
+    const int sweeps = c->opts.band_sweeps;
+    T *buf = reinterpret_cast<T *>(c->btmp);   // (10 doubles per band cell: room for either precision)
+    constexpr int MAX = BandRows<T>::MAX;
+    const int64_t one = (int64_t)BAND_THREADS * MAX;
+    int ncta = 1;
+    if (b.nb > one)
+        while (ncta < c->bot_ctas && (int64_t)ncta * BAND_THREADS < b.nb) ncta *= 2;
+    const int it = (int)((b.nb + (int64_t)ncta * BAND_THREADS - 1) / ((int64_t)ncta * BAND_THREADS));
+    if (it > MAX) {
+        const unsigned gb = (unsigned)((b.nb + 255) / 256);
+        T *cur = buf, *nxt = buf + b.nb, *zh = buf + 2 * (size_t)b.nb;
+        KL(-1, k_band_start<T>, gb, 256, c->g, c->gh, o, b, c->type, v, z, omega, cur, zh);
+        for (int s = 0; s < sweeps; ++s) {
+            KL(-1, k_band_sweep<T>, gb, 256, c->g, c->gh, o, b, v, omega, cur, zh, nxt, s + 1 == sweeps ? z : nullptr);
+            std::swap(cur, nxt);
+        }
+        IBM_LAUNCHED(c);
+        return IBM_OK;
+    }
+    typedef void (*Fn)(GridDev, GhostDev, OpT<T>, BandDev, const uint8_t *, const T *, T *, T, int, T *, int);
+    Fn fn;
+    if (ncta == 1) fn = it == 1 ? k_band_sweeps<T, 1, true> : (it == 2 ? k_band_sweeps<T, 2, true> : k_band_sweeps<T, MAX, true>);
+    else fn = it == 1 ? k_band_sweeps<T, 1, false> : (it == 2 ? k_band_sweeps<T, 2, false> : k_band_sweeps<T, MAX, false>);
+    const bool ahead = overlap_launch(c);
+    const size_t dyn = ncta == 1 ? sizeof(T) * 10 * (size_t)b.nb : 0;
+    if (dyn > 0) IBM_CUDA(c, cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(10 * one * sizeof(T))));
+    if (ncta > 8) IBM_CUDA(c, cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)ncta, 1, 1);
+    cfg.blockDim = dim3(BAND_THREADS, 1, 1);
+    cfg.dynamicSmemBytes = dyn;
+    cfg.stream = c->s;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)ncta;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = ahead ? 2 : 1;
+    kt_begin(c, -1);
+    ++c->nlaunch;
+    IBM_CUDA(c, cudaLaunchKernelEx(&cfg, fn, c->g, c->gh, o, b, (const uint8_t *)c->type, v, z, omega, sweeps, buf, ncta));
+    c->chain = true;
+    kt_end(c, -1);
+    return IBM_OK;
+}
+
 // z = M^{-1} v, vectors and multigrid in precision T
 template <typename T>
 static ibm_status precond(Ctx *c, MGHier<T> &H, const T *v, T *z) {
@@ -3170,24 +3166,10 @@ static ibm_status precond(Ctx *c, MGHier<T> &H, const T *v, T *z) {
         IBM_LAUNCHED(c);
     }
     const OpT<T> o = op_of<T>(c);
+    if (c->nband > 0 && c->opts.band_sweeps > 0) return band_sweeps<T>(c, v, z);
     if (c->ng > 0) {
         KL(-1, k_pre_ghost<T>, (unsigned)((c->ng + 255) / 256), 256, c->gh, o.wp, c->type, v, z);
         IBM_LAUNCHED(c);
-    }
-    if (c->nband > 0 && c->opts.band_sweeps > 0 && c->nband <= (int64_t)BAND_BLOCK * BAND_PER_THREAD) {
-        KL(-1, k_band_block<T>, 1, BAND_BLOCK, c->g, c->gh, o, c->nband, c->band, c->band_g, v, z,
-           (T)c->opts.band_omega, c->opts.band_sweeps);
-        IBM_LAUNCHED(c);
-    } else if (c->nband > 0) {
-        // (btmp holds nband doubles: room for either precision)
-        const unsigned gb = (unsigned)((c->nband + 255) / 256);
-        T *tmp = reinterpret_cast<T *>(c->btmp);
-        for (int s = 0; s < c->opts.band_sweeps; ++s) {
-            KL(-1, k_band_jacobi<T>, gb, 256, c->g, c->gh, o, c->nband, c->band, c->band_g, v, (const T *)z,
-               (T)c->opts.band_omega, tmp);
-            KL(-1, k_band_scatter<T>, gb, 256, c->nband, c->band, (const T *)tmp, z);
-            IBM_LAUNCHED(c);
-        }
     }
     return IBM_OK;
 }
