@@ -2920,15 +2920,23 @@ static ibm_status vcycle(Ctx *c, MGHier<T> &H, const T *f0, T *x0) {
 }
 
 // The V-cycle pr -> pz as one CUDA graph: captured from the stream the
-// first time (and again after a multigrid rebuild or a change of its
-// settings), then replayed with a single launch. Its buffers are fixed, so
-// the graph stays valid for the life of the hierarchy.
+// first time (and again after a change of its settings), then replayed with a
+// single launch. Its kernels' arguments (buffers, extents, tables) are fixed
+// for the life of the hierarchy, and a new classification rewrites the buffers
+// in place, so the graphs stay valid over it: capturing the 17 of a solve
+// again took 5 ms of every body move.
 template <typename T>
 static ibm_status vcycle_graph(Ctx *c, MGHier<T> &H, T *out) {
     const ibm_solver_opts &o = c->opts;
-    const uint64_t key = ((((((c->mg_gen * 64 + (uint64_t)o.nu1) * 64 + (uint64_t)o.nu2) * 4096 +
-                           (uint64_t)o.coarse_sweeps) * 1024 + (uint64_t)o.tile_x) * 4 + (uint64_t)o.mg_interp * 2 +
-                         (uint64_t)o.fine_split) * 1000003 + (uint64_t)o.tail_cells) * 16 + (uint64_t)o.nu_coarse + 1;
+    // FNV-1a over the settings that the cycle's launches depend on
+    uint64_t key = 1469598103934665603ull;
+    auto mix = [&](const void *p, size_t n) {
+        for (size_t i = 0; i < n; ++i) key = (key ^ ((const unsigned char *)p)[i]) * 1099511628211ull;
+    };
+    const int set[7] = {o.nu1, o.nu2, o.nu_coarse, o.tile_x, o.mg_interp, o.fine_split, o.tail_cells};
+    mix(set, sizeof(set));
+    mix(&o.smooth_omega, sizeof(o.smooth_omega));
+    key |= 1ull;
     auto drop_all = [&]() -> ibm_status {
         IBM_CUDA(c, cudaStreamSynchronize(c->s));
         for (int i = 0; i < MGHier<T>::NVG; ++i) {

@@ -49,3 +49,30 @@ def test_captured_steps_repeat_bit_for_bit(precision):
     for _ in range(4):
         b = _run(case, precision, torch.cuda.Stream(), 2)
         assert all(np.array_equal(ref[k], b[k]) for k in ref)
+
+
+@pytest.mark.parametrize("precision", [ibm.IBM_FP64, ibm.IBM_MIXED])
+def test_graphs_kept_over_classifications_and_options(precision):
+    """V-cycle graphs captured for one body position and option set, used
+    again after a move, a new classification and a changed relaxation factor:
+    the bits of a context that launches every kernel."""
+    case = synth.wing_case(112, 96, 98, n_chord=30, n_span=10)   # above 2^20 cells: a graph per Krylov vector
+    verts = np.array(case.verts)
+    verts[:, 1] += 0.03
+    outs = []
+    for graph in (0, 1):
+        s = ibm.Solver(case, precision=precision, stream=torch.cuda.Stream())
+        s.set_opts(precision=precision, graph=graph)
+        s.set_body(case.verts, case.elems)
+        s.classify()
+        s.step(1)
+        s.move_body(verts, U=(0.0, 0.1, 0.0))
+        s.step(1)
+        s.set_opts(smooth_omega=1.1)
+        s.step(1)
+        u = s.get("u")
+        s.classify()
+        s.step(1)
+        outs.append((u, s.get("p")))
+        s.close()
+    assert all(np.array_equal(a, b) for a, b in zip(*outs))
