@@ -395,10 +395,16 @@ static ibm_status create_impl(Ctx *c, const ibm_grid_desc *d) {
     c->NFy = (int64_t)c->nx * (c->ny + 1) * c->nz;
     c->NFz = (int64_t)c->nx * c->ny * (c->nz + 1);
     {
-        const int64_t r = (c->N + 8 * RED_THREADS - 1) / (8 * RED_THREADS);
-        c->nred = (int)(r < 1 ? 1 : (r > RED_BLOCKS ? RED_BLOCKS : r));
-        const int64_t w = (c->N + 2 * RED_THREADS - 1) / (2 * RED_THREADS);
-        c->nred_wide = (int)(w < 1 ? 1 : (w > RED_BLOCKS_MAX ? RED_BLOCKS_MAX : w));
+        // (a small grid is spread over up to two blocks per SM: its FP64
+        // reductions are bound by the FP64 pipe of the SMs they run on. At 8
+        // cells per thread a 128x64 grid had four blocks: 10 us for a
+        // five-column multi-dot, 18 us for the Helmholtz residual.)
+        const int64_t cells = (c->N + RED_THREADS - 1) / RED_THREADS;
+        const int64_t spread = cells < 2 * 152 ? cells : 2 * 152;
+        const int64_t r = std::max((c->N + 8 * RED_THREADS - 1) / (8 * RED_THREADS), spread);
+        c->nred = (int)(r > RED_BLOCKS ? RED_BLOCKS : r);
+        const int64_t w = std::max((c->N + 2 * RED_THREADS - 1) / (2 * RED_THREADS), spread);
+        c->nred_wide = (int)(w > RED_BLOCKS_MAX ? RED_BLOCKS_MAX : w);
         const int64_t e = (c->N + 255) / 256;
         c->nelem = (unsigned)(e < 1 ? 1 : (e > 152 * 16 ? 152 * 16 : e));
     }

@@ -231,7 +231,8 @@ struct Ctx {
     bool chain = false;    // the last thing put on the stream was a kernel of launch()
     int64_t nlaunch = 0;   // kernels launched by this context so far
     // launch sizes that follow the grid: reduction kernels run nred blocks of
-    // RED_THREADS (about 8 cells per thread, at most RED_BLOCKS; a function
+    // RED_THREADS (one cell per thread up to two blocks per SM, then about 8
+    // cells per thread, at most RED_BLOCKS; a function
     // of N only, so reductions stay deterministic); the FP32 operator product
     // and the Krylov/preconditioner vector kernels nred_wide (about 2 cells
     // per thread, at most RED_BLOCKS_MAX: a thread walking tens of cells is

@@ -512,9 +512,12 @@ __device__ __forceinline__ void scale_f32(int64_t n, float * dst, const float * 
 // grid of the multi-dot: each block ends with one FP64 tree sum per column,
 // which on GB300's FP64 pipe costs about as much as a few hundred elements, so
 // the FP64 kernel takes half the usual blocks (each thread streams twice the
-// elements)
+// elements), down to one per SM
 template <typename T>
-static unsigned mdot_blocks(const Ctx *c) { return sizeof(T) == 8 ? (unsigned)((c->nred + 1) / 2) : (unsigned)c->nred; }
+static unsigned mdot_blocks(const Ctx *c) {
+    if (sizeof(T) == 4) return (unsigned)c->nred;
+    return (unsigned)(c->nred > 2 * 152 ? (c->nred + 1) / 2 : (c->nred > 152 ? 152 : c->nred));
+}
 
 template <typename T, typename S>
 __global__ void k_scale(int64_t n, T * dst, const S * src, double a) {
