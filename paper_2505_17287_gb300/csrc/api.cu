@@ -92,7 +92,7 @@ static void release_all(Ctx *c) {
     std::vector<void *> a = c->allocs;
     for (void *p : a) dev_free(c, p);
     if (c->hscal) cudaFreeHost(c->hscal);
-    cudaEvent_t ev[6] = {c->ev0, c->ev1, c->ev2, c->ev3, c->ev4, c->ev5};
+    cudaEvent_t ev[7] = {c->ev0, c->ev1, c->ev2, c->ev3, c->ev4, c->ev5, c->ev6};
     for (auto e : ev)
         if (e) cudaEventDestroy(e);
     for (auto e : c->kt.pool) cudaEventDestroy(e);
@@ -421,7 +421,8 @@ static ibm_status create_impl(Ctx *c, const ibm_grid_desc *d) {
     IBM_CUDA(c, cudaEventCreate(&c->ev3));
     IBM_CUDA(c, cudaEventCreate(&c->ev4));
     IBM_CUDA(c, cudaEventCreate(&c->ev5));
-    IBM_CUDA(c, cudaMallocHost((void **)&c->hscal, sizeof(double) * 64));
+    IBM_CUDA(c, cudaEventCreateWithFlags(&c->ev6, cudaEventDisableTiming));
+    IBM_CUDA(c, cudaMallocHost((void **)&c->hscal, sizeof(double) * 128));
     c->xf = upload(c, c->hxf); c->yf = upload(c, c->hyf); c->zf = upload(c, c->hzf);
     c->xc = upload(c, c->hxc); c->yc = upload(c, c->hyc); c->zc = upload(c, c->hzc);
     c->dx = upload(c, c->hdx); c->dy = upload(c, c->hdy); c->dz = upload(c, c->hdz);
@@ -495,13 +496,13 @@ static ibm_status create_impl(Ctx *c, const ibm_grid_desc *d) {
     c->w = (double *)dev_alloc(c, nb);
     c->rr = (double *)dev_alloc(c, nb);
     c->part = (double *)dev_alloc(c, sizeof(double) * RED_BLOCKS_MAX * 40);
-    c->scal = (double *)dev_alloc(c, sizeof(double) * 64);
+    c->scal = (double *)dev_alloc(c, sizeof(double) * 128);
     if (!c->p || !c->p_prev || !c->p_prev2 || !c->b || !c->w || !c->rr || !c->part || !c->scal)
         return c->fail(IBM_ERR_OOM, "solver vector allocation failed");
     IBM_CUDA(c, cudaMemsetAsync(c->p, 0, nb, c->s));
     IBM_CUDA(c, cudaMemsetAsync(c->p_prev, 0, nb, c->s));
     IBM_CUDA(c, cudaMemsetAsync(c->p_prev2, 0, nb, c->s));
-    IBM_CUDA(c, cudaMemsetAsync(c->scal, 0, sizeof(double) * 64, c->s));
+    IBM_CUDA(c, cudaMemsetAsync(c->scal, 0, sizeof(double) * 128, c->s));
     IBM_TRY(build_levels(c));
     IBM_CUDA(c, cudaStreamSynchronize(c->s));
     return IBM_OK;

@@ -163,8 +163,8 @@ struct Ctx {
 
     // reductions and scalars
     double *part = nullptr;      // partials: RED_BLOCKS * 32
-    double *scal = nullptr;      // device scalars (64)
-    double *hscal = nullptr;     // pinned host mirror (64)
+    double *scal = nullptr;      // device scalars (128)
+    double *hscal = nullptr;     // pinned host mirror (128)
 
     // Poisson (FP64 FGMRES)
     int m_cap = 0;
@@ -209,6 +209,7 @@ struct Ctx {
 
     cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev2 = nullptr, ev3 = nullptr;
     cudaEvent_t ev4 = nullptr, ev5 = nullptr;   // Poisson solve timing
+    cudaEvent_t ev6 = nullptr;                  // scalars published (no timing)
 
     // device-controlled step (opts.graph == 2): the whole fractional step is
     // captured once per buffer parity into a CUDA graph whose loops are
@@ -299,7 +300,8 @@ ibm_status poisson_solve(Ctx *c, const double *rhs, double *phi, double rtol, in
                          ibm_solve_stats *st);
 ibm_status fluid_mean(Ctx *c, const double *x, bool ghosts_too, double *mean_host);
 ibm_status sync_scalars(Ctx *c, int n);
-ibm_status finalize(Ctx *c, const double *part, int nparts, int ncols, double scale, double *out_dev);
+ibm_status finalize(Ctx *c, const double *part, int nparts, int ncols, double scale, double *out_dev,
+                    const double *flag = nullptr);
 
 // geom.cu
 ibm_status geom_classify(Ctx *c);

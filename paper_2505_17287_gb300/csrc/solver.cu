@@ -34,6 +34,8 @@ namespace ibm {
 // device scalar slots
 enum {
     S_RZ = 0, S_PQ = 1, S_AL = 2, S_RZN = 3, S_BE = 4, S_MEAN = 5, S_TMP = 8, S_MD = 16,
+    S_MD2 = 64, S_FLAG = 81,   // second Gram-Schmidt pass: its dots, whether it runs
+    S_COUNT = 128,
     B_RHO = 34, B_ALPHA = 35, B_OMEGA = 36, B_BETA = 37, B_RHO1 = 38, B_DEN = 39, B_TS = 58, B_TT = 59,
     B_FLAG = 60
 };
@@ -62,9 +64,10 @@ static inline dim3 rows_grid(int nx, int ny, int nz, int per_thread, int bx) {
 // ---------------------------------------------------------------------------
 
 // out[col] = scale * sum_i part[col*nparts + i], in a fixed order; one block
-// per column
-__global__ void k_finalize(const double * part, int nparts, double scale, double * out) {
+// per column (with flag: only if *flag is set)
+__global__ void k_finalize(const double * part, int nparts, double scale, double * out, const double *flag) {
     grid_begin();
+    if (flag && *flag == 0.0) return;
     __shared__ double sh[32];
     const int col = blockIdx.x;
     double v = 0.0;
@@ -74,8 +77,8 @@ __global__ void k_finalize(const double * part, int nparts, double scale, double
     if (threadIdx.x == 0) out[col] = v * scale;
 }
 
-ibm_status finalize(Ctx *c, const double *part, int nparts, int ncols, double scale, double *out_dev) {
-    KL(-1, k_finalize, (unsigned)ncols, RED_THREADS, part, nparts, scale, out_dev);
+ibm_status finalize(Ctx *c, const double *part, int nparts, int ncols, double scale, double *out_dev, const double *flag) {
+    KL(-1, k_finalize, (unsigned)ncols, RED_THREADS, part, nparts, scale, out_dev, flag);
     IBM_LAUNCHED(c);
     return IBM_OK;
 }
@@ -84,8 +87,17 @@ ibm_status reduce_sum(Ctx *c, const double *partials, int nparts, double *out_de
     return finalize(c, partials, nparts, 1, 1.0, out_dev);
 }
 
+// the first n scalars into the pinned host mirror: a kernel writes them over
+// the coherent link (1-2 us behind the kernel before it, a copy engine's
+// transfer about 9)
+__global__ void k_publish(const double *scal, double *host, int n) {
+    grid_begin();
+    if ((int)threadIdx.x < n) host[threadIdx.x] = scal[threadIdx.x];
+}
+
 ibm_status sync_scalars(Ctx *c, int n) {
-    IBM_CUDA(c, cudaMemcpyAsync(c->hscal, c->scal, sizeof(double) * n, cudaMemcpyDeviceToHost, c->s));
+    KL(-1, k_publish, 1, S_COUNT, c->scal, c->hscal, n);
+    IBM_LAUNCHED(c);
     IBM_CUDA(c, cudaStreamSynchronize(c->s));
     return IBM_OK;
 }
@@ -184,17 +196,34 @@ __device__ __forceinline__ T A_row(const GridDev &g, const OpT<T> &o, const T * 
     return s - o.dg[c] * xc;
 }
 
+// GHOST row q: y_g = sgn * (x_g - sum_m wp_m x_m) + b_g (b may be null = 0;
+// the pressure equation has b_g = 0, a defect-correction right-hand side not)
+template <typename T>
+__device__ __forceinline__ void ghost_row(const GhostDev &gh, const OpT<T> &o, const T *x, const T *b, T sgn, T *y,
+                                          int64_t q) {
+    if (q >= gh.ng) return;
+    const int64_t gi = gh.gidx[q];
+    T s = x[gi];
+    for (int m = 0; m < 8; ++m) s -= o.wp[8 * q + m] * x[gh.sidx[8 * q + m]];
+    y[gi] = sgn * s + (b ? b[gi] : T(0));
+}
+
 // y = sgn * (A x) + b  on FLUID and DEAD rows (b may be null = 0); GHOST rows
-// are written by k_ghost_rows. Partials (FP64): sum over FLUID of vol * y.
+// are written by the blocks past the first nb. Partials (FP64): sum over FLUID
+// of vol * y.
 // (PLAIN: b null and sgn = 1, the product of every Krylov step; two FP64
 // operations per cell fewer)
 template <typename T, bool PLAIN = false>
 __global__ void k_apply_A(GridDev g, OpT<T> o, const uint8_t * type, const T * x,
-                          const T * b, T sgn, T * y, double * part) {
+                          const T * b, T sgn, T * y, double * part, int nb, GhostDev gh) {
     grid_begin();
     __shared__ double sh[32];
+    if ((int)blockIdx.x >= nb) {
+        ghost_row(gh, o, x, b, sgn, y, (blockIdx.x - nb) * (int64_t)blockDim.x + threadIdx.x);
+        return;
+    }
     typename Acc<T>::type acc = 0;
-    GRID_STRIDE(c, g.n) {
+    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < g.n; c += (int64_t)nb * blockDim.x) {
         const uint8_t t = type[c];
         if (t == GHOST) continue;
         if (t == DEAD) { y[c] = T(0); continue; }
@@ -221,12 +250,16 @@ __device__ __forceinline__ uint8_t u4get(const uchar4 &v, int e) { return e == 0
 
 __global__ void __launch_bounds__(RED_THREADS)
     k_apply_A4(GridDev g, OpT<float> o, const uint8_t * type, const float * x,
-               const float * b, float sgn, float * y, double * part) {
+               const float * b, float sgn, float * y, double * part, int nb, GhostDev gh) {
     grid_begin();
     __shared__ double sh[32];
+    if ((int)blockIdx.x >= nb) {
+        ghost_row(gh, o, x, b, sgn, y, (blockIdx.x - nb) * (int64_t)blockDim.x + threadIdx.x);
+        return;
+    }
     double acc = 0.0;
     const int64_t sy = g.nx, sz = (int64_t)g.nx * g.ny;
-    GRID_STRIDE(q, g.n / 4) {
+    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < g.n / 4; q += (int64_t)nb * blockDim.x) {
         const int64_t c = 4 * q;
         const uchar4 t4 = reinterpret_cast<const uchar4 *>(type)[q];
         int i, j, k;
@@ -277,20 +310,6 @@ __global__ void __launch_bounds__(RED_THREADS)
 
 static inline bool al16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
-// GHOST rows: y_g = sgn * (x_g - sum_m wp_m x_m) + b_g (b may be null = 0;
-// the pressure equation has b_g = 0, a defect-correction right-hand side not)
-template <typename T>
-__global__ void k_ghost_rows(GhostDev gh, OpT<T> o, const T * x, const T * b, T sgn,
-                             T * y) {
-    grid_begin();
-    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q >= gh.ng) return;
-    const int64_t gi = gh.gidx[q];
-    T s = x[gi];
-    for (int m = 0; m < 8; ++m) s -= o.wp[8 * q + m] * x[gh.sidx[8 * q + m]];
-    y[gi] = sgn * s + (b ? b[gi] : T(0));
-}
-
 __global__ void k_zero_at(int64_t m, const int64_t * idx, double * x) {
     grid_begin();
     const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -338,27 +357,30 @@ OpT<float> op_of<float>(Ctx *c) {
                       nullptr, nullptr};
 }
 
+// y = sgn * A x + b, its volume-weighted FLUID mean in scal[S_MEAN]
+template <typename T>
+static ibm_status apply_A(Ctx *c, const T *x, const T *b, T sgn, T *y) {
+    const OpT<T> o = op_of<T>(c);
+    const int nb = sizeof(T) == 4 ? c->nred_wide : c->nred;
+    const unsigned grid = (unsigned)nb + (unsigned)((c->ng + RED_THREADS - 1) / RED_THREADS);
+    if constexpr (sizeof(T) == 4) {
+        if (c->g.nx % 4 == 0 && al16(x) && al16(y) && (!b || al16(b)))
+            KL(K_APPLY_A, k_apply_A4, grid, RED_THREADS, c->g, o, c->type, x, b, sgn, y, c->part, nb, c->gh);
+        else
+            KL(K_APPLY_A, k_apply_A<T>, grid, RED_THREADS, c->g, o, c->type, x, b, sgn, y, c->part, nb, c->gh);
+    } else if (!b && sgn == T(1)) {
+        KL(K_APPLY_A, (k_apply_A<T, true>), grid, RED_THREADS, c->g, o, c->type, x, b, sgn, y, c->part, nb, c->gh);
+    } else {
+        KL(K_APPLY_A, k_apply_A<T>, grid, RED_THREADS, c->g, o, c->type, x, b, sgn, y, c->part, nb, c->gh);
+    }
+    IBM_LAUNCHED(c);
+    return finalize(c, c->part, nb, 1, 1.0 / c->fluid_vol, c->scal + S_MEAN);
+}
+
 // y = P(sgn * A x + b)
 template <typename T>
 static ibm_status apply_PA(Ctx *c, const T *x, const T *b, T sgn, T *y) {
-    const OpT<T> o = op_of<T>(c);
-    const int nb = sizeof(T) == 4 ? c->nred_wide : c->nred;
-    if constexpr (sizeof(T) == 4) {
-        if (c->g.nx % 4 == 0 && al16(x) && al16(y) && (!b || al16(b)))
-            KL(K_APPLY_A, k_apply_A4, nb, RED_THREADS, c->g, o, c->type, x, b, sgn, y, c->part);
-        else
-            KL(K_APPLY_A, k_apply_A<T>, nb, RED_THREADS, c->g, o, c->type, x, b, sgn, y, c->part);
-    } else if (!b && sgn == T(1)) {
-        KL(K_APPLY_A, (k_apply_A<T, true>), nb, RED_THREADS, c->g, o, c->type, x, b, sgn, y, c->part);
-    } else {
-        KL(K_APPLY_A, k_apply_A<T>, nb, RED_THREADS, c->g, o, c->type, x, b, sgn, y, c->part);
-    }
-    IBM_LAUNCHED(c);
-    if (c->ng > 0) {
-        KL(-1, k_ghost_rows<T>, (unsigned)((c->ng + 255) / 256), 256, c->gh, o, x, b, sgn, y);
-        IBM_LAUNCHED(c);
-    }
-    IBM_TRY(finalize(c, c->part, nb, 1, 1.0 / c->fluid_vol, c->scal + S_MEAN));
+    IBM_TRY(apply_A<T>(c, x, b, sgn, y));
     KL(-1, k_sub_meanT<T>, c->nred_wide, RED_THREADS, c->N, c->type, y, c->scal + S_MEAN);
     IBM_LAUNCHED(c);
     return IBM_OK;
@@ -390,13 +412,40 @@ struct VPtrs {
     const T *p[17];
 };
 
+// mean removal of a vector's elements v W ... v W + W - 1 as they are read:
+// a - m on FLUID cells (the projection P; DEAD cells hold 0 already)
+__device__ __forceinline__ float4 minus_mean(float4 a, const uint8_t *type, int64_t v, float m) {
+    const uchar4 t = reinterpret_cast<const uchar4 *>(type)[v];
+    a.x = t.x == FLUID ? a.x - m : a.x;
+    a.y = t.y == FLUID ? a.y - m : a.y;
+    a.z = t.z == FLUID ? a.z - m : a.z;
+    a.w = t.w == FLUID ? a.w - m : a.w;
+    return a;
+}
+__device__ __forceinline__ double2 minus_mean(double2 a, const uint8_t *type, int64_t v, double m) {
+    const uchar2 t = reinterpret_cast<const uchar2 *>(type)[v];
+    a.x = t.x == FLUID ? a.x - m : a.x;
+    a.y = t.y == FLUID ? a.y - m : a.y;
+    return a;
+}
+
+// A Gram-Schmidt kernel's conditions: flag not null: it runs only if *flag is
+// set; type not null: w is the operator product before its FLUID mean *mean
+// is removed, which the kernel does as it reads w (k_orth_dev writes it so)
+struct GsArgs {
+    const double *flag;
+    const uint8_t *type;
+    const double *mean;
+};
+
 // partial dots: col q < NC: (w, V_q). The column count is a template
 // parameter so every loop is unrolled without predicates; 16-byte loads (the
 // vectors come from cudaMalloc or PyTorch's allocator, 256-byte aligned)
 template <typename T, int NC>
-__global__ void __launch_bounds__(RED_THREADS) k_mdot(int64_t n, const T * w, VPtrs<T> V,
-                                                      double * part) {
+__global__ void __launch_bounds__(RED_THREADS) k_mdot(int64_t n, const T * w, VPtrs<T> V, double * part, GsArgs gs) {
     grid_begin();
+    if (gs.flag && *gs.flag == 0.0) return;
+    const T mean = gs.type ? (T)*gs.mean : T(0);
     typedef typename Acc<T>::type A;
     typedef typename Vec16<T>::type VT;
     constexpr int W = Vec16<T>::W;
@@ -406,10 +455,11 @@ __global__ void __launch_bounds__(RED_THREADS) k_mdot(int64_t n, const T * w, VP
     for (int q = 0; q < NC; ++q) acc[q] = A(0);
     const int64_t nv = n / W;
     GRID_STRIDE(v, nv) {
-        const VT a = reinterpret_cast<const VT *>(w)[v];
+        VT a = reinterpret_cast<const VT *>(w)[v];
         VT b[NC];
 #pragma unroll
         for (int q = 0; q < NC; ++q) b[q] = reinterpret_cast<const VT *>(V.p[q])[v];
+        if (gs.type) a = minus_mean(a, gs.type, v, mean);
 #pragma unroll
         for (int q = 0; q < NC; ++q) {
             if constexpr (sizeof(T) == 4) {
@@ -424,8 +474,9 @@ __global__ void __launch_bounds__(RED_THREADS) k_mdot(int64_t n, const T * w, VP
         }
     }
     for (int64_t c = nv * W + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x) {
+        const T a = gs.type && gs.type[c] == FLUID ? w[c] - mean : w[c];
 #pragma unroll
-        for (int q = 0; q < NC; ++q) acc[q] += (A)(w[c] * V.p[q][c]);
+        for (int q = 0; q < NC; ++q) acc[q] += (A)(a * V.p[q][c]);
     }
 #pragma unroll
     for (int q = 0; q < NC; ++q) {
@@ -434,15 +485,20 @@ __global__ void __launch_bounds__(RED_THREADS) k_mdot(int64_t n, const T * w, VP
     }
 }
 
-// w -= sum_q h_q V_q ; partial (w, w)
+// w -= sum_q h_q V_q with h in device memory; partial (w, w)
 template <typename T, int NC>
-__global__ void __launch_bounds__(RED_THREADS) k_orth(int64_t n, T * w, VPtrs<T> V, Coef h,
-                                                      double * part) {
+__global__ void __launch_bounds__(RED_THREADS) k_orth_dev(int64_t n, T * w, VPtrs<T> V, const double * h, double * part,
+                                                          GsArgs gs) {
     grid_begin();
+    if (gs.flag && *gs.flag == 0.0) return;
+    const T mean = gs.type ? (T)*gs.mean : T(0);
     typedef typename Acc<T>::type A;
     typedef typename Vec16<T>::type VT;
     constexpr int W = Vec16<T>::W;
     __shared__ double sh[32];
+    T hv[NC];
+#pragma unroll
+    for (int q = 0; q < NC; ++q) hv[q] = (T)h[q];
     A ww = A(0);
     const int64_t nv = n / W;
     GRID_STRIDE(v, nv) {
@@ -450,10 +506,11 @@ __global__ void __launch_bounds__(RED_THREADS) k_orth(int64_t n, T * w, VPtrs<T>
         VT b[NC];
 #pragma unroll
         for (int q = 0; q < NC; ++q) b[q] = reinterpret_cast<const VT *>(V.p[q])[v];
+        if (gs.type) a = minus_mean(a, gs.type, v, mean);
 #pragma unroll
         for (int q = 0; q < NC; ++q)
 #pragma unroll
-            for (int e = 0; e < W; ++e) vset(a, e, vget(a, e) - (T)h.v[q] * vget(b[q], e));
+            for (int e = 0; e < W; ++e) vset(a, e, vget(a, e) - hv[q] * vget(b[q], e));
         reinterpret_cast<VT *>(w)[v] = a;
         if constexpr (sizeof(T) == 4) {
             T leaf = T(0);
@@ -466,9 +523,9 @@ __global__ void __launch_bounds__(RED_THREADS) k_orth(int64_t n, T * w, VPtrs<T>
         }
     }
     for (int64_t c = nv * W + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x) {
-        T a = w[c];
+        T a = gs.type && gs.type[c] == FLUID ? w[c] - mean : w[c];
 #pragma unroll
-        for (int q = 0; q < NC; ++q) a -= (T)h.v[q] * V.p[q][c];
+        for (int q = 0; q < NC; ++q) a -= hv[q] * V.p[q][c];
         w[c] = a;
         ww += (A)(a * a);
     }
@@ -476,11 +533,29 @@ __global__ void __launch_bounds__(RED_THREADS) k_orth(int64_t n, T * w, VPtrs<T>
     if (threadIdx.x == 0) part[blockIdx.x] = t;
 }
 
+// after the first pass of step j: *wa = ||w||^2 from the partials, and whether
+// a second pass follows: ||w||^2 dropped to eta2 of its value before the pass
+// (||w||^2 + sum h^2, the orthogonal decomposition) or below
+__global__ void k_gs_test(const double *part, int nparts, const double *h, int j, double eta2, double *wa, double *flag) {
+    grid_begin();
+    __shared__ double sh[32];
+    double v = 0.0;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < nparts; i += blockDim.x) v += part[i];
+    v = block_sum<RED_THREADS>(v, sh);
+    if (threadIdx.x == 0) {
+        double h2 = 0.0;
+        for (int i = 0; i <= j; ++i) h2 += h[i] * h[i];
+        *wa = v;
+        *flag = v <= eta2 * (v + h2) ? 1.0 : 0.0;
+    }
+}
+
 // kernel tables indexed by the column count - 1
 template <typename T>
-using MdotFn = void (*)(int64_t, const T *, VPtrs<T>, double *);
+using MdotFn = void (*)(int64_t, const T *, VPtrs<T>, double *, GsArgs);
 template <typename T>
-using OrthFn = void (*)(int64_t, T *, VPtrs<T>, Coef, double *);
+using OrthFn = void (*)(int64_t, T *, VPtrs<T>, const double *, double *, GsArgs);
 template <typename T, int... I>
 static const MdotFn<T> *mdot_table(std::integer_sequence<int, I...>) {
     static const MdotFn<T> t[] = {&k_mdot<T, I + 1>...};
@@ -488,9 +563,13 @@ static const MdotFn<T> *mdot_table(std::integer_sequence<int, I...>) {
 }
 template <typename T, int... I>
 static const OrthFn<T> *orth_table(std::integer_sequence<int, I...>) {
-    static const OrthFn<T> t[] = {&k_orth<T, I + 1>...};
+    static const OrthFn<T> t[] = {&k_orth_dev<T, I + 1>...};
     return t;
 }
+template <typename T>
+static inline MdotFn<T> mdot_fn(int ncols) { return mdot_table<T>(std::make_integer_sequence<int, 17>())[ncols - 1]; }
+template <typename T>
+static inline OrthFn<T> orth_fn(int ncols) { return orth_table<T>(std::make_integer_sequence<int, 17>())[ncols - 1]; }
 
 // dst = a src. FP32 to FP32 in FP32 arithmetic, four elements per 16-byte
 // access (per-element FP64 arithmetic makes an FP32 stream FP64-bound)
@@ -524,6 +603,15 @@ __global__ void k_scale(int64_t n, T * dst, const S * src, double a) {
     grid_begin();
     if constexpr (sizeof(T) == 4 && sizeof(S) == 4) scale_f32(n, dst, src, (float)a);
     else GRID_STRIDE(c, n) dst[c] = (T)(a * (double)src[c]);
+}
+
+// dst = src / sqrt(*n2) (0 where the norm is 0), one product per element
+template <typename T>
+__global__ void k_normalise(int64_t n, T *dst, const T *src, const double *n2) {
+    grid_begin();
+    const double h = sqrt(*n2), a = h > 0.0 ? 1.0 / h : 0.0;
+    if constexpr (sizeof(T) == 4) scale_f32(n, dst, src, (float)a);
+    else GRID_STRIDE(c, n) dst[c] = a * src[c];
 }
 
 // x += sum_i y_i Z_i
@@ -3205,6 +3293,34 @@ struct Krylov {
 static Krylov<double> kry64(Ctx *c) { return Krylov<double>{c->V, c->Z, c->Vdev, c->Zdev, c->w, c->rr, &c->mg64}; }
 static Krylov<float> kry32(Ctx *c) { return Krylov<float>{c->V32, c->Z32, c->Vdev32, c->Zdev32, c->w32, c->r32, &c->mg32}; }
 
+// Step j of the Arnoldi process: w = P A Z_j orthogonalised against V_0..V_j by
+// classical Gram-Schmidt, with a second pass when the norm drops below
+// reorth_eta (default 0.3) of its value (the test of Daniel, Gragg, Kaufman
+// and Stewart 1976, with a looser threshold). The dots stay on the device
+// (S_MD; second pass S_MD2, S_FLAG whether it ran; S_TMP ||w||^2), and the
+// second pass's kernels look at the flag themselves, so no pass waits for the
+// host: with a host read after each reduction a step of a small 2D grid spent
+// 88 of its 205 us on four round trips. The product's mean removal is part of
+// the first pass's reads.
+template <typename T>
+static ibm_status gs_step(Ctx *c, Krylov<T> &K, int j) {
+    const int64_t n = c->N;
+    VPtrs<T> vp{};
+    for (int i = 0; i <= j; ++i) vp.p[i] = K.V[i];
+    IBM_TRY(apply_A<T>(c, K.Z[j], nullptr, T(1), K.w));
+    const GsArgs first{nullptr, c->type, c->scal + S_MEAN}, again{c->scal + S_FLAG, nullptr, nullptr};
+    const int mb = (int)mdot_blocks<T>(c);
+    KL(K_MDOT, mdot_fn<T>(j + 1), mb, RED_THREADS, n, K.w, vp, c->part, first);
+    IBM_TRY(finalize(c, c->part, mb, j + 1, 1.0, c->scal + S_MD));
+    KL(K_ORTH, orth_fn<T>(j + 1), c->nred, RED_THREADS, n, K.w, vp, c->scal + S_MD, c->part, first);
+    KL(-1, k_gs_test, 1, RED_THREADS, c->part, c->nred, c->scal + S_MD, j, c->opts.reorth_eta * c->opts.reorth_eta,
+       c->scal + S_TMP, c->scal + S_FLAG);
+    KL(K_MDOT, mdot_fn<T>(j + 1), mb, RED_THREADS, n, K.w, vp, c->part, again);
+    IBM_TRY(finalize(c, c->part, mb, j + 1, 1.0, c->scal + S_MD2, again.flag));
+    KL(K_ORTH, orth_fn<T>(j + 1), c->nred, RED_THREADS, n, K.w, vp, c->scal + S_MD2, c->part, again);
+    return finalize(c, c->part, c->nred, 1, 1.0, c->scal + S_TMP, again.flag);
+}
+
 // Restarted FGMRES in precision T on P A x = b, x in/out. Stops at
 // ||P(b - A x)|| <= rtol * bnorm, after maxit steps, or (single_cycle)
 // after one restart cycle. Dot products accumulate in FP64.
@@ -3237,36 +3353,20 @@ static ibm_status fgmres(Ctx *c, Krylov<T> K, T *x, const T *b, double bnorm, do
         for (int j = 0; j < m && outer < maxit; ++j) {
             IBM_TRY(precond<T>(c, *K.H, K.V[j], K.Z[j]));
             inner += c->opts.inner_iters;
-            IBM_TRY(apply_PA<T>(c, K.Z[j], nullptr, T(1), K.w));
-            // classical Gram-Schmidt, with a second pass when the norm drops
-            // below reorth_eta (default 0.3) of its value (the test of Daniel,
-            // Gragg, Kaufman and Stewart 1976, with a looser threshold)
-            VPtrs<T> vp{};
-            for (int i = 0; i <= j; ++i) vp.p[i] = K.V[i];
-            double hcol[17] = {0};
-            double wbefore2 = 0.0, wafter2 = 0.0;
-            for (int pass = 0; pass < 2; ++pass) {
-                KL(K_MDOT, mdot_table<T>(std::make_integer_sequence<int, 17>())[j], mdot_blocks<T>(c), RED_THREADS,
-                   n, K.w, vp, c->part);
-                IBM_TRY(finalize(c, c->part, mdot_blocks<T>(c), j + 1, 1.0, c->scal + S_MD));
-                IBM_TRY(sync_scalars(c, S_MD + j + 1));
-                Coef h{};
-                double h2 = 0.0;
-                for (int i = 0; i <= j; ++i) {
-                    h.v[i] = c->hscal[S_MD + i];
-                    h2 += h.v[i] * h.v[i];
-                }
-                KL(K_ORTH, orth_table<T>(std::make_integer_sequence<int, 17>())[j], c->nred, RED_THREADS, n,
-                   K.w, vp, h, c->part);
-                IBM_TRY(finalize(c, c->part, c->nred, 1, 1.0, c->scal + S_TMP));
-                IBM_TRY(sync_scalars(c, S_TMP + 1));
-                wafter2 = c->hscal[S_TMP];
-                // ||w||^2 before the pass, from the orthogonal decomposition
-                wbefore2 = wafter2 + h2;
-                for (int i = 0; i <= j; ++i) hcol[i] += h.v[i];
-                const double eta = c->opts.reorth_eta;
-                if (!(wafter2 <= eta * eta * wbefore2)) break;
+            IBM_TRY(gs_step<T>(c, K, j));
+            // the host reads the column while the device normalises w
+            KL(-1, k_publish, 1, S_COUNT, c->scal, c->hscal, (int)S_FLAG + 1);
+            IBM_LAUNCHED(c);
+            IBM_CUDA(c, cudaEventRecord(c->ev6, c->s));
+            if (j + 1 < m) {
+                KL(-1, k_normalise<T>, c->nred_wide, RED_THREADS, n, K.V[j + 1], K.w, c->scal + S_TMP);
+                IBM_LAUNCHED(c);
             }
+            IBM_CUDA(c, cudaEventSynchronize(c->ev6));
+            const bool again = c->hscal[S_FLAG] != 0.0;
+            double hcol[17] = {0};
+            for (int i = 0; i <= j; ++i) hcol[i] = c->hscal[S_MD + i] + (again ? c->hscal[S_MD2 + i] : 0.0);
+            const double wafter2 = c->hscal[S_TMP];
             const double hn = sqrt(wafter2);
             ++outer;
             for (int i = 0; i <= j; ++i) H[(size_t)i * m + j] = hcol[i];
@@ -3287,10 +3387,6 @@ static ibm_status fgmres(Ctx *c, Krylov<T> K, T *x, const T *b, double bnorm, do
             gv[j] = cs[j] * gv[j];
             jlast = j;
             const double est = fabs(gv[j + 1]) / bnorm;
-            if (hn > 0.0 && j + 1 < m) {
-                KL(-1, (k_scale<T, T>), c->nred_wide, RED_THREADS, n, K.V[j + 1], K.w, 1.0 / hn);
-                IBM_LAUNCHED(c);
-            }
             if (est <= rtol || hn == 0.0) break;
         }
         if (done) break;
@@ -3509,9 +3605,9 @@ static ibm_status bicgstab(Ctx *c, double *phi, double bnorm, double rtol, int m
 // ---------------------------------------------------------------------------
 
 struct DevFG {
-    double H[17 * 16], cs[16], sn[16], g[17], y[16], hcol[17];
-    double beta, bnorm, rtol, rel, scale, wb, wa;
-    int outer, maxit, jlast, active, reorth, go, cycles, single, status, ncols, zero;
+    double H[17 * 16], cs[16], sn[16], g[17], y[16];
+    double beta, bnorm, rtol, rel, scale;
+    int outer, maxit, jlast, active, go, cycles, single, status, ncols, zero;
     // mixed-precision refinement (outer block only)
     double rn, last_rel, inner_rtol;
     int refinements, stalls, steps, stop;
@@ -3581,59 +3677,6 @@ __global__ void k_scale_dev(int64_t n, T * dst, const S * src, const double * a)
     const double f = *a;
     if constexpr (sizeof(T) == 4 && sizeof(S) == 4) scale_f32(n, dst, src, (float)f);
     else GRID_STRIDE(c, n) dst[c] = (T)(f * (double)src[c]);
-}
-
-// w -= sum_q h_q V_q with h in device memory; partial (w, w)
-template <typename T, int NC>
-__global__ void __launch_bounds__(RED_THREADS) k_orth_dev(int64_t n, T * w, VPtrs<T> V,
-                                                          const double * h, double * part) {
-    grid_begin();
-    typedef typename Acc<T>::type A;
-    typedef typename Vec16<T>::type VT;
-    constexpr int W = Vec16<T>::W;
-    __shared__ double sh[32];
-    T hv[NC];
-#pragma unroll
-    for (int q = 0; q < NC; ++q) hv[q] = (T)h[q];
-    A ww = A(0);
-    const int64_t nv = n / W;
-    GRID_STRIDE(v, nv) {
-        VT a = reinterpret_cast<const VT *>(w)[v];
-        VT b[NC];
-#pragma unroll
-        for (int q = 0; q < NC; ++q) b[q] = reinterpret_cast<const VT *>(V.p[q])[v];
-#pragma unroll
-        for (int q = 0; q < NC; ++q)
-#pragma unroll
-            for (int e = 0; e < W; ++e) vset(a, e, vget(a, e) - hv[q] * vget(b[q], e));
-        reinterpret_cast<VT *>(w)[v] = a;
-        if constexpr (sizeof(T) == 4) {
-            T leaf = T(0);
-#pragma unroll
-            for (int e = 0; e < W; ++e) leaf += vget(a, e) * vget(a, e);
-            ww += (A)leaf;
-        } else {
-#pragma unroll
-            for (int e = 0; e < W; ++e) ww += (A)vget(a, e) * (A)vget(a, e);
-        }
-    }
-    for (int64_t c = nv * W + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x) {
-        T a = w[c];
-#pragma unroll
-        for (int q = 0; q < NC; ++q) a -= hv[q] * V.p[q][c];
-        w[c] = a;
-        ww += (A)(a * a);
-    }
-    const double t = block_sum<RED_THREADS>(ww, sh);
-    if (threadIdx.x == 0) part[blockIdx.x] = t;
-}
-
-template <typename T>
-using OrthDevFn = void (*)(int64_t, T *, VPtrs<T>, const double *, double *);
-template <typename T, int... I>
-static const OrthDevFn<T> *orth_dev_table(std::integer_sequence<int, I...>) {
-    static const OrthDevFn<T> t[] = {&k_orth_dev<T, I + 1>...};
-    return t;
 }
 
 // x += sum_{q < ncols} y_q Z_q with y and ncols from the control block
@@ -3718,35 +3761,16 @@ __global__ void k_fg_cycle(DevFG *F, const double *rn2, cudaGraphConditionalHand
     cudaGraphSetConditional(h, go ? 1u : 0u);
 }
 
-// after the first Gram-Schmidt pass of step j: h in md[0..j], ||w||^2 after
-// in *wa2; a second pass when ||w||^2 dropped to eta2 of its value before the
-// pass (||w_after||^2 + sum h^2) or below
-__global__ void k_fg_post1(DevFG *F, const double *md, const double *wa2, int j, double eta2) {
-    grid_begin();
-    double h2 = 0.0;
-    for (int i = 0; i <= j; ++i) {
-        F->hcol[i] = md[i];
-        h2 += md[i] * md[i];
-    }
-    F->wa = *wa2;
-    F->wb = F->wa + h2;   // ||w||^2 before the pass, from the orthogonal decomposition
-    F->reorth = F->wa <= eta2 * F->wb;
-}
-
-__global__ void k_fg_post2(DevFG *F, const double *md, const double *wa2, int j) {
-    grid_begin();
-    for (int i = 0; i <= j; ++i) F->hcol[i] += md[i];
-    F->wa = *wa2;
-}
-
 // Hessenberg column j, Givens rotations, residual estimate and the decision
 // to take step j + 1
-__global__ void k_fg_givens(DevFG *F, int j, int m) {
+// (the column from gs_step's scalars)
+__global__ void k_fg_givens(DevFG *F, const double *scal, int j, int m) {
     grid_begin();
-    const double hn = sqrt(F->wa);
+    const double hn = sqrt(scal[S_TMP]);
+    const bool again = scal[S_FLAG] != 0.0;
     F->outer += 1;
     double *H = F->H;
-    for (int i = 0; i <= j; ++i) H[i * m + j] = F->hcol[i];
+    for (int i = 0; i <= j; ++i) H[i * m + j] = scal[S_MD + i] + (again ? scal[S_MD2 + i] : 0.0);
     H[(j + 1) * m + j] = hn;
     if (!isfinite(hn)) {
         F->status = IBM_ERR_DIVERGED;
@@ -3848,11 +3872,10 @@ template <typename T>
 static ibm_status fgmres_dev_cycle(Ctx *c, Krylov<T> K, T *x, DevFG *F) {
     const int64_t n = c->N;
     const int m = c->opts.restart;
-    VPtrs<T> vp{}, zp{};
-    for (int i = 0; i <= m && i < 17; ++i) vp.p[i] = K.V[i];
+    VPtrs<T> zp{};
     for (int i = 0; i < m; ++i) zp.p[i] = K.Z[i];
     for (int j = 0; j < m; ++j) {
-        cudaGraphConditionalHandle hj, hr;
+        cudaGraphConditionalHandle hj;
         IBM_TRY(cond_handle(c, &hj));
         KL(-1, k_set_cond, 1, 1, hj, &F->active);
         CondScope sj;
@@ -3861,30 +3884,8 @@ static ibm_status fgmres_dev_cycle(Ctx *c, Krylov<T> K, T *x, DevFG *F) {
             // V_j = (j == 0 ? r : w) / norm
             KL(-1, (k_scale_dev<T, T>), c->nred_wide, RED_THREADS, n, K.V[j], j == 0 ? K.r : K.w, &F->scale);
             IBM_TRY(precond<T>(c, *K.H, K.V[j], K.Z[j]));
-            IBM_TRY(apply_PA<T>(c, K.Z[j], nullptr, T(1), K.w));
-            KL(K_MDOT, mdot_table<T>(std::make_integer_sequence<int, 17>())[j], mdot_blocks<T>(c), RED_THREADS, n,
-               K.w, vp, c->part);
-            IBM_TRY(finalize(c, c->part, mdot_blocks<T>(c), j + 1, 1.0, c->scal + S_MD));
-            KL(K_ORTH, orth_dev_table<T>(std::make_integer_sequence<int, 17>())[j], c->nred, RED_THREADS, n, K.w,
-               vp, c->scal + S_MD, c->part);
-            IBM_TRY(finalize(c, c->part, c->nred, 1, 1.0, c->scal + S_TMP));
-            KL(-1, k_fg_post1, 1, 1, F, c->scal + S_MD, c->scal + S_TMP, j,
-               c->opts.reorth_eta * c->opts.reorth_eta);
-            IBM_TRY(cond_handle(c, &hr));
-            KL(-1, k_set_cond, 1, 1, hr, &F->reorth);
-            CondScope sr;
-            IBM_TRY(cond_open(c, cudaGraphCondTypeIf, hr, &sr));
-            {
-                KL(K_MDOT, mdot_table<T>(std::make_integer_sequence<int, 17>())[j], mdot_blocks<T>(c), RED_THREADS,
-                   n, K.w, vp, c->part);
-                IBM_TRY(finalize(c, c->part, mdot_blocks<T>(c), j + 1, 1.0, c->scal + S_MD));
-                KL(K_ORTH, orth_dev_table<T>(std::make_integer_sequence<int, 17>())[j], c->nred, RED_THREADS, n,
-                   K.w, vp, c->scal + S_MD, c->part);
-                IBM_TRY(finalize(c, c->part, c->nred, 1, 1.0, c->scal + S_TMP));
-                KL(-1, k_fg_post2, 1, 1, F, c->scal + S_MD, c->scal + S_TMP, j);
-            }
-            IBM_TRY(cond_close(c, &sr));
-            KL(-1, k_fg_givens, 1, 1, F, j, m);
+            IBM_TRY(gs_step<T>(c, K, j));
+            KL(-1, k_fg_givens, 1, 1, F, c->scal, j, m);
         }
         IBM_TRY(cond_close(c, &sj));
     }
@@ -4050,11 +4051,6 @@ ibm_status step_stats_read(Ctx *c, ibm_step_stats *st) {
 // (G + eps I) c = (b_i, P b) are solved by Cholesky in one thread. All of it
 // runs on the device, so the captured step graph holds it as well.
 
-template <typename T>
-static inline const MdotFn<T> *mdot_fns() {
-    return mdot_table<T>(std::make_integer_sequence<int, 17>());
-}
-
 // rhs - mean on FLUID cells, 0 elsewhere (the solver's P rhs)
 __global__ void k_hist_bp(int64_t n, const uint8_t * type, const double * rhs,
                           const HistCtl * H, double * bp) {
@@ -4195,7 +4191,8 @@ ibm_status hist_guess(Ctx *c, const double *rhs, double *phi) {
     vp.p[L] = c->hist_bp;
     for (int i = 0; i <= L; ++i)
         if (!al16(vp.p[i])) return c->fail(IBM_ERR_STATE, "Poisson history column not 16-byte aligned");
-    KL(-1, mdot_fns<double>()[L], mdot_blocks<double>(c), RED_THREADS, c->N, c->hist_bp, vp, c->part);
+    KL(-1, mdot_fn<double>(L + 1), mdot_blocks<double>(c), RED_THREADS, c->N, c->hist_bp, vp, c->part,
+       GsArgs{nullptr, nullptr, nullptr});
     IBM_TRY(finalize(c, c->part, mdot_blocks<double>(c), L + 1, 1.0, H->d));
     KL(-1, k_hist_solve, 1, 1, H);
     KL(-1, k_hist_guess, c->nelem, 256, c->N, c->hist_ld, H, c->hist_x, phi);
