@@ -355,6 +355,51 @@ __global__ void k_vghost_scatter(GhostDev gh, Fields3 u, int ncomp, const double
     if (q >= gh.ng) return;
     for (int cq = 0; cq < ncomp; ++cq) u.p[cq][gh.gidx[q]] = tmp[cq * gh.ng + q];
 }
+// A Jacobi pass of the ghost rows in one launch of one block, for at most
+// VGHOST_ONE ghosts: every new value is formed before a block barrier and
+// written after it (the values of k_vghost_compute and k_vghost_scatter); res,
+// if not null, takes the largest change
+constexpr int VGHOST_THREADS = 512, VGHOST_PER = 4, VGHOST_ONE = VGHOST_THREADS * VGHOST_PER;
+__global__ void __launch_bounds__(VGHOST_THREADS)
+    k_vghost_pass(GhostDev gh, Fields3 u, int ncomp, const double * ubi, int comp0, double * res, int scatter) {
+    grid_begin();
+    __shared__ double sh[32];
+    double r = 0.0;
+    for (int cq = 0; cq < ncomp; ++cq) {
+        double *uu = pick3(cq, u.p[0], u.p[1], u.p[2]);
+        double nv[VGHOST_PER];
+#pragma unroll
+        for (int e = 0; e < VGHOST_PER; ++e) {
+            const int64_t q = threadIdx.x + (int64_t)e * VGHOST_THREADS;
+            nv[e] = 0.0;
+            if (q >= gh.ng) continue;
+            double s = ubi ? (2.0 - gh.bv[q]) * ubi[3 * q + comp0 + cq] : 0.0;
+#pragma unroll
+            for (int m = 0; m < 8; ++m) s -= gh.wv[8 * q + m] * uu[gh.sidx[8 * q + m]];
+            nv[e] = s;
+            if (res) r = fmax(r, fabs(s - uu[gh.gidx[q]]));
+        }
+        if (scatter) {
+            __syncthreads();
+#pragma unroll
+            for (int e = 0; e < VGHOST_PER; ++e) {
+                const int64_t q = threadIdx.x + (int64_t)e * VGHOST_THREADS;
+                if (q < gh.ng) uu[gh.gidx[q]] = nv[e];
+            }
+        }
+    }
+    if (res) {
+        r = warp_max(r);
+        if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = r;
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            double t = threadIdx.x < VGHOST_THREADS / 32 ? sh[threadIdx.x] : 0.0;
+            t = warp_max(t);
+            if (threadIdx.x == 0) *res = t;
+        }
+    }
+}
+
 __global__ void k_max_final(const double * part, int n, double * out) {
     grid_begin();
     double m = 0.0;
@@ -597,6 +642,22 @@ static inline dim3 rb_grid(const Ctx *c) {
 // body velocity at the ghosts' intercepts (null while the body is at rest)
 static const double *ghost_ubi(const Ctx *c) { return c->moving ? c->ubi : nullptr; }
 
+// A pass of the velocity ghost rows of ncomp components from comp0 (scatter:
+// the values are written) and, if res is not null, the largest change a pass
+// makes into *res. One launch for the few ghosts of a 2D body, whose pass is
+// all latency (2.3 + 0.9 us as two launches, 2.4 as one).
+static void vghost_pass(Ctx *c, Fields3 U, int ncomp, int comp0, double *res, bool scatter) {
+    if (c->ng <= VGHOST_ONE) {
+        ++c->nlaunch, launch(c, k_vghost_pass, 1, VGHOST_THREADS, c->gh, U, ncomp, ghost_ubi(c), comp0, res, scatter ? 1 : 0);
+        return;
+    }
+    const unsigned gb = (unsigned)((c->ng + 255) / 256);
+    double *part = c->part + 2 * RED_BLOCKS_MAX;
+    ++c->nlaunch, launch(c, k_vghost_compute, gb, 256, c->gh, U, ncomp, ghost_ubi(c), comp0, c->gtmp, part, res ? 1 : 0);
+    if (scatter) ++c->nlaunch, launch(c, k_vghost_scatter, gb, 256, c->gh, U, ncomp, c->gtmp);
+    if (res) ++c->nlaunch, launch(c, k_max_final, 1, 256, part, (int)gb, res);
+}
+
 static ibm_status faces_from(Ctx *c, double *const *ucell) {
     const BCInfo bc = make_bc(c);
     for (int a = 0; a < c->ndim; ++a) {
@@ -624,19 +685,15 @@ static ibm_status ghost_refresh_all(Ctx *c, double *const *ucell, int *passes) {
     if (c->ng == 0) return IBM_OK;
     const int nc = c->ndim;
     Fields3 U{{ucell[0], ucell[1], nc == 3 ? ucell[2] : ucell[1]}};
-    const unsigned gb = (unsigned)((c->ng + 255) / 256);
     double scale = 1.0;
     for (int a = 0; a < 3; ++a) scale = fmax(scale, fabs(c->desc.u_inf[a]));
     const int check_every = 4;
     for (int it = 0; it < c->opts.ghost_maxit; ++it) {
         const int want = ((it + 1) % check_every == 0) || it + 1 == c->opts.ghost_maxit;
-        ++c->nlaunch, launch(c, k_vghost_compute, gb, 256, c->gh, U, nc, ghost_ubi(c), 0, c->gtmp, c->part, want);
-        ++c->nlaunch, launch(c, k_vghost_scatter, gb, 256, c->gh, U, nc, c->gtmp);
+        vghost_pass(c, U, nc, 0, want ? c->scal + 40 : nullptr, true);
         IBM_LAUNCHED(c);
         ++*passes;
         if (want) {
-            ++c->nlaunch, launch(c, k_max_final, 1, 256, c->part, (int)gb, c->scal + 40);
-            IBM_LAUNCHED(c);
             IBM_TRY(sync_scalars(c, 41));
             const double d = c->hscal[40];
             if (!isfinite(d)) return c->fail(IBM_ERR_DIVERGED, "velocity ghost refresh produced a non-finite value");
@@ -754,7 +811,6 @@ static ibm_status helmholtz_srj(Ctx *c, int q, int *sweeps) {
     const double *hinv = c->hinv[q];
     double *u = c->ustar[q], *t = c->htmp;
     const double *rhs = c->rhs[q];
-    const unsigned gb = (unsigned)((c->ng + 255) / 256);
     *sweeps = 0;
     double rhs2 = -1.0;
     for (int it = 0; it < c->opts.helm_maxit; it += M) {
@@ -764,8 +820,7 @@ static ibm_status helmholtz_srj(Ctx *c, int q, int *sweeps) {
             kt_end(c, K_HELM);
             if (c->ng > 0) {
                 Fields3 T3{{t, t, t}};
-                ++c->nlaunch, launch(c, k_vghost_compute, gb, 256, c->gh, T3, 1, ghost_ubi(c), q, c->gtmp, c->part, 0);
-                ++c->nlaunch, launch(c, k_vghost_scatter, gb, 256, c->gh, T3, 1, c->gtmp);
+                vghost_pass(c, T3, 1, q, nullptr, true);
             }
             IBM_LAUNCHED(c);
             double *x = u;
@@ -780,8 +835,7 @@ static ibm_status helmholtz_srj(Ctx *c, int q, int *sweeps) {
         IBM_TRY(finalize(c, c->part, c->nred, 2, 1.0, c->scal + 48));
         double gmax = 0.0;
         if (c->ng > 0) {
-            ++c->nlaunch, launch(c, k_vghost_compute, gb, 256, c->gh, U, 1, ghost_ubi(c), q, c->gtmp, c->part + 2 * RED_BLOCKS_MAX, 1);
-            ++c->nlaunch, launch(c, k_max_final, 1, 256, c->part + 2 * RED_BLOCKS_MAX, (int)gb, c->scal + 50);
+            vghost_pass(c, U, 1, q, c->scal + 50, false);
             IBM_LAUNCHED(c);
         }
         IBM_TRY(sync_scalars(c, 51));
@@ -811,10 +865,8 @@ static void helm_rb(Ctx *c, const double *rhs, const double *hinv, double *u, in
 // between the colours, not once per sweep, takes the 25.2M-cell wing from 6
 // to 4 sweeps per component at a 1e-12 residual (the 201M-cell wing, whose
 // finer cells converge more slowly, still needs 6).
-static void helm_ghost_pass(Ctx *c, int q, Fields3 U, unsigned gb) {
-    if (c->ng == 0) return;
-    ++c->nlaunch, launch(c, k_vghost_compute, gb, 256, c->gh, U, 1, ghost_ubi(c), q, c->gtmp, c->part, 0);
-    ++c->nlaunch, launch(c, k_vghost_scatter, gb, 256, c->gh, U, 1, c->gtmp);
+static void helm_ghost_pass(Ctx *c, int q, Fields3 U) {
+    if (c->ng > 0) vghost_pass(c, U, 1, q, nullptr, true);
 }
 
 static ibm_status helmholtz(Ctx *c, int q, int *sweeps) {
@@ -827,7 +879,6 @@ static ibm_status helmholtz(Ctx *c, int q, int *sweeps) {
     int next_check = c->opts.helm_check_first;
     *sweeps = 0;
     double rhs2 = -1.0;
-    const unsigned gb = (unsigned)((c->ng + 255) / 256);
     Fields3 U{{u, u, u}};
     for (int it = 0; it < c->opts.helm_maxit; ++it) {
         // each colour pass is followed by a Jacobi pass of the ghost rows
@@ -836,7 +887,7 @@ static ibm_status helmholtz(Ctx *c, int q, int *sweeps) {
             ++c->nlaunch, helm_rb(c, rhs, hinv, u, col);
             kt_end(c, K_HELM);
             IBM_LAUNCHED(c);
-            helm_ghost_pass(c, q, U, gb);
+            helm_ghost_pass(c, q, U);
         }
         ++*sweeps;
         if (*sweeps == next_check || it + 1 == c->opts.helm_maxit) {
@@ -847,8 +898,7 @@ static ibm_status helmholtz(Ctx *c, int q, int *sweeps) {
             double gmax = 0.0;
             if (c->ng > 0) {
                 // ghost-row residual: largest change a further Jacobi pass would make
-                ++c->nlaunch, launch(c, k_vghost_compute, gb, 256, c->gh, U, 1, ghost_ubi(c), q, c->gtmp, c->part + 2 * RED_BLOCKS_MAX, 1);
-                ++c->nlaunch, launch(c, k_max_final, 1, 256, c->part + 2 * RED_BLOCKS_MAX, (int)gb, c->scal + 50);
+                vghost_pass(c, U, 1, q, c->scal + 50, false);
                 IBM_LAUNCHED(c);
             }
             IBM_TRY(sync_scalars(c, 51));
@@ -1140,17 +1190,15 @@ struct HelmCtl {
     int due;          // a test runs after the current sweep
 };
 
-__global__ void k_hc_reset(HelmCtl *H, int q, int first_check, cudaGraphConditionalHandle h) {
+// start of component q's solve: `done` sweeps follow as plain nodes, then the
+// first residual test
+__global__ void k_hc_reset(HelmCtl *H, int q, int done, int next_check) {
     grid_begin();
     if (q == 0) H->status = 0;
-    if (q >= 0) {
-        H->sweeps[q] = 0;
-        H->rhs2 = -1.0;
-        H->next_check = first_check;
-    } else {
-        H->passes = 0;
-    }
-    cudaGraphSetConditional(h, 1u);
+    H->sweeps[q] = done;
+    H->rhs2 = -1.0;
+    H->next_check = next_check;
+    H->due = 1;
 }
 
 // after each sweep: count it and open the residual test when it is due
@@ -1161,6 +1209,11 @@ __global__ void k_helm_tick(HelmCtl *H, int q, int maxit, cudaGraphConditionalHa
     if (due) H->next_check = helm_next_check(H->next_check);
     H->due = due;
     cudaGraphSetConditional(hif, due ? 1u : 0u);
+}
+
+__global__ void k_helm_go(cudaGraphConditionalHandle h) {
+    grid_begin();
+    cudaGraphSetConditional(h, 1u);
 }
 
 __global__ void k_helm_decide(HelmCtl *H, int q, const double * scal, int has_ghost, double tol,
@@ -1185,10 +1238,10 @@ __global__ void k_helm_decide(HelmCtl *H, int q, const double * scal, int has_gh
     cudaGraphSetConditional(h, go ? 1u : 0u);
 }
 
-__global__ void k_ghost_decide(HelmCtl *H, const double * d, double tol, int maxit, int trip,
+__global__ void k_ghost_decide(HelmCtl *H, const double * d, double tol, int maxit, int trip, int first,
                                cudaGraphConditionalHandle h) {
     grid_begin();
-    H->passes += trip;
+    H->passes = (first ? 0 : H->passes) + trip;
     const double v = *d;
     if (!isfinite(v)) {
         H->status = IBM_ERR_DIVERGED;
@@ -1210,38 +1263,57 @@ static ibm_status helmholtz_dev(Ctx *c, int q) {
     const double *hinv = c->hinv[q];
     double *u = c->ustar[q];
     const double *rhs = c->rhs[q];
-    const unsigned gb = (unsigned)((c->ng + 255) / 256);
     Fields3 U{{u, u, u}};
     cudaGraphConditionalHandle h, hif;
     IBM_TRY(cond_handle(c, &h));
-    IBM_TRY(cond_handle(c, &hif));
-    ++c->nlaunch, launch(c, k_hc_reset, 1, 1, H, q, c->opts.helm_check_first, h);
+    auto sweep = [&]() {
+        for (int col = 0; col < 2; ++col) {
+            ++c->nlaunch, helm_rb(c, rhs, hinv, u, col);
+            helm_ghost_pass(c, q, U);
+        }
+    };
+    auto test = [&]() -> ibm_status {
+        ++c->nlaunch, launch(c, k_helm_resid, c->nred, RED_THREADS, c->g, helm_coef(c), c->type, rhs, make_bc(c), q, u, alpha,
+                             c->part);
+        IBM_LAUNCHED(c);
+        IBM_TRY(finalize(c, c->part, c->nred, 2, 1.0, c->scal + 48));
+        if (c->ng > 0) vghost_pass(c, U, 1, q, c->scal + 50, false);
+        IBM_LAUNCHED(c);
+        return IBM_OK;
+    };
+    auto decide = [&]() -> ibm_status {
+        ++c->nlaunch, launch(c, k_helm_decide, 1, 1, H, q, c->scal, c->ng > 0, c->opts.helm_rtol, u_scale(c),
+                             c->opts.helm_maxit, h);
+        IBM_LAUNCHED(c);
+        return IBM_OK;
+    };
+    // the sweeps up to the first residual test need no decision: plain nodes
+    // (a trip of the WHILE node costs 10 us beside its kernels), as long as
+    // there are not many; then one sweep per trip, the residual test (an IF
+    // node) on the same sweep counts as the host-driven solve
+    const int first = c->opts.helm_check_first, upto = first < c->opts.helm_maxit ? first : c->opts.helm_maxit;
+    const int plain = upto <= 32 ? upto : 1;
+    ++c->nlaunch, launch(c, k_hc_reset, 1, 1, H, q, plain, plain == first ? helm_next_check(first) : first);
+    for (int s = 0; s < plain; ++s) sweep();
+    IBM_LAUNCHED(c);
+    if (plain == upto) {
+        IBM_TRY(test());
+        IBM_TRY(decide());
+    } else {
+        ++c->nlaunch, launch(c, k_helm_go, 1, 1, h);
+    }
     CondScope sc;
     IBM_TRY(cond_open(c, cudaGraphCondTypeWhile, h, &sc));
     {
-        // one sweep per trip; the residual test (an IF node) on the same
-        // sweep counts as the host-driven solve
-        for (int col = 0; col < 2; ++col) {
-            ++c->nlaunch, helm_rb(c, rhs, hinv, u, col);
-            helm_ghost_pass(c, q, U, gb);
-        }
+        IBM_TRY(cond_handle(c, &hif));
+        sweep();
         ++c->nlaunch, launch(c, k_helm_tick, 1, 1, H, q, c->opts.helm_maxit, hif);
         IBM_LAUNCHED(c);
         CondScope si;
         IBM_TRY(cond_open(c, cudaGraphCondTypeIf, hif, &si));
-        ++c->nlaunch, launch(c, k_helm_resid, c->nred, RED_THREADS, c->g, helm_coef(c), c->type, rhs, make_bc(c), q, u, alpha,
-                                                                     c->part);
-        IBM_LAUNCHED(c);
-        IBM_TRY(finalize(c, c->part, c->nred, 2, 1.0, c->scal + 48));
-        if (c->ng > 0) {
-            ++c->nlaunch, launch(c, k_vghost_compute, gb, 256, c->gh, U, 1, ghost_ubi(c), q, c->gtmp, c->part + 2 * RED_BLOCKS_MAX, 1);
-            ++c->nlaunch, launch(c, k_max_final, 1, 256, c->part + 2 * RED_BLOCKS_MAX, (int)gb, c->scal + 50);
-            IBM_LAUNCHED(c);
-        }
+        IBM_TRY(test());
         IBM_TRY(cond_close(c, &si));
-        ++c->nlaunch, launch(c, k_helm_decide, 1, 1, H, q, c->scal, c->ng > 0, c->opts.helm_rtol, u_scale(c),
-                                                     c->opts.helm_maxit, h);
-        IBM_LAUNCHED(c);
+        IBM_TRY(decide());
     }
     IBM_TRY(cond_close(c, &sc));
     return IBM_OK;
@@ -1252,21 +1324,21 @@ static ibm_status ghost_refresh_dev(Ctx *c) {
     HelmCtl *H = (HelmCtl *)c->hctl;
     const int nc = c->ndim;
     Fields3 U{{c->u[0], c->u[1], nc == 3 ? c->u[2] : c->u[1]}};
-    const unsigned gb = (unsigned)((c->ng + 255) / 256);
     const int trip = 4;
     cudaGraphConditionalHandle h;
     IBM_TRY(cond_handle(c, &h));
-    ++c->nlaunch, launch(c, k_hc_reset, 1, 1, H, -1, 0, h);
+    // the first trip runs as plain nodes, further ones in the WHILE node
+    auto passes = [&](int first) -> ibm_status {
+        for (int t = 0; t < trip; ++t) vghost_pass(c, U, nc, 0, t == trip - 1 ? c->scal + 40 : nullptr, true);
+        ++c->nlaunch, launch(c, k_ghost_decide, 1, 1, H, c->scal + 40, c->opts.ghost_tol * u_scale(c),
+                                                      c->opts.ghost_maxit, trip, first, h);
+        IBM_LAUNCHED(c);
+        return IBM_OK;
+    };
+    IBM_TRY(passes(1));
     CondScope sc;
     IBM_TRY(cond_open(c, cudaGraphCondTypeWhile, h, &sc));
-    for (int t = 0; t < trip; ++t) {
-        ++c->nlaunch, launch(c, k_vghost_compute, gb, 256, c->gh, U, nc, ghost_ubi(c), 0, c->gtmp, c->part, t == trip - 1);
-        ++c->nlaunch, launch(c, k_vghost_scatter, gb, 256, c->gh, U, nc, c->gtmp);
-    }
-    ++c->nlaunch, launch(c, k_max_final, 1, 256, c->part, (int)gb, c->scal + 40);
-    ++c->nlaunch, launch(c, k_ghost_decide, 1, 1, H, c->scal + 40, c->opts.ghost_tol * u_scale(c),
-                                                  c->opts.ghost_maxit, trip, h);
-    IBM_LAUNCHED(c);
+    IBM_TRY(passes(0));
     IBM_TRY(cond_close(c, &sc));
     return IBM_OK;
 }
