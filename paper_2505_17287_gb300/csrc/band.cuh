@@ -23,9 +23,9 @@
 namespace ibm {
 
 constexpr int BAND_THREADS = 512, BAND_MAX_CTAS = 16;
-// rows a thread may own (their coefficients and neighbours take 20 registers
-// each, 30 in FP64)
-template <typename T> struct BandRows { enum { MAX = sizeof(T) == 4 ? 4 : 2 }; };
+// rows a thread of one block may own (their coefficients and neighbours take 20
+// registers each, 30 in FP64)
+template <typename T> struct BandRows { enum { MAX = sizeof(T) == 4 ? 4 : 1 }; };
 
 // nbr[m nb + q]: band position of neighbour m of band cell q (FLUID: -x, +x,
 // -y, +y, -z, +z, itself where there is no cell; GHOST: its eight stencil

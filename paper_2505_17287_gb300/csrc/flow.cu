@@ -356,10 +356,12 @@ __global__ void k_vghost_scatter(GhostDev gh, Fields3 u, int ncomp, const double
     for (int cq = 0; cq < ncomp; ++cq) u.p[cq][gh.gidx[q]] = tmp[cq * gh.ng + q];
 }
 // A Jacobi pass of the ghost rows in one launch of one block, for at most
-// VGHOST_ONE ghosts: every new value is formed before a block barrier and
+// VGHOST_ONE ghosts (a pass takes the block 9 FP64 operations a ghost and
+// component at 2 per clock: 2000 ghosts took 12-20 us, two launches on the
+// whole device 6): every new value is formed before a block barrier and
 // written after it (the values of k_vghost_compute and k_vghost_scatter); res,
 // if not null, takes the largest change
-constexpr int VGHOST_THREADS = 512, VGHOST_PER = 4, VGHOST_ONE = VGHOST_THREADS * VGHOST_PER;
+constexpr int VGHOST_THREADS = 512, VGHOST_ONE = VGHOST_THREADS;
 __global__ void __launch_bounds__(VGHOST_THREADS)
     k_vghost_pass(GhostDev gh, Fields3 u, int ncomp, const double * ubi, int comp0, double * res, int scatter) {
     grid_begin();
@@ -367,25 +369,17 @@ __global__ void __launch_bounds__(VGHOST_THREADS)
     double r = 0.0;
     for (int cq = 0; cq < ncomp; ++cq) {
         double *uu = pick3(cq, u.p[0], u.p[1], u.p[2]);
-        double nv[VGHOST_PER];
+        const int64_t q = threadIdx.x;
+        double nv = 0.0;
+        if (q < gh.ng) {
+            nv = ubi ? (2.0 - gh.bv[q]) * ubi[3 * q + comp0 + cq] : 0.0;
 #pragma unroll
-        for (int e = 0; e < VGHOST_PER; ++e) {
-            const int64_t q = threadIdx.x + (int64_t)e * VGHOST_THREADS;
-            nv[e] = 0.0;
-            if (q >= gh.ng) continue;
-            double s = ubi ? (2.0 - gh.bv[q]) * ubi[3 * q + comp0 + cq] : 0.0;
-#pragma unroll
-            for (int m = 0; m < 8; ++m) s -= gh.wv[8 * q + m] * uu[gh.sidx[8 * q + m]];
-            nv[e] = s;
-            if (res) r = fmax(r, fabs(s - uu[gh.gidx[q]]));
+            for (int m = 0; m < 8; ++m) nv -= gh.wv[8 * q + m] * uu[gh.sidx[8 * q + m]];
+            if (res) r = fmax(r, fabs(nv - uu[gh.gidx[q]]));
         }
         if (scatter) {
             __syncthreads();
-#pragma unroll
-            for (int e = 0; e < VGHOST_PER; ++e) {
-                const int64_t q = threadIdx.x + (int64_t)e * VGHOST_THREADS;
-                if (q < gh.ng) uu[gh.gidx[q]] = nv[e];
-            }
+            if (q < gh.ng) uu[gh.gidx[q]] = nv;
         }
     }
     if (res) {

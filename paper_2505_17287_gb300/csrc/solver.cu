@@ -35,6 +35,7 @@ namespace ibm {
 enum {
     S_RZ = 0, S_PQ = 1, S_AL = 2, S_RZN = 3, S_BE = 4, S_MEAN = 5, S_TMP = 8, S_MD = 16,
     S_MD2 = 64, S_FLAG = 81,   // second Gram-Schmidt pass: its dots, whether it runs
+    S_INV = 82,                // 1 / ||w|| of the Arnoldi step
     S_COUNT = 128,
     B_RHO = 34, B_ALPHA = 35, B_OMEGA = 36, B_BETA = 37, B_RHO1 = 38, B_DEN = 39, B_TS = 58, B_TT = 59,
     B_FLAG = 60
@@ -89,14 +90,20 @@ ibm_status reduce_sum(Ctx *c, const double *partials, int nparts, double *out_de
 
 // the first n scalars into the pinned host mirror: a kernel writes them over
 // the coherent link (1-2 us behind the kernel before it, a copy engine's
-// transfer about 9)
-__global__ void k_publish(const double *scal, double *host, int n) {
+// transfer about 9). inv: also scal[S_INV] = 1 / sqrt(scal[S_TMP]) (0 where
+// that is 0), for the normalisation that follows: a square root and a division
+// in each of its threads made that kernel FP64-bound (35 us instead of 7 at 4.1M cells)
+__global__ void k_publish(double *scal, double *host, int n, int inv) {
     grid_begin();
     if ((int)threadIdx.x < n) host[threadIdx.x] = scal[threadIdx.x];
+    if (inv && threadIdx.x == 0) {
+        const double h = sqrt(scal[S_TMP]);
+        scal[S_INV] = h > 0.0 ? 1.0 / h : 0.0;
+    }
 }
 
 ibm_status sync_scalars(Ctx *c, int n) {
-    KL(-1, k_publish, 1, S_COUNT, c->scal, c->hscal, n);
+    KL(-1, k_publish, 1, S_COUNT, c->scal, c->hscal, n, 0);
     IBM_LAUNCHED(c);
     IBM_CUDA(c, cudaStreamSynchronize(c->s));
     return IBM_OK;
@@ -605,13 +612,13 @@ __global__ void k_scale(int64_t n, T * dst, const S * src, double a) {
     else GRID_STRIDE(c, n) dst[c] = (T)(a * (double)src[c]);
 }
 
-// dst = src / sqrt(*n2) (0 where the norm is 0), one product per element
-template <typename T>
-__global__ void k_normalise(int64_t n, T *dst, const T *src, const double *n2) {
+// dst = *a src
+template <typename T, typename S>
+__global__ void k_scale_dev(int64_t n, T * dst, const S * src, const double * a) {
     grid_begin();
-    const double h = sqrt(*n2), a = h > 0.0 ? 1.0 / h : 0.0;
-    if constexpr (sizeof(T) == 4) scale_f32(n, dst, src, (float)a);
-    else GRID_STRIDE(c, n) dst[c] = a * src[c];
+    const double f = *a;
+    if constexpr (sizeof(T) == 4 && sizeof(S) == 4) scale_f32(n, dst, src, (float)f);
+    else GRID_STRIDE(c, n) dst[c] = (T)(f * (double)src[c]);
 }
 
 // x += sum_i y_i Z_i
@@ -3171,9 +3178,13 @@ static ibm_status pcg(Ctx *c, MGHier<T> &H, int iters) {
     return IBM_OK;
 }
 
-// The ghost rows of z and the band sweeps. One block while it can own the
-// band (2048 cells in FP32, 1024 in FP64), a cluster of up to 16 blocks up to
-// 16 times that, one launch per sweep above.
+// The ghost rows of z and the band sweeps. One block while its sweep is short
+// (2048 rows in FP32; 512 in FP64, whose sweep takes a block 10 operations a row
+// at 2 per clock), then a cluster of up to 16 blocks (16,384 rows in FP32, two a
+// thread: 24 us for the 192x128x128 wing's band; 8,192 in FP64: 34 us at 6,000
+// rows), else one launch per sweep on the whole device, about 3 us each in FP32
+// and 4-5 in FP64, where a cluster took 36 us with four FP32 rows a thread and
+// 55 us with two FP64 rows.
 template <typename T>
 static ibm_status band_sweeps(Ctx *c, const T *v, T *z) {
     const OpT<T> o = op_of<T>(c);
@@ -3181,13 +3192,13 @@ static ibm_status band_sweeps(Ctx *c, const T *v, T *z) {
     const T omega = (T)c->opts.band_omega;
     const int sweeps = c->opts.band_sweeps;
     T *buf = reinterpret_cast<T *>(c->btmp);   // (10 doubles per band cell: room for either precision)
-    constexpr int MAX = BandRows<T>::MAX;
+    constexpr int MAX = BandRows<T>::MAX, WIDE = sizeof(T) == 4 ? 2 : 1;   // rows a thread: one block, a cluster
     const int64_t one = (int64_t)BAND_THREADS * MAX;
     int ncta = 1;
     if (b.nb > one)
         while (ncta < c->bot_ctas && (int64_t)ncta * BAND_THREADS < b.nb) ncta *= 2;
     const int it = (int)((b.nb + (int64_t)ncta * BAND_THREADS - 1) / ((int64_t)ncta * BAND_THREADS));
-    if (it > MAX) {
+    if (it > (ncta == 1 ? MAX : WIDE)) {
         const unsigned gb = (unsigned)((b.nb + 255) / 256);
         T *cur = buf, *nxt = buf + b.nb, *zh = buf + 2 * (size_t)b.nb;
         KL(-1, k_band_start<T>, gb, 256, c->g, c->gh, o, b, c->type, v, z, omega, cur, zh);
@@ -3199,9 +3210,10 @@ static ibm_status band_sweeps(Ctx *c, const T *v, T *z) {
         return IBM_OK;
     }
     typedef void (*Fn)(GridDev, GhostDev, OpT<T>, BandDev, const uint8_t *, const T *, T *, T, int, T *, int);
-    Fn fn;
-    if (ncta == 1) fn = it == 1 ? k_band_sweeps<T, 1, true> : (it == 2 ? k_band_sweeps<T, 2, true> : k_band_sweeps<T, MAX, true>);
-    else fn = it == 1 ? k_band_sweeps<T, 1, false> : (it == 2 ? k_band_sweeps<T, 2, false> : k_band_sweeps<T, MAX, false>);
+    Fn fn = ncta == 1 ? k_band_sweeps<T, 1, true> : k_band_sweeps<T, 1, false>;
+    if constexpr (sizeof(T) == 4) {
+        if (it > 1) fn = ncta > 1 ? k_band_sweeps<T, WIDE, false> : (it == 2 ? k_band_sweeps<T, 2, true> : k_band_sweeps<T, MAX, true>);
+    }
     const bool ahead = overlap_launch(c);
     const size_t dyn = ncta == 1 ? sizeof(T) * 10 * (size_t)b.nb : 0;
     if (dyn > 0) IBM_CUDA(c, cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(10 * one * sizeof(T))));
@@ -3355,11 +3367,11 @@ static ibm_status fgmres(Ctx *c, Krylov<T> K, T *x, const T *b, double bnorm, do
             inner += c->opts.inner_iters;
             IBM_TRY(gs_step<T>(c, K, j));
             // the host reads the column while the device normalises w
-            KL(-1, k_publish, 1, S_COUNT, c->scal, c->hscal, (int)S_FLAG + 1);
+            KL(-1, k_publish, 1, S_COUNT, c->scal, c->hscal, (int)S_FLAG + 1, 1);
             IBM_LAUNCHED(c);
             IBM_CUDA(c, cudaEventRecord(c->ev6, c->s));
             if (j + 1 < m) {
-                KL(-1, k_normalise<T>, c->nred_wide, RED_THREADS, n, K.V[j + 1], K.w, c->scal + S_TMP);
+                KL(-1, (k_scale_dev<T, T>), c->nred_wide, RED_THREADS, n, K.V[j + 1], K.w, c->scal + S_INV);
                 IBM_LAUNCHED(c);
             }
             IBM_CUDA(c, cudaEventSynchronize(c->ev6));
@@ -3671,13 +3683,6 @@ ibm_status cond_close(Ctx *c, CondScope *sc) {
 __global__ void k_set_cond(cudaGraphConditionalHandle h, const int *flag) {
     grid_begin(); cudaGraphSetConditional(h, *flag ? 1u : 0u); }
 
-template <typename T, typename S>
-__global__ void k_scale_dev(int64_t n, T * dst, const S * src, const double * a) {
-    grid_begin();
-    const double f = *a;
-    if constexpr (sizeof(T) == 4 && sizeof(S) == 4) scale_f32(n, dst, src, (float)f);
-    else GRID_STRIDE(c, n) dst[c] = (T)(f * (double)src[c]);
-}
 
 // x += sum_{q < ncols} y_q Z_q with y and ncols from the control block
 template <typename T>
