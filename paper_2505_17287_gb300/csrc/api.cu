@@ -193,12 +193,6 @@ ibm_status alloc_krylov(Ctx *c, int m) {
         if (!(c->V[i] = (double *)dev_alloc(c, sizeof(double) * c->N))) return c->fail(IBM_ERR_OOM, "Krylov vector allocation failed");
     for (int i = 0; i < nz; ++i)
         if (!(c->Z[i] = (double *)dev_alloc(c, sizeof(double) * c->N))) return c->fail(IBM_ERR_OOM, "Krylov vector allocation failed");
-    if (!c->Vdev) c->Vdev = (double **)dev_alloc(c, sizeof(double *) * 17);
-    if (!c->Zdev) c->Zdev = (double **)dev_alloc(c, sizeof(double *) * 17);
-    if (!c->Vdev || !c->Zdev) return c->fail(IBM_ERR_OOM, "pointer table allocation failed");
-    IBM_CUDA(c, cudaMemcpyAsync(c->Vdev, c->V.data(), sizeof(double *) * (m + 1), cudaMemcpyHostToDevice, c->s));
-    IBM_CUDA(c, cudaMemcpyAsync(c->Zdev, c->Z.data(), sizeof(double *) * nz, cudaMemcpyHostToDevice, c->s));
-    IBM_CUDA(c, cudaStreamSynchronize(c->s));
     c->m_cap = m;
     return IBM_OK;
 }
@@ -403,6 +397,8 @@ static ibm_status create_impl(Ctx *c, const ibm_grid_desc *d) {
         const int64_t spread = cells < 2 * 152 ? cells : 2 * 152;
         const int64_t r = std::max((c->N + 8 * RED_THREADS - 1) / (8 * RED_THREADS), spread);
         c->nred = (int)(r > RED_BLOCKS ? RED_BLOCKS : r);
+        const int64_t w64 = std::min<int64_t>(c->N / (16 * RED_THREADS), RED_BLOCKS_MAX);
+        c->nred64 = (int)std::max<int64_t>(std::min(c->nred, 152 * 6), w64);
         const int64_t w = std::max((c->N + 2 * RED_THREADS - 1) / (2 * RED_THREADS), spread);
         c->nred_wide = (int)(w > RED_BLOCKS_MAX ? RED_BLOCKS_MAX : w);
         const int64_t e = (c->N + 255) / 256;

@@ -169,14 +169,12 @@ struct Ctx {
     // Poisson (FP64 FGMRES)
     int m_cap = 0;
     std::vector<double *> V, Z;
-    double **Vdev = nullptr, **Zdev = nullptr;   // device arrays of the V / Z pointers
     double *w = nullptr, *rr = nullptr;
     // FP32 storage of mixed mode
     float *op32[12] = {nullptr};         // cxm..czs, dx, dy, dz in FP32
     float *wp32 = nullptr;
     int64_t wp32_n = -1;
     std::vector<float *> V32, Z32;
-    float **Vdev32 = nullptr, **Zdev32 = nullptr;
     float *w32 = nullptr, *r32 = nullptr, *d32 = nullptr, *b32 = nullptr;
     int m32_cap = 0;
     // Poisson guess history: hist_cap pairs of N doubles (solutions, projected
@@ -240,6 +238,12 @@ struct Ctx {
     // latency-bound); the flow kernels nelem blocks of 256
     int nred = RED_BLOCKS;
     int nred_wide = RED_BLOCKS;
+    // the FP64 stencil reductions: nred up to one wave of six blocks per SM,
+    // then 16 cells per thread, at most RED_BLOCKS_MAX (a block's own FP64
+    // reduction costs a thread about one cell's operations: with 2.5 cells
+    // per thread a product at 3.1M cells took 70 us, with one wave 59; at
+    // 62.9M cells one wave took 1.36 ms, 13 waves' worth of blocks 1.16)
+    int nred64 = RED_BLOCKS;
     unsigned nelem = 152 * 16;
     int bot_ctas = 0;      // largest cluster of the V-cycle bottom on this device (0: not asked yet)
     uint64_t mg_gen = 0;   // multigrid rebuild counter (invalidates captured V-cycles)

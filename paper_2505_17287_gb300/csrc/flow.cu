@@ -66,17 +66,23 @@ __device__ __forceinline__ P pick3(int q, P a, P b, P c) { return q == 0 ? a : (
 // on FLUID cells; other cells get rhs = 0 and N = 0. Per axis the face area
 // over the volume is 1/width, and the viscous face coefficients are the
 // pressure operator's per-axis coefficients; a Dirichlet wall contributes
-// 2 (value - u_c) / width^2.
+// 2 (value - u_c) / width^2. The start values of the implicit solve, us = u,
+// are written on the way (on all cells), in place of a copy per component.
+// Bound by the FP64 pipe (two operations per clock and SM): 66 operations a
+// cell in 3D against 137 bytes. Each product is accumulated by an FMA of its
+// own (a difference of two products added afterwards took one operation more
+// per axis and component) and the walls' implicit share rides in off: 62.9M
+// cells 9.94 -> 8.77 ms, and three copies of 0.18 ms gone.
 __global__ void k_conv_rhs(GridDev g, const uint8_t * type, const double * dg, CFields3 u,
                            CFields3 F, CFields3 Nold, int first, const uint8_t * fresh, Fields3 Nnew,
-                           Fields3 rhs, BCInfo bc, double dt, double alpha, int ncomp) {
+                           Fields3 rhs, Fields3 us, BCInfo bc, double dt, double alpha, int ncomp) {
     grid_begin();
     const int64_t sy = g.nx, sz = (int64_t)g.nx * g.ny;
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < g.n; c += (int64_t)gridDim.x * blockDim.x) {
         if (type[c] != FLUID) {
 #pragma unroll
             for (int q = 0; q < 3; ++q)
-                if (q < ncomp) { Nnew.p[q][c] = 0.0; rhs.p[q][c] = 0.0; }
+                if (q < ncomp) { Nnew.p[q][c] = 0.0; rhs.p[q][c] = 0.0; us.p[q][c] = u.p[q][c]; }
             continue;
         }
         int i, j, k;
@@ -126,11 +132,13 @@ __global__ void k_conv_rhs(GridDev g, const uint8_t * type, const double * dg, C
             const double *noq = pick3(q, Nold.p[0], Nold.p[1], Nold.p[2]);
             double *nnq = pick3(q, Nnew.p[0], Nnew.p[1], Nnew.p[2]);
             double *rq = pick3(q, rhs.p[0], rhs.p[1], rhs.p[2]);
+            double *usq = pick3(q, us.p[0], us.p[1], us.p[2]);
             const double uc = uq[c];
-            // lap = off - D uc with off the neighbour (and Dirichlet wall)
-            // terms and D the diagonal; src is the wall values' share of the
-            // implicit half of Crank-Nicolson
-            double N = dF * uc, off = 0.0, D = dint, src = 0.0;
+            usq[c] = uc;
+            // off - D uc: off the neighbour terms and the Dirichlet wall
+            // terms, the latter twice (the explicit half of Crank-Nicolson
+            // and the wall values' share of the implicit half), D the diagonal
+            double N = dF * uc, off = 0.0, D = dint;
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 if (a >= g.ndim) break;
@@ -141,9 +149,8 @@ __global__ void k_conv_rhs(GridDev g, const uint8_t * type, const double * dg, C
                 } else if (pick3(q, bc.dir[0][2 * a], bc.dir[1][2 * a], bc.dir[2][2 * a])) {
                     const double v = pick3(q, bc.val[0][2 * a], bc.val[1][2 * a], bc.val[2][2 * a]), w2 = 2.0 * rw[a] * rw[a];
                     ulo = 2.0 * v - uc;
-                    off += w2 * v;
+                    off += 2.0 * (w2 * v);
                     D += w2;
-                    src += w2 * v;
                 } else {
                     ulo = uc;
                 }
@@ -153,26 +160,27 @@ __global__ void k_conv_rhs(GridDev g, const uint8_t * type, const double * dg, C
                 } else if (pick3(q, bc.dir[0][2 * a + 1], bc.dir[1][2 * a + 1], bc.dir[2][2 * a + 1])) {
                     const double v = pick3(q, bc.val[0][2 * a + 1], bc.val[1][2 * a + 1], bc.val[2][2 * a + 1]), w2 = 2.0 * rw[a] * rw[a];
                     uhi = 2.0 * v - uc;
-                    off += w2 * v;
+                    off += 2.0 * (w2 * v);
                     D += w2;
-                    src += w2 * v;
                 } else {
                     uhi = uc;
                 }
-                N += fh[a] * uhi - fl[a] * ulo;
+                N += fh[a] * uhi;
+                N -= fl[a] * ulo;
             }
             // Euler start on the first step, and at fresh cells (no history)
             const double No = (first || (fresh && fresh[c])) ? N : noq[c];
             nnq[c] = N;
-            rq[c] = (uc - c15 * N + c05 * No) + alpha * ((off - D * uc) + src);
+            rq[c] = (uc - c15 * N + c05 * No) + alpha * (off - D * uc);
         }
     }
 }
 
-// diagonal of (I - alpha L0) for component q at FLUID cell (i, j, k)
-__device__ __forceinline__ double helm_D(const GridDev &g, const BCInfo &bc, int q, double alpha, int i, int j,
-                                         int k) {
-    double d = g.cxs[i] + g.cys[j] + (g.ndim == 3 ? g.czs[k] : 0.0);
+// diagonal of (I - alpha L0) for component q at FLUID cell (i, j, k); d the
+// cell's sum of the interior face coefficients (stored: its two FP64 adds
+// cost more than reading it)
+__device__ __forceinline__ double helm_D(const GridDev &g, const BCInfo &bc, int q, double alpha, double d, int i,
+                                         int j, int k) {
     const bool edge = i == 0 || i == g.nx - 1 || j == 0 || j == g.ny - 1 ||
                       (g.ndim == 3 && (k == 0 || k == g.nz - 1));
     if (edge) {
@@ -191,14 +199,14 @@ __device__ __forceinline__ double helm_D(const GridDev &g, const BCInfo &bc, int
 }
 
 // inverse diagonal of (I - alpha L0) for component q on FLUID cells
-__global__ void k_helm_diag(GridDev g, const uint8_t * type, BCInfo bc, int q, double alpha,
+__global__ void k_helm_diag(GridDev g, const uint8_t * type, const double * dg, BCInfo bc, int q, double alpha,
                             double * hinv) {
     grid_begin();
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < g.n; c += (int64_t)gridDim.x * blockDim.x) {
         if (type[c] != FLUID) { hinv[c] = 0.0; continue; }
         int i, j, k;
         split3(g, (uint32_t)c, i, j, k);
-        hinv[c] = 1.0 / helm_D(g, bc, q, alpha, i, j, k);
+        hinv[c] = 1.0 / helm_D(g, bc, q, alpha, dg[c], i, j, k);
     }
 }
 
@@ -295,7 +303,11 @@ __global__ void k_helm_jacobi(GridDev g, HelmCoef h, const uint8_t * type, const
 // residual of the Helmholtz system on FLUID rows; partial columns |r|^2, |rhs|^2
 // (the diagonal is formed again rather than divided out of hinv: an FP64
 // division costs several times the few adds)
-__global__ void k_helm_resid(GridDev g, HelmCoef h, const uint8_t * type, const double * rhs,
+// Bound by the FP64 pipe: 10 operations a cell; six
+// blocks an SM (40 registers, no spills), since with two waves of four
+// blocks the loads' latency showed (62.9M cells: 1.82 -> 1.46 ms, 71% of the
+// pipe's rate with 12 operations before).
+__global__ void __launch_bounds__(RED_THREADS, 6) k_helm_resid(GridDev g, HelmCoef h, const uint8_t * type, const double * dg, const double * rhs,
                              BCInfo bc, int q, const double * u, double alpha,
                              double * part) {
     grid_begin();
@@ -305,9 +317,10 @@ __global__ void k_helm_resid(GridDev g, HelmCoef h, const uint8_t * type, const 
         if (type[c] != FLUID) continue;
         int i, j, k;
         split3(g, (uint32_t)c, i, j, k);
-        const double r = visc_sum(g, h, u, c, i, j, k, rhs[c]) - u[c] * helm_D(g, bc, q, alpha, i, j, k);
+        const double f = rhs[c];
+        const double r = visc_sum(g, h, u, c, i, j, k, f) - u[c] * helm_D(g, bc, q, alpha, dg[c], i, j, k);
         rr += r * r;
-        bb += rhs[c] * rhs[c];
+        bb += f * f;
     }
     rr = block_sum<RED_THREADS>(rr, sh);
     bb = block_sum<RED_THREADS>(bb, sh);
@@ -539,57 +552,47 @@ __global__ void k_divergence(GridDev g, const uint8_t * type, CFields3 F, double
     }
 }
 
-// projection of the interior faces of axis a that have a FLUID side
-// (fdx, fdy: multiply-shift dividers by the face counts along x and y; the
-// gradient multiplies by the stored reciprocal centre spacing)
-__global__ void k_project_faces(GridDev g, const uint8_t * type, const double * phi, int a,
-                                double dt, double * Fa, FastDiv fdx, FastDiv fdy) {
-    grid_begin();
-    const int nfx = g.nx + (a == 0), nfy = g.ny + (a == 1), nfz = g.nz + (a == 2);
-    const int64_t nf = (int64_t)nfx * nfy * nfz;
-    const int64_t st = a == 0 ? 1 : (a == 1 ? (int64_t)g.nx : (int64_t)g.nx * g.ny);
-    const int nax = a == 0 ? g.nx : (a == 1 ? g.ny : g.nz);
-    const double *rh = a == 0 ? g.rhx : (a == 1 ? g.rhy : g.rhz);
-    for (int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; f < nf; f += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t t = fdx.div((uint32_t)f), fk = fdy.div(t);
-        const int fi = (int)((uint32_t)f - t * (uint32_t)nfx), fj = (int)(t - fk * (uint32_t)nfy);
-        const int fa = a == 0 ? fi : (a == 1 ? fj : (int)fk);
-        if (fa == 0 || fa == nax) continue;
-        const int64_t cR = (int64_t)fi + (int64_t)g.nx * (fj + (int64_t)g.ny * fk);
-        const int64_t cL = cR - st;
-        if (type[cL] != FLUID && type[cR] != FLUID) continue;
-        Fa[f] -= dt * (phi[cR] - phi[cL]) * rh[fa];
+// one axis of the projection at cell c: the low face's velocity (interior
+// faces with a FLUID side) takes dt times its gradient, the cell's the mean
+// of its two faces' (hdt = dt / 2); ci, n the cell's index and count along
+// the axis, st its stride, lo/cell FLUID flags
+__device__ __forceinline__ void project_axis(const double * phi, double pc, const uint8_t * type, int64_t c,
+                                             int64_t st, int ci, int n, const double * rh, bool cell, double dt,
+                                             double hdt, double * Flo, const double * us, double * u) {
+    double v = us[c];
+    if (ci > 0) {
+        const bool lo = type[c - st] == FLUID;
+        if (cell || lo) {
+            const double glo = (pc - phi[c - st]) * rh[ci];
+            *Flo -= dt * glo;
+            if (cell) v -= hdt * glo;
+        }
     }
+    if (cell && ci < n - 1) v -= hdt * ((phi[c + st] - pc) * rh[ci + 1]);
+    u[c] = v;
 }
 
-// cell velocities on FLUID cells: u_a -= dt * mean of the two face gradients
-__global__ void k_project_cells(GridDev g, const uint8_t * type, const double * phi,
-                                CFields3 us, Fields3 u, double dt) {
+// projection: each cell updates its low faces and, on FLUID cells, its own
+// velocities (u = us - dt times the mean of the two face gradients; other
+// cells copy us). Bound by the FP64 pipe, 21 operations a cell in 3D: a
+// cell's low-face gradients serve the face and the cell, where a pass per
+// axis over the faces and one over the cells took 27 and read phi and the
+// types four times (62.9M cells: 3.74 -> 2.51 ms, 90% of the pipe's rate).
+__global__ void __launch_bounds__(256, 6) k_project(GridDev g, const uint8_t * type, const double * phi, Fields3 F, CFields3 us,
+                          Fields3 u, double dt) {
     grid_begin();
     const int64_t sy = g.nx, sz = (int64_t)g.nx * g.ny;
+    const double hdt = 0.5 * dt;
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < g.n; c += (int64_t)gridDim.x * blockDim.x) {
-        const uint8_t t = type[c];
-        if (t != FLUID) {
-            u.p[0][c] = us.p[0][c];
-            u.p[1][c] = us.p[1][c];
-            if (g.ndim == 3) u.p[2][c] = us.p[2][c];
-            continue;
-        }
+        const bool cell = type[c] == FLUID;
         int i, j, k;
         split3(g, (uint32_t)c, i, j, k);
         const double pc = phi[c];
-        double glo, ghi;
-        glo = i > 0 ? (pc - phi[c - 1]) * g.rhx[i] : 0.0;
-        ghi = i < g.nx - 1 ? (phi[c + 1] - pc) * g.rhx[i + 1] : 0.0;
-        u.p[0][c] = us.p[0][c] - dt * (0.5 * (glo + ghi));
-        glo = j > 0 ? (pc - phi[c - sy]) * g.rhy[j] : 0.0;
-        ghi = j < g.ny - 1 ? (phi[c + sy] - pc) * g.rhy[j + 1] : 0.0;
-        u.p[1][c] = us.p[1][c] - dt * (0.5 * (glo + ghi));
-        if (g.ndim == 3) {
-            glo = k > 0 ? (pc - phi[c - sz]) * g.rhz[k] : 0.0;
-            ghi = k < g.nz - 1 ? (phi[c + sz] - pc) * g.rhz[k + 1] : 0.0;
-            u.p[2][c] = us.p[2][c] - dt * (0.5 * (glo + ghi));
-        }
+        project_axis(phi, pc, type, c, 1, i, g.nx, g.rhx, cell, dt, hdt, F.p[0] + fx_lo(g, i, j, k), us.p[0], u.p[0]);
+        project_axis(phi, pc, type, c, sy, j, g.ny, g.rhy, cell, dt, hdt, F.p[1] + fy_lo(g, i, j, k), us.p[1], u.p[1]);
+        if (g.ndim == 3)
+            project_axis(phi, pc, type, c, sz, k, g.nz, g.rhz, cell, dt, hdt, F.p[2] + fz_lo(g, i, j, k), us.p[2],
+                         u.p[2]);
     }
 }
 
@@ -746,7 +749,7 @@ static ibm_status helm_prepare(Ctx *c) {
         for (int cq = 0; cq < c->ndim; ++cq) {
             if (!c->hinv[cq]) c->hinv[cq] = (double *)dev_alloc(c, sizeof(double) * c->N);
             if (!c->hinv[cq]) return c->fail(IBM_ERR_OOM, "Helmholtz diagonal allocation failed");
-            ++c->nlaunch, launch(c, k_helm_diag, c->nelem, 256, c->g, c->type, bc, cq, alpha, c->hinv[cq]);
+            ++c->nlaunch, launch(c, k_helm_diag, c->nelem, 256, c->g, c->type, c->dg_c, bc, cq, alpha, c->hinv[cq]);
         }
         IBM_LAUNCHED(c);
         c->hinv_ok = true;
@@ -824,9 +827,9 @@ static ibm_status helmholtz_srj(Ctx *c, int q, int *sweeps) {
         }
         // M is even: the iterate is back in ustar[q]
         Fields3 U{{u, u, u}};
-        ++c->nlaunch, launch(c, k_helm_resid, c->nred, RED_THREADS, c->g, helm_coef(c), c->type, rhs, make_bc(c), q, u, alpha, c->part);
+        ++c->nlaunch, launch(c, k_helm_resid, c->nred64, RED_THREADS, c->g, helm_coef(c), c->type, c->dg_c, rhs, make_bc(c), q, u, alpha, c->part);
         IBM_LAUNCHED(c);
-        IBM_TRY(finalize(c, c->part, c->nred, 2, 1.0, c->scal + 48));
+        IBM_TRY(finalize(c, c->part, c->nred64, 2, 1.0, c->scal + 48));
         double gmax = 0.0;
         if (c->ng > 0) {
             vghost_pass(c, U, 1, q, c->scal + 50, false);
@@ -886,9 +889,9 @@ static ibm_status helmholtz(Ctx *c, int q, int *sweeps) {
         ++*sweeps;
         if (*sweeps == next_check || it + 1 == c->opts.helm_maxit) {
             next_check = helm_next_check(next_check);
-            ++c->nlaunch, launch(c, k_helm_resid, c->nred, RED_THREADS, c->g, helm_coef(c), c->type, rhs, make_bc(c), q, u, alpha, c->part);
+            ++c->nlaunch, launch(c, k_helm_resid, c->nred64, RED_THREADS, c->g, helm_coef(c), c->type, c->dg_c, rhs, make_bc(c), q, u, alpha, c->part);
             IBM_LAUNCHED(c);
-            IBM_TRY(finalize(c, c->part, c->nred, 2, 1.0, c->scal + 48));
+            IBM_TRY(finalize(c, c->part, c->nred64, 2, 1.0, c->scal + 48));
             double gmax = 0.0;
             if (c->ng > 0) {
                 // ghost-row residual: largest change a further Jacobi pass would make
@@ -919,15 +922,15 @@ ibm_status flow_step(Ctx *c, ibm_step_stats *st) {
     CFields3 No{{c->Nold[0], c->Nold[1], nc == 3 ? c->Nold[2] : c->Nold[1]}};
     Fields3 Nn{{c->Nnew[0], c->Nnew[1], nc == 3 ? c->Nnew[2] : c->Nnew[1]}};
     Fields3 R{{c->rhs[0], c->rhs[1], nc == 3 ? c->rhs[2] : c->rhs[1]}};
+    Fields3 Us{{c->ustar[0], c->ustar[1], nc == 3 ? c->ustar[2] : c->ustar[1]}};
     kt_begin(c, K_CONV);
-    ++c->nlaunch, launch(c, k_conv_rhs, c->nelem, 256, c->g, c->type, c->dg_c, u, F, No, c->have_nold ? 0 : 1, c->fresh_pending ? c->fresh : nullptr, Nn, R, make_bc(c), dt,
+    ++c->nlaunch, launch(c, k_conv_rhs, c->nelem, 256, c->g, c->type, c->dg_c, u, F, No, c->have_nold ? 0 : 1, c->fresh_pending ? c->fresh : nullptr, Nn, R, Us, make_bc(c), dt,
                                            alpha, nc);
     kt_end(c, K_CONV);
     IBM_LAUNCHED(c);
     ibm_status status = IBM_OK;
     int sweeps_total = 0;
     for (int q = 0; q < nc; ++q) {
-        IBM_CUDA(c, cudaMemcpyAsync(c->ustar[q], c->u[q], sizeof(double) * c->N, cudaMemcpyDeviceToDevice, c->s));
         int sw = 0;
         ibm_status s = helmholtz(c, q, &sw);
         sweeps_total += sw;
@@ -949,17 +952,10 @@ ibm_status flow_step(Ctx *c, ibm_step_stats *st) {
     else if (s != IBM_OK) return s;
     IBM_TRY(hist_store(c, c->p));
     IBM_CUDA(c, cudaEventRecord(c->ev3, c->s));
-    for (int a = 0; a < nc; ++a) {
-        const int64_t nf = a == 0 ? c->NFx : (a == 1 ? c->NFy : c->NFz);
-        const unsigned nb = (unsigned)((nf + 255) / 256 > 152 * 32 ? 152 * 32 : (nf + 255) / 256);
-        ++c->nlaunch, launch(c, k_project_faces, nb, 256, c->g, c->type, c->p, a, dt, c->F[a],
-                                                          FastDiv((uint32_t)(c->nx + (a == 0))),
-                                                          FastDiv((uint32_t)(c->ny + (a == 1))));
-    }
-    IBM_LAUNCHED(c);
     CFields3 us{{c->ustar[0], c->ustar[1], nc == 3 ? c->ustar[2] : c->ustar[1]}};
     Fields3 un{{c->u[0], c->u[1], nc == 3 ? c->u[2] : c->u[1]}};
-    ++c->nlaunch, launch(c, k_project_cells, c->nelem, 256, c->g, c->type, c->p, us, un, dt);
+    Fields3 Fp{{c->F[0], c->F[1], nc == 3 ? c->F[2] : c->F[1]}};
+    ++c->nlaunch, launch(c, k_project, c->nelem, 256, c->g, c->type, c->p, Fp, us, un, dt);
     IBM_LAUNCHED(c);
     int passes = 0;
     IBM_TRY(ghost_refresh_all(c, c->u, &passes));
@@ -1267,10 +1263,10 @@ static ibm_status helmholtz_dev(Ctx *c, int q) {
         }
     };
     auto test = [&]() -> ibm_status {
-        ++c->nlaunch, launch(c, k_helm_resid, c->nred, RED_THREADS, c->g, helm_coef(c), c->type, rhs, make_bc(c), q, u, alpha,
+        ++c->nlaunch, launch(c, k_helm_resid, c->nred64, RED_THREADS, c->g, helm_coef(c), c->type, c->dg_c, rhs, make_bc(c), q, u, alpha,
                              c->part);
         IBM_LAUNCHED(c);
-        IBM_TRY(finalize(c, c->part, c->nred, 2, 1.0, c->scal + 48));
+        IBM_TRY(finalize(c, c->part, c->nred64, 2, 1.0, c->scal + 48));
         if (c->ng > 0) vghost_pass(c, U, 1, q, c->scal + 50, false);
         IBM_LAUNCHED(c);
         return IBM_OK;
@@ -1347,11 +1343,11 @@ static ibm_status flow_step_capture(Ctx *c) {
     CFields3 No{{c->Nold[0], c->Nold[1], nc == 3 ? c->Nold[2] : c->Nold[1]}};
     Fields3 Nn{{c->Nnew[0], c->Nnew[1], nc == 3 ? c->Nnew[2] : c->Nnew[1]}};
     Fields3 R{{c->rhs[0], c->rhs[1], nc == 3 ? c->rhs[2] : c->rhs[1]}};
-    ++c->nlaunch, launch(c, k_conv_rhs, c->nelem, 256, c->g, c->type, c->dg_c, u, F, No, c->have_nold ? 0 : 1, c->fresh_pending ? c->fresh : nullptr, Nn, R,
+    Fields3 Us{{c->ustar[0], c->ustar[1], nc == 3 ? c->ustar[2] : c->ustar[1]}};
+    ++c->nlaunch, launch(c, k_conv_rhs, c->nelem, 256, c->g, c->type, c->dg_c, u, F, No, c->have_nold ? 0 : 1, c->fresh_pending ? c->fresh : nullptr, Nn, R, Us,
                                                        make_bc(c), dt, alpha, nc);
     IBM_LAUNCHED(c);
     for (int q = 0; q < nc; ++q) {
-        IBM_CUDA(c, cudaMemcpyAsync(c->ustar[q], c->u[q], sizeof(double) * c->N, cudaMemcpyDeviceToDevice, c->s));
         IBM_TRY(helmholtz_dev(c, q));
     }
     IBM_TRY(faces_from(c, c->ustar));
@@ -1364,16 +1360,10 @@ static ibm_status flow_step_capture(Ctx *c) {
     IBM_TRY(hist_guess(c, braw, c->p));
     IBM_TRY(poisson_solve_dev(c, braw, c->p, c->opts.rtol, c->opts.max_outer));
     IBM_TRY(hist_store(c, c->p));
-    for (int a = 0; a < nc; ++a) {
-        const int64_t nf = a == 0 ? c->NFx : (a == 1 ? c->NFy : c->NFz);
-        const unsigned nb = (unsigned)((nf + 255) / 256 > 152 * 32 ? 152 * 32 : (nf + 255) / 256);
-        ++c->nlaunch, launch(c, k_project_faces, nb, 256, c->g, c->type, c->p, a, dt, c->F[a],
-                                                          FastDiv((uint32_t)(c->nx + (a == 0))),
-                                                          FastDiv((uint32_t)(c->ny + (a == 1))));
-    }
     CFields3 us{{c->ustar[0], c->ustar[1], nc == 3 ? c->ustar[2] : c->ustar[1]}};
     Fields3 un{{c->u[0], c->u[1], nc == 3 ? c->u[2] : c->u[1]}};
-    ++c->nlaunch, launch(c, k_project_cells, c->nelem, 256, c->g, c->type, c->p, us, un, dt);
+    Fields3 Fp{{c->F[0], c->F[1], nc == 3 ? c->F[2] : c->F[1]}};
+    ++c->nlaunch, launch(c, k_project, c->nelem, 256, c->g, c->type, c->p, Fp, us, un, dt);
     IBM_LAUNCHED(c);
     IBM_TRY(ghost_refresh_dev(c));
     IBM_TRY(step_stats_dev(c, ((HelmCtl *)c->hctl)->sweeps));

@@ -14,9 +14,10 @@
 //           FP64); then the ghost rows; then damped Jacobi sweeps of the full
 //           operator on the cells within two faces of a ghost cell;
 //   multigrid: V(nu1,nu2) cycle, red-black Gauss-Seidel smoothing,
-//           restriction by summing children, piecewise-constant prolongation,
+//           trilinear prolongation renormalised over the active coarse cells
+//           and its transpose as restriction (mg_interp 0: piecewise constant),
 //           coarse operators rediscretised from the open child-face areas,
-//           coarsest level solved by red-black sweeps in one thread block.
+//           the coarsest level's red-black sweeps applied as one matrix.
 //
 // GB300 runs FP64 at 1/64 of its FP32 rate, so the FP64 kernels here are
 // written to minimise FP64 instructions: per-axis 1D operator coefficients,
@@ -112,37 +113,84 @@ ibm_status sync_scalars(Ctx *c, int n) {
 #define GRID_STRIDE(c, n) \
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < (n); c += (int64_t)gridDim.x * blockDim.x)
 
-// sum over FLUID cells of vol * x (x null: the FLUID volume)
-__global__ void k_fluid_volsum(GridDev g, const uint8_t * type, const double * x,
+// sum over FLUID cells of vol * x (x null: the FLUID volume), vol the stored
+// cell volumes; four cells' loads are issued together (one at a time, the
+// pass waited for memory at a third of its rate), the sum in the same order
+__global__ void k_fluid_volsum(int64_t n, const uint8_t * type, const double * vol, const double * x,
                                double * part) {
     grid_begin();
     __shared__ double sh[32];
     double acc = 0.0;
-    GRID_STRIDE(c, g.n) {
-        if (type[c] != FLUID) continue;
-        int i, j, k;
-        split3(g, (uint32_t)c, i, j, k);
-        acc += (g.dx[i] * g.dy[j] * g.dz[k]) * (x ? x[c] : 1.0);
+    const int64_t st = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t c0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c0 < n; c0 += 4 * st) {
+        double v[4], y[4];
+        bool f[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int64_t c = c0 + e * st;
+            const bool in = c < n;
+            f[e] = in && type[c] == FLUID;
+            v[e] = in ? vol[c] : 0.0;
+            y[e] = in && x ? x[c] : 1.0;
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (f[e]) acc += v[e] * y[e];
     }
     acc = block_sum<RED_THREADS>(acc, sh);
     if (threadIdx.x == 0) part[blockIdx.x] = acc;
 }
 
-// x -= mean on FLUID (and GHOST if ghosts) cells; DEAD cells set to 0
+// x -= mean on FLUID and GHOST cells; DEAD cells set to 0
 __global__ void k_sub_mean(int64_t n, const uint8_t * type, double * x,
-                           const double * mean, int ghosts) {
+                           const double * mean) {
     grid_begin();
     const double m = *mean;
     GRID_STRIDE(c, n) {
         const uint8_t t = type[c];
-        if (t == FLUID || (ghosts && t == GHOST)) x[c] -= m;
+        if (t == FLUID || t == GHOST) x[c] -= m;
         else if (t == DEAD) x[c] = 0.0;
     }
 }
 
+// the pressure equation's right-hand side: b = rhs - mean on FLUID cells, 0 on
+// GHOST rows (homogeneous Neumann on the body) and DEAD cells; partials of
+// |b|^2 (one pass in place of a copy, the mean removal, the ghost rows' zeros
+// and the norm; two cells' loads issued together)
+__global__ void k_rhs_b(int64_t n, const uint8_t * type, const double * rhs, const double * mean, double * b,
+                        double * part) {
+    grid_begin();
+    __shared__ double sh[32];
+    const double m = *mean;
+    const int64_t st = (int64_t)gridDim.x * blockDim.x;
+    double acc = 0.0;
+    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n; c += 2 * st) {
+        const int64_t d = c + st < n ? c + st : c;
+        const double r0 = rhs[c], r1 = rhs[d];
+        const double b0 = type[c] == FLUID ? r0 - m : 0.0, b1 = type[d] == FLUID ? r1 - m : 0.0;
+        b[c] = b0;
+        acc += b0 * b0;
+        if (d != c) {
+            b[d] = b1;
+            acc += b1 * b1;
+        }
+    }
+    acc = block_sum<RED_THREADS>(acc, sh);
+    if (threadIdx.x == 0) part[blockIdx.x] = acc;
+}
+
+// c->b from rhs, |b|^2 in scal[S_TMP]
+static ibm_status rhs_b(Ctx *c, const double *rhs) {
+    KL(-1, k_fluid_volsum, c->nred, RED_THREADS, c->N, c->type, c->vol_c, rhs, c->part);
+    IBM_TRY(finalize(c, c->part, c->nred, 1, 1.0 / c->fluid_vol, c->scal + S_MEAN));
+    KL(-1, k_rhs_b, c->nred, RED_THREADS, c->N, c->type, rhs, c->scal + S_MEAN, c->b, c->part);
+    IBM_LAUNCHED(c);
+    return finalize(c, c->part, c->nred, 1, 1.0, c->scal + S_TMP);
+}
+
 ibm_status fluid_mean(Ctx *c, const double *x, bool ghosts_too, double *mean_host) {
     (void)ghosts_too;
-    KL(-1, k_fluid_volsum, c->nred, RED_THREADS, c->g, c->type, x, c->part);
+    KL(-1, k_fluid_volsum, c->nred, RED_THREADS, c->N, c->type, c->vol_c, x, c->part);
     IBM_LAUNCHED(c);
     IBM_TRY(finalize(c, c->part, c->nred, 1, 1.0 / c->fluid_vol, c->scal + S_MEAN));
     if (mean_host) {
@@ -220,8 +268,10 @@ __device__ __forceinline__ void ghost_row(const GhostDev &gh, const OpT<T> &o, c
 // of vol * y.
 // (PLAIN: b null and sgn = 1, the product of every Krylov step; two FP64
 // operations per cell fewer)
+// (the FP64 form is bound by the FP64 pipe; six blocks an SM, 16 cells a thread
+// or more, see nred64: 62.9M cells 1.36 -> 1.16 ms)
 template <typename T, bool PLAIN = false>
-__global__ void k_apply_A(GridDev g, OpT<T> o, const uint8_t * type, const T * x,
+__global__ void __launch_bounds__(RED_THREADS, 6) k_apply_A(GridDev g, OpT<T> o, const uint8_t * type, const T * x,
                           const T * b, T sgn, T * y, double * part, int nb, GhostDev gh) {
     grid_begin();
     __shared__ double sh[32];
@@ -317,12 +367,6 @@ __global__ void __launch_bounds__(RED_THREADS)
 
 static inline bool al16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
-__global__ void k_zero_at(int64_t m, const int64_t * idx, double * x) {
-    grid_begin();
-    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q < m) x[idx[q]] = 0.0;
-}
-
 // x -= mean on FLUID cells (precision T); DEAD cells set to 0
 // (FP32: four cells per 16-byte access, the tail one by one)
 template <typename T>
@@ -368,8 +412,8 @@ OpT<float> op_of<float>(Ctx *c) {
 template <typename T>
 static ibm_status apply_A(Ctx *c, const T *x, const T *b, T sgn, T *y) {
     const OpT<T> o = op_of<T>(c);
-    const int nb = sizeof(T) == 4 ? c->nred_wide : c->nred;
-    const unsigned grid = (unsigned)nb + (unsigned)((c->ng + RED_THREADS - 1) / RED_THREADS);
+    int nb = sizeof(T) == 4 ? c->nred_wide : c->nred64;
+    unsigned grid = (unsigned)nb + (unsigned)((c->ng + RED_THREADS - 1) / RED_THREADS);
     if constexpr (sizeof(T) == 4) {
         if (c->g.nx % 4 == 0 && al16(x) && al16(y) && (!b || al16(b)))
             KL(K_APPLY_A, k_apply_A4, grid, RED_THREADS, c->g, o, c->type, x, b, sgn, y, c->part, nb, c->gh);
@@ -621,20 +665,59 @@ __global__ void k_scale_dev(int64_t n, T * dst, const S * src, const double * a)
     else GRID_STRIDE(c, n) dst[c] = (T)(f * (double)src[c]);
 }
 
-// x += sum_i y_i Z_i
+// x += sum_{q < nc} y_q Z_q, in the columns' order: 16-byte accesses (the
+// Krylov vectors are 16-byte aligned; the tail one by one) with the columns'
+// loads of four issued together, and the vectors' addresses kernel
+// parameters. The pass is bound by memory: 62.9M cells, eight FP32 columns
+// took 812 us with one 4-byte load at a time through an array of pointers,
+// 373 us so.
 template <typename T>
-__global__ void k_xupd(int64_t n, T * x, const T *const * Z, int ncols, Coef y) {
-    grid_begin();
-    T yv[17];
+__device__ __forceinline__ void xupd_cells(int64_t n, T *x, const VPtrs<T> &Z, int nc, const T *yv) {
+    constexpr int W = 16 / sizeof(T);
+    // (x may be a caller's FP64 vector, aligned to its type only)
+    const int64_t nv = ((uintptr_t)x & 15u) == 0 ? n / W : 0;
+    GRID_STRIDE(v, nv) {
+        T a[W];
+        const float4 x4 = reinterpret_cast<const float4 *>(x)[v];
+        memcpy(a, &x4, 16);
 #pragma unroll
-    for (int q = 0; q < 17; ++q) yv[q] = (T)y.v[q];
-    GRID_STRIDE(c, n) {
+        for (int q = 0; q < 16; q += 4) {
+            if (q >= nc) break;
+            float4 z[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (q + e < nc) z[e] = reinterpret_cast<const float4 *>(Z.p[q + e])[v];
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (q + e < nc) {
+                    T w[W];
+                    memcpy(w, &z[e], 16);
+#pragma unroll
+                    for (int i = 0; i < W; ++i) a[i] += yv[q + e] * w[i];
+                }
+        }
+        float4 o;
+        memcpy(&o, a, 16);
+        reinterpret_cast<float4 *>(x)[v] = o;
+    }
+    for (int64_t c = nv * W + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n;
+         c += (int64_t)gridDim.x * blockDim.x) {
         T a = x[c];
 #pragma unroll
-        for (int q = 0; q < 17; ++q)
-            if (q < ncols) a += yv[q] * Z[q][c];
+        for (int q = 0; q < 16; ++q)
+            if (q < nc) a += yv[q] * Z.p[q][c];
         x[c] = a;
     }
+}
+
+// x += sum_i y_i Z_i
+template <typename T>
+__global__ void k_xupd(int64_t n, T * x, VPtrs<T> Z, int ncols, Coef y) {
+    grid_begin();
+    T yv[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) yv[q] = (T)y.v[q];
+    xupd_cells<T>(n, x, Z, ncols, yv);
 }
 
 // phi += a * ((double) d - mean) on FLUID and GHOST cells (FP64 update of the
@@ -3298,12 +3381,11 @@ static ibm_status norm2(Ctx *c, const T *x, double *out) {
 template <typename T>
 struct Krylov {
     std::vector<T *> V, Z;
-    T **Vdev, **Zdev;
     T *w, *r;
     MGHier<T> *H;
 };
-static Krylov<double> kry64(Ctx *c) { return Krylov<double>{c->V, c->Z, c->Vdev, c->Zdev, c->w, c->rr, &c->mg64}; }
-static Krylov<float> kry32(Ctx *c) { return Krylov<float>{c->V32, c->Z32, c->Vdev32, c->Zdev32, c->w32, c->r32, &c->mg32}; }
+static Krylov<double> kry64(Ctx *c) { return Krylov<double>{c->V, c->Z, c->w, c->rr, &c->mg64}; }
+static Krylov<float> kry32(Ctx *c) { return Krylov<float>{c->V32, c->Z32, c->w32, c->r32, &c->mg32}; }
 
 // Step j of the Arnoldi process: w = P A Z_j orthogonalised against V_0..V_j by
 // classical Gram-Schmidt, with a second pass when the norm drops below
@@ -3426,7 +3508,9 @@ static ibm_status fgmres(Ctx *c, Krylov<T> K, T *x, const T *b, double bnorm, do
         }
         Coef yc{};
         for (int i = 0; i <= jlast; ++i) yc.v[i] = y[i];
-        KL(-1, k_xupd<T>, c->nred_wide, RED_THREADS, n, x, (const T *const *)K.Zdev, jlast + 1, yc);
+        VPtrs<T> zp{};
+        for (int i = 0; i <= jlast; ++i) zp.p[i] = K.Z[i];
+        KL(-1, k_xupd<T>, c->nred_wide, RED_THREADS, n, x, zp, jlast + 1, yc);
         IBM_LAUNCHED(c);
     }
     *outer_out = outer;
@@ -3473,17 +3557,12 @@ static ibm_status ensure_mixed(Ctx *c) {
             if (!(c->V32[i] = (float *)dev_alloc(c, sizeof(float) * c->N))) return c->fail(IBM_ERR_OOM, "FP32 Krylov allocation failed");
         for (int i = 0; i < m; ++i)
             if (!(c->Z32[i] = (float *)dev_alloc(c, sizeof(float) * c->N))) return c->fail(IBM_ERR_OOM, "FP32 Krylov allocation failed");
-        if (!c->Vdev32) c->Vdev32 = (float **)dev_alloc(c, sizeof(float *) * 17);
-        if (!c->Zdev32) c->Zdev32 = (float **)dev_alloc(c, sizeof(float *) * 17);
         if (!c->w32) c->w32 = (float *)dev_alloc(c, sizeof(float) * c->N);
         if (!c->r32) c->r32 = (float *)dev_alloc(c, sizeof(float) * c->N);
         if (!c->d32) c->d32 = (float *)dev_alloc(c, sizeof(float) * c->N);
         if (!c->b32) c->b32 = (float *)dev_alloc(c, sizeof(float) * c->N);
-        if (!c->Vdev32 || !c->Zdev32 || !c->w32 || !c->r32 || !c->d32 || !c->b32)
+        if (!c->w32 || !c->r32 || !c->d32 || !c->b32)
             return c->fail(IBM_ERR_OOM, "FP32 Krylov allocation failed");
-        IBM_CUDA(c, cudaMemcpyAsync(c->Vdev32, c->V32.data(), sizeof(float *) * (m + 1), cudaMemcpyHostToDevice, c->s));
-        IBM_CUDA(c, cudaMemcpyAsync(c->Zdev32, c->Z32.data(), sizeof(float *) * m, cudaMemcpyHostToDevice, c->s));
-        IBM_CUDA(c, cudaStreamSynchronize(c->s));
         c->m32_cap = m;
     }
     return IBM_OK;
@@ -3709,13 +3788,7 @@ __global__ void k_xupd_dev(int64_t n, T * x, VPtrs<T> Z, const DevFG * F) {
     T yv[16];
 #pragma unroll
     for (int q = 0; q < 16; ++q) yv[q] = q < nc ? (T)F->y[q] : T(0);
-    GRID_STRIDE(c, n) {
-        T a = x[c];
-#pragma unroll
-        for (int q = 0; q < 16; ++q)
-            if (q < nc) a += yv[q] * Z.p[q][c];
-        x[c] = a;
-    }
+    xupd_cells<T>(n, x, Z, nc, yv);
 }
 
 __global__ void k_zero_if(int64_t n, double * x, const int * flag) {
@@ -3995,12 +4068,7 @@ ibm_status poisson_dev_prepare(Ctx *c) {
 ibm_status poisson_solve_dev(Ctx *c, const double *rhs, double *phi, double rtol, int maxit) {
     const int64_t n = c->N;
     DevFG *R = dfg(c, 0), *F = dfg(c, 1);
-    KL(-1, k_fluid_volsum, c->nred, RED_THREADS, c->g, c->type, rhs, c->part);
-    IBM_TRY(finalize(c, c->part, c->nred, 1, 1.0 / c->fluid_vol, c->scal + S_MEAN));
-    IBM_CUDA(c, cudaMemcpyAsync(c->b, rhs, sizeof(double) * n, cudaMemcpyDeviceToDevice, c->s));
-    KL(-1, k_sub_mean, c->nred_wide, RED_THREADS, n, c->type, c->b, c->scal + S_MEAN, 0);
-    if (c->ng > 0) KL(-1, k_zero_at, (unsigned)((c->ng + 255) / 256), 256, c->ng, c->gidx, c->b);
-    IBM_TRY(norm2_dev<double>(c, c->b, S_TMP));
+    IBM_TRY(rhs_b(c, rhs));
     KL(-1, k_fg_setup, 1, 1, R, c->scal + S_TMP, rtol, maxit);
     IBM_LAUNCHED(c);
     if (c->opts.precision == IBM_MIXED) {
@@ -4010,9 +4078,9 @@ ibm_status poisson_solve_dev(Ctx *c, const double *rhs, double *phi, double rtol
         IBM_TRY(fgmres64_dev(c, phi, R));
     }
     KL(-1, k_zero_if, c->nred_wide, RED_THREADS, n, phi, &R->zero);
-    KL(-1, k_fluid_volsum, c->nred, RED_THREADS, c->g, c->type, phi, c->part);
+    KL(-1, k_fluid_volsum, c->nred, RED_THREADS, c->N, c->type, c->vol_c, phi, c->part);
     IBM_TRY(finalize(c, c->part, c->nred, 1, 1.0 / c->fluid_vol, c->scal + S_MEAN));
-    KL(-1, k_sub_mean, c->nred_wide, RED_THREADS, n, c->type, phi, c->scal + S_MEAN, 1);
+    KL(-1, k_sub_mean, c->nred_wide, RED_THREADS, n, c->type, phi, c->scal + S_MEAN);
     IBM_LAUNCHED(c);
     return IBM_OK;
 }
@@ -4204,7 +4272,7 @@ ibm_status hist_guess(Ctx *c, const double *rhs, double *phi) {
     if (L <= 0) return IBM_OK;
     if (L > c->hist_cap || L != c->hist_len) return c->fail(IBM_ERR_STATE, "Poisson history not prepared");
     HistCtl *H = reinterpret_cast<HistCtl *>(c->hist_ctl);
-    KL(-1, k_fluid_volsum, c->nred, RED_THREADS, c->g, c->type, rhs, c->part);
+    KL(-1, k_fluid_volsum, c->nred, RED_THREADS, c->N, c->type, c->vol_c, rhs, c->part);
     IBM_TRY(finalize(c, c->part, c->nred, 1, 1.0 / c->fluid_vol, &H->mean));
     KL(-1, k_hist_bp, c->nelem, 256, c->N, c->type, rhs, H, c->hist_bp);
     VPtrs<double> vp{};
@@ -4238,20 +4306,9 @@ ibm_status poisson_solve(Ctx *c, const double *rhs, double *phi, double rtol, in
     IBM_TRY(mg_coarse_ready(c));
     const int64_t n = c->N;
     IBM_CUDA(c, cudaEventRecord(c->ev4, c->s));
-    // b = P rhs on FLUID rows, 0 elsewhere
-    KL(-1, k_fluid_volsum, c->nred, RED_THREADS, c->g, c->type, rhs, c->part);
-    IBM_TRY(finalize(c, c->part, c->nred, 1, 1.0 / c->fluid_vol, c->scal + S_MEAN));
-    IBM_CUDA(c, cudaMemcpyAsync(c->b, rhs, sizeof(double) * n, cudaMemcpyDeviceToDevice, c->s));
-    KL(-1, k_sub_mean, c->nred_wide, RED_THREADS, n, c->type, c->b, c->scal + S_MEAN, 0);
-    IBM_LAUNCHED(c);
-    // GHOST rows of b are 0 (homogeneous Neumann on the body)
-    if (c->ng > 0) {
-        KL(-1, k_zero_at, (unsigned)((c->ng + 255) / 256), 256, c->ng, c->gidx, c->b);
-        IBM_LAUNCHED(c);
-    }
-    double bn2;
-    IBM_TRY(norm2<double>(c, c->b, &bn2));
-    const double bnorm = sqrt(bn2);
+    IBM_TRY(rhs_b(c, rhs));
+    IBM_TRY(sync_scalars(c, S_TMP + 1));
+    const double bnorm = sqrt(c->hscal[S_TMP]);
     if (!isfinite(bnorm)) return c->fail(IBM_ERR_DIVERGED, "Poisson right-hand side is not finite");
     int outer = 0, inner = 0;
     double rel = 0.0;
@@ -4266,9 +4323,9 @@ ibm_status poisson_solve(Ctx *c, const double *rhs, double *phi, double rtol, in
         else status = fgmres<double>(c, kry64(c), phi, c->b, bnorm, rtol, maxit, false, &outer, &inner, &rel);
         if (status != IBM_OK && status != IBM_ERR_NOT_CONVERGED) return status;
         // normalise: zero volume-weighted FLUID mean, shift ghosts too
-        KL(-1, k_fluid_volsum, c->nred, RED_THREADS, c->g, c->type, phi, c->part);
+        KL(-1, k_fluid_volsum, c->nred, RED_THREADS, c->N, c->type, c->vol_c, phi, c->part);
         IBM_TRY(finalize(c, c->part, c->nred, 1, 1.0 / c->fluid_vol, c->scal + S_MEAN));
-        KL(-1, k_sub_mean, c->nred_wide, RED_THREADS, n, c->type, phi, c->scal + S_MEAN, 1);
+        KL(-1, k_sub_mean, c->nred_wide, RED_THREADS, n, c->type, phi, c->scal + S_MEAN);
         IBM_LAUNCHED(c);
     }
     IBM_TRY(kt_flush(c));
