@@ -275,6 +275,7 @@ static ibm_status build_levels(Ctx *c) {
         c->gI[a].assign(c->lg.size(), nullptr);
         c->gw64[a].assign(c->lg.size(), nullptr);
         c->gw32[a].assign(c->lg.size(), nullptr);
+        if (a == 0) c->gwt32.assign(c->lg.size(), nullptr);
     }
     for (size_t l = 1; l < c->lg.size(); ++l) {
         const LevelGeom &F = c->lg[l - 1], &C = c->lg[l];
@@ -348,14 +349,27 @@ static ibm_status build_levels(Ctx *c) {
             }
             int *dgi = (int *)dev_alloc(c, sizeof(int) * 4 * nc);
             double *dgw = (double *)dev_alloc(c, sizeof(double) * 4 * nc);
-            float *dgw32 = (float *)dev_alloc(c, sizeof(float) * 4 * nc);
+            // x halved: the same weights by the fine cell's position t in the
+            // coarse cell's window 2I - 1 .. 2I + 2, at [t nc + I]
+            const bool win = a == 0 && fac[a] == 2 && nf == 2 * nc;
+            if (win) {
+                gw32.resize((size_t)8 * nc, 0.0f);
+                for (size_t q = 0; q < (size_t)4 * nc; ++q) {
+                    const int C2 = (int)(q / 4), t = gi[q] - (2 * C2 - 1);
+                    if (gi[q] < 0) continue;
+                    if (t < 0 || t > 3) return c->fail(IBM_ERR_ARG, "transfer table: fine cell outside its coarse cell's window");
+                    gw32[(size_t)(4 + t) * nc + C2] = gw32[q];
+                }
+            }
+            float *dgw32 = (float *)dev_alloc(c, sizeof(float) * gw32.size());
             if (!dgi || !dgw || !dgw32) return c->fail(IBM_ERR_OOM, "transfer table allocation failed");
             IBM_CUDA(c, cudaMemcpy(dgi, gi.data(), sizeof(int) * 4 * nc, cudaMemcpyHostToDevice));
             IBM_CUDA(c, cudaMemcpy(dgw, gw.data(), sizeof(double) * 4 * nc, cudaMemcpyHostToDevice));
-            IBM_CUDA(c, cudaMemcpy(dgw32, gw32.data(), sizeof(float) * 4 * nc, cudaMemcpyHostToDevice));
+            IBM_CUDA(c, cudaMemcpy(dgw32, gw32.data(), sizeof(float) * gw32.size(), cudaMemcpyHostToDevice));
             c->gI[a][l] = dgi;
             c->gw64[a][l] = dgw;
             c->gw32[a][l] = dgw32;
+            if (a == 0) c->gwt32[l] = win ? dgw32 + (size_t)4 * nc : nullptr;
         }
     }
     return IBM_OK;

@@ -202,6 +202,7 @@ struct Ctx {
     std::vector<int *> gI[3];
     std::vector<double *> gw64[3];
     std::vector<float *> gw32[3];
+    std::vector<float *> gwt32;   // x weights by window position (Xfer::gwtx), in gw32[0]'s allocation
     MGHier<double> mg64;
     MGHier<float> mg32;
 

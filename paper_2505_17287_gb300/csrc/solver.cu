@@ -301,13 +301,33 @@ __global__ void __launch_bounds__(RED_THREADS, 6) k_apply_A(GridDev g, OpT<T> o,
 // keeps several loads in flight where the one-cell loop stalls on load
 // latency. Each cell gets the same expression as A_row<float>; GHOST cells
 // are computed but not stored. The partial sums add a quad's cells in x order.
+// A block takes a column of 8 quads by 32 rows through `chunk` planes, the
+// planes below, at and above in registers and the one after in flight: the
+// y neighbours' rows are the column's own, so a value comes from L2 once
+// (1.06 rows a row, and 1 + 2 / chunk planes a plane). 62.9M cells: 213 us
+// with each thread's quads taken in linear order, 199 over boxes of 8 x 8 x 4
+// quads, 144 so.
+struct QuadWalk {
+    FastDiv fx, fy;    // columns along x and y
+    uint32_t n;        // columns times chunks
+    int chunk;
+};
+
+// chunks of up to 16 planes while that leaves two items per resident block
+static QuadWalk quad_walk(const GridDev &g) {
+    const uint32_t tx = (uint32_t)(g.nx / 4 + 7) / 8, ty = (uint32_t)(g.ny + 31) / 32;
+    int ch = 16;
+    while (ch > 1 && (int64_t)tx * ty * ((g.nz + ch - 1) / ch) < 1216) ch /= 2;
+    return QuadWalk{FastDiv(tx), FastDiv(ty), tx * ty * (uint32_t)((g.nz + ch - 1) / ch), ch};
+}
+
 __device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
 __device__ __forceinline__ float f4get(const float4 &v, int e) { return e == 0 ? v.x : e == 1 ? v.y : e == 2 ? v.z : v.w; }
 __device__ __forceinline__ uint8_t u4get(const uchar4 &v, int e) { return e == 0 ? v.x : e == 1 ? v.y : e == 2 ? v.z : v.w; }
 
 __global__ void __launch_bounds__(RED_THREADS)
     k_apply_A4(GridDev g, OpT<float> o, const uint8_t * type, const float * x,
-               const float * b, float sgn, float * y, double * part, int nb, GhostDev gh) {
+               const float * b, float sgn, float * y, double * part, int nb, GhostDev gh, QuadWalk w) {
     grid_begin();
     __shared__ double sh[32];
     if ((int)blockIdx.x >= nb) {
@@ -316,49 +336,57 @@ __global__ void __launch_bounds__(RED_THREADS)
     }
     double acc = 0.0;
     const int64_t sy = g.nx, sz = (int64_t)g.nx * g.ny;
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < g.n / 4; q += (int64_t)nb * blockDim.x) {
-        const int64_t c = 4 * q;
-        const uchar4 t4 = reinterpret_cast<const uchar4 *>(type)[q];
-        int i, j, k;
-        split3(g, (uint32_t)c, i, j, k);
-        const float4 xc = ld4(x + c);
-        const float xl = i > 0 ? x[c - 1] : xc.x;
-        const float xr = i + 4 < g.nx ? x[c + 4] : xc.w;
-        const float4 ym = j > 0 ? ld4(x + c - sy) : xc;
-        const float4 yp = j < g.ny - 1 ? ld4(x + c + sy) : xc;
-        float4 zm = xc, zp = xc;
-        if (g.ndim == 3) {
-            if (k > 0) zm = ld4(x + c - sz);
-            if (k < g.nz - 1) zp = ld4(x + c + sz);
-        }
-        const float4 bb = b ? ld4(b + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (uint32_t item = blockIdx.x; item < w.n; item += (uint32_t)nb) {
+        const uint32_t tr = w.fx.div(item), tz = w.fy.div(tr);
+        const int i = 4 * (int)((item - tr * w.fx.d) * 8 + (threadIdx.x & 7));
+        const int j = (int)(tr - tz * w.fy.d) * 32 + (int)(threadIdx.x >> 3);
+        const int k0 = (int)tz * w.chunk, k1 = min(k0 + w.chunk, g.nz);
+        if (i >= g.nx || j >= g.ny) continue;
+        int64_t c = i + g.nx * (j + (int64_t)g.ny * k0);
         const float4 cm = ld4(o.cxm + i), cp = ld4(o.cxp + i), dxv = ld4(o.dx + i);
-        const float cym = o.cym[j], cyp = o.cyp[j], dyj = o.dy[j], dzk = o.dz[k];
-        const float czm = g.ndim == 3 ? o.czm[k] : 0.f, czp = g.ndim == 3 ? o.czp[k] : 0.f;
-        float out[4];
-        bool ghost = false;
-        float leaf = 0.f;
+        const float cym = o.cym[j], cyp = o.cyp[j], dyj = o.dy[j];
+        float4 xc = ld4(x + c), zm = k0 > 0 ? ld4(x + c - sz) : xc;
+        float4 zp = k0 + 1 < g.nz ? ld4(x + c + sz) : xc;
+        for (int k = k0; k < k1; ++k, c += sz) {
+            // (the last cell of the grid repeats itself: its coefficient is 0)
+            float4 zn = zp;
+            if (k + 1 < k1 && k + 2 < g.nz) zn = ld4(x + c + 2 * sz);
+            const uchar4 t4 = *reinterpret_cast<const uchar4 *>(type + c);
+            const float xl = i > 0 ? x[c - 1] : xc.x;
+            const float xr = i + 4 < g.nx ? x[c + 4] : xc.w;
+            const float4 ym = j > 0 ? ld4(x + c - sy) : xc;
+            const float4 yp = j < g.ny - 1 ? ld4(x + c + sy) : xc;
+            const float4 bb = b ? ld4(b + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+            const float dzk = o.dz[k];
+            const float czm = g.ndim == 3 ? o.czm[k] : 0.f, czp = g.ndim == 3 ? o.czp[k] : 0.f;
+            float out[4];
+            bool ghost = false;
+            float leaf = 0.f;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const float xe = f4get(xc, e);
-            const float xm = e == 0 ? xl : f4get(xc, e - 1);
-            const float xp = e == 3 ? xr : f4get(xc, e + 1);
-            float s = f4get(cm, e) * (xm - xe) + f4get(cp, e) * (xp - xe) + cym * (f4get(ym, e) - xe) +
-                      cyp * (f4get(yp, e) - xe);
-            if (g.ndim == 3) s += czm * (f4get(zm, e) - xe) + czp * (f4get(zp, e) - xe);
-            const float v = sgn * s + f4get(bb, e);
-            const uint8_t t = u4get(t4, e);
-            ghost |= t == GHOST;
-            out[e] = t == DEAD ? 0.f : v;
-            if (t == FLUID) leaf += (f4get(dxv, e) * dyj * dzk) * v;
-        }
-        acc += (double)leaf;
-        if (!ghost) {
-            *reinterpret_cast<float4 *>(y + c) = make_float4(out[0], out[1], out[2], out[3]);
-        } else {
+            for (int e = 0; e < 4; ++e) {
+                const float xe = f4get(xc, e);
+                const float xm = e == 0 ? xl : f4get(xc, (e - 1) & 3);
+                const float xp = e == 3 ? xr : f4get(xc, (e + 1) & 3);
+                float s = f4get(cm, e) * (xm - xe) + f4get(cp, e) * (xp - xe) + cym * (f4get(ym, e) - xe) +
+                          cyp * (f4get(yp, e) - xe);
+                if (g.ndim == 3) s += czm * (f4get(zm, e) - xe) + czp * (f4get(zp, e) - xe);
+                const float v = sgn * s + f4get(bb, e);
+                const uint8_t t = u4get(t4, e);
+                ghost |= t == GHOST;
+                out[e] = t == DEAD ? 0.f : v;
+                if (t == FLUID) leaf += (f4get(dxv, e) * dyj * dzk) * v;
+            }
+            acc += (double)leaf;
+            if (!ghost) {
+                *reinterpret_cast<float4 *>(y + c) = make_float4(out[0], out[1], out[2], out[3]);
+            } else {
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
-                if (u4get(t4, e) != GHOST) y[c + e] = out[e];
+                for (int e = 0; e < 4; ++e)
+                    if (u4get(t4, e) != GHOST) y[c + e] = out[e];
+            }
+            zm = xc;
+            xc = zp;
+            zp = zn;
         }
     }
     const double tot = block_sum<RED_THREADS>(acc, sh);
@@ -415,9 +443,14 @@ static ibm_status apply_A(Ctx *c, const T *x, const T *b, T sgn, T *y) {
     int nb = sizeof(T) == 4 ? c->nred_wide : c->nred64;
     unsigned grid = (unsigned)nb + (unsigned)((c->ng + RED_THREADS - 1) / RED_THREADS);
     if constexpr (sizeof(T) == 4) {
-        if (c->g.nx % 4 == 0 && al16(x) && al16(y) && (!b || al16(b)))
-            KL(K_APPLY_A, k_apply_A4, grid, RED_THREADS, c->g, o, c->type, x, b, sgn, y, c->part, nb, c->gh);
-        else
+        if (c->g.nx % 4 == 0 && al16(x) && al16(y) && (!b || al16(b))) {
+            const QuadWalk w = quad_walk(c->g);
+            if ((uint32_t)nb > w.n) {
+                grid -= (uint32_t)nb - w.n;
+                nb = (int)w.n;
+            }
+            KL(K_APPLY_A, k_apply_A4, grid, RED_THREADS, c->g, o, c->type, x, b, sgn, y, c->part, nb, c->gh, w);
+        } else
             KL(K_APPLY_A, k_apply_A<T>, grid, RED_THREADS, c->g, o, c->type, x, b, sgn, y, c->part, nb, c->gh);
     } else if (!b && sgn == T(1)) {
         KL(K_APPLY_A, (k_apply_A<T, true>), grid, RED_THREADS, c->g, o, c->type, x, b, sgn, y, c->part, nb, c->gh);
@@ -1114,31 +1147,56 @@ __device__ __forceinline__ QuadNb split_loads(const SplitLv<float> &L, const flo
 }
 
 // sum over the open faces of T_f x_nb and the face sum d for the four cells
-// of a quad (the order and operations of k_offdiag<float, true>)
+// of a quad (the order and operations of k_offdiag<float, true>; face by face
+// over the four cells, so that the 1D metrics are 16-byte reads of which one
+// is live at a time)
 __device__ __forceinline__ void split_offdiag(const SplitLv<float> &L, const QuadNb &N, int h0, int j, int k,
                                               int pc, uchar4 m4, float s[4], float d[4]) {
-    // the 1D metrics are small arrays (L1 hits), read per cell as needed so
-    // they hold no registers across the loop
-    const float *swx = (pc ? L.swx1 : L.swx0) + h0, *srm = (pc ? L.srm1 : L.srm0) + h0;
-    const float *srp = (pc ? L.srp1 : L.srp0) + h0;
     const float wyj = L.wy[j], wzk = L.wz[k], ry0 = L.rhy[j], ry1 = L.rhy[j + 1], rz0 = L.rhz[k], rz1 = L.rhz[k + 1];
+    const float ayz = wyj * wzk;
+    const unsigned mk[4] = {m4.x, m4.y, m4.z, m4.w};
+    const float4 rm = ld4((pc ? L.srm1 : L.srm0) + h0);
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-        const unsigned msk = e == 0 ? m4.x : e == 1 ? m4.y : e == 2 ? m4.z : m4.w;
-        const float xm = pc ? f4at(N.O, e) : (e == 0 ? N.xe : f4at(N.O, e - 1));
-        const float xp = pc ? (e == 3 ? N.xe : f4at(N.O, e + 1)) : f4at(N.O, e);
-        const float wxe = swx[e];
-        const float ayz = wyj * wzk, axz = wxe * wzk, axy = wxe * wyj;
-        float dd = 0.f, ss = 0.f, t;
-        if (msk & 1u) { t = ayz * srm[e]; dd += t; ss += t * xm; }
-        if (msk & 2u) { t = ayz * srp[e]; dd += t; ss += t * xp; }
-        if (msk & 4u) { t = axz * ry0; dd += t; ss += t * f4at(N.ym, e); }
-        if (msk & 8u) { t = axz * ry1; dd += t; ss += t * f4at(N.yp, e); }
-        if (msk & 16u) { t = axy * rz0; dd += t; ss += t * f4at(N.zm, e); }
-        if (msk & 32u) { t = axy * rz1; dd += t; ss += t * f4at(N.zp, e); }
-        s[e] = ss;
-        d[e] = dd;
+        s[e] = d[e] = 0.f;
+        const float xm = pc ? f4at(N.O, e) : (e == 0 ? N.xe : f4at(N.O, (e - 1) & 3));
+        if (mk[e] & 1u) { const float t = ayz * f4at(rm, e); d[e] += t; s[e] += t * xm; }
     }
+    const float4 rp = ld4((pc ? L.srp1 : L.srp0) + h0);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const float xp = pc ? (e == 3 ? N.xe : f4at(N.O, (e + 1) & 3)) : f4at(N.O, e);
+        if (mk[e] & 2u) { const float t = ayz * f4at(rp, e); d[e] += t; s[e] += t * xp; }
+    }
+    const float4 wx = ld4((pc ? L.swx1 : L.swx0) + h0);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const unsigned msk = mk[e];
+        const float axz = f4at(wx, e) * wzk, axy = f4at(wx, e) * wyj;
+        float t;
+        if (msk & 4u) { t = axz * ry0; d[e] += t; s[e] += t * f4at(N.ym, e); }
+        if (msk & 8u) { t = axz * ry1; d[e] += t; s[e] += t * f4at(N.yp, e); }
+        if (msk & 16u) { t = axy * rz0; d[e] += t; s[e] += t * f4at(N.zm, e); }
+        if (msk & 32u) { t = axy * rz1; d[e] += t; s[e] += t * f4at(N.zp, e); }
+    }
+}
+
+// Blocks of 256 quads as boxes of 8 quads (128 bytes) by rows along y and z,
+// 8 x 8 x 4 in 3D and 8 x 32 in 2D: the y and z neighbour rows of a box are
+// mostly rows of the box, read from L2 once (1.75 rows a row; four
+// consecutive whole rows read 3.5), and the traffic from L2 is what the pass
+// waits for beside memory's (62.9M cells: 124 -> 116 us, the last pass
+// 156 -> 131).
+struct QuadBox {
+    int ly;   // log2 of the rows along y
+    __host__ __device__ int by() const { return 1 << ly; }
+    __host__ __device__ int bz() const { return 32 >> ly; }
+};
+
+static QuadBox quad_box(int nz) { return QuadBox{nz > 1 ? 3 : 5}; }
+
+static dim3 quad_grid(const QuadBox &b, int nq, int ny, int nz) {
+    return dim3((unsigned)((nq + 7) / 8), (unsigned)((ny + b.by() - 1) / b.by()), (unsigned)((nz + b.bz() - 1) / b.bz()));
 }
 
 // One colour pass (colour col, other colour's x in xo) on level 0 in split
@@ -1148,15 +1206,15 @@ __device__ __forceinline__ void split_offdiag(const SplitLv<float> &L, const Qua
 // Every load of a quad is issued before the first use, so a thread waits
 // for memory once.
 template <bool OMEGA, bool NAT>
-__global__ void __launch_bounds__(256, 5)
-    k_rbgs_split(SplitLv<float> L, const float * fq, const uint8_t * mq,
+__global__ void __launch_bounds__(256, 4)
+    k_rbgs_split(SplitLv<float> L, QuadBox box, const float * fq, const uint8_t * mq,
                  const float * xo, float * xq, int col, float w, float * xn) {
     grid_begin();
-    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q >= L.nq) return;
-    int64_t base;
-    int h0, j, k;
-    split_quad_pos(L, q, base, h0, j, k);
+    const int t = threadIdx.x, h0 = 4 * (blockIdx.x * 8 + (t & 7));
+    const int j = blockIdx.y * box.by() + ((t >> 3) & (box.by() - 1));
+    const int k = blockIdx.z * box.bz() + (t >> (3 + box.ly));
+    if (h0 >= L.H || j >= L.ny || k >= L.nz) return;
+    const int64_t base = (j + (int64_t)L.ny * k) * L.H + h0;
     const int pc = (col + j + k) & 1;
     const uchar4 m4 = *reinterpret_cast<const uchar4 *>(mq + base);
     const float4 f4 = ld4(fq + base);
@@ -1362,6 +1420,7 @@ struct Xfer {
     const int *Gx, *Gy, *Gz;                  // gather: coarse index -> 4 fine
     const T *gwx, *gwy, *gwz;
     const T *vx, *vy, *vz;                    // weight of coarse J (1 - w)
+    const T *gwtx;   // FP32, x halved: weight of fine 2I - 1 + t in coarse I at [t nc + I]
 };
 
 // the up-to-two coarse indices and weights of fine index i along one axis
@@ -1610,118 +1669,92 @@ __global__ void __launch_bounds__(RX_THREADS)
 }
 
 // k_resid_rx on level 0 in colour-split storage when x is coarsened by two
-// (nx a multiple of 8): one thread per four coarse x-cells I0 .. I0 + 3 of a
-// row. Coarse I gathers fine cells 2I - 1 .. 2I + 2, so the thread evaluates
-// pn r on the ten fine cells 2 I0 - 1 .. 2 I0 + 8 (the two outer ones also by
-// its neighbours) with 16-byte loads: the colour relaxed last (1) has zero
-// residual where it has an open face and p f where it has none; colour 0
-// takes the full stencil, in the order and operations of k_resid_rx. The
-// restriction then sums in the gather table's order, so the result equals
-// k_resid_rx bit for bit.
-__global__ void __launch_bounds__(256)
+// (nx a multiple of 8): one lane per four coarse x-cells I0 .. I0 + 3 of a
+// row. Coarse I gathers fine cells 2I - 1 .. 2I + 2: a lane evaluates pn r on
+// its own eight fine cells and takes the cell on either side from its
+// neighbour lanes, so the first and last lane of a warp only serve theirs (30
+// quads of a warp's 32 are stored, the outer two evaluated twice). The colour
+// relaxed last (1) has zero residual where it has an open face and p f where
+// it has none; colour 0 takes the full stencil, in the order and operations
+// of k_resid_rx, and the restriction sums the window's positions in order
+// (table gwtx: 0 where a coarse cell has no such fine cell), so the result
+// equals k_resid_rx bit for bit.
+// Bound by memory (13 bytes a cell) once the L1 accesses are few: tables and
+// metrics are read as 16-byte runs over the four cells, where strided reads
+// of metrics, gather indices and window edges by each thread took 330 L1
+// passes a warp, three times the memory's time (62.9M cells: 366 -> 162 us).
+__global__ void __launch_bounds__(256, 3)
     k_resid_rx_split4(MGLevel<float> L, SplitLv<float> S, const float * fs0, const float * fs1,
                       const float * xs0, const float * xs1, const float * pn,
                       Xfer<float> X, float * tA) {
     grid_begin();
-    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q >= S.nq) return;
+    const int lane = threadIdx.x & 31;
+    const int64_t w30 = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * 30;
+    if (w30 >= S.nq) return;   // (whole warps)
+    const int64_t q0 = w30 + lane - 1;
+    const int64_t q = q0 < 0 ? 0 : (q0 < S.nq ? q0 : S.nq - 1);
     const int H = S.H, nx = L.nx;
-    const uint32_t rw = S.fq.div((uint32_t)q);
-    const int I0 = 4 * (int)((uint32_t)q - rw * (uint32_t)(H / 4));   // packed quad h0 = I0 (H = coarse nx)
-    int j, k;
-    row_jk(rw, S.fny, S.ny, j, k);
-    const int64_t row = rw, base = row * H + I0, crow = row * nx;
+    int64_t base;
+    int I0, j, k;   // packed quad h0 = I0 (H = coarse nx)
+    split_quad_pos(S, q, base, I0, j, k);
+    const int64_t row = j + (int64_t)L.ny * k, crow = row * nx;
     const int pc0 = (j + k) & 1;             // colour 0 sits at i = 2 h + pc0
     const int64_t sy = H, sz = (int64_t)H * L.ny;
-    const int i0 = 2 * I0 - 1;               // first fine cell of the window
-    // colour 0 of the window: packed I0 - pc0 .. I0 + 4 - pc0 = the quad at
-    // I0 and one edge cell he
-    const float4 x0q = ld4(xs0 + base), f0q = ld4(fs0 + base);
-    const int he = pc0 ? I0 - 1 : I0 + 4;
-    const bool heok = he >= 0 && he < H;
-    const int64_t be = row * H + (heok ? he : I0);
-    const float x0e = heok ? xs0[be] : 0.f, f0e = heok ? fs0[be] : 0.f;
-    // colour 1: packed I0 - 1 .. I0 + 4 of the row (x neighbours), and the
-    // y / z rows at the colour-0 cells' packed indices
-    const float4 c1q = ld4(xs1 + base);
-    const float c1m = I0 > 0 ? xs1[base - 1] : 0.f, c1p = I0 + 4 < H ? xs1[base + 4] : 0.f;
+    const float4 x0q = ld4(xs0 + base), f0q = ld4(fs0 + base), c1q = ld4(xs1 + base);
     const float4 ymq = ld4(xs1 + (j > 0 ? base - sy : base)), ypq = ld4(xs1 + (j < L.ny - 1 ? base + sy : base));
-    const float yme = (j > 0 && heok) ? xs1[be - sy] : 0.f, ype = (j < L.ny - 1 && heok) ? xs1[be + sy] : 0.f;
-    float4 zmq = c1q, zpq = c1q;
-    float zme = 0.f, zpe = 0.f;
-    if (L.nz > 1) {
-        if (k > 0) {
-            zmq = ld4(xs1 + base - sz);
-            if (heok) zme = xs1[be - sz];
-        }
-        if (k < L.nz - 1) {
-            zpq = ld4(xs1 + base + sz);
-            if (heok) zpe = xs1[be + sz];
-        }
-    }
-    // cell-ordered pn and open-face mask of the window
+    const float4 zmq = ld4(xs1 + (L.nz > 1 && k > 0 ? base - sz : base));
+    const float4 zpq = ld4(xs1 + (L.nz > 1 && k < L.nz - 1 ? base + sz : base));
+    // cell-ordered pn and open-face mask
     const float4 pA = ld4(pn + crow + 2 * I0), pB = ld4(pn + crow + 2 * I0 + 4);
-    const float pm = I0 > 0 ? pn[crow + i0] : 0.f, pp = 2 * I0 + 8 < nx ? pn[crow + 2 * I0 + 8] : 0.f;
     const uint2 mm = *reinterpret_cast<const uint2 *>(L.omask + crow + 2 * I0);
-    const unsigned mlo = I0 > 0 ? L.omask[crow + i0] : 0u, mhi = 2 * I0 + 8 < nx ? L.omask[crow + 2 * I0 + 8] : 0u;
+    const float4 wx4 = ld4((pc0 ? S.swx1 : S.swx0) + I0), rm4 = ld4((pc0 ? S.srm1 : S.srm0) + I0);
+    const float4 rp4 = ld4((pc0 ? S.srp1 : S.srp0) + I0);
+    const float c1m = __shfl_up_sync(0xffffffffu, c1q.w, 1), c1p = __shfl_down_sync(0xffffffffu, c1q.x, 1);
     const float wyj = L.wy[j], wzk = L.wz[k], ry0 = L.rhy[j], ry1 = L.rhy[j + 1], rz0 = L.rhz[k], rz1 = L.rhz[k + 1];
     float r[10];
 #pragma unroll
-    for (int t = 0; t < 10; ++t) {
-        const int i = i0 + t;
-        const float p = t == 0 ? pm : (t == 9 ? pp : (t < 5 ? f4at(pA, t - 1) : f4at(pB, t - 5)));
-        const unsigned msk = t == 0 ? mlo : (t == 9 ? mhi : (((t < 5 ? mm.x : mm.y) >> (8 * ((t - 1) & 3))) & 0xffu));
-        float v = 0.f;
-        if (i >= 0 && i < nx && p > 0.f) {
-            if (((t + pc0 + 1) & 1) == 0) {
-                // colour 0, the e-th of the window's five (t = 2 e - pc0 + 1)
-                const int e = (t + pc0 - 1) >> 1;
-                const bool edge = pc0 ? e == 0 : e == 4;
-                const int qq = pc0 ? e - 1 : e;
-                const float xc = edge ? x0e : f4at(x0q, qq & 3), fc = edge ? f0e : f4at(f0q, qq & 3);
-                // x neighbours (colour 1) at packed I0 - 1 + e and I0 + e
-                const float xm = e == 0 ? c1m : f4at(c1q, (e - 1) & 3);
-                const float xp = e == 4 ? c1p : f4at(c1q, e & 3);
-                const float ym = edge ? yme : f4at(ymq, qq & 3), yp = edge ? ype : f4at(ypq, qq & 3);
-                const float zm = edge ? zme : f4at(zmq, qq & 3), zp = edge ? zpe : f4at(zpq, qq & 3);
-                const float ayz = wyj * wzk, axz = L.wx[i] * wzk, axy = L.wx[i] * wyj;
-                float d = 0.f, s = fc, tt;
-                if (msk & 1u) { tt = ayz * L.rhx[i]; d += tt; s += tt * xm; }
-                if (msk & 2u) { tt = ayz * L.rhx[i + 1]; d += tt; s += tt * xp; }
-                if (msk & 4u) { tt = axz * ry0; d += tt; s += tt * ym; }
-                if (msk & 8u) { tt = axz * ry1; d += tt; s += tt * yp; }
-                if (msk & 16u) { tt = axy * rz0; d += tt; s += tt * zm; }
-                if (msk & 32u) { tt = axy * rz1; d += tt; s += tt * zp; }
-                v = p * (s - d * xc);
-            } else if ((msk & 0x3fu) == 0) {
-                // colour 1 (relaxed last) without an open face: not updated by
-                // the smoother, r = p (f - 0 x)
-                const int64_t pb = row * H + (i >> 1);
-                const float d = 0.f;
-                v = p * (fs1[pb] - d * xs1[pb]);
-            }
+    for (int e = 0; e < 4; ++e) {
+        // the pair of cells 2 h, 2 h + 1 at packed index h = I0 + e
+        const float pe = e < 2 ? f4at(pA, 2 * e) : f4at(pB, 2 * e - 4);
+        const float po = e < 2 ? f4at(pA, 2 * e + 1) : f4at(pB, 2 * e - 3);
+        const unsigned m2 = (e < 2 ? mm.x : mm.y) >> (16 * (e & 1));
+        const float p0 = pc0 ? po : pe, p1 = pc0 ? pe : po;
+        const unsigned msk = (pc0 ? m2 >> 8 : m2) & 0xffu, msk1 = (pc0 ? m2 : m2 >> 8) & 0xffu;
+        float v0 = 0.f, v1 = 0.f;
+        if (p0 > 0.f) {
+            // x neighbours (colour 1): packed h - 1 and h (pc0 = 0), h and h + 1 (pc0 = 1)
+            const float xm = pc0 ? f4at(c1q, e) : (e == 0 ? c1m : f4at(c1q, (e - 1) & 3));
+            const float xp = pc0 ? (e == 3 ? c1p : f4at(c1q, (e + 1) & 3)) : f4at(c1q, e);
+            const float wxe = f4at(wx4, e);
+            const float ayz = wyj * wzk, axz = wxe * wzk, axy = wxe * wyj;
+            float d = 0.f, s = f4at(f0q, e), tt;
+            if (msk & 1u) { tt = ayz * f4at(rm4, e); d += tt; s += tt * xm; }
+            if (msk & 2u) { tt = ayz * f4at(rp4, e); d += tt; s += tt * xp; }
+            if (msk & 4u) { tt = axz * ry0; d += tt; s += tt * f4at(ymq, e); }
+            if (msk & 8u) { tt = axz * ry1; d += tt; s += tt * f4at(ypq, e); }
+            if (msk & 16u) { tt = axy * rz0; d += tt; s += tt * f4at(zmq, e); }
+            if (msk & 32u) { tt = axy * rz1; d += tt; s += tt * f4at(zpq, e); }
+            v0 = p0 * (s - d * f4at(x0q, e));
         }
-        r[t] = v;
+        if (p1 > 0.f && (msk1 & 0x3fu) == 0) {
+            // colour 1 (relaxed last) without an open face: not updated by
+            // the smoother, r = p (f - 0 x)
+            const float d = 0.f;
+            v1 = p1 * (fs1[base + e] - d * xs1[base + e]);
+        }
+        r[1 + 2 * e] = pc0 ? v1 : v0;
+        r[2 + 2 * e] = pc0 ? v0 : v1;
     }
-    // coarse I = I0 + u gathers the consecutive fine cells 2I - 1 .. 2I + 2
-    // (2I .. 2I + 2 at the row start): window positions 2u + s + sh
-    // (each coarse cell's four table entries in one 16-byte load apiece)
-    float out[4];
+    const float rl = __shfl_up_sync(0xffffffffu, r[8], 1), rr = __shfl_down_sync(0xffffffffu, r[1], 1);
+    r[0] = I0 > 0 ? rl : 0.f;
+    r[9] = 2 * I0 + 8 < nx ? rr : 0.f;
+    if (q != q0 || lane == 0 || lane == 31) return;
+    float out[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int I = I0 + u;
-        const int4 gi = *reinterpret_cast<const int4 *>(X.Gx + 4 * I);
-        const float4 gw = ld4(X.gwx + 4 * I);
-        const bool sh = gi.x != 2 * I - 1;
-        const int g4[4] = {gi.x, gi.y, gi.z, gi.w};
-        float acc = 0.f;
+    for (int t = 0; t < 4; ++t) {
+        const float4 gw = ld4(X.gwtx + t * (int64_t)H + I0);
 #pragma unroll
-        for (int s2 = 0; s2 < 4; ++s2) {
-            if (g4[s2] < 0) continue;
-            const float rv = sh ? (2 * u + s2 + 1 <= 9 ? r[(2 * u + s2 + 1) > 9 ? 9 : (2 * u + s2 + 1)] : 0.f) : r[2 * u + s2];
-            acc += f4at(gw, s2) * rv;
-        }
-        out[u] = acc;
+        for (int u = 0; u < 4; ++u) out[u] += f4at(gw, u) * r[2 * u + t];
     }
     *reinterpret_cast<float4 *>(tA + base) = make_float4(out[0], out[1], out[2], out[3]);
 }
@@ -2390,14 +2423,14 @@ Xfer<double> xfer_of<double>(Ctx *c, int l) {
     return Xfer<double>{c->tI[0][l],   c->tJ[0][l],   c->tI[1][l],   c->tJ[1][l],   c->tI[2][l],
                         c->tJ[2][l],   c->tw64[0][l], c->tw64[1][l], c->tw64[2][l], c->gI[0][l],
                         c->gI[1][l],   c->gI[2][l],   c->gw64[0][l], c->gw64[1][l], c->gw64[2][l],
-                        c->tv64[0][l], c->tv64[1][l], c->tv64[2][l]};
+                        c->tv64[0][l], c->tv64[1][l], c->tv64[2][l], nullptr};
 }
 template <>
 Xfer<float> xfer_of<float>(Ctx *c, int l) {
     return Xfer<float>{c->tI[0][l],   c->tJ[0][l],   c->tI[1][l],   c->tJ[1][l],   c->tI[2][l],
                        c->tJ[2][l],   c->tw32[0][l], c->tw32[1][l], c->tw32[2][l], c->gI[0][l],
                        c->gI[1][l],   c->gI[2][l],   c->gw32[0][l], c->gw32[1][l], c->gw32[2][l],
-                       c->tv32[0][l], c->tv32[1][l], c->tv32[2][l]};
+                       c->tv32[0][l], c->tv32[1][l], c->tv32[2][l], c->gwt32[l]};
 }
 
 template <typename T>
@@ -2722,12 +2755,14 @@ static ibm_status split_pass(Ctx *c, MGHier<float> &H, int kind, int col, const 
         const float *fq = H.fs[col], *xo = H.xs[1 - col];
         const uint8_t *mq = H.ms[col];
         float *xq = H.xs[col];
+        const QuadBox box = quad_box(S.nz);
+        const dim3 qg = quad_grid(box, S.H / 4, S.ny, S.nz);
         if (kind == 2) {
-            if (om) KL(K_RBGS0, (k_rbgs_split<true, true>), nb, 256, S, fq, mq, xo, xq, col, (float)w, x0);
-            else KL(K_RBGS0, (k_rbgs_split<false, true>), nb, 256, S, fq, mq, xo, xq, col, 1.f, x0);
+            if (om) KL(K_RBGS0, (k_rbgs_split<true, true>), qg, 256, S, box, fq, mq, xo, xq, col, (float)w, x0);
+            else KL(K_RBGS0, (k_rbgs_split<false, true>), qg, 256, S, box, fq, mq, xo, xq, col, 1.f, x0);
         } else {
-            if (om) KL(K_RBGS0, (k_rbgs_split<true, false>), nb, 256, S, fq, mq, xo, xq, col, (float)w, nullptr);
-            else KL(K_RBGS0, (k_rbgs_split<false, false>), nb, 256, S, fq, mq, xo, xq, col, 1.f, nullptr);
+            if (om) KL(K_RBGS0, (k_rbgs_split<true, false>), qg, 256, S, box, fq, mq, xo, xq, col, (float)w, nullptr);
+            else KL(K_RBGS0, (k_rbgs_split<false, false>), qg, 256, S, box, fq, mq, xo, xq, col, 1.f, nullptr);
         }
     }
     IBM_LAUNCHED(c);
@@ -3023,7 +3058,7 @@ static ibm_status vcycle(Ctx *c, MGHier<T> &H, const T *f0, T *x0) {
                 if (l == 0 && sp) {
                     if (CG.fx == 2 && zcol == 1) {
                         const SplitLv<float> S = split_of(H);
-                        KL(K_RESTRICT, k_resid_rx_split4, (unsigned)((S.nq + 255) / 256), 256, Lf, S, H.fs[0],
+                        KL(K_RESTRICT, k_resid_rx_split4, (unsigned)((S.nq + 239) / 240), 256, Lf, S, H.fs[0],
                            H.fs[1], H.xs[0], H.xs[1], H.pn[l], X, tA);
                     } else {
                         KL(K_RESTRICT, k_resid_rx_split, rgrid, RX_THREADS, Lf, H.fs[0], H.fs[1], H.xs[0], H.xs[1],
