@@ -94,7 +94,9 @@ typedef struct {
     int inner_iters;    /* Poisson: MG-PCG iterations per preconditioner call */
     int nu1, nu2;       /* multigrid pre/post red-black Gauss-Seidel sweeps, 1..8; equal
                            when inner_iters > 1 (CG needs a symmetric V-cycle) */
-    int coarse_sweeps;  /* red-black sweep pairs on the coarsest level */
+    int coarse_sweeps;  /* red-black sweep pairs on the coarsest level (at most 64 cells
+                           where the grid coarsens that far; the sweeps are applied
+                           as one operator, formed once per classification) */
     double helm_rtol;   /* Crank-Nicolson Helmholtz: relative residual target */
     int helm_maxit;     /* Helmholtz: sweep limit */
     double ghost_tol;   /* velocity ghost refresh: max relative change */
@@ -117,7 +119,8 @@ typedef struct {
                            transfer kernels (one block per grid row segment):
                            32, 64, 128, 256 or 512 */
     int graph;          /* 1: the multigrid V-cycle is captured once into a CUDA graph
-                           and replayed at every preconditioner call (one launch
+                           (again only when an option that shapes it changes) and
+                           replayed at every preconditioner call (one launch
                            instead of ~10 per level; not on the legacy default
                            stream, which cannot be captured, nor while the kernel
                            timer runs); 2: the whole fractional step is one captured
@@ -182,14 +185,17 @@ typedef struct {
                            saves IBM_FIELD_P_HIST_*. Costs 16 bytes per cell and
                            pair */
     int tail_cells;     /* multigrid levels below the finest with at most tail_cells
-                           cells run as one persistent launch per V-cycle (a
+                           cells (at least those of the launch that always runs a
+                           cycle's smallest levels in shared memory) run as one
+                           persistent launch per V-cycle (a
                            cluster of up to 8 blocks walks their passes with
                            hardware cluster barriers between them; same values as
                            the per-level kernels, bit for bit); 0 = every level
                            launched on its own, the default: on GB300 the
                            per-level kernels replayed from CUDA graphs measured
                            faster (2D 256x128 cylinder step 2.28 ms without the
-                           tail, 2.42-2.58 ms with it). Needs mg_interp 1 and
+                           tail, 2.42-2.58 ms with it, before the smallest levels
+                           had a launch of their own). Needs mg_interp 1 and
                            three levels or more */
     int nu_coarse;      /* red-black sweeps before and after the coarse-grid correction on
                            the multigrid levels below the finest, 1..8; 0 = nu1 and nu2

@@ -83,3 +83,19 @@ def test_solution_update_on_an_odd_address():
         out.append(phi.cpu().numpy())
     assert np.array_equal(out[0], out[1])
     s.close()
+
+
+# coarse rows of a multiple of the access width and not, planes 1 and odd
+@pytest.mark.parametrize("precision", [ibm.IBM_FP64, ibm.IBM_MIXED])
+@pytest.mark.parametrize("shape", [(104, 70, 34), (84, 61, 47), (90, 66, 38), (300, 129, 1), (328, 130, 1)],
+                         ids=lambda s: "x".join(map(str, s)))
+def test_restriction_by_columns_equals_the_tail(shape, precision):
+    """The restriction's column walk against the tail's cell-by-cell one."""
+    case = _case(*shape)
+    out = []
+    for tail in (0, 1 << 20):
+        s = _solver(case, precision=precision, tail_cells=tail, poisson_hist=0)
+        assert s.step(2)["status"] == ibm.IBM_OK
+        out.append((s.get("u"), s.get("p")))
+        s.close()
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
