@@ -3934,6 +3934,7 @@ __global__ void k_add_scaled_dev(int64_t n, const uint8_t * type, double * phi,
                                  const float * d, const DevFG * R,
                                  const double * mean) {
     grid_begin();
+    if (!R->go) return;
     const double a = R->rn, m = *mean;
     GRID_STRIDE(c, n) if (type[c] != DEAD) phi[c] += a * ((double)d[c] - m);
 }
@@ -3983,6 +3984,10 @@ __global__ void k_fg_cycle(DevFG *F, const double *rn2, cudaGraphConditionalHand
         F->jlast = -1;
         F->active = 1;
         F->ncols = 0;
+    } else {
+        // (the kernels of a first cycle run as plain nodes look at these)
+        F->active = 0;
+        F->ncols = 0;
     }
     cudaGraphSetConditional(h, go ? 1u : 0u);
 }
@@ -3992,6 +3997,7 @@ __global__ void k_fg_cycle(DevFG *F, const double *rn2, cudaGraphConditionalHand
 // (the column from gs_step's scalars)
 __global__ void k_fg_givens(DevFG *F, const double *scal, int j, int m) {
     grid_begin();
+    if (!F->active) return;
     const double hn = sqrt(scal[S_TMP]);
     const bool again = scal[S_FLAG] != 0.0;
     F->outer += 1;
@@ -4025,6 +4031,7 @@ __global__ void k_fg_givens(DevFG *F, const double *scal, int j, int m) {
 // back substitution H y = g over the steps taken
 __global__ void k_fg_ysolve(DevFG *F, int m) {
     grid_begin();
+    if (!F->go) return;
     const int jl = F->jlast;
     if (F->status != 0 || jl < 0) {
         if (F->status == 0) F->status = IBM_ERR_NOT_CONVERGED;
@@ -4063,12 +4070,16 @@ __global__ void k_ref_start(DevFG *R, DevFG *F, const double *rn2, cudaGraphCond
         F->single = 1;
         F->status = 0;
         F->ncols = 0;
+    } else {
+        F->zero = 1;   // (no cycle)
     }
+    R->go = go;
     cudaGraphSetConditional(h, go ? 1u : 0u);
 }
 
 __global__ void k_ref_after(DevFG *R, const DevFG *F) {
     grid_begin();
+    if (!R->go) return;
     R->steps += F->outer;
     if (F->outer == 0) {
         R->status = IBM_ERR_NOT_CONVERGED;
@@ -4093,19 +4104,28 @@ static ibm_status norm2_dev(Ctx *c, const T *x, int slot) {
 }
 
 // one restart cycle of device-controlled FGMRES on control block F (the
-// cycle's residual r must be in K.r and F->scale = 1 / ||r||), then x update
+// cycle's residual r must be in K.r and F->scale = 1 / ||r||), then x update:
+// steps j < plain as plain nodes, the others each in an IF node, those from
+// the seventh on together in one more (passing an IF node by costs 6 us: ten
+// of them, for a cycle that takes four steps, as much as a step's work)
 template <typename T>
-static ibm_status fgmres_dev_cycle(Ctx *c, Krylov<T> K, T *x, DevFG *F) {
+static ibm_status fgmres_dev_cycle(Ctx *c, Krylov<T> K, T *x, DevFG *F, int plain) {
     const int64_t n = c->N;
     const int m = c->opts.restart;
     VPtrs<T> zp{};
     for (int i = 0; i < m; ++i) zp.p[i] = K.Z[i];
+    auto open = [&](CondScope *sc) -> ibm_status {
+        cudaGraphConditionalHandle h;
+        IBM_TRY(cond_handle(c, &h));
+        KL(-1, k_set_cond, 1, 1, h, &F->active);
+        return cond_open(c, cudaGraphCondTypeIf, h, sc);
+    };
+    const int rest = m > 8 ? 6 : m;
+    CondScope sr;
     for (int j = 0; j < m; ++j) {
-        cudaGraphConditionalHandle hj;
-        IBM_TRY(cond_handle(c, &hj));
-        KL(-1, k_set_cond, 1, 1, hj, &F->active);
         CondScope sj;
-        IBM_TRY(cond_open(c, cudaGraphCondTypeIf, hj, &sj));
+        if (j == rest) IBM_TRY(open(&sr));
+        if (j >= plain) IBM_TRY(open(&sj));
         {
             // V_j = (j == 0 ? r : w) / norm
             KL(-1, (k_scale_dev<T, T>), c->nred_wide, RED_THREADS, n, K.V[j], j == 0 ? K.r : K.w, &F->scale);
@@ -4113,15 +4133,30 @@ static ibm_status fgmres_dev_cycle(Ctx *c, Krylov<T> K, T *x, DevFG *F) {
             IBM_TRY(gs_step<T>(c, K, j));
             KL(-1, k_fg_givens, 1, 1, F, c->scal, j, m);
         }
-        IBM_TRY(cond_close(c, &sj));
+        if (j >= plain) IBM_TRY(cond_close(c, &sj));
     }
+    if (rest < m) IBM_TRY(cond_close(c, &sr));
     KL(-1, k_fg_ysolve, 1, 1, F, m);
     KL(-1, k_xupd_dev<T>, c->nred_wide, RED_THREADS, n, x, zp, F);
     IBM_LAUNCHED(c);
     return IBM_OK;
 }
 
-// FP64 FGMRES(m) with restarts, all on the device (control block 0)
+// Steps of a solve's first cycle that run as plain nodes, whether it still
+// needs them or not (what they compute is not used then). A conditional body
+// costs about 20 us to enter, an Arnoldi step 100 us or more: a step is plain
+// where nearly every solve takes it (256x128 with the first pass out of its
+// WHILE node and two of its four steps plain: 1.59 -> 1.53 ms a step; with the
+// later IF nodes of a cycle under one more 1.35). A cycle inside a conditional
+// body always takes its first step.
+static int plain_steps(const Ctx *c) {
+    const int p = c->N <= (int64_t)1 << 18 ? 2 : 1;
+    return p < c->opts.restart ? p : c->opts.restart;
+}
+
+// FP64 FGMRES(m) with restarts, all on the device (control block 0): the
+// first cycle as plain nodes (without effect where the guess is good enough),
+// further ones in the WHILE node
 static ibm_status fgmres64_dev(Ctx *c, double *x, DevFG *F) {
     Krylov<double> K = kry64(c);
     cudaGraphConditionalHandle hw;
@@ -4129,20 +4164,23 @@ static ibm_status fgmres64_dev(Ctx *c, double *x, DevFG *F) {
     IBM_TRY(apply_PA<double>(c, x, c->b, -1.0, K.r));
     IBM_TRY(norm2_dev<double>(c, K.r, S_TMP));
     KL(-1, k_fg_cycle, 1, 1, F, c->scal + S_TMP, hw);
-    CondScope sw;
-    IBM_TRY(cond_open(c, cudaGraphCondTypeWhile, hw, &sw));
-    {
-        IBM_TRY(fgmres_dev_cycle<double>(c, K, x, F));
+    auto cycle = [&](int plain) -> ibm_status {
+        IBM_TRY(fgmres_dev_cycle<double>(c, K, x, F, plain));
         IBM_TRY(apply_PA<double>(c, x, c->b, -1.0, K.r));
         IBM_TRY(norm2_dev<double>(c, K.r, S_TMP));
         KL(-1, k_fg_cycle, 1, 1, F, c->scal + S_TMP, hw);
-    }
+        return IBM_OK;
+    };
+    IBM_TRY(cycle(plain_steps(c)));
+    CondScope sw;
+    IBM_TRY(cond_open(c, cudaGraphCondTypeWhile, hw, &sw));
+    IBM_TRY(cycle(1));
     IBM_TRY(cond_close(c, &sw));
     return IBM_OK;
 }
 
 // FP64 defect correction around one FP32 FGMRES cycle per pass (control
-// blocks 0: refinement, 1: FP32 cycle)
+// blocks 0: refinement, 1: FP32 cycle); the first pass as plain nodes
 static ibm_status mixed_dev(Ctx *c, double *phi, DevFG *R, DevFG *F) {
     const int64_t n = c->N;
     Krylov<float> K = kry32(c);
@@ -4151,21 +4189,25 @@ static ibm_status mixed_dev(Ctx *c, double *phi, DevFG *R, DevFG *F) {
     IBM_TRY(apply_PA<double>(c, phi, c->b, -1.0, c->rr));
     IBM_TRY(norm2_dev<double>(c, c->rr, S_TMP));
     KL(-1, k_ref_start, 1, 1, R, F, c->scal + S_TMP, hr);
-    CondScope sr;
-    IBM_TRY(cond_open(c, cudaGraphCondTypeWhile, hr, &sr));
-    {
+    auto pass = [&](bool first) -> ibm_status {
         KL(-1, (k_scale_dev<float, double>), c->nred_wide, RED_THREADS, n, c->b32, c->rr, &R->scale);
         IBM_CUDA(c, cudaMemsetAsync(c->d32, 0, sizeof(float) * n, c->s));
         // the FP32 cycle: r32 = P(b32 - A d32), then one restart cycle if needed
-        cudaGraphConditionalHandle hi;
-        IBM_TRY(cond_handle(c, &hi));
+        // (the first pass's is unconditional: its decision, written to hr, is
+        // overwritten by the refinement test that follows)
+        cudaGraphConditionalHandle hi = hr;
+        if (!first) IBM_TRY(cond_handle(c, &hi));
         IBM_TRY(apply_PA<float>(c, c->d32, c->b32, -1.0f, K.r));
         IBM_TRY(norm2_dev<float>(c, K.r, S_TMP));
         KL(-1, k_fg_cycle, 1, 1, F, c->scal + S_TMP, hi);
-        CondScope si;
-        IBM_TRY(cond_open(c, cudaGraphCondTypeIf, hi, &si));
-        IBM_TRY(fgmres_dev_cycle<float>(c, K, c->d32, F));
-        IBM_TRY(cond_close(c, &si));
+        if (first) {
+            IBM_TRY(fgmres_dev_cycle<float>(c, K, c->d32, F, plain_steps(c)));
+        } else {
+            CondScope si;
+            IBM_TRY(cond_open(c, cudaGraphCondTypeIf, hi, &si));
+            IBM_TRY(fgmres_dev_cycle<float>(c, K, c->d32, F, 1));
+            IBM_TRY(cond_close(c, &si));
+        }
         KL(-1, k_fluid_volsum32, c->nred, RED_THREADS, c->g, op_of<float>(c), c->type, c->d32, c->part);
         IBM_TRY(finalize(c, c->part, c->nred, 1, 1.0 / c->fluid_vol, c->scal + S_MEAN));
         KL(-1, k_add_scaled_dev, c->nred_wide, RED_THREADS, n, c->type, phi, c->d32, R, c->scal + S_MEAN);
@@ -4173,7 +4215,12 @@ static ibm_status mixed_dev(Ctx *c, double *phi, DevFG *R, DevFG *F) {
         IBM_TRY(apply_PA<double>(c, phi, c->b, -1.0, c->rr));
         IBM_TRY(norm2_dev<double>(c, c->rr, S_TMP));
         KL(-1, k_ref_start, 1, 1, R, F, c->scal + S_TMP, hr);
-    }
+        return IBM_OK;
+    };
+    IBM_TRY(pass(true));
+    CondScope sr;
+    IBM_TRY(cond_open(c, cudaGraphCondTypeWhile, hr, &sr));
+    IBM_TRY(pass(false));
     IBM_TRY(cond_close(c, &sr));
     IBM_LAUNCHED(c);
     return IBM_OK;

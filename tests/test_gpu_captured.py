@@ -39,3 +39,26 @@ def test_captured_step_equals_host_driven(n, first):
         # operator's condition, below 1e4 on these grids
         scale = max(1.0, np.abs(a[k]).max())
         assert np.abs(a[k] - b[k]).max() <= 1e-9 * scale, k
+
+
+# the first cycle's plain steps: fewer and more steps than a solve needs, and
+# none (the guess passes the test at once)
+@pytest.mark.parametrize("precision", [ibm.IBM_FP64, ibm.IBM_MIXED])
+@pytest.mark.parametrize("rtol", [0.9, 1e-2, 1e-10])
+@pytest.mark.parametrize("restart", [2, 16])
+def test_first_cycle_takes_the_host_driven_steps(precision, rtol, restart):
+    case = synth.cylinder_case(96, 48, nseg=256, dt=0.02)
+    out = []
+    for graph in (0, 2):
+        s = ibm.Solver(case, precision=precision, stream=torch.cuda.Stream())
+        s.set_opts(precision=precision, rtol=rtol, restart=restart, graph=graph, max_outer=400)
+        s.set_body(case.verts, case.elems)
+        s.classify()
+        r = s.step(6)
+        assert r["status"] == ibm.IBM_OK, r
+        out.append((r["poisson_outer"], s.get("u"), s.get("p")))
+        s.close()
+    assert out[0][0] == out[1][0]
+    # (the rotations are formed on the host and on the device: rounding)
+    for a, b in zip(out[0][1:], out[1][1:]):
+        assert np.abs(a - b).max() <= 1e-9 * max(1.0, np.abs(a).max())
