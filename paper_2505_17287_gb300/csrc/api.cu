@@ -302,32 +302,11 @@ static ibm_status build_levels(Ctx *c) {
                 }
                 w32[i] = (float)w[i];
             }
-            int *dI = (int *)dev_alloc(c, sizeof(int) * nf), *dJ = (int *)dev_alloc(c, sizeof(int) * nf);
-            double *dw = (double *)dev_alloc(c, sizeof(double) * nf);
-            float *dw32 = (float *)dev_alloc(c, sizeof(float) * nf);
-            if (!dI || !dJ || !dw || !dw32) return c->fail(IBM_ERR_OOM, "transfer table allocation failed");
-            IBM_CUDA(c, cudaMemcpy(dI, I.data(), sizeof(int) * nf, cudaMemcpyHostToDevice));
-            IBM_CUDA(c, cudaMemcpy(dJ, J.data(), sizeof(int) * nf, cudaMemcpyHostToDevice));
-            IBM_CUDA(c, cudaMemcpy(dw, w.data(), sizeof(double) * nf, cudaMemcpyHostToDevice));
-            IBM_CUDA(c, cudaMemcpy(dw32, w32.data(), sizeof(float) * nf, cudaMemcpyHostToDevice));
-            c->tI[a][l] = dI;
-            c->tJ[a][l] = dJ;
-            c->tw64[a][l] = dw;
-            c->tw32[a][l] = dw32;
-            {
-                std::vector<double> v(nf);
-                std::vector<float> v32(nf);
-                for (int i = 0; i < nf; ++i) {
-                    v[i] = 1.0 - w[i];
-                    v32[i] = 1.0f - w32[i];
-                }
-                double *dv = (double *)dev_alloc(c, sizeof(double) * nf);
-                float *dv32 = (float *)dev_alloc(c, sizeof(float) * nf);
-                if (!dv || !dv32) return c->fail(IBM_ERR_OOM, "transfer table allocation failed");
-                IBM_CUDA(c, cudaMemcpy(dv, v.data(), sizeof(double) * nf, cudaMemcpyHostToDevice));
-                IBM_CUDA(c, cudaMemcpy(dv32, v32.data(), sizeof(float) * nf, cudaMemcpyHostToDevice));
-                c->tv64[a][l] = dv;
-                c->tv32[a][l] = dv32;
+            std::vector<double> v(nf);
+            std::vector<float> v32(nf);
+            for (int i = 0; i < nf; ++i) {
+                v[i] = 1.0 - w[i];
+                v32[i] = 1.0f - w32[i];
             }
             // transpose: the weight of fine i in coarse I[i] is w, in J[i] it
             // is 1 - w, rounded in each precision as the prolongation rounds it
@@ -347,8 +326,6 @@ static ibm_status build_levels(Ctx *c) {
                     gw32[q] = t == 0 ? w32[i] : 1.0f - w32[i];
                 }
             }
-            int *dgi = (int *)dev_alloc(c, sizeof(int) * 4 * nc);
-            double *dgw = (double *)dev_alloc(c, sizeof(double) * 4 * nc);
             // x halved: the same weights by the fine cell's position t in the
             // coarse cell's window 2I - 1 .. 2I + 2, at [t nc + I]
             const bool win = a == 0 && fac[a] == 2 && nf == 2 * nc;
@@ -361,15 +338,33 @@ static ibm_status build_levels(Ctx *c) {
                     gw32[(size_t)(4 + t) * nc + C2] = gw32[q];
                 }
             }
-            float *dgw32 = (float *)dev_alloc(c, sizeof(float) * gw32.size());
-            if (!dgi || !dgw || !dgw32) return c->fail(IBM_ERR_OOM, "transfer table allocation failed");
-            IBM_CUDA(c, cudaMemcpy(dgi, gi.data(), sizeof(int) * 4 * nc, cudaMemcpyHostToDevice));
-            IBM_CUDA(c, cudaMemcpy(dgw, gw.data(), sizeof(double) * 4 * nc, cudaMemcpyHostToDevice));
-            IBM_CUDA(c, cudaMemcpy(dgw32, gw32.data(), sizeof(float) * gw32.size(), cudaMemcpyHostToDevice));
-            c->gI[a][l] = dgi;
-            c->gw64[a][l] = dgw;
-            c->gw32[a][l] = dgw32;
-            if (a == 0) c->gwt32[l] = win ? dgw32 + (size_t)4 * nc : nullptr;
+            // the axis's tables in one allocation and one copy (nine of each
+            // took a fifth of a small grid's creation)
+            std::vector<unsigned char> pack;
+            auto put = [&](const void *src, size_t bytes) {
+                const size_t at = (pack.size() + 63) / 64 * 64;
+                pack.resize(at + bytes);
+                memcpy(pack.data() + at, src, bytes);
+                return at;
+            };
+            const size_t oI = put(I.data(), sizeof(int) * nf), oJ = put(J.data(), sizeof(int) * nf);
+            const size_t ow = put(w.data(), sizeof(double) * nf), ow32 = put(w32.data(), sizeof(float) * nf);
+            const size_t ov = put(v.data(), sizeof(double) * nf), ov32 = put(v32.data(), sizeof(float) * nf);
+            const size_t ogi = put(gi.data(), sizeof(int) * 4 * nc), ogw = put(gw.data(), sizeof(double) * 4 * nc);
+            const size_t ogw32 = put(gw32.data(), sizeof(float) * gw32.size());
+            unsigned char *d = (unsigned char *)dev_alloc(c, pack.size());
+            if (!d) return c->fail(IBM_ERR_OOM, "transfer table allocation failed");
+            IBM_CUDA(c, cudaMemcpy(d, pack.data(), pack.size(), cudaMemcpyHostToDevice));
+            c->tI[a][l] = (int *)(d + oI);
+            c->tJ[a][l] = (int *)(d + oJ);
+            c->tw64[a][l] = (double *)(d + ow);
+            c->tw32[a][l] = (float *)(d + ow32);
+            c->tv64[a][l] = (double *)(d + ov);
+            c->tv32[a][l] = (float *)(d + ov32);
+            c->gI[a][l] = (int *)(d + ogi);
+            c->gw64[a][l] = (double *)(d + ogw);
+            c->gw32[a][l] = (float *)(d + ogw32);
+            if (a == 0) c->gwt32[l] = win ? c->gw32[a][l] + (size_t)4 * nc : nullptr;
         }
     }
     return IBM_OK;
