@@ -46,8 +46,8 @@ UNIT = "Mcell-steps/s"
 # DRAM traffic per launch of the roofline kernel (dram__bytes_read.sum +
 # dram__bytes_write.sum of one launch, per cell), keyed by (kernel, precision);
 # valid for the kernel as captured (removed when the kernel changes). The split
-# colour pass: a one-pass capture at 201,326,592 cells, 906.7 MB read and
-# 377.1 MB written per launch.
+# colour pass: one-pass captures at 201,326,592 cells, 906.6 MB read and
+# 375-380 MB written per launch (linear quad order: 906.7 and 377.1).
 SPLIT_PASS = "k_rbgs_split (finest FP32 level in colour-split storage, one colour pass)"
 TRAFFIC_BYTES_PER_CELL = {(SPLIT_PASS, 4): (906.67e6 + 377.14e6) / 201326592}
 
