@@ -167,10 +167,15 @@ __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;
 // 152 SMs) are launched plainly and skip both: the two instructions cost each
 // block a few hundred cycles, 5-10% of a many-wave streaming pass whose blocks
 // live about 2 us (k_helm_rb at 25.2M cells: 159 us without, 177 with), while
-// such a pass hardly notices the launch gap.
+// such a pass hardly notices the launch gap (the finest FP32 colour pass, on a
+// 3D grid, not at all: 116 us at 62.9M cells with the two and without).
+// launch() applies the same rule to all three extents; it multiplies them in
+// 64 bits, so that a kernel it starts early always waits (32 bits here: 64
+// made k_apply_A<double> 2% slower; a product that wraps only adds a wait that
+// returns at once).
 constexpr unsigned OVERLAP_BLOCKS = 152 * 8;
 __device__ __forceinline__ void grid_begin() {
-    if (gridDim.x * gridDim.y <= OVERLAP_BLOCKS) {
+    if (gridDim.x * gridDim.y * gridDim.z <= OVERLAP_BLOCKS) {
         grid_release();
         grid_wait();
     }
