@@ -21,7 +21,10 @@
  *   - An admitted case keeps all its fields resident on the device from
  *     classification to its last step; only its results are copied back.
  *   - Device memory comes from a stream-ordered pool owned by the server, so
- *     creating and releasing cases never synchronises the whole device.
+ *     creating and releasing cases never synchronises the whole device. A
+ *     case takes one block of its estimated footprint for its whole time;
+ *     what does not fit in it comes from the pool beside it and is counted
+ *     against the budget while the case runs.
  *   - Every kernel of the library uses a fixed launch shape and fixed-order
  *     reductions, so a case gives the same bits alone and in a mix.
  *
@@ -79,7 +82,9 @@ typedef struct {
     double t_admit;
     double t_done;
     size_t bytes_estimate; /* footprint used for admission */
-    size_t bytes_peak;     /* device bytes the case actually held at most */
+    size_t bytes_peak;     /* device bytes the case held at most: the block of its
+                              estimated footprint, taken at its start and kept to its
+                              end, and what did not fit in it */
     ibm_step_stats step;   /* IBM_REQ_STEP */
     ibm_solve_stats solve; /* IBM_REQ_POISSON */
     int slot;              /* slot that ran it */
@@ -90,7 +95,8 @@ typedef struct {
     int64_t submitted, completed, failed, queued, running;
     int peak_running;      /* most cases resident at once */
     size_t budget;         /* byte budget in force */
-    size_t admitted_bytes; /* summed footprint of the running cases */
+    size_t admitted_bytes; /* summed footprint of the running cases (what one holds
+                              beyond its estimate included) */
     size_t peak_admitted_bytes;
 } ibm_server_stats;
 

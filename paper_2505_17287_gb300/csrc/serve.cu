@@ -11,8 +11,6 @@
 #include <chrono>
 #include <condition_variable>
 #include <deque>
-#include <iterator>
-#include <map>
 #include <mutex>
 #include <string>
 #include <thread>
@@ -21,6 +19,9 @@
 
 #include "../../include/ibm.h"
 #include "../../include/ibm_serve.h"
+#include "slab.h"
+
+struct ibm_server;
 
 namespace {
 
@@ -45,121 +46,21 @@ struct Req {
 
 struct Slot {
     int index = 0;
+    ibm_server *srv = nullptr;
     cudaStream_t s = nullptr;
     cudaMemPool_t pool = nullptr;
     std::thread th;
-    // device bytes the running case holds, through the allocator hooks
-    std::unordered_map<void *, size_t> sizes;
-    size_t cur = 0, peak = 0;
+    std::unordered_map<void *, size_t> sizes;   // live blocks of the running case
     bool oom = false;
     // the running case's slab: one pool block of its estimated footprint,
-    // held from its start to its end, and the free ranges in it (offset ->
-    // length, neighbours merged); reused: a range was given back since the
+    // held from its start to its end; reused: a block was given back since the
     // stream was last waited for
-    char *slab = nullptr;
-    std::map<size_t, size_t> ranges;
-    size_t slab_bytes = 0;
+    ibm::Slab slab;
     bool reused = false;
+    // device bytes the case holds (the slab and what went to the pool beside
+    // it), the most it held, and the bytes it is admitted with
+    size_t held = 0, peak = 0, admitted = 0;
 };
-
-constexpr size_t SLAB_ALIGN = 256;
-
-// A case makes a few hundred allocations, each of which cost a pool call and a
-// stream wait. So a case takes one block of its estimated footprint and the
-// hooks carve that; what does not fit goes to the pool. (Four sphere requests
-// of 58^3 to 96^3 cells at a time, two steps each: 33 ms a round before, 30 ms
-// now.)
-void slab_open(Slot *s, size_t bytes) {
-    void *p = nullptr;
-    s->ranges.clear();
-    s->slab = nullptr;
-    s->reused = false;
-    if (cudaMallocFromPoolAsync(&p, bytes, s->pool, s->s) != cudaSuccess) {
-        cudaGetLastError();
-        return;   // every allocation goes to the pool
-    }
-    if (cudaStreamSynchronize(s->s) != cudaSuccess) {
-        cudaGetLastError();
-        cudaFreeAsync(p, s->s);
-        return;
-    }
-    s->slab = (char *)p;
-    s->slab_bytes = bytes / SLAB_ALIGN * SLAB_ALIGN;
-    s->ranges[0] = s->slab_bytes;
-}
-
-void slab_close(Slot *s) {
-    if (s->slab) cudaFreeAsync(s->slab, s->s);
-    s->slab = nullptr;
-    s->ranges.clear();
-}
-
-// allocator hooks handed to ibm_create_grid: the first free range of the slab
-// that holds the block, else a pool allocation ordered on the slot stream; in
-// either case memory that earlier work on the stream may still use is waited
-// for, so that the library's synchronous copies may write it
-void *slot_alloc(size_t bytes, void *ctx) {
-    Slot *s = (Slot *)ctx;
-    void *p = nullptr;
-    const size_t need = (bytes + SLAB_ALIGN - 1) / SLAB_ALIGN * SLAB_ALIGN;
-    for (auto it = s->ranges.begin(); it != s->ranges.end(); ++it) {
-        if (it->second < need) continue;
-        const size_t off = it->first, len = it->second;
-        s->ranges.erase(it);
-        if (len > need) s->ranges[off + need] = len - need;
-        p = s->slab + off;
-        break;
-    }
-    if (!p) {
-        if (cudaMallocFromPoolAsync(&p, bytes, s->pool, s->s) != cudaSuccess) {
-            cudaGetLastError();
-            s->oom = true;
-            return nullptr;
-        }
-        s->reused = true;
-    }
-    if (s->reused) {
-        if (cudaStreamSynchronize(s->s) != cudaSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-        s->reused = false;
-    }
-    s->sizes[p] = bytes;
-    s->cur += bytes;
-    s->peak = std::max(s->peak, s->cur);
-    return p;
-}
-
-void slot_free(void *p, void *ctx) {
-    Slot *s = (Slot *)ctx;
-    size_t bytes = 0;
-    auto it = s->sizes.find(p);
-    if (it != s->sizes.end()) {
-        bytes = it->second;
-        s->cur -= bytes;
-        s->sizes.erase(it);
-    }
-    if (!s->slab || (char *)p < s->slab || (char *)p >= s->slab + s->slab_bytes) {
-        cudaFreeAsync(p, s->s);
-        return;
-    }
-    s->reused = true;
-    size_t off = (size_t)((char *)p - s->slab), len = (bytes + SLAB_ALIGN - 1) / SLAB_ALIGN * SLAB_ALIGN;
-    auto next = s->ranges.lower_bound(off);
-    if (next != s->ranges.end() && next->first == off + len) {
-        len += next->second;
-        next = s->ranges.erase(next);
-    }
-    if (next != s->ranges.begin()) {
-        auto prev = std::prev(next);
-        if (prev->first + prev->second == off) {
-            prev->second += len;
-            return;
-        }
-    }
-    s->ranges[off] = len;
-}
 
 }  // namespace
 
@@ -203,9 +104,95 @@ struct ibm_server {
 
     void worker(Slot *sl);
     void run(Req *q, Slot *sl);
+    // what a case holds beyond its estimate counts against the budget too,
+    // from here to its end
+    void held_more(Slot *sl);
 };
 
+void ibm_server::held_more(Slot *sl) {
+    sl->peak = std::max(sl->peak, sl->held);
+    if (sl->held <= sl->admitted) return;
+    std::lock_guard<std::mutex> lk(mu);
+    admitted += sl->held - sl->admitted;
+    sl->admitted = sl->held;
+    peak_admitted = std::max(peak_admitted, admitted);
+}
+
 namespace {
+
+// A case makes a few hundred allocations, each of which cost a pool call and a
+// stream wait. So a case takes one block of its estimated footprint and the
+// hooks carve that; what does not fit goes to the pool. (Four sphere requests
+// of 58^3 to 96^3 cells at a time, two steps each: 33 ms a round before, 30 ms
+// now.)
+void slab_open(Slot *s, size_t bytes) {
+    void *p = nullptr;
+    s->slab.open(nullptr, 0);
+    s->reused = false;
+    s->held = s->peak = 0;
+    if (cudaMallocFromPoolAsync(&p, bytes, s->pool, s->s) != cudaSuccess) {
+        cudaGetLastError();
+        return;   // every allocation goes to the pool
+    }
+    if (cudaStreamSynchronize(s->s) != cudaSuccess) {
+        cudaGetLastError();
+        cudaFreeAsync(p, s->s);
+        return;
+    }
+    s->slab.open(p, bytes);
+    s->held = bytes;
+    s->srv->held_more(s);
+}
+
+void slab_close(Slot *s) {
+    if (s->slab.base) cudaFreeAsync(s->slab.base, s->s);
+    s->slab.open(nullptr, 0);
+}
+
+// allocator hooks handed to ibm_create_grid: a block of the slab, else a pool
+// allocation ordered on the slot stream; in either case memory that earlier
+// work on the stream may still use is waited for, so that the library's
+// synchronous copies may write it
+void *slot_alloc(size_t bytes, void *ctx) {
+    Slot *s = (Slot *)ctx;
+    void *p = s->slab.take(bytes);
+    if (!p) {
+        if (cudaMallocFromPoolAsync(&p, bytes, s->pool, s->s) != cudaSuccess) {
+            cudaGetLastError();
+            s->oom = true;
+            return nullptr;
+        }
+        s->reused = true;
+        s->held += bytes;
+        s->srv->held_more(s);
+    }
+    s->sizes[p] = bytes;
+    if (s->reused) {
+        if (cudaStreamSynchronize(s->s) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        s->reused = false;
+    }
+    return p;
+}
+
+void slot_free(void *p, void *ctx) {
+    Slot *s = (Slot *)ctx;
+    size_t bytes = 0;
+    auto it = s->sizes.find(p);
+    if (it != s->sizes.end()) {
+        bytes = it->second;
+        s->sizes.erase(it);
+    }
+    if (s->slab.holds(p)) {
+        s->reused = true;
+        s->slab.give(p, bytes);
+    } else {
+        cudaFreeAsync(p, s->s);
+        s->held -= bytes;
+    }
+}
 
 void set_error(ibm_result &r, ibm_status st, const char *where, const char *msg) {
     r.status = st;
@@ -226,8 +213,8 @@ void ibm_server::run(Req *q, Slot *sl) {
     d.alloc = slot_alloc;
     d.free = slot_free;
     d.alloc_ctx = sl;
-    sl->cur = sl->peak = 0;
     sl->oom = false;
+    sl->admitted = q->est;
     slab_open(sl, q->est);
     ibm_ctx *ctx = nullptr;
     ibm_status st = ibm_create_grid(&d, &ctx);
@@ -333,7 +320,7 @@ void ibm_server::worker(Slot *sl) {
         run(q, sl);
         {
             std::lock_guard<std::mutex> lk(mu);
-            admitted -= q->est;
+            admitted -= sl->admitted;
             --running;
             q->res.t_done = now();
             q->done = true;
@@ -399,6 +386,7 @@ extern "C" ibm_status ibm_server_create(const ibm_server_opts *o, ibm_server **o
     for (int i = 0; i < o->max_slots; ++i) {
         Slot *sl = new Slot();
         sl->index = i;
+        sl->srv = s;
         sl->pool = s->pool;
         if (cudaStreamCreateWithFlags(&sl->s, cudaStreamNonBlocking) != cudaSuccess) {
             cudaGetLastError();
