@@ -336,7 +336,12 @@ void ibm_server::worker(Slot *sl) {
 // predictor and Poisson vectors, ghost-row scratch and the multigrid
 // hierarchy of the chosen precision (coarse levels add 1/7 in 3D, 1/3 in
 // 2D), the FGMRES(16) basis in the Krylov precision, and the transient
-// open-area arrays of the hierarchy build; plus the body and table storage.
+// open-area arrays of the hierarchy build; per ghost cell its tables (390 B)
+// and some four rows of the near-body band (128 B each); the body, the
+// reductions' partial sums and the images of the V-cycle bottom's blocks.
+// Ghost cells are taken as the bounding box's half surface, 1.6 times those
+// of the largest sphere in the box. The quarter and the constant on top are
+// margin: tests/test_gpu_serve_memory.py counts the allocations.
 extern "C" size_t ibm_case_bytes(int ndim, int nx, int ny, int nz, int precision, int64_t nelems_total) {
     const double n = (double)nx * ny * (ndim == 3 ? nz : 1);
     const double coarse = ndim == 3 ? 8.0 / 7.0 : 4.0 / 3.0;
@@ -347,8 +352,11 @@ extern "C" size_t ibm_case_bytes(int ndim, int nx, int ny, int nz, int precision
     else
         per_cell += 33 * 8 + 90 * coarse;       // FP64 basis and hierarchy
     per_cell += 8 + 16 * 8;                   // Poisson guess history, default 8 pairs
+    const double surface = ndim == 3 ? (double)nx * ny + (double)ny * nz + (double)nx * nz : (double)nx + ny;
+    const double ghosts = (390.0 + 4 * 128.0) * std::min(surface, n);
     const double body = 256.0 * (double)nelems_total;
-    return (size_t)(1.25 * (per_cell * n + body)) + ((size_t)64 << 20);
+    const double fixed = 8.0 * 40 * 152 * 32 + 16 * 226 * 1024.0;   // partial sums, block images
+    return (size_t)(1.25 * (per_cell * n + ghosts + body + fixed)) + ((size_t)56 << 20);
 }
 
 extern "C" ibm_status ibm_server_create(const ibm_server_opts *o, ibm_server **out) {
