@@ -63,7 +63,7 @@ __global__ void k_band_nbr(GridDev g, GhostDev gh, int nb, const int64_t *band, 
         if (band[mid] < n) lo = mid + 1;
         else hi = mid;
     }
-    nbr[(size_t)m * nb + t] = lo < nb && band[lo] == n ? lo : -1;
+    nbr[band_slot(nb, m, t)] = lo < nb && band[lo] == n ? lo : -1;
 }
 
 // one row of the band: v - (A z) and the damped inverse diagonal
@@ -73,7 +73,8 @@ struct BandRow {
     int idx[8];
     bool ghost;
 
-    // row of band cell q; zh[m nb + q] takes the values outside the band
+    // row of band cell q; zh[m nb + q] takes the values outside the band (their
+    // entries in idx serve the sweeps of one launch, whose bands are small)
     __device__ __forceinline__ void load(const GridDev &g, const GhostDev &gh, const OpT<T> &o, const BandDev &b,
                                          const uint8_t *type, const T *vv, const T *z, T omega, int q, T *zh) {
         const int64_t c = b.cell[q], gq = b.gpos[q];
@@ -82,7 +83,7 @@ struct BandRow {
         v = vv[c];
         dg = T(0);
 #pragma unroll
-        for (int m = 0; m < 8; ++m) idx[m] = b.nbr[(size_t)m * b.nb + q];
+        for (int m = 0; m < 8; ++m) idx[m] = b.nbr[band_slot(b.nb, m, q)];
         if (ghost) {
             // the ghost row solved for its value from the FLUID corners
             zc = v;
@@ -113,9 +114,9 @@ struct BandRow {
 #pragma unroll
         for (int m = 0; m < 8; ++m)
             if (idx[m] < 0) {
-                const int h = m * b.nb + q;
+                const size_t h = band_slot(b.nb, m, q);
                 zh[h] = z[n[m]];
-                idx[m] = -1 - h;
+                idx[m] = -1 - (int)h;
             }
     }
 
@@ -213,8 +214,9 @@ __global__ void k_band_sweep(GridDev g, GhostDev gh, OpT<T> o, BandDev b, const 
     const T zc = cur[q];
 #pragma unroll
     for (int m = 0; m < 8; ++m) {
-        const int n = b.nbr[(size_t)m * b.nb + q];
-        x[m] = n >= 0 ? cur[n] : zh[(size_t)m * b.nb + q];
+        const size_t h = band_slot(b.nb, m, q);
+        const int n = b.nbr[h];
+        x[m] = n >= 0 ? cur[n] : zh[h];
     }
     T s, wd;
     if (gq >= 0) {

@@ -181,6 +181,10 @@ __device__ __forceinline__ void grid_begin() {
     }
 }
 
+// entry of neighbour m of band row q in the band's neighbour-major arrays
+// (band.cuh; eight entries a row: past 32 bits from 2^28 rows)
+__host__ __device__ __forceinline__ size_t band_slot(int nb, int m, int q) { return (size_t)m * (size_t)nb + (size_t)q; }
+
 __device__ __forceinline__ double warp_sum(double v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     return v;
