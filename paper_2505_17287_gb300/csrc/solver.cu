@@ -4144,13 +4144,20 @@ static ibm_status fgmres_dev_cycle(Ctx *c, Krylov<T> K, T *x, DevFG *F, int plai
 
 // Steps of a solve's first cycle that run as plain nodes, whether it still
 // needs them or not (what they compute is not used then). A conditional body
-// costs about 20 us to enter, an Arnoldi step 100 us or more: a step is plain
-// where nearly every solve takes it (256x128 with the first pass out of its
-// WHILE node and two of its four steps plain: 1.59 -> 1.53 ms a step; with the
-// later IF nodes of a cycle under one more 1.35). A cycle inside a conditional
-// body always takes its first step.
+// costs about 20 us to enter, an Arnoldi step 60 us or more: a step is plain
+// where nearly every solve takes it, which the residual target decides. Steps
+// a solve takes in a long run (all 8 pairs of the guess history, 8K to 884K
+// cells, 2D and 3D, both precisions) and ms a step of the 720x360 cylinder in
+// FP64 with 2, 1 and 0 of them plain:
+//   rtol 1e-2, 1e-4:  0.5-0.9   0.956  0.745  0.704
+//   rtol 1e-6:        1.0-1.2   0.966  0.751  0.772
+//   rtol 1e-8:        2.0-3.0   1.056  1.063  1.082
+//   rtol 1e-10:       4.0-6.9   1.477  1.483  1.497
+// Above 2^18 cells a second one gains nothing (1024x512: 1.867 and 1.866). A
+// cycle inside a conditional body always takes its first step.
 static int plain_steps(const Ctx *c) {
-    const int p = c->N <= (int64_t)1 << 18 ? 2 : 1;
+    const int need = c->opts.rtol > 1e-5 ? 0 : (c->opts.rtol > 1e-7 ? 1 : 2);
+    const int p = std::min(need, c->N <= (int64_t)1 << 18 ? 2 : 1);
     return p < c->opts.restart ? p : c->opts.restart;
 }
 
