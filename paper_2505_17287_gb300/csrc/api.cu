@@ -221,7 +221,7 @@ static ibm_status build_levels(Ctx *c) {
     c->lg.clear();
     LevelGeom L0{c->nx, c->ny, c->nz, 1, 1, 1, c->hxf, c->hyf, c->hzf};
     c->lg.push_back(L0);
-    while ((int)c->lg.size() < 24) {
+    for (;;) {
         const LevelGeom &L = c->lg.back();
         const int64_t n = (int64_t)L.nx * L.ny * L.nz;
         // (64 cells: the coarsest solve is a small dense product. Stopping at
@@ -247,10 +247,6 @@ static ibm_status build_levels(Ctx *c) {
         C.yf = coarsen(L.yf, L.ny, C.fy, C.ny);
         C.zf = coarsen(L.zf, L.nz, C.fz, C.nz);
         c->lg.push_back(C);
-    }
-    {
-        const LevelGeom &L = c->lg.back();
-        if ((int64_t)L.nx * L.ny * L.nz > 512) return c->fail(IBM_ERR_ARG, "grid too anisotropic to coarsen to 512 cells");
     }
     for (auto &L : c->lg) {
         std::vector<double> cc, w, h;

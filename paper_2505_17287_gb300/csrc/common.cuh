@@ -144,9 +144,6 @@ struct Ctx;
 void *dev_alloc(Ctx *c, size_t bytes);
 void dev_free(Ctx *c, void *p);
 
-// reduction helper: block partials to one value (device function kernels in solver.cu)
-ibm_status reduce_sum(Ctx *c, const double *partials, int nparts, double *out_dev);
-
 }  // namespace ibm
 
 // ---------------------------------------------------------------------------

@@ -85,10 +85,6 @@ ibm_status finalize(Ctx *c, const double *part, int nparts, int ncols, double sc
     return IBM_OK;
 }
 
-ibm_status reduce_sum(Ctx *c, const double *partials, int nparts, double *out_dev) {
-    return finalize(c, partials, nparts, 1, 1.0, out_dev);
-}
-
 // the first n scalars into the pinned host mirror: a kernel writes them over
 // the coherent link (1-2 us behind the kernel before it, a copy engine's
 // transfer about 9). inv: also scal[S_INV] = 1 / sqrt(scal[S_TMP]) (0 where
@@ -1879,136 +1875,95 @@ __global__ void __launch_bounds__(256)
     *reinterpret_cast<float4 *>(xs1 + base) = make_float4(o1[0], o1[1], o1[2], o1[3]);
 }
 
-// coarsest level: red-black sweeps in one block, all data in shared memory.
+// coarsest level (at most COARSE_STOP cells): red-black sweeps in one block.
 // The level operator is singular (constants); the right-hand side is made
 // compatible by removing its mean over the active cells, and the solution is
 // returned with zero mean there, so no constant mode builds up in the
 // preconditioner (which would swamp FP32 corrections).
-constexpr int COARSE_MAX = 512;
 
-// Shared memory of the solve: x with zero padding of half the largest level
-// on either side (a neighbour offset is at most n / 2), and the partial sums.
-constexpr int COARSE_PAD = COARSE_MAX / 2;
+// mean over the active cells, one cell per thread of a block of COARSE_STOP:
+// the sums of its warps, added in order
 template <typename T>
-struct CoarseSmem {
-    T sx[COARSE_MAX + 2 * COARSE_PAD];
-    T red[COARSE_MAX / 32];
-    int cnt[COARSE_MAX / 32];
-};
-
-// mean over the active cells (thread c < COARSE_MAX holds cell c): sums of
-// the 16 warps, added in order
-template <typename T>
-__device__ __forceinline__ T block_mean_active(T v, bool act, CoarseSmem<T> &S) {
+__device__ __forceinline__ T block_mean_active(T v, bool act) {
+    __shared__ T red[COARSE_STOP / 32];
+    __shared__ int cnt[COARSE_STOP / 32];
     T a = act ? v : T(0);
     for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    const int cnt = __popc(__ballot_sync(0xffffffffu, act));
-    if (threadIdx.x < COARSE_MAX && (threadIdx.x & 31) == 0) {
-        S.red[threadIdx.x >> 5] = a;
-        S.cnt[threadIdx.x >> 5] = cnt;
+    const int n = __popc(__ballot_sync(0xffffffffu, act));
+    if ((threadIdx.x & 31) == 0) {
+        red[threadIdx.x >> 5] = a;
+        cnt[threadIdx.x >> 5] = n;
     }
     __syncthreads();
     T t = T(0);
     int m = 0;
 #pragma unroll
-    for (int w = 0; w < COARSE_MAX / 32; ++w) {
-        t += S.red[w];
-        m += S.cnt[w];
+    for (int w = 0; w < COARSE_STOP / 32; ++w) {
+        t += red[w];
+        m += cnt[w];
     }
     __syncthreads();
     return m > 0 ? t / T(m) : T(0);
 }
 
-// the coarsest-level solve by the threads of one block (at least COARSE_MAX).
-// Bound by the latency of one colour pass (4 sweeps of them, each waiting for
-// the last), in FP64 by the pipe: so a thread owns one cell of each colour
-// (no lane idles in a pass), keeps their coefficients in registers, reads its
-// six neighbours unconditionally (a closed or outer face has coefficient 0)
-// and only the warps that hold cells meet at the barrier. A 512-cell level
-// with 32 sweeps: 25 us before, with one thread per cell of either colour and
-// the coefficients in shared memory.
-template <typename T>
-__device__ void coarse_solve_dev(const MGLevel<T> &L, const T * f, T * x, int sweeps,
-                                 CoarseSmem<T> &S) {
-    const int n = (int)L.n, tid = threadIdx.x;
-    const int sy = L.nx, sz = L.nz > 1 ? L.nx * L.ny : 0;   // (at most n / 2: two cells or more per axis)
-    const bool act = tid < n && L.dinv[tid] > T(0);
-    for (int q = tid; q < COARSE_MAX + 2 * COARSE_PAD; q += blockDim.x) S.sx[q] = T(0);
-    const T fm = block_mean_active<T>(tid < n ? f[tid] : T(0), act, S);
-    const int nh = (L.nx + 1) >> 1, items = nh * L.ny * L.nz;   // at most 2 n / 3 (nx >= 2)
-    const int nthr = (items + 31) & ~31;
-    if (tid < nthr) {
-        int cc[2];
-        T k[2][6], di[2], ff[2];
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int row = tid / nh, j = row % L.ny, z = row / L.ny;
-            const int i = 2 * (tid - row * nh) + ((q + j + z) & 1);
-            const int c = row * L.nx + i;
-            const bool in = tid < items && i < L.nx;
-            cc[q] = in && L.dinv[c] > T(0) ? c : -1;
-            k[q][0] = in && i > 0 ? L.tx[c] : T(0);
-            k[q][1] = in && i < L.nx - 1 ? L.tx[c + 1] : T(0);
-            k[q][2] = in && j > 0 ? L.ty[c] : T(0);
-            k[q][3] = in && j < L.ny - 1 ? L.ty[c + sy] : T(0);
-            k[q][4] = in && z > 0 ? L.tz[c] : T(0);
-            k[q][5] = in && z < L.nz - 1 ? L.tz[c + sz] : T(0);
-            di[q] = cc[q] >= 0 ? L.dinv[c] : T(0);
-            ff[q] = cc[q] >= 0 ? f[c] - fm : T(0);
-        }
-        auto half = [&](int q) {
-            if (cc[q] >= 0) {
-                T *xc = S.sx + COARSE_PAD + cc[q];
-                T s = ff[q];
-                s += k[q][0] * xc[-1];
-                s += k[q][1] * xc[1];
-                s += k[q][2] * xc[-sy];
-                s += k[q][3] * xc[sy];
-                s += k[q][4] * xc[-sz];
-                s += k[q][5] * xc[sz];
-                *xc = s * di[q];
-            }
-            asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
-        };
-        // sweeps x (red, black) then sweeps x (black, red): a palindrome
-        for (int p = 0; p < sweeps; ++p) {
-            half(0);
-            half(1);
-        }
-        for (int p = 0; p < sweeps; ++p) {
-            half(1);
-            half(0);
-        }
-    }
-    __syncthreads();
-    const T xc = tid < n ? S.sx[COARSE_PAD + tid] : T(0);
-    const T xm = block_mean_active<T>(xc, act, S);
-    if (tid < n) x[tid] = act ? xc - xm : T(0);
-    __syncthreads();
-}
-
 // The sweeps are a linear operator of the right-hand side, fixed between two
-// classifications, so their matrix M (n x n) is formed once per hierarchy,
-// one block per column, and a cycle applies it: 128 dependent passes of about
-// 0.1 us each (FP64 0.4 us) become one small matrix-vector product.
+// classifications, so their matrix M (n x n) is formed once per hierarchy and a
+// cycle applies it: 128 dependent passes of about 0.1 us each (FP64 0.4 us)
+// become one small matrix-vector product. One block per column, whose
+// right-hand side is a unit vector; a thread holds one cell and reads its
+// neighbours unconditionally (a closed or outer face has coefficient 0, the
+// ends are padded with zeros).
 template <typename T>
-__global__ void __launch_bounds__(COARSE_MAX) k_coarse_matrix(MGLevel<T> L, int sweeps, T * M) {
+__global__ void __launch_bounds__(COARSE_STOP) k_coarse_matrix(MGLevel<T> L, int sweeps, T * M) {
     grid_begin();
-    __shared__ CoarseSmem<T> S;
-    __shared__ T e[COARSE_MAX], x[COARSE_MAX];
-    const int n = (int)L.n, col = blockIdx.x;
-    e[threadIdx.x] = (int)threadIdx.x == col ? T(1) : T(0);
+    constexpr int PAD = COARSE_STOP / 2;   // (a neighbour is at most n / 2 away: two cells or more per axis)
+    __shared__ T sx[COARSE_STOP + 2 * PAD];
+    const int n = (int)L.n, c = threadIdx.x, col = blockIdx.x;
+    const int sy = L.nx, sz = L.nz > 1 ? L.nx * L.ny : 0;
+    const bool in = c < n, act = in && L.dinv[c] > T(0);
+    const int row = c / L.nx, i = c - row * L.nx, z = row / L.ny, j = row - z * L.ny;
+    const T e = c == col ? T(1) : T(0);
+    const T f = e - block_mean_active<T>(e, act);
+    const T k0 = in && i > 0 ? L.tx[c] : T(0), k1 = in && i < L.nx - 1 ? L.tx[c + 1] : T(0);
+    const T k2 = in && j > 0 ? L.ty[c] : T(0), k3 = in && j < L.ny - 1 ? L.ty[c + sy] : T(0);
+    const T k4 = in && z > 0 ? L.tz[c] : T(0), k5 = in && z < L.nz - 1 ? L.tz[c + sz] : T(0);
+    const T di = act ? L.dinv[c] : T(0);
+    for (int q = c; q < COARSE_STOP + 2 * PAD; q += COARSE_STOP) sx[q] = T(0);
     __syncthreads();
-    coarse_solve_dev<T>(L, e, x, sweeps, S);
-    if ((int)threadIdx.x < n) M[(size_t)threadIdx.x * n + col] = x[threadIdx.x];
+    T *x = sx + PAD + c;
+    auto half = [&](int colour) {
+        if (act && ((i + j + z) & 1) == colour) {
+            T s = f;
+            s += k0 * x[-1];
+            s += k1 * x[1];
+            s += k2 * x[-sy];
+            s += k3 * x[sy];
+            s += k4 * x[-sz];
+            s += k5 * x[sz];
+            *x = s * di;
+        }
+        __syncthreads();
+    };
+    // sweeps x (red, black) then sweeps x (black, red): a palindrome
+    for (int p = 0; p < sweeps; ++p) {
+        half(0);
+        half(1);
+    }
+    for (int p = 0; p < sweeps; ++p) {
+        half(1);
+        half(0);
+    }
+    const T xm = block_mean_active<T>(*x, act);
+    if (in) M[(size_t)c * n + col] = act ? *x - xm : T(0);
 }
 
 }  // namespace ibm
 #include "vbottom.cuh"
 namespace ibm {
 
+constexpr int COARSE_THREADS = 512;   // a warp per row, 16 rows at a time
 template <typename T>
-__global__ void __launch_bounds__(COARSE_MAX) k_coarse_apply(int n, const T * M, const T * f,
+__global__ void __launch_bounds__(COARSE_THREADS) k_coarse_apply(int n, const T * M, const T * f,
                                                              T * x) {
     grid_begin();
     coarse_apply_dev<T>(n, M, f, x);
@@ -2670,7 +2625,7 @@ static ibm_status coarse_matrix(Ctx *c, MGHier<T> &H) {
     const MGLevel<T> &L = H.lv.back();
     if (!H.cm) H.cm = dev_alloc(c, sizeof(T) * (size_t)(L.n * L.n));
     if (!H.cm) return c->fail(IBM_ERR_OOM, "coarsest operator allocation failed");
-    KL(-1, k_coarse_matrix<T>, (unsigned)L.n, COARSE_MAX, L, c->opts.coarse_sweeps, (T *)H.cm);
+    KL(-1, k_coarse_matrix<T>, (unsigned)L.n, COARSE_STOP, L, c->opts.coarse_sweeps, (T *)H.cm);
     IBM_LAUNCHED(c);
     // the images of the V-cycle bottom's blocks (their layout is fixed by the grid)
     BotPar<T> P;
@@ -2983,7 +2938,7 @@ static int bottom_setup(Ctx *c, const MGHier<T> &H, BotPar<T> *out) {
         if (!fits) continue;
         P.nc = (int)H.lv[L - 1].n;
         P.cm = (const T *)H.cm;
-        P.ocm = P.nc <= COARSE_STOP ? take((int64_t)P.nc * P.nc) : -1;
+        P.ocm = take((int64_t)P.nc * P.nc);
         P.oint = (int)off;
         off = (off * (int64_t)sizeof(T) + ioff * (int64_t)sizeof(int) + 15) / 16 * 16;
         if (off > BOT_SMEM) continue;
@@ -3081,7 +3036,7 @@ static ibm_status vcycle(Ctx *c, MGHier<T> &H, const T *f0, T *x0, bool started 
     const int nuc2 = c->opts.nu_coarse > 0 ? c->opts.nu_coarse : nu2;
     const int bx = c->opts.tile_x;
     if (L == 1) {
-        KL(-1, k_coarse_apply<T>, 1, COARSE_MAX, (int)H.lv[0].n, (const T *)H.cm, f0, x0);
+        KL(-1, k_coarse_apply<T>, 1, COARSE_THREADS, (int)H.lv[0].n, (const T *)H.cm, f0, x0);
         IBM_LAUNCHED(c);
         return IBM_OK;
     }
@@ -3169,7 +3124,7 @@ static ibm_status vcycle(Ctx *c, MGHier<T> &H, const T *f0, T *x0, bool started 
     } else if (lb > 0) {
         IBM_TRY(launch_bottom<T>(c, bot));
     } else {
-        KL(-1, k_coarse_apply<T>, 1, COARSE_MAX, (int)H.lv[L - 1].n, (const T *)H.cm, H.lv[L - 1].f, H.lv[L - 1].x);
+        KL(-1, k_coarse_apply<T>, 1, COARSE_THREADS, (int)H.lv[L - 1].n, (const T *)H.cm, H.lv[L - 1].f, H.lv[L - 1].x);
         IBM_LAUNCHED(c);
     }
     for (int l = lt - 1; l >= 0; --l) {

@@ -324,8 +324,7 @@ __global__ void __launch_bounds__(BOT_THREADS) k_bottom_image(const __grid_const
         axis(v.ax[1], v.ny, c.ny, X.Gy, X.gwy, X.Iy, X.Jy, X.wy, X.vy);
         axis(v.ax[2], v.nz, c.nz, X.Gz, X.gwz, X.Iz, X.Jz, X.wz, X.vz);
     }
-    if (P.ocm >= 0)
-        for (int q = tid; q < P.nc * P.nc; q += BOT_THREADS) sm[P.ocm + q] = P.cm[q];
+    for (int q = tid; q < P.nc * P.nc; q += BOT_THREADS) sm[P.ocm + q] = P.cm[q];
 }
 
 template <typename T, bool OMEGA, bool D3>
@@ -429,7 +428,7 @@ __global__ void __launch_bounds__(BOT_THREADS, 1) k_vbottom(const __grid_constan
         __syncthreads();
     }
     if (r == 0) {
-        coarse_apply_dev<T>(P.nc, P.ocm >= 0 ? sm + P.ocm : P.cm, sm + P.ocf, sm + P.ocx);
+        coarse_apply_dev<T>(P.nc, sm + P.ocm, sm + P.ocf, sm + P.ocx);
         __syncthreads();
     }
     for (int l = lend - 1; l >= 0; --l) {
