@@ -69,7 +69,7 @@ __device__ __forceinline__ P pick3(int q, P a, P b, P c) { return q == 0 ? a : (
 // 2 (value - u_c) / width^2. The start values of the implicit solve, us = u,
 // are written on the way (on all cells), in place of a copy per component.
 // Bound by the FP64 pipe (two operations per clock and SM): 66 operations a
-// cell in 3D against 137 bytes. Each product is accumulated by an FMA of its
+// cell in 3D against 153 bytes. Each product is accumulated by an FMA of its
 // own (a difference of two products added afterwards took one operation more
 // per axis and component) and the walls' implicit share rides in off: 62.9M
 // cells 9.94 -> 8.77 ms, and three copies of 0.18 ms gone.
@@ -301,8 +301,8 @@ __global__ void k_helm_jacobi(GridDev g, HelmCoef h, const uint8_t * type, const
 }
 
 // residual of the Helmholtz system on FLUID rows; partial columns |r|^2, |rhs|^2
-// (the diagonal is formed again rather than divided out of hinv: an FP64
-// division costs several times the few adds)
+// (the diagonal comes from the stored sum of the face coefficients, not from
+// hinv: an FP64 division costs several times the multiply and add)
 // Bound by the FP64 pipe: 10 operations a cell; six
 // blocks an SM (40 registers, no spills), since with two waves of four
 // blocks the loads' latency showed (62.9M cells: 1.82 -> 1.46 ms, 71% of the

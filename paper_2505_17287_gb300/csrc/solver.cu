@@ -1555,7 +1555,9 @@ struct alignas(sizeof(T) * W) Pack {
 // access where nx allows it) up through a chunk of coarse planes and keeps
 // the last two fine planes summed along y, which the next coarse plane needs
 // again: 8 loads per W cells in place of 16 per cell. Bound by memory (tA
-// read once, f and x written); 62.9M -> 7.9M cells in FP32: see restrict_yz.
+// and the inverse diagonal read once, f and x written): 201M -> 25M cells in
+// FP32 129 us, 5.5 TB/s; all levels of a 62.9M-cell cycle 33 -> 15 us a launch
+// against one cell a thread.
 template <typename T, int W>
 __global__ void __launch_bounds__(256) k_restrict_yz(MGLevel<T> C, const T * tA, int fny, Xfer<T> X, QuadWalk w) {
     grid_begin();
@@ -1744,10 +1746,10 @@ __global__ void __launch_bounds__(RX_THREADS)
 // of k_resid_rx, and the restriction sums the window's positions in order
 // (table gwtx: 0 where a coarse cell has no such fine cell), so the result
 // equals k_resid_rx bit for bit.
-// Bound by memory (13 bytes a cell) once the L1 accesses are few: tables and
-// metrics are read as 16-byte runs over the four cells, where strided reads
-// of metrics, gather indices and window edges by each thread took 330 L1
-// passes a warp, three times the memory's time (62.9M cells: 366 -> 162 us).
+// Bound by memory (13 bytes a cell, 120 us at 62.9M) once the L1 accesses are
+// few: tables and metrics are read as 16-byte runs over the four cells, where
+// strided reads of metrics, gather indices and window edges by each thread
+// took three times the memory's time (62.9M cells: 366 -> 162 us).
 __global__ void __launch_bounds__(256, 3)
     k_resid_rx_split4(MGLevel<float> L, SplitLv<float> S, const float * fs0, const float * fs1,
                       const float * xs0, const float * xs1, const float * pn,
