@@ -94,9 +94,9 @@ typedef struct {
     int inner_iters;    /* Poisson: MG-PCG iterations per preconditioner call */
     int nu1, nu2;       /* multigrid pre/post red-black Gauss-Seidel sweeps, 1..8; equal
                            when inner_iters > 1 (CG needs a symmetric V-cycle) */
-    int coarse_sweeps;  /* red-black sweep pairs on the coarsest level (at most 64 cells
-                           where the grid coarsens that far; the sweeps are applied
-                           as one operator, formed once per classification) */
+    int coarse_sweeps;  /* red-black sweep pairs on the coarsest level (at most 64 cells;
+                           the sweeps are applied as one operator, formed once per
+                           classification) */
     double helm_rtol;   /* Crank-Nicolson Helmholtz: relative residual target */
     int helm_maxit;     /* Helmholtz: sweep limit */
     double ghost_tol;   /* velocity ghost refresh: max relative change */
